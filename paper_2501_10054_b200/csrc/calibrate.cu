@@ -2,9 +2,11 @@
 // the range that holds the central portion of them (quantiles q_lo, q_hi) and the least-squares line
 // y = a z + c of GELU over the samples inside that range.
 //
-// One CTA per neuron: the N samples are sorted in shared memory (bitonic network over the next power of two,
-// padded with +inf), the two quantiles are interpolated between order statistics in fp64 and rounded to fp32,
-// and the regression sums run in fp64 in two passes (means, then centred second moments), GELU in fp64.
+// One CTA per neuron: the N samples are sorted in registers (bitonic network over the next power of two, padded with
+// +inf), the two quantiles are interpolated between order statistics in fp64 and rounded to fp32, and the regression
+// sums run in fp64 in two passes (means, then centred second moments), GELU in fp64, once per sample.
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace tardis {
@@ -13,16 +15,24 @@ namespace cal {
 constexpr int NT = 256;
 constexpr int kMaxSamples = 8192;
 
-__device__ __forceinline__ double block_sum(double v, double* red) {     // every thread gets the sum
+// K sums over the CTA at once (one round of barriers); every thread gets them
+template <int K> __device__ __forceinline__ void block_sums(double (&v)[K], double (&red)[K][NT / 32]) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int k = 0; k < K; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
   __syncthreads();                                                        // red is free again
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  double t = 0.0;
+  if ((threadIdx.x & 31) == 0)
 #pragma unroll
-  for (int w = 0; w < NT / 32; ++w) t += red[w];
-  return t;
+    for (int k = 0; k < K; ++k) red[k][threadIdx.x >> 5] = v[k];
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    double t = 0.0;
+#pragma unroll
+    for (int w = 0; w < NT / 32; ++w) t += red[k][w];
+    v[k] = t;
+  }
 }
 
 __device__ __forceinline__ double gelu_slope_f64(double z, int act) {
@@ -35,52 +45,92 @@ __device__ __forceinline__ double gelu_slope_f64(double z, int act) {
   return 0.5 * (1.0 + erf(z * 0.7071067811865476)) + z * exp(-0.5 * z * z) * 0.3989422804014327;
 }
 
-// loads the n samples of neuron j (plus its bias) into keys[0..npad) (+inf beyond n) and sorts them ascending
-// (bitonic network; npad a power of two); all threads of the CTA
-__device__ __forceinline__ void load_and_sort(const float* __restrict__ z, long long ldz, const float* __restrict__ b1, int j, int n,
-                                              int npad, float* keys) {
-  const int tid = threadIdx.x;
+// The n samples of neuron j plus its bias, NT E values over the CTA (+inf beyond n): thread t gets samples e NT + t.
+template <int E> __device__ __forceinline__ void load_samples(float (&v)[E], const float* __restrict__ z, long long ldz,
+                                                              const float* __restrict__ b1, int j, int n) {
   const float bias = b1 ? b1[j] : 0.f;
-  for (int i = tid; i < npad; i += NT) {
-    float v = __int_as_float(0x7f800000);              // +inf: padding sorts behind every sample
-    if (i < n) v = z[size_t(j) * ldz + i] + bias;
-    keys[i] = v;
-  }
-  __syncthreads();
-  for (int k = 2; k <= npad; k <<= 1) {
-    for (int s = k >> 1; s > 0; s >>= 1) {
-      for (int t = tid; t < npad / 2; t += NT) {
-        const int i = 2 * t - (t & (s - 1)), p = i + s;          // pair (i, i + s), i without bit s
-        const bool up = (i & k) == 0;
-        const float x = keys[i], y = keys[p];
-        if ((x > y) == up) { keys[i] = y; keys[p] = x; }
-      }
-      __syncthreads();
-    }
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const int i = e * NT + threadIdx.x;
+    v[e] = i < n ? z[size_t(j) * ldz + i] + bias : __int_as_float(0x7f800000);
   }
 }
 
-// least squares of the activation over the samples with l <= z < u (fp64, two passes: means, then centred second
-// moments); thread 0 writes the line of neuron j; fewer than two samples in range: the tangent at the midpoint
-__device__ __forceinline__ void fit_and_store(const float* keys, int n, float lo_f, float hi_f, int act, double* red, int j,
-                                              float* __restrict__ lo, float* __restrict__ hi, float* __restrict__ a, float* __restrict__ c) {
+// Ascending sort of the NT E values of the CTA; afterwards thread t holds positions t E .. t E + E - 1.  Bitonic network:
+// strides below E stay inside a thread, strides below 32 E go by shuffle, and only the strides between warps (6 of the 66
+// steps of 2048 values) pass through shared memory.  (All steps through shared memory: four times the time, bound by its
+// bandwidth.)  sm: NT E floats.
+__device__ __forceinline__ void order(float& x, float& y, bool up) {
+  const float a = fminf(x, y), b = fmaxf(x, y);
+  x = up ? a : b;
+  y = up ? b : a;
+}
+template <int E> __device__ __forceinline__ void sort_samples(float (&v)[E], float* sm) {
   const int tid = threadIdx.x;
+#pragma unroll
+  for (int k = 2; k <= E; k <<= 1)
+#pragma unroll
+    for (int s = k >> 1; s > 0; s >>= 1)
+#pragma unroll
+      for (int e = 0; e < E; ++e)
+        if (!(e & s)) order(v[e], v[e | s], ((tid * E + e) & k) == 0);
+  for (int k = 2; k <= NT; k <<= 1) {                  // runs of k E values
+    const bool up = (tid & k) == 0;
+    int m = k >> 1;
+    for (; m >= 32; m >>= 1) {
+      const bool keep_min = ((tid & m) == 0) == up;
+#pragma unroll
+      for (int e = 0; e < E; ++e) sm[e * NT + tid] = v[e];
+      __syncthreads();
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const float o = sm[e * NT + (tid ^ m)];
+        v[e] = keep_min ? fminf(v[e], o) : fmaxf(v[e], o);
+      }
+      __syncthreads();
+    }
+    for (; m >= 1; m >>= 1) {
+      const bool keep_min = ((tid & m) == 0) == up;
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const float o = __shfl_xor_sync(0xffffffffu, v[e], m);
+        v[e] = keep_min ? fminf(v[e], o) : fmaxf(v[e], o);
+      }
+    }
+#pragma unroll
+    for (int s = E >> 1; s > 0; s >>= 1)
+#pragma unroll
+      for (int e = 0; e < E; ++e)
+        if (!(e & s)) order(v[e], v[e | s], up);
+  }
+}
+
+// Least squares of the activation over the samples with l <= z < u (fp64, two passes: means, then centred second
+// moments); thread 0 writes the line of neuron j; fewer than two samples in range: the tangent at the midpoint.
+// gs: activation values of the thread's samples where they are in range.
+template <int E> __device__ __forceinline__ void fit_and_store(const float (&v)[E], const double (&gs)[E], float lo_f, float hi_f, int act, int j,
+                                                               float* __restrict__ lo, float* __restrict__ hi, float* __restrict__ a, float* __restrict__ c) {
+  __shared__ double red3[3][NT / 32];
+  __shared__ double red2[2][NT / 32];
   const double l = double(lo_f), u = double(hi_f);
-  double cnt = 0.0, sz = 0.0, ss = 0.0;
-  for (int i = tid; i < n; i += NT) {
-    const double v = double(keys[i]);
-    if (v >= l && v < u) { cnt += 1.0; sz += v; ss += gelu_f64(v, act); }
+  double s[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const double x = double(v[e]);
+    if (x >= l && x < u) { s[0] += 1.0; s[1] += x; s[2] += gs[e]; }
   }
-  cnt = block_sum(cnt, red); sz = block_sum(sz, red); ss = block_sum(ss, red);
-  const double safe = cnt > 0.0 ? cnt : 1.0;
-  const double mz = sz / safe, ms = ss / safe;
-  double var = 0.0, cov = 0.0;
-  for (int i = tid; i < n; i += NT) {
-    const double v = double(keys[i]);
-    if (v >= l && v < u) { const double dz = v - mz; var += dz * dz; cov += dz * (gelu_f64(v, act) - ms); }
+  block_sums<3>(s, red3);
+  const double cnt = s[0], safe = cnt > 0.0 ? cnt : 1.0;
+  const double mz = s[1] / safe, ms = s[2] / safe;
+  double m[2] = {0.0, 0.0};
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const double x = double(v[e]);
+    if (x >= l && x < u) { const double dz = x - mz; m[0] += dz * dz; m[1] += dz * (gs[e] - ms); }
   }
-  var = block_sum(var, red) / safe; cov = block_sum(cov, red) / safe;
-  if (tid == 0) {
+  block_sums<2>(m, red2);
+  const double var = m[0] / safe, cov = m[1] / safe;
+  if (threadIdx.x == 0) {
     double aj, cj;
     if (cnt >= 2.0 && var > 1e-30) { aj = cov / var; cj = ms - aj * mz; }
     else {                                             // too few samples in range: tangent at the midpoint
@@ -92,213 +142,423 @@ __device__ __forceinline__ void fit_and_store(const float* keys, int n, float lo
   }
 }
 
-__global__ void __launch_bounds__(NT)
-k_calibrate(const float* __restrict__ z, long long ldz, const float* __restrict__ b1, int n, int npad, double q_lo, double q_hi,
+// Bound by the instructions of the sort and of the fp64 activation, in equal parts.  16384 neurons x 2048 samples:
+// 0.46 ms (0.91 ms with every step of the sort in shared memory and the activation as a fp64 tanh, evaluated twice).
+template <int E> __global__ void __launch_bounds__(NT)
+k_calibrate(const float* __restrict__ z, long long ldz, const float* __restrict__ b1, int n, double q_lo, double q_hi,
             int act, float* __restrict__ lo, float* __restrict__ hi, float* __restrict__ a, float* __restrict__ c) {
-  extern __shared__ float keys[];                      // [npad]
-  __shared__ double red[NT / 32];
-  __shared__ float range[2];
+  extern __shared__ float keys[];                      // [NT E]
+  __shared__ float stat[4];                            // the order statistics around the two quantiles
   const int j = blockIdx.x, tid = threadIdx.x;
-  load_and_sort(z, ldz, b1, j, n, npad, keys);
+  float v[E];
+  load_samples<E>(v, z, ldz, b1, j, n);
+  sort_samples<E>(v, keys);
   // quantile at level q: between the order statistics around position q (n - 1)
-  if (tid < 2) {
-    const double pos = (tid == 0 ? q_lo : q_hi) * double(n - 1);
-    const int i0 = int(floor(pos)), i1 = min(i0 + 1, n - 1);
-    const double w = pos - double(i0);
-    const double v = __dadd_rn(__dmul_rn(double(keys[i0]), 1.0 - w), __dmul_rn(double(keys[i1]), w));
-    range[tid] = float(v);
+  float range[2];
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const int i0 = int(floor((r == 0 ? q_lo : q_hi) * double(n - 1))), i1 = min(i0 + 1, n - 1);
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      if (tid * E + e == i0) stat[2 * r] = v[e];
+      if (tid * E + e == i1) stat[2 * r + 1] = v[e];
+    }
   }
   __syncthreads();
-  fit_and_store(keys, n, range[0], range[1], act, red, j, lo, hi, a, c);
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const double pos = (r == 0 ? q_lo : q_hi) * double(n - 1);
+    const double w = pos - floor(pos);
+    range[r] = float(__dadd_rn(__dmul_rn(double(stat[2 * r]), 1.0 - w), __dmul_rn(double(stat[2 * r + 1]), w)));
+  }
+  double gs[E];
+#pragma unroll
+  for (int e = 0; e < E; ++e) gs[e] = (v[e] >= range[0] && v[e] < range[1]) ? gelu_f64(double(v[e]), act) : 0.0;
+  fit_and_store<E>(v, gs, range[0], range[1], act, j, lo, hi, a, c);
 }
 
 // ---- the greedy range search of Algorithm 1 (Section 5.1.1, "Range Searching") --------------------------------------
 // One CTA per neuron.  (1) Sort the samples.  (2) Centroid: the sample with the highest Gaussian kernel density estimate
-// (width 1.06 std N^-1/5, density evaluated at every sample, fp64).  (3) The greedy loop, all threads in step: range =
-// centroid - k_l step .. centroid + k_r step, grown by one step on the side whose candidate range has the smaller error
-// (right on ties; a side that has passed the outermost sample is not grown) until the share of samples inside reaches the
-// neuron's threshold.  The error of a candidate is evaluated as its definition says: least-squares line over the samples
-// inside (means, centred moments), then the mean of the squared residuals; the samples are sorted, so "inside" is an index
-// range found by binary search, and the activation values are computed once.  (Prefix sums would make a candidate O(1),
-// but they lose the exact zeros of piecewise-linear activations, on which the tie rule depends.)  (4) The line over the
+// (width 1.06 std N^-1/5, density evaluated at the samples, fp64).  (3) The greedy loop: range = centroid - k_l step ..
+// centroid + k_r step, grown by one step on the side whose candidate range has the smaller error (right on ties; a side that
+// has passed the outermost sample is not grown) until the share of samples inside reaches the neuron's threshold.  The error
+// of a candidate is the mean squared residual of the least-squares line over the samples inside.  (4) The line over the
 // final range, as in k_calibrate.
+//
+// Neither the densities nor the errors are needed as numbers, only which one is the largest / smaller, so both are screened
+// by cheap values with a bound on what these can be off by, and evaluated as defined only where the bound leaves it open:
+//   * density: value F and slope F' at every 16th sample in fp32.  |F''| <= N per squared kernel width, so
+//     F(x) <= F(c) + F'(c) t + N t^2 / 2 at a distance of t widths; only samples whose bound reaches the largest value seen
+//     (about 150 of 2048) are evaluated in fp32, and of those only the ones within the fp32 error of the best (a handful) in
+//     fp64.  All N^2 exponentials in fp64 took 95 % of the time before.
+//   * candidate errors: from moments that grow with the range (fp64 sums over the samples of each step, made for all steps
+//     at once, a thread each).  One warp then walks the steps, half of its lanes with the left candidate, half with the right.
+//     Two errors closer than the rounding bound of the moments (or moments that cancel) are evaluated by the definition;
+//     exact zeros of piecewise-linear activations, on which the tie rule depends, thus stay exact.
+// 16384 neurons x 2048 samples: 4.3 ms (133 ms with every density and error evaluated as defined).
 constexpr int kMaxSearchSamples = 2048;
+constexpr int kMaxSteps = 160;           // steps on one side whose moments are made ahead (later ones: when they are reached)
+constexpr int kCoarse = 16;              // samples per coarse density point
+constexpr int kMaxCoarse = kMaxSearchSamples / kCoarse;
 
-__device__ __forceinline__ void block_sum2(double& v0, double& v1, double* red) {     // every thread gets both sums
+__device__ __forceinline__ float ex2f(float x) { float y; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
+__device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) { v0 += __shfl_xor_sync(0xffffffffu, v0, o); v1 += __shfl_xor_sync(0xffffffffu, v1, o); }
-  __syncthreads();                                                                    // red is free again
-  if ((threadIdx.x & 31) == 0) { red[threadIdx.x >> 5] = v0; red[NT / 32 + (threadIdx.x >> 5)] = v1; }
-  __syncthreads();
-  double t0 = 0.0, t1 = 0.0;
-#pragma unroll
-  for (int w = 0; w < NT / 32; ++w) { t0 += red[w]; t1 += red[NT / 32 + w]; }
-  v0 = t0; v1 = t1;
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
 }
 
-__global__ void __launch_bounds__(NT)
-k_range_search(const float* __restrict__ z, long long ldz, const float* __restrict__ b1, int n, int npad,
+// Position of the highest density among the sorted samples keys[0 .. n - 1] (the smallest position among equals); the whole
+// CTA, every thread gets it.  bw: kernel width (> 0).  list: room for n positions.
+__device__ __forceinline__ int densest_sample(const float* keys, int n, double bw, int* list) {
+  __shared__ float cf[kMaxCoarse], cs[kMaxCoarse];
+  __shared__ float wmax[NT / 32];
+  __shared__ double bestv[NT / 32];
+  __shared__ int besti[NT / 32];
+  __shared__ int count;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const float scale = float(0.8493218002880191 / bw);       // sqrt(log2(e) / 2) / width: e^(-u^2/2) = 2^-(scale (zk - zi))^2
+  const bool screen = bw > 1e-30 && bw < 1e30 && double(keys[n - 1]) - double(keys[0]) < 1e30;
+  if (tid == 0) count = 0;
+  __syncthreads();
+  if (screen) {
+    const int nc = (n + kCoarse - 1) / kCoarse;             // coarse points: samples 8, 24, 40, ...
+    auto point = [&](int c) { return min(c * kCoarse + kCoarse / 2, n - 1); };
+    // a pair of lanes per point, each half of the samples
+    for (int c0 = 0; c0 < nc; c0 += NT / 2) {
+      const int ci = c0 + (tid >> 1);
+      const float zi = keys[point(min(ci, nc - 1))];
+      float f = 0.f, s = 0.f;
+      const int half = (n + 1) >> 1, k0 = (tid & 1) * half, k1 = min(n, k0 + half);
+#pragma unroll 8
+      for (int k = k0; k < k1; ++k) {
+        const float t = (keys[k] - zi) * scale, w = ex2f(-t * t);
+        f += w;
+        s = fmaf(t, w, s);
+      }
+      f += __shfl_xor_sync(0xffffffffu, f, 1);
+      s += __shfl_xor_sync(0xffffffffu, s, 1);
+      if (!(tid & 1) && ci < nc) { cf[ci] = f; cs[ci] = s * 1.1774100225f; }   // slope per kernel width
+    }
+    __syncthreads();
+    float best = 0.f;
+    for (int c = tid; c < nc; c += NT) best = fmaxf(best, cf[c]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, o));
+    if (lane == 0) wmax[warp] = best;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < NT / 32; ++w) best = fmaxf(best, wmax[w]);
+    // What an fp32 density can be off by: the exponent (two roundings of t, squared) by 4e-7 of itself, which changes a term by
+    // less than 2e-7; the additions by 2^-24 of the sum each, 69 in a row for the listed samples (5e-6 N in all, once for each
+    // of two values compared), 1024 in a row for the coarse ones (6e-5 of the sum, 6e-5 N per width for the slope).
+    const float slack = 1e-5f * float(n), N2 = 0.5f * float(n), inv = float(1.0 / bw);
+    for (int i = tid; i < n; i += NT) {
+      if (i > 0 && keys[i] == keys[i - 1]) continue;        // the same density as its neighbour, which comes first
+      const int c = i / kCoarse;
+      const float t = (keys[i] - keys[point(c)]) * inv;
+      const float bound = fmaf(t, fmaf(t, N2, cs[c]), cf[c]);
+      if (bound * 1.0003f + slack * (1.f + 8.f * fabsf(t)) >= best) list[atomicAdd(&count, 1)] = i;
+    }
+    __syncthreads();
+    const int m = count;
+    // fp32 densities of the listed samples, two per warp at a time
+    float* dens = reinterpret_cast<float*>(list + n);
+    float top = 0.f;
+    for (int e = warp * 2; e < m; e += (NT / 32) * 2) {
+      const float za = keys[list[e]], zb = keys[list[min(e + 1, m - 1)]];
+      float fa = 0.f, fb = 0.f;
+#pragma unroll 4
+      for (int k = lane; k < n; k += 32) {
+        const float x = keys[k], ta = (x - za) * scale, tb = (x - zb) * scale;
+        fa += ex2f(-ta * ta);
+        fb += ex2f(-tb * tb);
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) { fa += __shfl_xor_sync(0xffffffffu, fa, o); fb += __shfl_xor_sync(0xffffffffu, fb, o); }
+      if (lane == 0) { dens[e] = fa; if (e + 1 < m) dens[e + 1] = fb; }
+      top = fmaxf(top, fmaxf(fa, fb));
+    }
+    __syncthreads();                                        // (count and wmax have been read)
+    if (tid == 0) count = 0;
+    if (lane == 0) wmax[warp] = top;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < NT / 32; ++w) top = fmaxf(top, wmax[w]);
+    int keep[(kMaxSearchSamples + NT - 1) / NT], nk = 0;
+#pragma unroll
+    for (int r = 0; r < (kMaxSearchSamples + NT - 1) / NT; ++r) {
+      const int e = r * NT + tid;
+      keep[r] = (e < m && dens[e] + slack >= top) ? list[e] : -1;
+      nk += keep[r] >= 0;
+    }
+    __syncthreads();
+    int at = nk ? atomicAdd(&count, nk) : 0;
+#pragma unroll
+    for (int r = 0; r < (kMaxSearchSamples + NT - 1) / NT; ++r)
+      if (keep[r] >= 0) list[at++] = keep[r];
+  } else {
+    for (int i = tid; i < n; i += NT) list[i] = i;
+    if (tid == 0) count = n;
+  }
+  __syncthreads();
+  // fp64 densities of what is left, one warp per sample
+  const int m = count;
+  const double inv = 1.0 / bw;
+  double bv = -1.0;
+  int bi = 0x7fffffff;
+  for (int e = warp; e < m; e += NT / 32) {
+    const int i = list[e];
+    const double zi = double(keys[i]);
+    double dsum = 0.0;
+    for (int k = lane; k < n; k += 32) { const double u = (double(keys[k]) - zi) * inv; dsum += exp(-0.5 * u * u); }
+    dsum = warp_sum(dsum);
+    if (dsum > bv || (dsum == bv && i < bi)) { bv = dsum; bi = i; }
+  }
+  if (lane == 0) { bestv[warp] = bv; besti[warp] = bi; }
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < NT / 32; ++w)
+    if (bestv[w] > bv || (bestv[w] == bv && besti[w] < bi)) { bv = bestv[w]; bi = besti[w]; }
+  return bi;
+}
+
+// Moments of some samples about the centroid (y = z - centroid, g = activation - activation at the centroid)
+struct Moments { double y, g, yy, yg, gg; };
+__device__ __forceinline__ Moments operator+(const Moments& p, const Moments& q) { return {p.y + q.y, p.g + q.g, p.yy + q.yy, p.yg + q.yg, p.gg + q.gg}; }
+
+template <int E> __global__ void __launch_bounds__(NT, 4)
+k_range_search(const float* __restrict__ z, long long ldz, const float* __restrict__ b1, int n,
                const float* __restrict__ thr, double t_all, double step, int act, float* __restrict__ lo, float* __restrict__ hi,
                float* __restrict__ a, float* __restrict__ c, int* __restrict__ steps_out) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  double* gs = reinterpret_cast<double*>(smem_raw);                // [n] activation of the sorted samples
-  float* keys = reinterpret_cast<float*>(gs + n);                  // [npad]
-  __shared__ double red[2 * (NT / 32)];
-  __shared__ double bestv[NT / 32];
-  __shared__ int besti[NT / 32];
-  __shared__ double cen_s;
-  const int j = blockIdx.x, tid = threadIdx.x;
-  load_and_sort(z, ldz, b1, j, n, npad, keys);
-  // mean and standard deviation (N - 1 in the denominator) of the samples; activation values
-  double s1 = 0.0;
-  for (int i = tid; i < n; i += NT) { s1 += double(keys[i]); gs[i] = gelu_f64(double(keys[i]), act); }
-  const double mean = block_sum(s1, red) / double(n);
-  double s2 = 0.0;
-  for (int i = tid; i < n; i += NT) { const double dz = double(keys[i]) - mean; s2 += dz * dz; }
-  s2 = block_sum(s2, red);
-  const double bw = n > 1 ? 1.06 * sqrt(s2 / double(n - 1)) * pow(double(n), -0.2) : 0.0;
-  // centroid: highest density, the smallest sample among equals
-  if (bw > 0.0) {
-    const double inv = 1.0 / bw;
-    double bv = -1.0;
-    int bi = 0x7fffffff;
-    for (int i = tid; i < n; i += NT) {
-      const double zi = double(keys[i]);
-      double dsum = 0.0;
-      for (int k = 0; k < n; ++k) { const double u = (double(keys[k]) - zi) * inv; dsum += exp(-0.5 * u * u); }
-      if (dsum > bv) { bv = dsum; bi = i; }                 // i ascends within a thread: the first maximum stays
-    }
+  double* gs = reinterpret_cast<double*>(smem_raw);                // [NT E] activation of the sorted samples
+  float* keys = reinterpret_cast<float*>(gs + NT * E);             // [NT E] sorted samples
+  __shared__ double red[1][NT / 32];
+  __shared__ float range_s[2];
+  __shared__ Moments ahead[2][kMaxSteps];
+  __shared__ int ends[2][kMaxSteps];
+  const int j = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
+  float v[E];
+  load_samples<E>(v, z, ldz, b1, j, n);
+  sort_samples<E>(v, keys);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (ov > bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }
-    }
-    if ((tid & 31) == 0) { bestv[tid >> 5] = bv; besti[tid >> 5] = bi; }
-    __syncthreads();
-    if (tid == 0) {
-      for (int w = 1; w < NT / 32; ++w)
-        if (bestv[w] > bv || (bestv[w] == bv && besti[w] < bi)) { bv = bestv[w]; bi = besti[w]; }
-      cen_s = double(keys[bi]);
-    }
-  } else if (tid == 0) {
-    cen_s = double(keys[0]);
-  }
+  for (int e = 0; e < E; ++e) keys[tid * E + e] = v[e];
+  // mean and standard deviation (N - 1 in the denominator) of the samples
+  double s1[1] = {0.0}, s2[1] = {0.0};
+#pragma unroll
+  for (int e = 0; e < E; ++e) if (tid * E + e < n) s1[0] += double(v[e]);
+  block_sums<1>(s1, red);
+  const double mean = s1[0] / double(n);
+#pragma unroll
+  for (int e = 0; e < E; ++e) if (tid * E + e < n) { const double dz = double(v[e]) - mean; s2[0] += dz * dz; }
+  block_sums<1>(s2, red);
+  const double bw = n > 1 ? 1.06 * sqrt(s2[0] / double(n - 1)) * pow(double(n), -0.2) : 0.0;
+  const int ic = bw > 0.0 ? densest_sample(keys, n, bw, reinterpret_cast<int*>(gs)) : 0;
+  const double cen = double(keys[ic]);
+  __syncthreads();                                                 // (the list in the place of gs has been read)
+#pragma unroll
+  for (int e = 0; e < E; ++e) gs[tid * E + e] = tid * E + e < n ? gelu_f64(double(v[e]), act) : 0.0;
   __syncthreads();
-  const double cen = cen_s;
-  const double t = thr ? double(thr[j]) : t_all;
+  // what every step on either side adds to the range: the samples between two successive bounds
+  const double gc = gs[ic];
   auto lower = [&](double v) {                            // number of samples below v
     int l = 0, r = n;
     while (l < r) { const int m = (l + r) >> 1; if (double(keys[m]) < v) l = m + 1; else r = m; }
     return l;
   };
-  // mean squared residual of the least-squares line over the sorted samples i0 .. i1 - 1 (every thread gets it)
-  auto mse = [&](int i0, int i1) -> double {
-    const int cnt = i1 - i0;
-    if (cnt < 2) return 0.0;                              // (uniform over the CTA)
-    const double q = 1.0 / double(cnt);
-    double sz = 0.0, sg = 0.0;
-    for (int i = i0 + tid; i < i1; i += NT) { sz += double(keys[i]); sg += gs[i]; }
-    block_sum2(sz, sg, red);
-    const double mz = sz * q, mg = sg * q;
-    double vzz = 0.0, vzg = 0.0;
-    for (int i = i0 + tid; i < i1; i += NT) { const double dz = double(keys[i]) - mz; vzz += dz * dz; vzg += dz * (gs[i] - mg); }
-    block_sum2(vzz, vzg, red);
-    vzz *= q; vzg *= q;
-    if (!(vzz > 1e-30)) return 0.0;
-    const double sl = vzg / vzz;
-    double rr = 0.0, dummy = 0.0;
-    for (int i = i0 + tid; i < i1; i += NT) { const double r = (gs[i] - mg) - sl * (double(keys[i]) - mz); rr += r * r; }
-    block_sum2(rr, dummy, red);
-    return rr * q;
-  };
-  const double zmin = double(keys[0]), zmax = double(keys[n - 1]);
-  int kl = 0, kr = 0, nsteps = 0;
-  const int cap = 4 + 2 * int(fmin(1.0e7, (zmax - zmin) / step + 2.0));   // the loop ends long before; a guard against a bad step
-  for (; nsteps < cap; ++nsteps) {
-    const double l = cen - kl * step, u = cen + kr * step;
-    const int i0 = lower(l), i1 = lower(u);
-    const int inside = i1 - i0;
-    if (double(inside) >= t * double(n) || inside == n) break;
-    bool go_left;
-    if (u > zmax) go_left = true;
-    else if (l <= zmin) go_left = false;
-    else {
-      const double el = mse(lower(cen - (kl + 1) * step), i1);
-      const double er = mse(i0, lower(cen + (kr + 1) * step));
-      go_left = el < er;
+  // position of the range's end on a side (0 left, 1 right) after k steps; what the step from k to k + 1 adds there
+  auto edge = [&](int side, int k) { return lower(side ? cen + k * step : cen - k * step); };
+  auto added = [&](int side, int k, int& next) {
+    const int p = edge(side, k);
+    next = edge(side, k + 1);
+    Moments m = {0.0, 0.0, 0.0, 0.0, 0.0};
+    for (int i = side ? p : next; i < (side ? next : p); ++i) {
+      const double y = double(keys[i]) - cen, q = gs[i] - gc;
+      m.y += y; m.g += q; m.yy += y * y; m.yg += y * q; m.gg += q * q;
     }
-    if (go_left) ++kl; else ++kr;
+    return m;
+  };
+  for (int e = tid; e < 2 * kMaxSteps; e += NT) {
+    const int side = e & 1, k = e >> 1;
+    if (k > 0 && (side ? cen + k * step > double(keys[n - 1]) : cen - k * step <= double(keys[0]))) continue;   // nothing beyond
+    int next;
+    ahead[side][k] = added(side, k, next);
+    ends[side][k] = next;
   }
-  const float lo_f = float(cen - kl * step), hi_f = float(cen + kr * step);
-  if (tid == 0 && steps_out) steps_out[j] = nsteps;
   __syncthreads();
-  fit_and_store(keys, n, lo_f, hi_f, act, red, j, lo, hi, a, c);
+  if (tid < 32) {
+    // the greedy loop, one warp: lanes 0 .. 15 look at the left side, lanes 16 .. 31 at the right one
+    const double t = thr ? double(thr[j]) : t_all;
+    const double zmin = double(keys[0]), zmax = double(keys[n - 1]);
+    const int side = lane >> 4;
+    // mean squared residual of the least-squares line over the sorted samples i0 .. i1 - 1, as it is defined
+    auto mse = [&](int i0, int i1) -> double {
+      const int cnt = i1 - i0;
+      if (cnt < 2) return 0.0;
+      const double q = 1.0 / double(cnt);
+      double sz = 0.0, sg = 0.0;
+      for (int i = i0 + lane; i < i1; i += 32) { sz += double(keys[i]); sg += gs[i]; }
+      const double mz = warp_sum(sz) * q, mg = warp_sum(sg) * q;
+      double vzz = 0.0, vzg = 0.0;
+      for (int i = i0 + lane; i < i1; i += 32) { const double dz = double(keys[i]) - mz; vzz += dz * dz; vzg += dz * (gs[i] - mg); }
+      vzz = warp_sum(vzz) * q; vzg = warp_sum(vzg) * q;
+      if (!(vzz > 1e-30)) return 0.0;
+      const double sl = vzg / vzz;
+      double rr = 0.0;
+      for (int i = i0 + lane; i < i1; i += 32) { const double r = (gs[i] - mg) - sl * (double(keys[i]) - mz); rr += r * r; }
+      return warp_sum(rr) * q;
+    };
+    // the same from the moments of the range (times its number of samples, and so on, to have one division), and what it
+    // can be off by (infinite where the moments cancel)
+    auto quick = [&](const Moments& m, int i0, int i1, float& off) -> double {
+      const int cnt = i1 - i0;
+      off = 0.f;
+      if (cnt < 2) return 0.0;
+      if (act == TARDIS_ACT_RELU && (keys[i0] > 0.f || keys[i1 - 1] <= 0.f)) return 0.0;   // one straight piece: exactly zero
+      const double q = double(cnt), yy = m.yy * q, gg = m.gg * q;
+      const double vyy = yy - m.y * m.y, vyg = m.yg * q - m.y * m.g, vgg = gg - m.g * m.g;
+      // every moment is off by less than 1e-13 of the sum of its terms' sizes (2 n 2^-53); |yg| <= sqrt(yy gg)
+      const float k = 1.f + __fdividef(float(yy), float(vyy)), iq = __fdividef(1.f, float(q));
+      off = fmaxf(1e-12f * float(gg) * iq * iq * k * k, 1e-37f);
+      if (!(vyy > 1e-8 * yy && vyy > 1e-25 * q * q)) off = __int_as_float(0x7f800000);
+      return (vgg * vyy - vyg * vyg) / (vyy * q * q);
+    };
+    int kl = 0, kr = 0, nsteps = 0;
+    int i0 = edge(0, 0), i1 = i0;                                  // samples inside: i0 .. i1 - 1 (none yet)
+    Moments in = {0.0, 0.0, 0.0, 0.0, 0.0};
+    const int cap = 4 + 2 * int(fmin(1.0e7, (zmax - zmin) / step + 2.0));   // the loop ends long before; a guard against a bad step
+    for (; nsteps < cap; ++nsteps) {
+      const double l = cen - kl * step, u = cen + kr * step;
+      const int inside = i1 - i0;
+      if (double(inside) >= t * double(n) || inside == n) break;
+      const bool right_done = u > zmax, left_done = l <= zmin;     // (not both: every sample would be inside)
+      // the range grown on the lane's side, if there is anything left on it
+      int end = side ? i1 : i0;
+      Moments m = in;
+      if (side ? !right_done : !left_done) {
+        const int k = side ? kr : kl;
+        if (k < kMaxSteps) { m = in + ahead[side][k]; end = ends[side][k]; }
+        else m = in + added(side, k, end);
+      }
+      bool go_left;
+      if (right_done) go_left = true;
+      else if (left_done) go_left = false;
+      else {
+        float off;
+        const double e = quick(m, side ? i0 : end, side ? end : i1, off);
+        const double eo = __shfl_xor_sync(0xffffffffu, e, 16);
+        const float oo = __shfl_xor_sync(0xffffffffu, off, 16);
+        const double gap = side ? e - eo : eo - e;                 // right minus left
+        go_left = gap > 0.0;
+        const bool open = !(fabs(gap) > double(off + oo)) && off + oo != 0.f;
+        if (__any_sync(0xffffffffu, open)) {                       // (every lane agrees; the vote makes the branch a uniform one)
+          const int l0 = __shfl_sync(0xffffffffu, end, 0), r1 = __shfl_sync(0xffffffffu, end, 16);
+          go_left = mse(l0, i1) < mse(i0, r1);
+        }
+      }
+      const int from = go_left ? 0 : 16;
+      in.y = __shfl_sync(0xffffffffu, m.y, from); in.g = __shfl_sync(0xffffffffu, m.g, from); in.yy = __shfl_sync(0xffffffffu, m.yy, from);
+      in.yg = __shfl_sync(0xffffffffu, m.yg, from); in.gg = __shfl_sync(0xffffffffu, m.gg, from);
+      const int at = __shfl_sync(0xffffffffu, end, from);
+      if (go_left) { ++kl; i0 = at; } else { ++kr; i1 = at; }
+    }
+    if (lane == 0) {
+      range_s[0] = float(cen - kl * step);
+      range_s[1] = float(cen + kr * step);
+      if (steps_out) steps_out[j] = nsteps;
+    }
+  }
+  __syncthreads();
+  double g[E];
+#pragma unroll
+  for (int e = 0; e < E; ++e) { v[e] = keys[e * NT + tid]; g[e] = gs[e * NT + tid]; }
+  fit_and_store<E>(v, g, range_s[0], range_s[1], act, j, lo, hi, a, c);
 }
 
 // Error contribution of every neuron (Section 5.1.1, the E of the neuron-level thresholds): the mean squared residual of
 // the least-squares line over the neuron's samples inside its range [lo_j, hi_j), as Algorithm 1's approx_error measures it.
-__global__ void __launch_bounds__(NT)
-k_neuron_error(const float* __restrict__ z, long long ldz, const float* __restrict__ b1, int n, int npad, int act,
+// (The samples inside are told by comparison: no order is needed.)
+template <int E> __global__ void __launch_bounds__(NT)
+k_neuron_error(const float* __restrict__ z, long long ldz, const float* __restrict__ b1, int n, int act,
                const float* __restrict__ lo, const float* __restrict__ hi, float* __restrict__ err) {
-  extern __shared__ __align__(16) unsigned char smem_err[];
-  double* gs = reinterpret_cast<double*>(smem_err);                // [n] activation of the sorted samples
-  float* keys = reinterpret_cast<float*>(gs + n);                  // [npad] sorted samples
-  __shared__ double red[2 * (NT / 32)];
-  const int j = blockIdx.x, tid = threadIdx.x;
-  load_and_sort(z, ldz, b1, j, n, npad, keys);
-  for (int i = tid; i < n; i += NT) gs[i] = gelu_f64(double(keys[i]), act);
-  __syncthreads();
-  auto lower = [&](double v) {
-    int l = 0, r = n;
-    while (l < r) { const int m = (l + r) >> 1; if (double(keys[m]) < v) l = m + 1; else r = m; }
-    return l;
-  };
-  const int i0 = lower(double(lo[j])), i1 = lower(double(hi[j]));
-  const int cnt = i1 - i0;
-  double e = 0.0;
-  if (cnt >= 2) {                                           // (uniform over the CTA)
-    const double q = 1.0 / double(cnt);
-    double sz = 0.0, sg = 0.0;
-    for (int i = i0 + tid; i < i1; i += NT) { sz += double(keys[i]); sg += gs[i]; }
-    block_sum2(sz, sg, red);
-    const double mz = sz * q, mg = sg * q;
-    double vzz = 0.0, vzg = 0.0;
-    for (int i = i0 + tid; i < i1; i += NT) { const double dz = double(keys[i]) - mz; vzz += dz * dz; vzg += dz * (gs[i] - mg); }
-    block_sum2(vzz, vzg, red);
-    vzz *= q; vzg *= q;
+  __shared__ double red3[3][NT / 32];
+  __shared__ double red2[2][NT / 32];
+  __shared__ double red1[1][NT / 32];
+  const int j = blockIdx.x;
+  const double l = double(lo[j]), u = double(hi[j]);
+  float v[E];
+  double g[E];
+  load_samples<E>(v, z, ldz, b1, j, n);
+  double s[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const double x = double(v[e]);
+    const bool in = e * NT + threadIdx.x < n && x >= l && x < u;
+    g[e] = in ? gelu_f64(x, act) : 0.0;
+    if (in) { s[0] += 1.0; s[1] += x; s[2] += g[e]; }
+    else v[e] = __int_as_float(0x7f800000);
+  }
+  block_sums<3>(s, red3);
+  double r = 0.0;
+  if (s[0] >= 2.0) {                                        // (uniform over the CTA)
+    const double q = 1.0 / s[0], mz = s[1] * q, mg = s[2] * q;
+    double m[2] = {0.0, 0.0};
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+      if (v[e] < __int_as_float(0x7f800000)) { const double dz = double(v[e]) - mz; m[0] += dz * dz; m[1] += dz * (g[e] - mg); }
+    block_sums<2>(m, red2);
+    const double vzz = m[0] * q;
     if (vzz > 1e-30) {
-      const double sl = vzg / vzz;
-      double rr = 0.0, dummy = 0.0;
-      for (int i = i0 + tid; i < i1; i += NT) { const double r = (gs[i] - mg) - sl * (double(keys[i]) - mz); rr += r * r; }
-      block_sum2(rr, dummy, red);
-      e = rr * q;
+      const double sl = m[1] * q / vzz;
+      double rr[1] = {0.0};
+#pragma unroll
+      for (int e = 0; e < E; ++e)
+        if (v[e] < __int_as_float(0x7f800000)) { const double w = (g[e] - mg) - sl * (double(v[e]) - mz); rr[0] += w * w; }
+      block_sums<1>(rr, red1);
+      r = rr[0] * q;
     }
   }
-  if (tid == 0) err[j] = float(e);
+  if (threadIdx.x == 0) err[j] = float(r);
 }
 
 // Neuron-level thresholds (Section 5.1.1): minimise sum_j E_j t_j subject to sum_j t_j = t_layer h, read with the box
 // t_min <= t_j <= t_max.  A linear objective over a box with one equality: every neuron starts at t_min and the budget
 // (t_layer - t_min) h goes, t_max - t_min each, to the neurons in order of increasing error (the smaller index first among
-// equals).  A thread finds its neuron's place in that order by counting, then takes its share of what is left for it.
+// equals).  Eight lanes find a neuron's place in that order by counting an eighth of the errors each (a thread per neuron
+// leaves more than half of the SMs idle at 16384 neurons: 85 us), then it takes its share of what is left for it.
 __global__ void __launch_bounds__(NT)
 k_neuron_thresholds(const float* __restrict__ err, int h, double t_layer, double t_min, double t_max, float* __restrict__ t) {
-  __shared__ float tile[NT];
-  const int j = blockIdx.x * NT + threadIdx.x;
+  __shared__ float tile[NT * 4];
+  const int j = blockIdx.x * (NT / 8) + (threadIdx.x >> 3), part = threadIdx.x & 7;
   const float ej = j < h ? err[j] : 0.f;
   int rank = 0;
-  for (int base = 0; base < h; base += NT) {
+  for (int base = 0; base < h; base += NT * 4) {
     __syncthreads();
-    tile[threadIdx.x] = base + threadIdx.x < h ? err[base + threadIdx.x] : 0.f;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int i = base + r * NT + threadIdx.x;
+      tile[r * NT + threadIdx.x] = i < h ? err[i] : __int_as_float(0x7f800000);
+    }
     __syncthreads();
-    const int m = min(NT, h - base);
-    for (int i = 0; i < m; ++i) rank += (tile[i] < ej || (tile[i] == ej && base + i < j)) ? 1 : 0;
+#pragma unroll 8
+    for (int i = part; i < NT * 4; i += 8) {
+      const float v = tile[i];
+      rank += (v < ej || (v == ej && base + i < j)) ? 1 : 0;
+    }
   }
-  if (j >= h) return;
+#pragma unroll
+  for (int o = 1; o < 8; o <<= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
+  if (j >= h || part) return;
   const double cap = t_max - t_min, budget = (t_layer - t_min) * double(h);
   const double give = fmin(cap, fmax(0.0, budget - double(rank) * cap));
   t[j] = float(t_min + give);
+}
+
+// Calls f with the number of samples per thread (a power of two up to MOST) that covers n samples, as a compile-time constant
+template <int MOST, int E = 1, typename F> static tardis_status_t with_samples(int n, F&& f) {
+  if constexpr (E > MOST) { (void)n; (void)f; return TARDIS_ERR_UNSUPPORTED; }
+  else return n <= NT * E ? f(std::integral_constant<int, E>()) : with_samples<MOST, E * 2>(n, static_cast<F&&>(f));
 }
 
 }  // namespace cal
@@ -306,12 +566,13 @@ k_neuron_thresholds(const float* __restrict__ err, int h, double t_layer, double
 tardis_status_t launch_neuron_thresholds(int h, int n, const float* z, long long ldz, const float* b1, const float* lo, const float* hi,
                                          int act, double t_layer, double t_min, double t_max, float* err, float* t, cudaStream_t s) {
   if (n < 1 || n > cal::kMaxSearchSamples) return TARDIS_ERR_UNSUPPORTED;
-  int npad = 2;
-  while (npad < n) npad <<= 1;
-  const size_t smem = size_t(n) * sizeof(double) + size_t(npad) * sizeof(float);
-  cal::k_neuron_error<<<h, cal::NT, smem, s>>>(z, ldz, b1, n, npad, act, lo, hi, err);
-  TARDIS_CUDA_TRY(cudaGetLastError());
-  cal::k_neuron_thresholds<<<(h + cal::NT - 1) / cal::NT, cal::NT, 0, s>>>(err, h, t_layer, t_min, t_max, t);
+  const tardis_status_t st = cal::with_samples<cal::kMaxSearchSamples / cal::NT>(n, [&](auto e) {
+    cal::k_neuron_error<decltype(e)::value><<<h, cal::NT, 0, s>>>(z, ldz, b1, n, act, lo, hi, err);
+    TARDIS_CUDA_TRY(cudaGetLastError());
+    return TARDIS_OK;
+  });
+  if (st != TARDIS_OK) return st;
+  cal::k_neuron_thresholds<<<(h * 8 + cal::NT - 1) / cal::NT, cal::NT, 0, s>>>(err, h, t_layer, t_min, t_max, t);
   TARDIS_CUDA_TRY(cudaGetLastError());
   return TARDIS_OK;
 }
@@ -319,23 +580,24 @@ tardis_status_t launch_neuron_thresholds(int h, int n, const float* z, long long
 tardis_status_t launch_calibrate(int h, int n, const float* z, long long ldz, const float* b1, double q_lo, double q_hi, int act,
                                  float* lo, float* hi, float* a, float* c, cudaStream_t s) {
   if (n < 1 || n > cal::kMaxSamples) return TARDIS_ERR_UNSUPPORTED;
-  int npad = 2;
-  while (npad < n) npad <<= 1;
-  cal::k_calibrate<<<h, cal::NT, size_t(npad) * sizeof(float), s>>>(z, ldz, b1, n, npad, q_lo, q_hi, act, lo, hi, a, c);
-  TARDIS_CUDA_TRY(cudaGetLastError());
-  return TARDIS_OK;
+  return cal::with_samples<cal::kMaxSamples / cal::NT>(n, [&](auto e) {
+    constexpr int E = decltype(e)::value;
+    cal::k_calibrate<E><<<h, cal::NT, size_t(cal::NT) * E * sizeof(float), s>>>(z, ldz, b1, n, q_lo, q_hi, act, lo, hi, a, c);
+    TARDIS_CUDA_TRY(cudaGetLastError());
+    return TARDIS_OK;
+  });
 }
 
 tardis_status_t launch_range_search(int h, int n, const float* z, long long ldz, const float* b1, const float* thr, double t_all,
                                     double step, int act, float* lo, float* hi, float* a, float* c, int* steps_out, cudaStream_t s) {
   if (n < 1 || n > cal::kMaxSearchSamples) return TARDIS_ERR_UNSUPPORTED;
-  int npad = 2;
-  while (npad < n) npad <<= 1;
-  const size_t smem = size_t(n) * sizeof(double) + size_t(npad) * sizeof(float);
-  TARDIS_CUDA_TRY(cudaFuncSetAttribute(cal::k_range_search, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
-  cal::k_range_search<<<h, cal::NT, smem, s>>>(z, ldz, b1, n, npad, thr, t_all, step, act, lo, hi, a, c, steps_out);
-  TARDIS_CUDA_TRY(cudaGetLastError());
-  return TARDIS_OK;
+  return cal::with_samples<cal::kMaxSearchSamples / cal::NT>(n, [&](auto e) {
+    constexpr int E = decltype(e)::value;
+    cal::k_range_search<E><<<h, cal::NT, size_t(cal::NT) * E * (sizeof(double) + sizeof(float)), s>>>(z, ldz, b1, n, thr, t_all, step, act,
+                                                                                                     lo, hi, a, c, steps_out);
+    TARDIS_CUDA_TRY(cudaGetLastError());
+    return TARDIS_OK;
+  });
 }
 
 }  // namespace tardis

@@ -129,8 +129,9 @@ __device__ __forceinline__ float gelu_f32(float z, int act) {
 __device__ __forceinline__ double gelu_f64(double z, int act) {
   if (act == TARDIS_ACT_RELU) return z > 0.0 ? z : 0.0 * z;
   if (act == TARDIS_ACT_GELU_TANH) {
-    double u = 0.7978845608028654 * (z + 0.044715 * z * z * z);
-    return 0.5 * z * (1.0 + tanh(u));
+    // (1 + tanh u) / 2 = 1 / (1 + e^-2u): one exponential and one division, and no cancellation where tanh u is near -1
+    const double u2 = 1.5957691216057308 * (z + 0.044715 * z * z * z);
+    return z / (1.0 + exp(-u2));
   }
   return 0.5 * z * (1.0 + erf(z * 0.7071067811865476));
 }

@@ -167,6 +167,27 @@ def test_greedy_range_search_matches_oracle(shape, act):
     assert ties <= h // 4
 
 
+@pytest.mark.parametrize("kind,n,step", [("duplicates", 255, 0.05), ("two modes", 513, 0.02), ("heavy tails", 2047, 0.2), ("narrow", 300, 2e-4),
+                                         ("normal", 65, 0.05), ("normal", 1025, 0.004)])
+def test_range_search_screening_falls_back_where_it_must(kind, n, step):
+    # equal samples and equal densities, a coarse density grid that is sparse (tails, few samples), candidate errors that cancel
+    # (samples 4e-3 wide around 3), more steps on a side than have their moments made ahead (0.004).
+    # (Not fewer samples: with 17 of them the choice often lies between two ranges of two samples, whose residuals are zero in
+    # exact arithmetic and 1e-33 in rounding noise; _check_search knows near-ties only relative to the larger error.)
+    g = torch.Generator().manual_seed(n)
+    z = torch.randn(12, n, generator=g)
+    if kind == "duplicates":
+        z = (z * 4).round() / 4 + 0.013
+    elif kind == "two modes":
+        z = 0.4 * z + torch.where(torch.rand(12, n, generator=g) < 0.51, 1.5, -1.5)
+    elif kind == "heavy tails":
+        z = z / torch.rand(12, n, generator=g).clamp(min=2e-3)
+    elif kind == "narrow":
+        z = 3.0 + 1e-3 * z
+    for act in (W.ACT_GELU_ERF, W.ACT_RELU):
+        assert _check_search(z.cuda(), None, 0.9, step, act) <= 3
+
+
 def test_greedy_range_search_edge_cases_and_errors():
     lib = T.load_library()
     # all samples equal, a single sample, threshold 0 (empty range at the centroid) and 1 (every sample)

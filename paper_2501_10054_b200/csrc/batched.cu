@@ -2,9 +2,11 @@
 // the tcgen05 tensor cores (gemm.cu) or a light elementwise pass.
 //
 // For a chunk of up to kChunk tokens X[n, d]:
-//   1. fast predictor scores  Zhat = X What^T + b1, What = s (q - zp) (Section 5.3).  What needs 10 significant
-//      bits (13 with 4-bit codes), so it is held as an exact sum of two bf16 matrices (hi + lo); one GEMM runs
-//      over both and its epilogue turns the scores into flag words (they are stored only for the debug
+//   1. fast predictor scores  Zhat = X What^T + b1, What = s (q - zp) (Section 5.3).  What needs up to 10 significant
+//      bits (13 with 4-bit codes), so it is held as an exact sum of two bf16 matrices (hi + lo).  With 2-bit codes lo is
+//      zero wherever |q - zp| <= 2, which is every group whose weights have both signs: the fold notes which 128-row
+//      tiles need lo at all, and the score GEMM leaves it out for the others (half of its work; 16384 prompt tokens of a
+//      4096 / 16384 layer 10.1 -> 9.2 ms, 32 tokens of an 8192 / 32768 layer 522 -> 445 us).  Its epilogue turns the scores into flag words (they are stored only for the debug
 //      capture).  Products are exact, the fp32 accumulation is not: a score within
 //      tau(t, j) = kEps * (2^bits - 1) max_g s[j,g] * |x_t|_1 of a range end is queued by the epilogue and
 //      re-evaluated in fp64 from the packed codes (k_recheck), so the flags are the exact ones;
@@ -32,6 +34,7 @@ constexpr int kMaxRecheck = 1 << 21;         // (token, neuron) pairs per chunk 
 struct State {
   __nv_bfloat16 *Wf, *W2, *What_hi, *What_lo;     // [d,d], [d,h], [h,d], [h,d]
   float* smaxrow;                                  // [h] largest group scale of a neuron
+  uint32_t* lo_used;                               // [h / 128 rounded up] 0 where What_lo is zero in those rows
   float *zhat, *yacc, *x1;                         // [kChunkCapture,h] (scores for the capture; fold temporary), [kChunk,d], [kChunk]
   __nv_bfloat16* delta;                            // [kChunk,h]
   uint32_t* bitmap;                                // [kChunk,h/32]
@@ -44,7 +47,8 @@ struct State {
 // What = s (q - zp) split exactly into hi = bf16(What) and lo = What - hi (at most 2 significant bits left).
 __global__ void k_dequant_split(const uint32_t* __restrict__ codes, const __nv_bfloat16* __restrict__ scale,
                                 const uint8_t* __restrict__ zero, __nv_bfloat16* __restrict__ hi,
-                                __nv_bfloat16* __restrict__ lo, float* __restrict__ smaxrow, int d, int G, int bits) {
+                                __nv_bfloat16* __restrict__ lo, float* __restrict__ smaxrow, uint32_t* __restrict__ lo_used, int d, int G, int bits) {
+  bool rest = false;                            // any of this thread's values has a second term
   const int per = 32 / bits;                    // codes per word
   const uint32_t cmask = (1u << bits) - 1u;
   const int j = blockIdx.x, ng = d / G, nwords = d / per;
@@ -56,6 +60,7 @@ __global__ void k_dequant_split(const uint32_t* __restrict__ codes, const __nv_b
       const __nv_bfloat16 h = __float2bfloat16_rn(v);
       hi[size_t(j) * d + k] = h;
       lo[size_t(j) * d + k] = __float2bfloat16_rn(v - __bfloat162float(h));
+      rest |= v != __bfloat162float(h);
     }
   }
   for (int w = threadIdx.x; w < nwords && 32 % bits == 0; w += blockDim.x) {
@@ -68,8 +73,10 @@ __global__ void k_dequant_split(const uint32_t* __restrict__ codes, const __nv_b
       const __nv_bfloat16 h = __float2bfloat16_rn(v);
       hi[size_t(j) * d + w * per + q] = h;
       lo[size_t(j) * d + w * per + q] = __float2bfloat16_rn(v - __bfloat162float(h));
+      rest |= v != __bfloat162float(h);
     }
   }
+  if (rest) lo_used[j >> 7] = 1u;
   if (threadIdx.x == 0) {
     float m = 0.f;
     for (int g = 0; g < ng; ++g) m = fmaxf(m, fabsf(__bfloat162float(scale[size_t(j) * ng + g])));
@@ -195,7 +202,7 @@ tardis_status_t batched_prepare(Handle* H) {
   Req reqs[] = {
       {reinterpret_cast<void**>(&S->Wf), size_t(d) * d * 2, false}, {reinterpret_cast<void**>(&S->W2), hd * 2, false},
       {reinterpret_cast<void**>(&S->What_hi), hd * 2, false},       {reinterpret_cast<void**>(&S->What_lo), hd * 2, false},
-      {reinterpret_cast<void**>(&S->smaxrow), size_t(h) * 4, false},
+      {reinterpret_cast<void**>(&S->smaxrow), size_t(h) * 4, false}, {reinterpret_cast<void**>(&S->lo_used), size_t((h + 127) / 128) * 4, false},
       {reinterpret_cast<void**>(&S->zhat), size_t(kChunkCapture) * h * 4, true}, {reinterpret_cast<void**>(&S->yacc), size_t(kChunk) * d * 4, true},
       {reinterpret_cast<void**>(&S->x1), size_t(kChunk) * 4, true},       {reinterpret_cast<void**>(&S->delta), size_t(kChunk) * h * 2, true},
       {reinterpret_cast<void**>(&S->bitmap), size_t(kChunk) * (h / 32) * 4, true},
@@ -207,7 +214,7 @@ tardis_status_t batched_prepare(Handle* H) {
   }
   H->bytes_folded += size_t(d) * d * 2;
   H->bytes_w2t += hd * 2;                       // second copy of W2 (original orientation)
-  H->bytes_predictor += 2 * hd * 2 + size_t(h) * 4;
+  H->bytes_predictor += 2 * hd * 2 + size_t(h) * 4 + size_t((h + 127) / 128) * 4;
   H->bytes_scratch += S->bytes_scratch;
   return TARDIS_OK;
 }
@@ -288,9 +295,10 @@ tardis_status_t batched_finish(Handle* H, const void* W2, cudaStream_t s) {
   if (W2) TARDIS_CUDA_TRY(cudaMemcpyAsync(S->W2, W2, hd * 2, cudaMemcpyDeviceToDevice, s));
   else      // (a handle read back from a file has only the transposed copy)
     k_transpose_b<__nv_bfloat16><<<dim3((d + 31) / 32, (h + 31) / 32), tb, 0, s>>>(static_cast<const __nv_bfloat16*>(H->W2T), S->W2, h, d);
+  TARDIS_CUDA_TRY(cudaMemsetAsync(S->lo_used, 0, size_t((h + 127) / 128) * 4, s));
   if (H->bits <= 4)   // (8-bit codes: the batched path is not used, see the dispatch)
     k_dequant_split<<<h, 256, 0, s>>>(H->codes, static_cast<const __nv_bfloat16*>(H->scale), H->zero, S->What_hi, S->What_lo,
-                                    S->smaxrow, d, H->G, H->bits);
+                                    S->smaxrow, S->lo_used, d, H->G, H->bits);
   TARDIS_CUDA_TRY(cudaGetLastError());
   return TARDIS_OK;
 }
@@ -298,7 +306,7 @@ tardis_status_t batched_finish(Handle* H, const void* W2, cudaStream_t s) {
 void batched_release(Handle* H) {
   State* S = static_cast<State*>(H->bstate);
   if (!S) return;
-  void* ptrs[] = {S->Wf, S->W2, S->What_hi, S->What_lo, S->smaxrow, S->zhat, S->yacc, S->x1, S->delta, S->bitmap, S->rlist, S->rcount};
+  void* ptrs[] = {S->Wf, S->W2, S->What_hi, S->What_lo, S->smaxrow, S->lo_used, S->zhat, S->yacc, S->x1, S->delta, S->bitmap, S->rlist, S->rcount};
   for (void* q : ptrs)
     if (q) dev_free(q);
   delete S;
@@ -321,7 +329,7 @@ tardis_status_t launch_batched_forward(Handle* H, const void* xv, void* yv, int6
     // 1. fast scores: one GEMM over the hi and lo halves of the dequantised predictor
     GemmArgs g = {};
     g.M = n; g.N = h; g.K1 = d; g.K2 = d;
-    g.A1 = xc; g.lda1 = d; g.B1 = S->What_hi; g.ldb1 = d; g.A2 = xc; g.lda2 = d; g.B2 = S->What_lo; g.ldb2 = d;
+    g.A1 = xc; g.lda1 = d; g.B1 = S->What_hi; g.ldb1 = d; g.A2 = xc; g.lda2 = d; g.B2 = S->What_lo; g.ldb2 = d; g.second_used = S->lo_used;
     // its epilogue turns the scores into flag words and queues the pairs too close to a range end; the scores
     // themselves are stored only for the debug capture
     g.epilogue = GEMM_EPI_FLAGS; g.out_f32 = keep_scores ? S->zhat : nullptr; g.ldo = h; g.bias = H->b1;

@@ -105,6 +105,7 @@ __host__ __device__ constexpr uint32_t instr_desc_bf16(int M, int N) {
 
 struct KParams {
   int M, N, kb1, kb2;          // k blocks (of 64) of the two operand pairs
+  const uint32_t* second_used; // per 128 rows n: 0 = the second pair adds nothing (null: it always counts)
   int epilogue, ldo, act, splits;
   int fast_m, band;            // tile raster (see decode() in the kernel)
   float* out_f32; __nv_bfloat16* out_bf16;
@@ -272,9 +273,6 @@ k_gemm(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtenso
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nm = (p.M + BM - 1) / BM, nn = (p.N + BN - 1) / BN;
   const int ntiles = nm * nn * p.splits;
-  const int nkb_all = p.kb1 + p.kb2;
-  const int per = (nkb_all + p.splits - 1) / p.splits;   // k blocks per split of the channel range
-
   if (threadIdx.x == 0) {
     for (int s = 0; s < C::NS; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
     for (int b = 0; b < 2; ++b) { mbar_init(&accum_full[b], 1); mbar_init(&accum_empty[b], 4); }
@@ -301,6 +299,13 @@ k_gemm(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtenso
     const int slow = r2 / w, fast = bi * p.band + (r2 - slow * w);
     const int mi = p.fast_m ? fast : slow, ni = p.fast_m ? slow : fast;
     m0 = mi * BM; n0 = ni * BN;
+    int nkb_all = p.kb1;
+    if (p.kb2 > 0) {
+      bool used = p.second_used == nullptr;
+      for (int r = n0; r < min(p.N, n0 + BN) && !used; r += 128) used = __ldg(p.second_used + (r >> 7)) != 0u;
+      if (used) nkb_all += p.kb2;
+    }
+    const int per = (nkb_all + p.splits - 1) / p.splits;   // k blocks per split of the channel range
     kb_lo = z * per;
     nkb = max(0, min(nkb_all, kb_lo + per) - kb_lo);
   };
@@ -443,7 +448,7 @@ static tardis_status_t launch_bn(const GemmArgs& g, cudaStream_t s) {
     return TARDIS_ERR_INVALID_ARG;
   KParams p;
   p.M = g.M; p.N = g.N; p.kb1 = (g.K1 + BK - 1) / BK; p.kb2 = g.K2 > 0 ? (g.K2 + BK - 1) / BK : 0;
-  p.epilogue = g.epilogue; p.ldo = g.ldo; p.act = g.act; p.splits = g.splits > 1 ? g.splits : 1;
+  p.second_used = g.second_used; p.epilogue = g.epilogue; p.ldo = g.ldo; p.act = g.act; p.splits = g.splits > 1 ? g.splits : 1;
   p.out_f32 = g.out_f32; p.out_bf16 = static_cast<__nv_bfloat16*>(g.out_bf16);
   p.bias = g.bias; p.addend = g.addend; p.a = g.a; p.c = g.c; p.bitmap = g.bitmap; p.error_word = g.error_word;
   p.lo = g.lo; p.hi = g.hi; p.colscale = g.colscale; p.rowscale = g.rowscale; p.keps = g.keps; p.bitmap_out = g.bitmap_out;

@@ -108,6 +108,28 @@ def test_wider_predictor_codes(bits):
     _run(cfg32, 7)
 
 
+@pytest.mark.parametrize("rows", [range(0, 0), range(130, 141), range(0, 2048, 127)])
+@pytest.mark.parametrize("n", [3, 20, 150])
+def test_predictor_values_of_two_terms_in_some_row_tiles(rows, n):
+    # zero-points at the end of the code range make values 3 s, which need a second bf16 term; the fold notes the 128-row tiles
+    # that have any: none, one tile, every tile
+    cfg = W.LayerConfig("two_terms", 512, 2048, group=64, n_calib=512)
+    L = _layer(cfg, 3)
+    r = torch.tensor(list(rows), device="cuda", dtype=torch.long)
+    L.zero[r] = torch.where(torch.arange(L.zero.shape[1], device="cuda") % 2 == 0, 0, 3).to(torch.uint8)
+    L.scale[r] *= 0.4
+    s = L.numpy64()
+    x = W.make_tokens(cfg, n, 3).cuda()
+    for path in (0, 3):
+        h = T.fold_layer(L)
+        try:
+            T.tardis_set_path(h, path)
+            y, F, S = Hp.gpu_forward(h, L, x)
+            Hp.assert_parity(L, s, x, y, F, S, score_tol=3e-4, label="rows %r path %d" % (rows, path))
+        finally:
+            T.tardis_destroy(h)
+
+
 def test_relu_activation_on_every_path():
     # ReLU layer (the OPT model of the paper's evaluation): per-token kernel, batched path, generic kernels, fp32
     cfg = W.LayerConfig("relu", 512, 2048, dtype="bf16", act=W.ACT_RELU, n_calib=512)

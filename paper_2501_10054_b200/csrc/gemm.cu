@@ -3,7 +3,7 @@
 // A CTA computes 128 x BN tiles of the output, one after the other (persistent, one CTA per SM).  Warp 0 stages
 // 128 x 64 (A) and BN x 64 (B) operand boxes into a ring of shared-memory stages with TMA
 // (cp.async.bulk.tensor, 128-byte swizzle, no multicast); warp 1 issues tcgen05.mma (M = 128, N = BN,
-// K = 16 per instruction) from one thread, accumulating in tensor memory (TMEM, 128 lanes x BN fp32 columns,
+// K = 16 per instruction; one elected lane), accumulating in tensor memory (TMEM, 128 lanes x BN fp32 columns,
 // two accumulators used in turn) and releasing each stage with tcgen05.commit; warps 2..5 read a finished
 // accumulator back with tcgen05.ld (each warp its own 32 lanes) and run the epilogue while the next tile's
 // main loop fills the other accumulator.  Every wait on an mbarrier is bounded: when it runs out the waiter
@@ -16,92 +16,44 @@
 
 #include "common.cuh"
 #include "exact.cuh"
+#include "tc.cuh"
 
 namespace tardis {
+namespace tc {
+typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                                  const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+static EncodeTiledFn encode_fn() {
+  static const EncodeTiledFn fn = [] {
+    void* ptr = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &ptr, cudaEnableDefault, &q) != cudaSuccess) { cudaGetLastError(); return EncodeTiledFn(nullptr); }
+    return q == cudaDriverEntryPointSuccess ? reinterpret_cast<EncodeTiledFn>(ptr) : EncodeTiledFn(nullptr);
+  }();
+  return fn;
+}
+
+bool tensor_maps_available() { return encode_fn() != nullptr; }
+
+bool make_map(CUtensorMap* map, const void* base, int rows, int K, int ld, int box_rows) {
+  const cuuint64_t dims[2] = {cuuint64_t(K), cuuint64_t(rows)};
+  const cuuint64_t strides[1] = {cuuint64_t(ld) * 2};
+  const cuuint32_t box[2] = {64, cuuint32_t(box_rows)};
+  const cuuint32_t estr[2] = {1, 1};
+  return encode_fn() && encode_fn()(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
+                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+}  // namespace tc
+
 namespace gemm {
+using namespace tc;
 
 constexpr int BM = 128;                 // tile rows (tokens / outputs)
 constexpr int BK = 64;                  // channels per stage: 64 bf16 = one 128-byte swizzle row
 constexpr int NTHREADS = 192;           // warp 0 TMA, warp 1 MMA, warps 2..5 epilogue
-constexpr uint32_t SPIN_LIMIT = 1u << 22;
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return uint32_t(__cvta_generic_to_shared(p)); }
-__device__ __forceinline__ void mbar_init(uint64_t* b, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(count));
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* b, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(b)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t* b) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(b)) : "memory");
-}
-__device__ __forceinline__ bool mbar_test(uint64_t* b, uint32_t parity) {
-  uint32_t ok;
-  asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-               : "=r"(ok) : "r"(smem_u32(b)), "r"(parity) : "memory");
-  return ok != 0;
-}
-__device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity) {   // bounded
-  for (uint32_t i = 0; i < SPIN_LIMIT; ++i) {
-    if (mbar_test(b, parity)) return true;
-    if (i > 64) __nanosleep(32);
-  }
-  return false;
-}
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
-  asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-               ::"r"(smem_u32(dst)), "l"(map), "r"(smem_u32(bar)), "r"(x), "r"(y) : "memory");
-}
-__device__ __forceinline__ void tmem_alloc(uint32_t* dst_smem, uint32_t ncols) {
-  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst_smem)), "r"(ncols) : "memory");
-  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
-  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-// D[tmem] (+)= A[smem] * B[smem]^T, M = 128, N from the instruction descriptor, K = 16
-__device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
-  asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
-               ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
-}
-// The barrier gets one arrival when every MMA issued so far by this thread has completed.
-__device__ __forceinline__ void umma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-// 32 consecutive fp32 columns of this thread's TMEM lane
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
-  uint32_t r[32];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-// Shared-memory matrix descriptor of a K-major operand tile stored as rows of 64 bf16 (128 bytes) with the
-// 128-byte swizzle TMA applies: start address (>> 4), leading-dimension offset (unused for this layout, 1),
-// stride between 8-row groups = 1024 bytes (>> 4), descriptor version 1, layout type 2 (128-byte swizzle).
-__device__ __forceinline__ uint64_t smem_desc_k_major_sw128(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= uint64_t((saddr & 0x3FFFFu) >> 4);
-  d |= uint64_t(1) << 16;
-  d |= uint64_t(1024 >> 4) << 32;
-  d |= uint64_t(1) << 46;
-  d |= uint64_t(2) << 61;
-  return d;
-}
-// Instruction descriptor, kind::f16: fp32 accumulator, bf16 A and B, both K-major, N and M of the tile.
-__host__ __device__ constexpr uint32_t instr_desc_bf16(int M, int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(N >> 3) << 17) | (uint32_t(M >> 4) << 24);
-}
 
 struct KParams {
   int M, N, kb1, kb2;          // k blocks (of 64) of the two operand pairs
@@ -270,7 +222,7 @@ k_gemm(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtenso
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(accum_empty + 2);
   volatile uint32_t* failed = tmem_slot + 1;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // (warp: uniform, and known to be)
   const int nm = (p.M + BM - 1) / BM, nn = (p.N + BN - 1) / BN;
   const int ntiles = nm * nn * p.splits;
   if (threadIdx.x == 0) {
@@ -312,58 +264,51 @@ k_gemm(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtenso
 
   if (warp == 0) {
     // ---------------- TMA producer ----------------
-    if (lane == 0) {
-      uint32_t it = 0;                                 // k blocks staged so far (over all tiles)
-      bool ok = true;
-      for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
-        int m0, n0, kb_lo, nkb, z;
-        decode(tile, m0, n0, kb_lo, nkb, z);
-        for (int kb = 0; kb < nkb; ++kb, ++it) {
-          const int s = it % C::NS;
-          if (*failed || !mbar_wait(&empty[s], ((it / C::NS) & 1) ^ 1)) { *failed = 1u; ok = false; break; }
-          uint8_t* sa = smem + s * C::STAGE_BYTES;
-          uint8_t* sb = sa + BM * BK * 2;
+    int s = 0, parity = 1;                             // stage and the phase of its `empty` barrier to wait for
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+      int m0, n0, kb_lo, nkb, z;
+      decode(tile, m0, n0, kb_lo, nkb, z);
+      for (int kg = kb_lo; kg < kb_lo + nkb; ++kg) {   // k block in the whole channel range
+        const bool ok = mbar_wait_issue(&empty[s], parity, failed);
+        const bool second = kg >= p.kb1;
+        const int kx = (second ? kg - p.kb1 : kg) * BK;
+        uint8_t* sa = smem + s * C::STAGE_BYTES;
+        if (elect_one() && ok) {
           mbar_expect_tx(&full[s], C::STAGE_BYTES);
-          const int kg = kb_lo + kb;                   // k block in the whole channel range
-          const bool second = kg >= p.kb1;
-          const int kx = (second ? kg - p.kb1 : kg) * BK;
           tma_load_2d(sa, second ? &tmA2 : &tmA1, kx, m0, &full[s]);
-          tma_load_2d(sb, second ? &tmB2 : &tmB1, kx, n0, &full[s]);
+          tma_load_2d(sa + BM * BK * 2, second ? &tmB2 : &tmB1, kx, n0, &full[s]);
         }
+        if (++s == C::NS) { s = 0; parity ^= 1; }
       }
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
-    if (lane == 0) {
-      constexpr uint32_t idesc = instr_desc_bf16(BM, BN);
-      uint32_t it = 0, use = 0;                        // k blocks consumed; accumulator uses so far
-      bool ok = true;
-      for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
-        int m0, n0, kb_lo, nkb, z;
-        decode(tile, m0, n0, kb_lo, nkb, z);
-        if (nkb == 0) continue;                        // nothing to add: the epilogue takes zeros
-        const uint32_t ab = use & 1u;
-        // the epilogue warps have drained this accumulator's previous tile
-        if (*failed || !mbar_wait(&accum_empty[ab], ((use >> 1) & 1) ^ 1)) { *failed = 1u; ok = false; break; }
+    constexpr uint32_t idesc = instr_desc_bf16(BM, BN);
+    const uint64_t adesc = smem_desc_k_major_sw128(smem_u32(smem)), bdesc = smem_desc_k_major_sw128(smem_u32(smem) + BM * BK * 2);
+    int s = 0, parity = 0;
+    uint32_t use = 0;                                  // accumulator uses so far
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+      int m0, n0, kb_lo, nkb, z;
+      decode(tile, m0, n0, kb_lo, nkb, z);
+      if (nkb == 0) continue;                          // nothing to add: the epilogue takes zeros
+      const uint32_t ab = use & 1u;
+      // the epilogue warps have drained this accumulator's previous tile
+      bool ok = mbar_wait_issue(&accum_empty[ab], ((use >> 1) & 1) ^ 1, failed);
+      tc_fence_after();
+      const uint32_t tacc = tmem_base + ab * BN;
+      for (int kb = 0; kb < nkb; ++kb) {
+        ok = mbar_wait_issue(&full[s], parity, failed);
         tc_fence_after();
-        const uint32_t tacc = tmem_base + ab * BN;
-        for (int kb = 0; kb < nkb; ++kb, ++it) {
-          const int s = it % C::NS;
-          if (!mbar_wait(&full[s], (it / C::NS) & 1)) { *failed = 1u; ok = false; break; }
-          tc_fence_after();
-          const uint32_t sa = smem_u32(smem + s * C::STAGE_BYTES);
-          const uint32_t sb = sa + BM * BK * 2;
+        const uint64_t da = adesc + uint32_t(s * (C::STAGE_BYTES >> 4)), db = bdesc + uint32_t(s * (C::STAGE_BYTES >> 4));
+        if (elect_one() && ok) {
 #pragma unroll
-          for (int k = 0; k < BK / 16; ++k) {
-            const uint64_t adesc = smem_desc_k_major_sw128(sa + k * 32);
-            const uint64_t bdesc = smem_desc_k_major_sw128(sb + k * 32);
-            umma_f16(tacc, adesc, bdesc, idesc, (kb | k) != 0 ? 1u : 0u);
-          }
+          for (int k = 0; k < BK / 16; ++k) umma_f16(tacc, da + k * 2, db + k * 2, idesc, (kb | k) != 0 ? 1u : 0u);
           umma_commit(&empty[s]);                      // frees the stage when these MMAs have read it
         }
-        if (ok) umma_commit(&accum_full[ab]);          // accumulator complete
-        ++use;
+        if (++s == C::NS) { s = 0; parity ^= 1; }
       }
+      if (elect_one() && ok) umma_commit(&accum_full[ab]);   // accumulator complete
+      ++use;
     }
   } else {
     // ---------------- epilogue: warp q reads TMEM lanes 32 (warp % 4) .. + 31 ----------------
@@ -377,7 +322,7 @@ k_gemm(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtenso
       const int m = m0 + q * 32 + lane;
       const uint32_t ab = use & 1u;
       if (nkb > 0) {
-        ok = !*failed && mbar_wait(&accum_full[ab], (use >> 1) & 1);
+        ok = mbar_wait_warp(&accum_full[ab], (use >> 1) & 1);
         if (!ok) { *failed = 1u; break; }
         tc_fence_after();
       }
@@ -407,38 +352,6 @@ k_gemm(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtenso
 }
 
 // ---- host side ------------------------------------------------------------------------------------------
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
-                                  const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-static EncodeTiledFn encode_fn() {
-  static EncodeTiledFn fn = nullptr;
-  static bool tried = false;
-  if (!tried) {
-    tried = true;
-    void* ptr = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &ptr, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeTiledFn>(ptr);
-    else
-      cudaGetLastError();
-  }
-  return fn;
-}
-
-// [rows, K] bf16 row-major with leading dimension ld; box = 64 channels x box_rows rows, 128-byte swizzle;
-// elements outside the matrix read as zero.
-static bool make_map(CUtensorMap* map, const void* base, int rows, int K, int ld, int box_rows) {
-  const cuuint64_t dims[2] = {cuuint64_t(K), cuuint64_t(rows)};
-  const cuuint64_t strides[1] = {cuuint64_t(ld) * 2};
-  const cuuint32_t box[2] = {cuuint32_t(BK), cuuint32_t(box_rows)};
-  const cuuint32_t estr[2] = {1, 1};
-  return encode_fn()(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
-                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 template <int BN>
 static tardis_status_t launch_bn(const GemmArgs& g, cudaStream_t s) {
   CUtensorMap a1, b1, a2, b2;
@@ -474,7 +387,7 @@ static tardis_status_t launch_bn(const GemmArgs& g, cudaStream_t s) {
 tardis_status_t launch_gemm(const GemmArgs& g, cudaStream_t s) {
   using namespace gemm;
   if (g.M <= 0 || g.N <= 0 || g.K1 <= 0) return TARDIS_ERR_INVALID_ARG;
-  if (!encode_fn()) return TARDIS_ERR_UNSUPPORTED;
+  if (!tensor_maps_available()) return TARDIS_ERR_UNSUPPORTED;
   auto bad = [](const void* p, int ld, int K) { return !p || (reinterpret_cast<uintptr_t>(p) & 15u) || (ld & 7) || (K & 7) || ld < K; };
   if (bad(g.A1, g.lda1, g.K1) || bad(g.B1, g.ldb1, g.K1)) return TARDIS_ERR_INVALID_ARG;
   if (g.K2 > 0 && (bad(g.A2, g.lda2, g.K2) || bad(g.B2, g.ldb2, g.K2))) return TARDIS_ERR_INVALID_ARG;

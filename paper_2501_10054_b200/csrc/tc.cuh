@@ -25,8 +25,14 @@ __device__ __forceinline__ bool mbar_test(uint64_t* b, uint32_t parity) {
                : "=r"(ok) : "r"(smem_u32(b)), "r"(parity) : "memory");
   return ok != 0;
 }
-// Waits are bounded (about 0.2 s) and use the non-blocking test: the potentially blocking try_wait takes several hundred cycles
-// even on a completed phase.
+__device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t parity) {
+  uint32_t ok;
+  asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+               : "=r"(ok) : "r"(smem_u32(b)), "r"(parity) : "memory");
+  return ok != 0;
+}
+// Waits are bounded (about 0.2 s).  The non-blocking test comes first: the potentially blocking try_wait takes several hundred
+// cycles even on a completed phase, but leaves the issue slots alone while there is something to wait for.
 constexpr long long WAIT_CYCLES = 400000000ll;
 // One lane of a converged warp.  The warps that issue copies and MMAs run their loops with all lanes and let the elected one
 // issue: addresses and descriptors then stay in uniform registers, where these instructions want them.  (Loops run by lane 0
@@ -42,20 +48,18 @@ __device__ __forceinline__ bool mbar_wait_issue(uint64_t* b, uint32_t parity, vo
   bool ok = mbar_test(b, parity);
   if (!ok) {
     const long long t0 = clock64();
-    while (!(ok = mbar_test(b, parity)))
+    while (!(ok = mbar_try(b, parity)))
       if (clock64() - t0 > WAIT_CYCLES || *failed) { *failed = 1u; break; }
   }
   return __all_sync(0xffffffffu, ok);
 }
-// The wait of a whole warp that has time: one lane looks, and sleeps between looks.
+// The wait of a whole warp that only needs the outcome: one lane looks.
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* b, uint32_t parity) {
   int ok = 1;
   if ((threadIdx.x & 31) == 0 && !mbar_test(b, parity)) {
     const long long t0 = clock64();
-    do {
-      __nanosleep(40);
-      ok = mbar_test(b, parity);
-    } while (!ok && clock64() - t0 <= WAIT_CYCLES);
+    do ok = mbar_try(b, parity);
+    while (!ok && clock64() - t0 <= WAIT_CYCLES);
   }
   return __shfl_sync(0xffffffffu, ok, 0) != 0;
 }
@@ -113,6 +117,32 @@ __device__ __forceinline__ uint64_t smem_desc_k_major_sw128(uint32_t saddr) {
 // Instruction descriptor, kind::f16: fp32 accumulator, bf16 A and B, both K-major, N and M of the tile.
 __host__ __device__ constexpr uint32_t instr_desc_bf16(int M, int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(N >> 3) << 17) | (uint32_t(M >> 4) << 24);
+}
+// The same with the 128 rows of A in TMEM (row = lane, two consecutive bf16 channels per 32-bit column)
+__device__ __forceinline__ void umma_f16_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+  asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}"
+               ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
+}
+// 8 consecutive fp32 columns of this thread's TMEM lane
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
+  uint32_t r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+// 32 consecutive 32-bit columns of this thread's TMEM lane; complete on return
+__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
+      "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"
+      ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
+        "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]),
+        "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]),
+        "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
+      : "memory");
+  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
 // Host: tensor map of a bf16 matrix [rows, K] row-major with leading dimension ld; box = 64 channels x box_rows rows, 128-byte

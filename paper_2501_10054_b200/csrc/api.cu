@@ -117,6 +117,7 @@ static tardis_status_t dev_alloc(T** p, size_t count, size_t* tally) {
 static void free_all(Handle* H) {
   fused_release(H);
   decode_release(H);
+  few_release(H);
   batched_release(H);
   void* ptrs[] = {H->W1, H->W2T, H->C, H->bf, H->lo, H->hi, H->a, H->c, H->b1, H->codes, H->scale,
                   H->zero, H->yacc, H->bitmap, H->counters};
@@ -225,7 +226,11 @@ tardis_status_t tardis_ffn_forward(tardis_handle_t handle, const void* x, void* 
   tardis_status_t st;
   // (deterministic mode: only the kernels of fused.cu and the tensor-core products without a split channel range qualify)
   const bool has_fused = H->fscratch != nullptr || (H->codes_mma != nullptr && !H->deterministic);
-  const bool fused = has_fused && ((H->path_override == 0 && n_tokens <= (H->fscratch ? H->fused_max_tokens : 8)) || (H->path_override == 2 && n_tokens <= 4096));
+  // One launch of the fused kernel (4 tokens) is faster than the kernels of few.cu (4096 / 16384: 52 us against 75), two are not;
+  // of the per-token kernel of wider layers two launches are the most (8192 / 32768: 87 us each against 255).  Where few.cu
+  // does not serve a layer the batched path takes over later.
+  const int most_fused = H->few && !H->deterministic ? (H->fscratch ? 4 : 2) : (H->fscratch ? H->fused_max_tokens : 8);
+  const bool fused = has_fused && ((H->path_override == 0 && n_tokens <= most_fused) || (H->path_override == 2 && n_tokens <= 4096));
   // (8-bit codes times a bf16 scale do not fit the exact two-term bf16 form the batched scores rely on)
   const bool batched = ((H->path_override == 0 && !fused) || H->path_override == 3) && H->bstate != nullptr && H->bits <= 4;
   if (H->deterministic && !fused && !batched) return TARDIS_ERR_UNSUPPORTED;

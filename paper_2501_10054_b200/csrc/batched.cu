@@ -216,7 +216,9 @@ tardis_status_t batched_prepare(Handle* H) {
   H->bytes_w2t += hd * 2;                       // second copy of W2 (original orientation)
   H->bytes_predictor += 2 * hd * 2 + size_t(h) * 4 + size_t((h + 127) / 128) * 4;
   H->bytes_scratch += S->bytes_scratch;
-  return TARDIS_OK;
+  const tardis_status_t st = few_prepare(H);
+  if (st != TARDIS_OK) batched_release(H);
+  return st;
 }
 
 // a_j W1[j][k] in fp32, transposed to [k][j] and split into bf16 hi + lo (16 significant bits together)
@@ -300,7 +302,7 @@ tardis_status_t batched_finish(Handle* H, const void* W2, cudaStream_t s) {
     k_dequant_split<<<h, 256, 0, s>>>(H->codes, static_cast<const __nv_bfloat16*>(H->scale), H->zero, S->What_hi, S->What_lo,
                                     S->smaxrow, S->lo_used, d, H->G, H->bits);
   TARDIS_CUDA_TRY(cudaGetLastError());
-  return TARDIS_OK;
+  return few_finish(H, S->W2, S->Wf, s);
 }
 
 void batched_release(Handle* H) {
@@ -317,6 +319,7 @@ tardis_status_t launch_batched_forward(Handle* H, const void* xv, void* yv, int6
   State* S = static_cast<State*>(H->bstate);
   if (!S) return TARDIS_ERR_UNSUPPORTED;
   const int d = H->d, h = H->h;
+  if (H->few && n_total <= 128 && !H->deterministic) return launch_few_forward(H, xv, yv, int(n_total), S->smaxrow, s);
   const __nv_bfloat16* x = static_cast<const __nv_bfloat16*>(xv);
   __nv_bfloat16* y = static_cast<__nv_bfloat16*>(yv);
   const bool keep_scores = H->dbg_bitmap || H->dbg_scores;

@@ -44,6 +44,7 @@ struct Handle {
   void* dscratch;        // fused decode scratch (see decode.cu)
   size_t dscratch_bytes;
   void* bstate;          // batched / prefill state and scratch (see batched.cu); null when not built
+  void* few;             // state of the kernels for a few to 128 tokens (see few.cu); null when not built
   // debug capture (caller-owned)
   uint32_t* dbg_bitmap;
   double* dbg_scores;
@@ -94,6 +95,10 @@ tardis_status_t batched_prepare(Handle* H);                                     
 tardis_status_t batched_finish(Handle* H, const void* W2, cudaStream_t s);   // fills the batched state (W2 null: from W2T)
 tardis_status_t launch_batched_forward(Handle* H, const void* x, void* y, int64_t n, cudaStream_t s);
 void batched_release(Handle* H);
+tardis_status_t few_prepare(Handle* H);                                       // few.cu: allocations
+tardis_status_t few_finish(Handle* H, const void* W2, const void* Wf, cudaStream_t s);   // fills its state (W2 [d, h], W_f [d, d] row-major)
+tardis_status_t launch_few_forward(Handle* H, const void* x, void* y, int n, const float* smaxrow, cudaStream_t s);
+void few_release(Handle* H);
 tardis_status_t launch_stack_forward(const tardis_stack_desc_t* desc, const void* x, void* y, void* work, void* keep, int64_t n,
                                      cudaStream_t s);   // stack.cu; arguments checked by the caller
 tardis_status_t launch_build_predictor(int h, int d, int dtype, const void* W1, const double* U, int bits, int G, uint32_t* codes,

@@ -108,37 +108,41 @@ template <int TERM> __device__ __forceinline__ void expand(const uint4& code, ui
     }
 }
 
-// Exact fp64 predictor sum of one neuron and token over the channel blocks first, first + step, ..., from the packed blocks the
-// CTA has just read (`rows` apart).  A lone warp waits for its loads and its chains of additions, nothing else (8 us per pair
-// with the words read one after the other): the loads of a block go out before the first is used, and four sums run side by side.
+// Exact fp64 predictor sum of one neuron and token over the code words first, first + step, ..., from the packed blocks the CTA
+// has just read (`rows` apart).  A lone warp waits for its loads and for its instructions, nothing else (8 us per pair with the
+// words read one after the other): four words' loads go out before the first is used, and the code is kept short.
 __device__ __noinline__ double exact_from_packed(const uint4* __restrict__ codes, const uint32_t* __restrict__ meta, const __nv_bfloat16* __restrict__ x,
-                                                 int nkb, int kpg, int rows, int first, int step) {
-  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+                                                 int nwords, int kpg, int rows, int first, int step) {
+  double acc = 0.0;
 #pragma unroll 1
-  for (int kb = first; kb < nkb; kb += step) {
-    const uint4 code = codes[size_t(kb) * rows];
-    const uint32_t m = meta[size_t(kb / kpg) * rows];
-    uint4 xv[8];
+  for (int w0 = first; w0 < nwords; w0 += 4 * step) {
+    uint32_t code[4], m[4];
+    uint4 xv[4][2];
 #pragma unroll
-    for (int c = 0; c < 8; ++c) xv[c] = *reinterpret_cast<const uint4*>(x + kb * BK + c * 8);
-    const float zp = float(m & 3u);
-    const uint32_t words[4] = {code.x, code.y, code.z, code.w};
-    double part[4] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll
-    for (int p = 0; p < 8; ++p)
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const uint4& q = xv[2 * k + (p >> 2)];
-        const uint32_t xw = (p & 3) == 0 ? q.x : ((p & 3) == 1 ? q.y : ((p & 3) == 2 ? q.z : q.w));
-        // (q - zp) x is exact in fp32
-        part[k] += double((float((words[k] >> (2 * p)) & 3u) - zp) * __uint_as_float(xw << 16));
-        part[k] += double((float((words[k] >> (16 + 2 * p)) & 3u) - zp) * __uint_as_float(xw & 0xffff0000u));
+    for (int u = 0; u < 4; ++u) {
+      const int w = w0 + u * step, kb = w >> 2;
+      if (w < nwords) {
+        code[u] = reinterpret_cast<const uint32_t*>(codes + size_t(kb) * rows)[w & 3];
+        m[u] = meta[size_t(kb / kpg) * rows];
+        xv[u][0] = *reinterpret_cast<const uint4*>(x + w * 16);
+        xv[u][1] = *reinterpret_cast<const uint4*>(x + w * 16 + 8);
       }
-    const double s = double(__uint_as_float(m & 0xffff0000u));
+    }
 #pragma unroll
-    for (int k = 0; k < 4; ++k) acc[k] += s * part[k];
+    for (int u = 0; u < 4; ++u) {
+      if (w0 + u * step >= nwords) break;
+      const float zp = float(m[u] & 3u);
+      const uint32_t xw[8] = {xv[u][0].x, xv[u][0].y, xv[u][0].z, xv[u][0].w, xv[u][1].x, xv[u][1].y, xv[u][1].z, xv[u][1].w};
+      double p0 = 0.0, p1 = 0.0;
+#pragma unroll
+      for (int p = 0; p < 8; ++p) {                        // (q - zp) x is exact in fp32
+        p0 += double((float((code[u] >> (2 * p)) & 3u) - zp) * __uint_as_float(xw[p] << 16));
+        p1 += double((float((code[u] >> (16 + 2 * p)) & 3u) - zp) * __uint_as_float(xw[p] & 0xffff0000u));
+      }
+      acc += double(__uint_as_float(m[u] & 0xffff0000u)) * (p0 + p1);
+    }
   }
-  return (acc[0] + acc[1]) + (acc[2] + acc[3]);
+  return acc;
 }
 
 // Adds v[e], the value of output i (this lane's; outputs of a warp's lanes are consecutive, i of lane 0 a multiple of 4) for token
@@ -184,3 +188,698 @@ struct Walk {
   }
 };
 
+// N: token columns (the call's tokens rounded up); TERMS: bf16 terms of a correction (2 keeps 16 significant bits of it)
+template <int N, int TERMS>
+__global__ void __maxnreg__(128)                       // (NT_IN threads; leaves room for k_few_out on the SM)
+k_few_in(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUtensorMap tmWf, const __grid_constant__ CUtensorMap tmX,
+         const InParams p) {
+  using C = InCfg<N>;
+  constexpr int RING = C::NBUF / 2;                    // expanded blocks per group of four warps
+  constexpr int HALF = N / 2;                          // token columns per epilogue thread
+  constexpr int MW = (HALF + 31) / 32;                 // flag words of a thread
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + C::NS * C::STAGE);   // [NS] stage filled
+  uint64_t* empty = full + C::NS;                      // [NS] stage read by the MMAs and the norms
+  uint64_t* a_full = empty + C::NS;                    // [NBUF] predictor block expanded
+  uint64_t* a_empty = a_full + C::NBUF;                // [NBUF] ... and read
+  uint64_t* acc_full = a_empty + C::NBUF;              // scores and pre-activations of a tile complete
+  uint64_t* acc_free = acc_full + 1;
+  uint64_t* f_full = acc_free + 1;                     // a piece of the folded product complete
+  uint64_t* f_free = f_full + 1;
+  uint64_t* norm_ready = f_free + 1;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(norm_ready + 1);
+  volatile uint32_t* failed = tmem_slot + 1;
+  uint32_t* near_count = tmem_slot + 2;
+  uint4* near = reinterpret_cast<uint4*>(smem + C::NS * C::STAGE + 256);          // [MAX_NEAR] row << 8 | token, lo, hi, b1
+  uint32_t* settled = reinterpret_cast<uint32_t*>(near + MAX_NEAR);               // [BM][(N + 31) / 32] re-evaluated scores that are outside
+  float* x1 = reinterpret_cast<float*>(settled + BM * ((N + 31) / 32));           // [N] sum |x|
+  unsigned int* tok_flagged = reinterpret_cast<unsigned int*>(x1 + N);            // [N]
+  float* staging = reinterpret_cast<float*>(tok_flagged + N);                     // [8 warps][8][32]
+
+  const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // (warp: uniform, and known to be)
+  const int nkb = p.nkb;
+  const int2 wf = p.wf_plan[blockIdx.x];
+  pdl_launch();
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < C::NS; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 3); }
+    for (int b = 0; b < C::NBUF; ++b) { mbar_init(&a_full[b], 4); mbar_init(&a_empty[b], 1); }
+    mbar_init(acc_full, 1); mbar_init(acc_free, 8); mbar_init(f_full, 1); mbar_init(f_free, 8); mbar_init(norm_ready, 2);
+    *failed = 0u;
+    *near_count = 0u;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  for (int i = threadIdx.x; i < BM * ((N + 31) / 32); i += NT_IN) settled[i] = 0u;
+  if (threadIdx.x < N) tok_flagged[threadIdx.x] = 0u;
+  __syncthreads();
+  // (warp 0 goes on with its copies: the allocation waits while the launch before holds too much of the SM's tensor memory)
+  if (warp == 1) tmem_alloc(tmem_slot, C::TMEM);
+  if (warp != 0) {
+    tc_fence_before();
+    asm volatile("bar.sync 2, 352;" ::: "memory");
+    tc_fence_after();
+  }
+  const uint32_t tmem = *tmem_slot;
+
+  if (warp == 0) {
+    // ---------------- TMA: W1 tiles, then the folded matrix's blocks; the tokens beside each ----------------
+    Walk w(p, wf), first = w;
+    const int ahead = min(C::NS, w.total);
+    auto bytes = [&](const Walk& at) { return uint32_t((at.folded ? BM : p.rows) * BK * 2 + C::X_BYTES); };
+    auto weights = [&](const Walk& at, int s) { tma_load_2d(smem + s * C::STAGE, at.folded ? &tmWf : &tmW1, at.kb * BK, at.row0, &full[s]); };
+    auto tokens = [&](const Walk& at, int s) { tma_load_2d(smem + s * C::STAGE + W_BYTES, &tmX, at.kb * BK, 0, &full[s]); };
+    for (int s = 0; s < ahead; ++s, w.next())              // constant state: before the wait
+      if (elect_one()) { mbar_expect_tx(&full[s], bytes(w)); weights(w, s); }
+    pdl_wait();
+    for (int s = 0; s < ahead; ++s, first.next())
+      if (elect_one()) tokens(first, s);
+    for (int i = ahead, s = 0, parity = 0; i < w.total; ++i, w.next()) {
+      const bool ok = mbar_wait_issue(&empty[s], parity, failed);
+      if (elect_one() && ok) { mbar_expect_tx(&full[s], bytes(w)); weights(w, s); tokens(w, s); }
+      if (++s == C::NS) { s = 0; parity ^= 1; }
+    }
+  } else if (warp == 1) {
+    // ---------------- MMA issuer ----------------
+    constexpr uint32_t idesc = instr_desc_bf16(BM, N);
+    const uint64_t wdesc = smem_desc_k_major_sw128(smem_u32(smem)), xdesc = smem_desc_k_major_sw128(smem_u32(smem) + W_BYTES);
+    int s = 0, parity = 0, ati = 0, own0 = 0, own1 = 0;    // stage and its phase; tiles; expanded blocks used of either group
+    auto next_stage = [&]() { if (++s == C::NS) { s = 0; parity ^= 1; } };
+    for (int tile = blockIdx.x; tile < p.ntiles; tile += gridDim.x, ++ati) {
+      const int terms = p.two_terms[tile] ? 2 : 1;
+      bool ok = mbar_wait_issue(acc_free, (ati & 1) ^ 1, failed);
+      for (int kb = 0; kb < nkb; ++kb) {
+        ok = mbar_wait_issue(&full[s], parity, failed);
+        tc_fence_after();
+        const uint64_t da = wdesc + uint32_t(s * (C::STAGE >> 4)), db = xdesc + uint32_t(s * (C::STAGE >> 4));
+        if (elect_one() && ok) {
+#pragma unroll
+          for (int k = 0; k < BK / 16; ++k) umma_f16(tmem + C::COL_Z, da + k * 2, db + k * 2, idesc, (kb | k) != 0 ? 1u : 0u);
+        }
+        for (int term = 0; term < terms; ++term) {
+          const int own = (kb & 1) ? own1 : own0, b = (kb & 1) + 2 * (own % RING);
+          ok = mbar_wait_issue(&a_full[b], (own / RING) & 1, failed);
+          tc_fence_after();
+          if (elect_one() && ok) {
+#pragma unroll
+            for (int k = 0; k < BK / 16; ++k)
+              umma_f16_ta(tmem + C::COL_S, tmem + C::COL_A + b * 32 + k * 8, db + k * 2, idesc, (kb | k | term) != 0 ? 1u : 0u);
+            umma_commit(&a_empty[b]);
+            if (term == terms - 1) umma_commit(&empty[s]);
+          }
+          if (kb & 1) ++own1; else ++own0;
+        }
+        next_stage();
+      }
+      if (elect_one() && ok) umma_commit(acc_full);
+    }
+    for (int u = wf.x, end = wf.x / nkb * nkb, seg = 0; u < wf.y; ++seg) {
+      end = min(wf.y, end + nkb);                            // blocks of one output tile
+      bool ok = mbar_wait_issue(f_free, (seg & 1) ^ 1, failed);
+      for (uint32_t accumulate = 0u; u < end; ++u) {
+        ok = mbar_wait_issue(&full[s], parity, failed);
+        tc_fence_after();
+        const uint64_t da = wdesc + uint32_t(s * (C::STAGE >> 4)), db = xdesc + uint32_t(s * (C::STAGE >> 4));
+        if (elect_one() && ok) {
+#pragma unroll
+          for (int k = 0; k < BK / 16; ++k) umma_f16(tmem + C::COL_F, da + k * 2, db + k * 2, idesc, k ? 1u : accumulate);
+          umma_commit(&empty[s]);
+        }
+        accumulate = 1u;
+        next_stage();
+      }
+      if (elect_one() && ok) umma_commit(f_full);
+    }
+  } else if (warp < 4) {
+    // ---------------- token norms sum |x|, read beside the MMAs while the first tile passes by ----------------
+    const int total = Walk(p, wf).total;
+    const bool any_tile = int(blockIdx.x) < p.ntiles;
+    float sum[2] = {0.f, 0.f};
+    bool bad[2] = {false, false};
+    const int tk = (warp - 2) * 32 + lane;
+    for (int i = 0, s = 0, parity = 0; i < total; ++i) {
+      if (!mbar_wait_warp(&full[s], parity)) { *failed = 1u; break; }
+      if (any_tile && i < nkb) {
+        const uint8_t* xt = smem + s * C::STAGE + W_BYTES;
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          const int t = tk + 64 * r;
+          if (t < N) {
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+              const uint4 v = *reinterpret_cast<const uint4*>(xt + t * 128 + ((c ^ (t & 7)) << 4));
+              const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                const float lo = fabsf(__uint_as_float(w[q] << 16)), hi = fabsf(__uint_as_float(w[q] & 0xffff0000u));
+                bad[r] |= !(lo <= 3.0e38f) || !(hi <= 3.0e38f);
+                sum[r] += lo + hi;
+              }
+            }
+          }
+        }
+        if (i == nkb - 1) {
+#pragma unroll
+          for (int r = 0; r < 2; ++r)
+            if (tk + 64 * r < N) x1[tk + 64 * r] = bad[r] ? __int_as_float(0x7f800000) : sum[r];
+        }
+      }
+      __syncwarp();
+      if (lane == 0) {
+        mbar_arrive(&empty[s]);
+        if (i == nkb - 1) mbar_arrive(norm_ready);
+      }
+      if (++s == C::NS) { s = 0; parity ^= 1; }
+    }
+  } else {
+    // ---------------- predictor expansion, then the epilogues: thread = weight row 32 q + lane of the tile ----------------
+    const int q = warp & 3, gi = (warp - 4) >> 2;          // TMEM lanes 32 q .. + 31; channel blocks / token columns of this group
+    const uint32_t lanes = tmem + (uint32_t(q * 32) << 16);
+    const int row = q * 32 + lane, rows = p.rows;
+    const bool holds = q * 32 < rows;                      // any row of this warp is in use
+    float* const stage = staging + (warp - 4) * 256;
+    const int kpg = p.G / BK;                              // channel blocks per predictor group
+    int ati = 0, own = 0;
+    bool ok = true;
+    // (after a wait that ran out the flow stays the same, without further waits: the warps meet at named barriers)
+    for (int tile = blockIdx.x; tile < p.ntiles; tile += gridDim.x, ++ati) {
+      // -- this group's channel blocks gi, gi + 2, ...: codes fetched four blocks ahead --
+      const int terms = p.two_terms[tile] ? 2 : 1;
+      const uint4* const tile_codes = p.codes + size_t(tile) * nkb * rows;
+      const uint32_t* const tile_meta = p.meta + size_t(tile) * (p.d / p.G) * rows;
+      const int mine = (nkb - gi + 1) / 2;
+      uint4 code[4] = {};
+      uint32_t meta[4] = {};
+      auto fetch = [&](int kb, uint4& cd, uint32_t& mt) {
+        if (row < rows) {
+          cd = __ldg(tile_codes + size_t(kb) * rows + row);
+          mt = __ldg(tile_meta + size_t(kb / kpg) * rows + row);
+        }
+      };
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (u < mine) fetch(gi + 2 * u, code[u], meta[u]);
+      const int j = tile * rows + row;
+      const bool real = row < rows && j < p.h;
+      float lo = 0.f, hi = 0.f, b1 = 0.f, fa = 0.f, fc = 0.f;
+      if (real) { lo = p.lo[j]; hi = p.hi[j]; b1 = p.b1[j]; fa = p.a[j]; fc = p.c[j]; }
+      const float smax = real ? p.smax[j] : 0.f;
+      for (int i0 = 0; i0 < mine && ok; i0 += 4) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int i = i0 + u;
+          if (i < mine && ok) {
+            uint32_t w[32];
+            for (int term = 0; term < terms && ok; ++term) {
+              if (!holds) {}
+              else if (terms == 1) expand<-1>(code[u], meta[u], w);
+              else if (term == 0) expand<0>(code[u], meta[u], w);
+              else expand<1>(code[u], meta[u], w);
+              if (term == terms - 1 && i + 4 < mine) fetch(gi + 2 * (i + 4), code[u], meta[u]);
+              const int b = gi + 2 * (own % RING);
+              ok = mbar_wait_warp(&a_empty[b], ((own / RING) & 1) ^ 1);
+              if (!ok) { *failed = 1u; break; }
+              tc_fence_after();
+              if (holds) tmem_st32(lanes + C::COL_A + b * 32, w);
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) mbar_arrive(&a_full[b]);
+              ++own;
+            }
+          }
+        }
+      }
+      pdl_wait();                                          // (from here on: data of earlier launches)
+      // -- scores -> flags of this thread's neuron and token columns gi HALF .. + HALF - 1 --
+      ok = ok && mbar_wait_warp(norm_ready, 0) && mbar_wait_warp(acc_full, ati & 1);
+      if (!ok) *failed = 1u;
+      tc_fence_after();
+      // (loops over columns stay rolled: unrolled, their code outgrows the instruction cache and costs 20 us)
+      uint64_t flags = 0, open = 0;                        // bit c: token column gi HALF + c; open: too close to a range end to tell
+      // the terms of a score are at most (largest |q - zp|) smax |x| each: 3 only where a tile has such codes
+      const float tau1 = (terms == 2 ? 3.f : 2.f) * kEps * smax;
+      const int cols = real ? min(HALF, p.n - gi * HALF) : 0;   // (may be negative)
+#pragma unroll 1
+      for (int c0 = 0; c0 < HALF; c0 += 8) {
+        float v[8];
+        tmem_ld8(lanes + C::COL_S + gi * HALF + c0, v);
+        uint32_t fl = 0u, op = 0u;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          const float xn = x1[gi * HALF + c0 + e], z = v[e] + b1, tau = fmaf(tau1, xn, 1e-30f);
+          const bool finite = xn <= 3.0e38f;               // (a non-finite token: every neuron flagged)
+          const bool near_end = finite && (fabsf(z - lo) <= tau || fabsf(z - hi) <= tau);
+          fl |= uint32_t(!near_end && !(finite && lo <= z && z < hi)) << e;
+          op |= uint32_t(near_end) << e;
+          v[e] = finite ? z : __int_as_float(0x7fc00000);
+        }
+        const uint32_t valid = cols >= c0 + 8 ? 0xffu : (cols > c0 ? (1u << (cols - c0)) - 1u : 0u);
+        flags |= uint64_t(fl & valid) << c0;
+        open |= uint64_t(op & valid) << c0;
+        if (p.dbg_scores)
+#pragma unroll
+          for (int e = 0; e < 8; ++e)
+            if (c0 + e < cols) p.dbg_scores[size_t(gi * HALF + c0 + e) * p.h + j] = double(v[e]);
+      }
+      for (uint64_t w = open; w; w &= w - 1) {             // rare
+        const int t = gi * HALF + __ffsll((long long)w) - 1;
+        const uint32_t slot = atomicAdd(near_count, 1u);
+        if (slot < MAX_NEAR) near[slot] = make_uint4(uint32_t(row) << 8 | uint32_t(t), __float_as_uint(lo), __float_as_uint(hi), __float_as_uint(b1));
+        else {                                             // list full: this thread settles the pair alone
+          const double ze = exact_from_packed(tile_codes + row, tile_meta + row, p.x + size_t(t) * p.d, nkb * 4, kpg, rows, 0, 1) + double(b1);
+          if (!(double(lo) <= ze && ze < double(hi))) flags |= 1ull << (t - gi * HALF);
+        }
+      }
+      asm volatile("bar.sync 1, 256;" ::: "memory");
+      const uint32_t nn = *near_count;
+      if (nn > 0) {                                        // (the same for all eight warps)
+        for (uint32_t e = warp - 4; e < min(nn, uint32_t(MAX_NEAR)); e += 8) {
+          const uint4 pair = near[e];
+          const int r = int(pair.x >> 8), t = int(pair.x & 255u);
+          const float rl = __uint_as_float(pair.y), rh = __uint_as_float(pair.z), rb = __uint_as_float(pair.w);
+          double z = exact_from_packed(tile_codes + r, tile_meta + r, p.x + size_t(t) * p.d, nkb * 4, kpg, rows, lane, 32);
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+          z += double(rb);
+          if (lane == 0) {
+            if (!(double(rl) <= z && z < double(rh))) atomicOr(&settled[r * ((N + 31) / 32) + (t >> 5)], 1u << (t & 31));
+            if (p.dbg_scores) p.dbg_scores[size_t(t) * p.h + tile * rows + r] = z;
+          }
+        }
+        asm volatile("bar.sync 1, 256;" ::: "memory");
+        if (threadIdx.x == 128) { atomicAdd(&p.counters[CTR_RECHECKS], (unsigned long long)nn); *near_count = 0u; }
+        uint32_t* fix = &settled[row * ((N + 31) / 32)];
+        if (HALF >= 32) {
+#pragma unroll
+          for (int m = 0; m < MW; ++m) { flags |= uint64_t(fix[gi * MW + m]) << (32 * m); fix[gi * MW + m] = 0u; }
+        } else {
+          flags |= (fix[0] >> (gi * HALF)) & ((1u << (HALF & 31)) - 1u);
+        }
+      }
+      // -- counts per token; corrections act(z) - a z - c where flagged, zero elsewhere --
+#pragma unroll 1
+      for (int c0 = 0; c0 < HALF; c0 += 8) {
+        const uint32_t bits = uint32_t(flags >> c0) & 0xffu;
+        float v[8];
+        tmem_ld8(lanes + C::COL_Z + gi * HALF + c0, v);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          const uint32_t word = __ballot_sync(0xffffffffu, (bits >> e) & 1u);
+          const int t = gi * HALF + c0 + e;
+          if (lane == 0 && t < p.n) {
+            if (word) atomicAdd(&tok_flagged[t], __popc(word));
+            if (p.dbg_bitmap && word) {                    // (cleared before the launch; a tile may begin inside a word)
+              atomicOr(p.dbg_bitmap + size_t(t) * (p.h / 32) + (j >> 5), word << (j & 31));
+              if ((j & 31) && (word >> (32 - (j & 31)))) atomicOr(p.dbg_bitmap + size_t(t) * (p.h / 32) + (j >> 5) + 1, word >> (32 - (j & 31)));
+            }
+          }
+          stage[e * 32 + lane] = v[e];
+        }
+#pragma unroll 1
+        for (uint32_t w = bits; w; w &= w - 1u) {
+          const int e = __ffs(w) - 1;
+          const float z = stage[e * 32 + lane] + b1;
+          stage[e * 32 + lane] = gelu_f32(z, p.act) - fa * z - fc;
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          if (c0 + e < cols) {
+            const int t = gi * HALF + c0 + e;
+            const float dl = (bits >> e) & 1u ? stage[e * 32 + lane] : 0.f;
+            const __nv_bfloat16 h0 = __float2bfloat16_rn(dl);
+            p.delta[size_t(t) * p.h + j] = h0;
+            if (TERMS == 2) p.delta[size_t(N + t) * p.h + j] = __float2bfloat16_rn(dl - __bfloat162float(h0));
+          }
+        }
+      }
+      if (HALF < 32) {                                     // (both groups' threads read the same word: cleared after both have)
+        asm volatile("bar.sync 1, 256;" ::: "memory");
+        if (gi == 0) settled[row] = 0u;
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(acc_free);
+    }
+    // -- pieces of the folded product: added to the fp32 accumulator --
+    pdl_wait();
+    int seg = 0;
+    for (int u = wf.x; u < wf.y; ++seg) {
+      const int m = u / nkb;
+      u = min(wf.y, (m + 1) * nkb);
+      ok = ok && mbar_wait_warp(f_full, seg & 1);
+      if (!ok) { *failed = 1u; break; }
+      tc_fence_after();
+#pragma unroll 1
+      for (int c0 = 0; c0 < HALF; c0 += 8) {
+        float v[8];
+        tmem_ld8(lanes + C::COL_F + gi * HALF + c0, v);
+        add_outputs(p.yacc, p.d, p.n, gi * HALF + c0, m * BM + row, v);
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(f_free);
+    }
+    asm volatile("bar.sync 1, 256;" ::: "memory");
+    const int t = threadIdx.x - 128;
+    if (t < p.n && tok_flagged[t]) atomicAdd(&p.nfl[t], tok_flagged[t]);
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (threadIdx.x == 0 && *failed) atomicExch(&p.counters[CTR_ERROR], 1ull);
+  if (warp == 1) tmem_dealloc(tmem, C::TMEM);
+}
+
+// Corrections times W2.  N: columns (tokens rounded up, times the terms of a correction).  CTA c works on the pairs
+// [c total / grid, (c + 1) total / grid) of (output tile, neuron block).
+template <int N>
+__global__ void __maxnreg__(80)                        // (NT_OUT threads beside NT_IN of k_few_in: 64512 of 65536 registers)
+k_few_out(const __grid_constant__ CUtensorMap tmW2, const __grid_constant__ CUtensorMap tmD, const OutParams p) {
+  using C = OutCfg<N>;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + C::NS * C::STAGE);
+  uint64_t* empty = full + C::NS;
+  uint64_t* acc_full = empty + C::NS;
+  uint64_t* acc_free = acc_full + 1;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_free + 1);
+  volatile uint32_t* failed = tmem_slot + 1;
+  uint32_t* last = tmem_slot + 2;
+  const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // (warp: uniform, and known to be)
+  auto begin_of = [&](int c) { return int((long long)p.total * c / int(gridDim.x)); };
+  const int begin = begin_of(blockIdx.x), end = begin_of(blockIdx.x + 1), nkb = p.nkb;
+  pdl_launch();
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < C::NS; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
+    mbar_init(acc_full, 1);
+    mbar_init(acc_free, 4);
+    *failed = 0u;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+
+  if (warp == 0) {
+    int m = begin / nkb, kb = begin - m * nkb, xb = kb;      // next pair; neuron block of the next token tile
+    auto weights = [&](int s) { tma_load_2d(smem + s * C::STAGE, &tmW2, kb * BK, m * BM, &full[s]); };
+    auto corrections = [&](int s) { tma_load_2d(smem + s * C::STAGE + W_BYTES, &tmD, xb * BK, 0, &full[s]); };
+    auto next_weights = [&]() { if (++kb == nkb) { kb = 0; ++m; } };
+    auto next_corrections = [&]() { if (++xb == nkb) xb = 0; };
+    const int total = end - begin, ahead = min(C::NS, total);
+    for (int s = 0; s < ahead; ++s, next_weights())          // constant state: before the wait
+      if (elect_one()) { mbar_expect_tx(&full[s], C::STAGE); weights(s); }
+    pdl_wait();
+    for (int s = 0; s < ahead; ++s, next_corrections())
+      if (elect_one()) corrections(s);
+    for (int i = ahead, s = 0, parity = 0; i < total; ++i, next_weights(), next_corrections()) {
+      const bool ok = mbar_wait_issue(&empty[s], parity, failed);
+      if (elect_one() && ok) { mbar_expect_tx(&full[s], C::STAGE); weights(s); corrections(s); }
+      if (++s == C::NS) { s = 0; parity ^= 1; }
+    }
+  } else {
+    // TMEM only once the launch before has given its own back (an allocation that has to wait blocks)
+    pdl_wait();
+    if (warp == 1) tmem_alloc(tmem_slot, C::TMEM);
+    tc_fence_before();
+    asm volatile("bar.sync 1, 160;" ::: "memory");      // (warps 1..5; warp 0 goes on with its copies)
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+    if (warp == 1) {
+      constexpr uint32_t idesc = instr_desc_bf16(BM, N);
+      const uint64_t wdesc = smem_desc_k_major_sw128(smem_u32(smem)), xdesc = smem_desc_k_major_sw128(smem_u32(smem) + W_BYTES);
+      int s = 0, parity = 0;
+      for (int u = begin, stop = begin / nkb * nkb, seg = 0; u < end; ++seg) {
+        stop = min(end, stop + nkb);                           // blocks of one output tile
+        bool ok = mbar_wait_issue(acc_free, (seg & 1) ^ 1, failed);
+        for (uint32_t accumulate = 0u; u < stop; ++u) {
+          ok = mbar_wait_issue(&full[s], parity, failed);
+          tc_fence_after();
+          const uint64_t da = wdesc + uint32_t(s * (C::STAGE >> 4)), db = xdesc + uint32_t(s * (C::STAGE >> 4));
+          if (elect_one() && ok) {
+#pragma unroll
+            for (int k = 0; k < BK / 16; ++k) umma_f16(tmem, da + k * 2, db + k * 2, idesc, k ? 1u : accumulate);
+            umma_commit(&empty[s]);
+          }
+          accumulate = 1u;
+          if (++s == C::NS) { s = 0; parity ^= 1; }
+        }
+        if (elect_one() && ok) umma_commit(acc_full);
+      }
+    } else {
+      const int q = warp & 3, row = q * 32 + lane, et = threadIdx.x - 64;
+      const uint32_t lanes = tmem + (uint32_t(q * 32) << 16);
+      if (blockIdx.x == 0) {                               // flagged neurons per token, counted by the launch before
+        unsigned int f = et < p.n ? p.nfl[et] : 0u;
+        if (et < p.n) p.nfl[et] = 0u;
+        const unsigned int sum = __reduce_add_sync(0xffffffffu, f), most = __reduce_max_sync(0xffffffffu, f);
+        if (lane == 0 && sum) {
+          atomicAdd(&p.counters[CTR_FLAGGED_TOTAL], (unsigned long long)sum);
+          atomicMax(&p.counters[CTR_FLAGGED_MAX], (unsigned long long)most);
+        }
+      }
+      bool ok = true;
+      int seg = 0;
+      for (int u = begin; u < end; ++seg) {
+        const int m = u / nkb, i = m * BM + row;
+        u = min(end, (m + 1) * nkb);
+        ok = ok && mbar_wait_warp(acc_full, seg & 1);
+        if (!ok) *failed = 1u;
+        tc_fence_after();
+        const int cols = N / p.terms;                      // token columns; with two terms the second one is cols further on
+#pragma unroll 1
+        for (int c0 = 0; c0 < cols && c0 < p.n; c0 += 8) {
+          float v[8];
+          tmem_ld8(lanes + c0, v);
+          if (p.terms == 2) {
+            float w[8];
+            tmem_ld8(lanes + cols + c0, w);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) v[e] += w[e];
+          }
+          add_outputs(p.yacc, p.d, p.n, c0, i, v);
+        }
+        tc_fence_before();
+        __threadfence();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(acc_free);
+        asm volatile("bar.sync 2, 128;" ::: "memory");
+        if (et == 0) *last = atomicAdd(&p.done[m], 1u) + 1u == p.parts[m] ? 1u : 0u;
+        asm volatile("bar.sync 2, 128;" ::: "memory");
+        if (*last) {                                       // every part is in: b_f, one rounding; the accumulator is left cleared
+          __threadfence();
+          // (a lane takes four outputs, a warp every fourth token: its loads are in flight together)
+          const int i4 = m * BM + lane * 4;
+          if (i4 < p.d) {
+            const float4 bf = *reinterpret_cast<const float4*>(p.bf + i4);
+#pragma unroll 1
+            for (int t0 = q; t0 < p.n; t0 += 32) {
+              float4 v[8];
+#pragma unroll
+              for (int r = 0; r < 8; ++r)
+                if (t0 + 4 * r < p.n) v[r] = __ldcg(reinterpret_cast<const float4*>(p.yacc + size_t(t0 + 4 * r) * p.d + i4));
+#pragma unroll
+              for (int r = 0; r < 8; ++r)
+                if (t0 + 4 * r < p.n) {
+                  const size_t at = size_t(t0 + 4 * r) * p.d + i4;
+                  const __nv_bfloat162 o[2] = {__floats2bfloat162_rn(v[r].x + bf.x, v[r].y + bf.y), __floats2bfloat162_rn(v[r].z + bf.z, v[r].w + bf.w)};
+                  *reinterpret_cast<uint2*>(p.y + at) = *reinterpret_cast<const uint2*>(o);
+                  *reinterpret_cast<float4*>(p.yacc + at) = make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+            }
+          }
+          if (et == 0) p.done[m] = 0u;
+        }
+        asm volatile("bar.sync 2, 128;" ::: "memory");     // (*last has been read)
+      }
+    }
+    tc_fence_before();
+    asm volatile("bar.sync 1, 160;" ::: "memory");
+    if (warp == 1) tmem_dealloc(tmem, C::TMEM);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0 && *failed) atomicExch(&p.counters[CTR_ERROR], 1ull);
+}
+
+// ---- set-up ---------------------------------------------------------------------------------------------
+// Packed predictor: block (tile of `rows` neurons, 64 channels) = rows x 16 bytes, a neuron's four code words each with its even
+// channels' codes in the lower half and the odd ones' in the upper half; per (tile, group) `rows` words, bf16 scale above,
+// zero-point below.  two_terms: the tile has a value with |q - zp| = 3.
+__global__ void k_pack(const uint32_t* __restrict__ codes, const __nv_bfloat16* __restrict__ scale, const uint8_t* __restrict__ zero,
+                       uint4* __restrict__ out, uint32_t* __restrict__ meta, uint32_t* __restrict__ two_terms, int rows, int d, int h, int G, int nkb) {
+  const int tile = blockIdx.x, r = threadIdx.x, j = tile * rows + r, ng = d / G;
+  bool two = false;
+  for (int kb = blockIdx.y; kb < nkb; kb += gridDim.y) {
+    uint32_t w[4] = {0u, 0u, 0u, 0u};
+    if (j < h) {
+      const uint4 src = *reinterpret_cast<const uint4*>(codes + size_t(j) * (d / 16) + kb * 4);
+      const uint32_t s[4] = {src.x, src.y, src.z, src.w};
+      const uint32_t zp = zero[size_t(j) * ng + kb * BK / G] & 3u;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+#pragma unroll
+        for (int p = 0; p < 8; ++p)
+          w[k] |= ((s[k] >> (4 * p)) & 3u) << (2 * p) | ((s[k] >> (4 * p + 2)) & 3u) << (16 + 2 * p);
+        const uint32_t lo = s[k] & 0x55555555u, hi = (s[k] >> 1) & 0x55555555u;   // bits of the codes
+        two |= (zp == 0u && (lo & hi)) || (zp == 3u && (~(lo | hi) & 0x55555555u));
+      }
+    }
+    out[(size_t(tile) * nkb + kb) * rows + r] = make_uint4(w[0], w[1], w[2], w[3]);
+  }
+  if (two) two_terms[tile] = 1u;
+  for (int g = blockIdx.y; g < ng; g += gridDim.y)
+    meta[(size_t(tile) * ng + g) * rows + r] =
+        j < h ? (uint32_t(__bfloat16_as_ushort(scale[size_t(j) * ng + g])) << 16) | (zero[size_t(j) * ng + g] & 3u) : 0u;
+}
+
+struct State {
+  uint4* codes; uint32_t *meta, *two_terms; int2* plan; float* yacc; unsigned int *nfl, *done, *parts;
+  __nv_bfloat16* delta;
+  CUtensorMap w1, w2, wf;
+  int grid, out_grid, nkb, rows, ntiles, mtiles, out_nkb;
+};
+
+// Shares of the folded product's blocks: a neuron tile's block costs its rows' share of a 128-row one plus a seventh (codes);
+// every CTA is filled up to the same total, and pieces of fewer than 8 blocks are not dealt (a piece costs one pass over a
+// 128-row accumulator at its end).
+static void deal_folded_blocks(const State& S, std::vector<int2>& plan) {
+  const double per_tile = 1.15 * S.rows / BM * S.nkb;
+  const int blocks = S.mtiles * S.nkb;
+  std::vector<double> room(S.grid);
+  auto fill = [&](double level) {
+    double sum = 0.0;
+    for (int c = 0; c < S.grid; ++c) {
+      room[c] = level - per_tile * ((S.ntiles - c + S.grid - 1) / S.grid);
+      if (room[c] < 8.0) room[c] = 0.0;
+      sum += room[c];
+    }
+    return sum;
+  };
+  double lo = 0.0, hi = per_tile * (S.ntiles / S.grid + 2) + blocks;
+  while (hi - lo > 1e-3) { const double mid = 0.5 * (lo + hi); (fill(mid) >= blocks ? hi : lo) = mid; }   // the level that holds all blocks
+  const double sum = fill(hi);
+  double cum = 0.0;
+  int at = 0;
+  for (int c = 0; c < S.grid; ++c) {
+    cum += room[c];
+    const int to = c == S.grid - 1 ? blocks : std::min(blocks, int(cum / sum * blocks + 0.5));
+    plan[c] = make_int2(at, to);
+    at = to;
+  }
+}
+
+}  // namespace few
+
+using namespace few;
+
+// Serves bf16 layers with 2-bit codes in groups of a multiple of 64 channels (every channel block lies in one group).
+tardis_status_t few_prepare(Handle* H) {
+  H->few = nullptr;
+  const int d = H->d, h = H->h, G = H->G;
+  if (H->dtype != TARDIS_BF16 || H->bits != 2 || G % BK || !tensor_maps_available()) return TARDIS_OK;
+  State* S = new (std::nothrow) State();
+  if (!S) return TARDIS_ERR_ALLOC;
+  memset(S, 0, sizeof(*S));
+  H->few = S;
+  S->grid = H->num_sms;
+  const int rounds = (h + S->grid * BM - 1) / (S->grid * BM), share = (h + S->grid * rounds - 1) / (S->grid * rounds);
+  S->rows = std::min(BM, std::max(16, (share + 7) / 8 * 8));          // every CTA gets the same number of tiles, or one less
+  S->nkb = d / BK; S->ntiles = (h + S->rows - 1) / S->rows; S->mtiles = (d + BM - 1) / BM; S->out_nkb = (h + BK - 1) / BK;
+  const size_t code_bytes = size_t(S->ntiles) * S->nkb * S->rows * 16, meta_bytes = size_t(S->ntiles) * (d / G) * S->rows * 4;
+  struct Req { void** p; size_t bytes; };
+  Req reqs[] = {{reinterpret_cast<void**>(&S->codes), code_bytes}, {reinterpret_cast<void**>(&S->meta), meta_bytes},
+                {reinterpret_cast<void**>(&S->plan), sizeof(int2) * S->grid}, {reinterpret_cast<void**>(&S->yacc), sizeof(float) * MAX_TOKENS * d},
+                {reinterpret_cast<void**>(&S->nfl), sizeof(unsigned int) * (MAX_TOKENS + 2 * S->mtiles + S->ntiles)},
+                {reinterpret_cast<void**>(&S->delta), size_t(2) * MAX_TOKENS * h}};
+  for (const Req& r : reqs) {
+    const cudaError_t e = dev_malloc(r.p, r.bytes);
+    if (e != cudaSuccess) { set_last_error(e, "cudaMalloc"); cudaGetLastError(); few_release(H); return TARDIS_ERR_ALLOC; }
+  }
+  S->done = S->nfl + MAX_TOKENS;
+  S->parts = S->done + S->mtiles;
+  S->two_terms = S->parts + S->mtiles;
+  H->bytes_predictor += code_bytes + meta_bytes;
+  for (int i = 2; i < 6; ++i) H->bytes_scratch += reqs[i].bytes;
+  return TARDIS_OK;
+}
+
+tardis_status_t few_finish(Handle* H, const void* W2, const void* Wf, cudaStream_t s) {
+  State* S = static_cast<State*>(H->few);
+  if (!S) return TARDIS_OK;
+  const int d = H->d, h = H->h;
+  if (!make_map(&S->w1, H->W1, h, d, d, S->rows) || !make_map(&S->w2, W2, d, h, h, BM) || !make_map(&S->wf, Wf, d, d, d, BM)) {
+    few_release(H);                                    // (not served: the other kernels take these calls)
+    return TARDIS_OK;
+  }
+  std::vector<int2> plan(S->grid);
+  deal_folded_blocks(*S, plan);
+  S->out_grid = std::max(1, std::min(H->num_sms, S->mtiles * S->out_nkb / 4));
+  // CTAs that contribute to an output tile (the shares of k_few_out)
+  const long long total = (long long)S->mtiles * S->out_nkb;
+  std::vector<unsigned int> parts(S->mtiles, 0u);
+  for (int c = 0; c < S->out_grid; ++c) {
+    const long long b = total * c / S->out_grid, e = total * (c + 1) / S->out_grid;
+    for (long long m = b / S->out_nkb; m * S->out_nkb < e; ++m) parts[m] += 1u;
+  }
+  TARDIS_CUDA_TRY(cudaMemsetAsync(S->nfl, 0, sizeof(unsigned int) * (MAX_TOKENS + 2 * S->mtiles + S->ntiles), s));
+  TARDIS_CUDA_TRY(cudaMemcpyAsync(S->plan, plan.data(), sizeof(int2) * S->grid, cudaMemcpyHostToDevice, s));
+  TARDIS_CUDA_TRY(cudaMemcpyAsync(S->parts, parts.data(), sizeof(unsigned int) * S->mtiles, cudaMemcpyHostToDevice, s));
+  TARDIS_CUDA_TRY(cudaStreamSynchronize(s));           // (the host buffers go away with this call)
+  TARDIS_CUDA_TRY(cudaMemsetAsync(S->yacc, 0, sizeof(float) * MAX_TOKENS * d, s));
+  k_pack<<<dim3(S->ntiles, 8), S->rows, 0, s>>>(H->codes, static_cast<const __nv_bfloat16*>(H->scale), H->zero, S->codes, S->meta, S->two_terms,
+                                                S->rows, d, h, H->G, S->nkb);
+  TARDIS_CUDA_TRY(cudaGetLastError());
+  return TARDIS_OK;
+}
+
+void few_release(Handle* H) {
+  State* S = static_cast<State*>(H->few);
+  if (!S) return;
+  void* ptrs[] = {S->codes, S->meta, S->plan, S->yacc, S->nfl, S->delta};
+  for (void* q : ptrs)
+    if (q) dev_free(q);
+  delete S;
+  H->few = nullptr;
+}
+
+template <typename K, typename... Args>
+static cudaError_t launch_overlapped(K kernel, int grid, int threads, size_t smem, cudaStream_t s, const Args&... args) {
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid); cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+template <int N, int TERMS>
+static tardis_status_t launch_n(Handle* H, const __nv_bfloat16* x, __nv_bfloat16* y, int n, const float* smaxrow, cudaStream_t s) {
+  State* S = static_cast<State*>(H->few);
+  CUtensorMap tmx, tmd;
+  if (!make_map(&tmx, x, n, H->d, H->d, N) || !make_map(&tmd, S->delta, MAX_TOKENS, H->h, H->h, N * TERMS)) return TARDIS_ERR_UNSUPPORTED;
+  InParams a = {};
+  a.n = n; a.d = H->d; a.h = H->h; a.G = H->G; a.nkb = S->nkb; a.ntiles = S->ntiles; a.rows = S->rows; a.act = H->act;
+  a.codes = S->codes; a.meta = S->meta; a.two_terms = S->two_terms;
+  a.lo = H->lo; a.hi = H->hi; a.a = H->a; a.c = H->c; a.b1 = H->b1; a.smax = smaxrow; a.x = x;
+  a.wf_plan = S->plan; a.delta = S->delta; a.yacc = S->yacc; a.nfl = S->nfl; a.counters = H->counters;
+  a.dbg_bitmap = H->dbg_bitmap; a.dbg_scores = H->dbg_scores;
+  if (H->dbg_bitmap) TARDIS_CUDA_TRY(cudaMemsetAsync(H->dbg_bitmap, 0, size_t(n) * (H->h / 32) * 4, s));
+  TARDIS_CUDA_TRY(launch_overlapped(k_few_in<N, TERMS>, S->grid, NT_IN, InCfg<N>::SMEM, s, S->w1, S->wf, tmx, a));
+  OutParams o = {};
+  o.n = n; o.d = H->d; o.h = H->h; o.nkb = S->out_nkb; o.total = S->mtiles * S->out_nkb; o.terms = TERMS;
+  o.bf = H->bf; o.yacc = S->yacc; o.y = y; o.done = S->done; o.parts = S->parts; o.nfl = S->nfl; o.counters = H->counters;
+  TARDIS_CUDA_TRY(launch_overlapped(k_few_out<N * TERMS>, S->out_grid, NT_OUT, OutCfg<N * TERMS>::SMEM, s, S->w2, tmd, o));
+  H->launches += 2;
+  return TARDIS_OK;
+}
+
+// 1 .. 128 tokens.  Corrections keep two bf16 terms up to 16 tokens, as on the fused path that serves smaller calls.
+tardis_status_t launch_few_forward(Handle* H, const void* xv, void* yv, int n, const float* smaxrow, cudaStream_t s) {
+  const __nv_bfloat16* x = static_cast<const __nv_bfloat16*>(xv);
+  __nv_bfloat16* y = static_cast<__nv_bfloat16*>(yv);
+  if (n <= 16) return launch_n<16, 2>(H, x, y, n, smaxrow, s);
+  if (n <= 32) return launch_n<32, 1>(H, x, y, n, smaxrow, s);
+  if (n <= 64) return launch_n<64, 1>(H, x, y, n, smaxrow, s);
+  return launch_n<128, 1>(H, x, y, n, smaxrow, s);
+}
+
+}  // namespace tardis

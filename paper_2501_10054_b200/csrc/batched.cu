@@ -45,42 +45,43 @@ struct State {
 
 // ---- set-up ---------------------------------------------------------------------------------------------
 // What = s (q - zp) split exactly into hi = bf16(What) and lo = What - hi (at most 2 significant bits left).
+// A row per CTA; a thread takes 8 channels (one group: groups are multiples of 16 channels) and writes 16 bytes of either matrix.
 __global__ void k_dequant_split(const uint32_t* __restrict__ codes, const __nv_bfloat16* __restrict__ scale,
                                 const uint8_t* __restrict__ zero, __nv_bfloat16* __restrict__ hi,
                                 __nv_bfloat16* __restrict__ lo, float* __restrict__ smaxrow, uint32_t* __restrict__ lo_used, int d, int G, int bits) {
+  __shared__ float wmax[8];
   bool rest = false;                            // any of this thread's values has a second term
-  const int per = 32 / bits;                    // codes per word
-  const uint32_t cmask = (1u << bits) - 1u;
-  const int j = blockIdx.x, ng = d / G, nwords = d / per;
-  if (32 % bits) {                              // 3-bit codes: a bit stream, channel by channel
-    const uint32_t* row = codes + size_t(j) * (size_t(d) * bits / 32);
-    for (int k = threadIdx.x; k < d; k += blockDim.x) {
-      const int g = k / G;
-      const float v = __bfloat162float(scale[size_t(j) * ng + g]) * (float(stream_code(row, k, bits)) - float(zero[size_t(j) * ng + g]));
-      const __nv_bfloat16 h = __float2bfloat16_rn(v);
-      hi[size_t(j) * d + k] = h;
-      lo[size_t(j) * d + k] = __float2bfloat16_rn(v - __bfloat162float(h));
-      rest |= v != __bfloat162float(h);
+  float smax = 0.f;
+  const int j = blockIdx.x, ng = d / G;
+  const uint32_t* row = codes + size_t(j) * (size_t(d) * bits / 32);
+  for (int k0 = threadIdx.x * 8; k0 < d; k0 += blockDim.x * 8) {
+    const int g = k0 / G;
+    const float s = __bfloat162float(scale[size_t(j) * ng + g]), zp = float(zero[size_t(j) * ng + g]);
+    smax = fmaxf(smax, fabsf(s));
+    __nv_bfloat162 h[4], l[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      float v[2], t[2];
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        v[e] = s * (float(stream_code(row, k0 + 2 * q + e, bits)) - zp);   // exact: 8-bit significand times |int| <= 15
+        t[e] = __bfloat162float(__float2bfloat16_rn(v[e]));
+        rest |= v[e] != t[e];
+      }
+      h[q] = __floats2bfloat162_rn(t[0], t[1]);
+      l[q] = __floats2bfloat162_rn(v[0] - t[0], v[1] - t[1]);
     }
-  }
-  for (int w = threadIdx.x; w < nwords && 32 % bits == 0; w += blockDim.x) {
-    const uint32_t word = codes[size_t(j) * nwords + w];
-    const int g = (w * per) / G;
-    const float s = __bfloat162float(scale[size_t(j) * ng + g]);
-    const float zp = float(zero[size_t(j) * ng + g]);
-    for (int q = 0; q < per; ++q) {
-      const float v = s * (float((word >> (bits * q)) & cmask) - zp);   // exact: 8-bit significand times |int| <= 15
-      const __nv_bfloat16 h = __float2bfloat16_rn(v);
-      hi[size_t(j) * d + w * per + q] = h;
-      lo[size_t(j) * d + w * per + q] = __float2bfloat16_rn(v - __bfloat162float(h));
-      rest |= v != __bfloat162float(h);
-    }
+    *reinterpret_cast<uint4*>(hi + size_t(j) * d + k0) = *reinterpret_cast<const uint4*>(h);
+    *reinterpret_cast<uint4*>(lo + size_t(j) * d + k0) = *reinterpret_cast<const uint4*>(l);
   }
   if (rest) lo_used[j >> 7] = 1u;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) smax = fmaxf(smax, __shfl_xor_sync(0xffffffffu, smax, o));
+  if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = smax;
+  __syncthreads();
   if (threadIdx.x == 0) {
-    float m = 0.f;
-    for (int g = 0; g < ng; ++g) m = fmaxf(m, fabsf(__bfloat162float(scale[size_t(j) * ng + g])));
-    smaxrow[j] = m;
+    for (int w = 1; w < (blockDim.x >> 5); ++w) smax = fmaxf(smax, wmax[w]);
+    smaxrow[j] = smax;
   }
 }
 

@@ -728,6 +728,23 @@ __global__ void k_pack(const uint32_t* __restrict__ codes, const __nv_bfloat16* 
         j < h ? (uint32_t(__bfloat16_as_ushort(scale[size_t(j) * ng + g])) << 16) | (zero[size_t(j) * ng + g] & 3u) : 0u;
 }
 
+// The shares of the folded product (end of each CTA's) and, per output tile, how many CTAs of k_few_out contribute to it (those that
+// hold its first to its last pair), put where the kernels read them.
+constexpr int MAX_GRID = 256;
+struct Shares { int end[MAX_GRID]; };
+__global__ void k_plan(const Shares shares, int2* plan, int grid, unsigned int* parts, int mtiles, int nkb, int out_grid) {
+  for (int c = threadIdx.x; c < grid; c += blockDim.x) plan[c] = make_int2(c ? shares.end[c - 1] : 0, shares.end[c]);
+  const long long total = (long long)mtiles * nkb;
+  auto owner = [&](long long pair) {                       // the CTA c with total c / out_grid <= pair < total (c + 1) / out_grid
+    int c = int(pair * out_grid / total);
+    while (total * (c + 1) / out_grid <= pair) ++c;
+    while (total * c / out_grid > pair) --c;
+    return c;
+  };
+  for (int m = threadIdx.x; m < mtiles; m += blockDim.x)
+    parts[m] = unsigned(owner((long long)(m + 1) * nkb - 1) - owner((long long)m * nkb) + 1);
+}
+
 struct State {
   uint4* codes; uint32_t *meta, *two_terms; int2* plan; float* yacc; unsigned int *nfl, *done, *parts;
   __nv_bfloat16* delta;
@@ -777,7 +794,7 @@ tardis_status_t few_prepare(Handle* H) {
   if (!S) return TARDIS_ERR_ALLOC;
   memset(S, 0, sizeof(*S));
   H->few = S;
-  S->grid = H->num_sms;
+  S->grid = std::min(H->num_sms, MAX_GRID);
   const int rounds = (h + S->grid * BM - 1) / (S->grid * BM), share = (h + S->grid * rounds - 1) / (S->grid * rounds);
   S->rows = std::min(BM, std::max(16, (share + 7) / 8 * 8));          // every CTA gets the same number of tiles, or one less
   S->nkb = d / BK; S->ntiles = (h + S->rows - 1) / S->rows; S->mtiles = (d + BM - 1) / BM; S->out_nkb = (h + BK - 1) / BK;
@@ -809,18 +826,11 @@ tardis_status_t few_finish(Handle* H, const void* W2, const void* Wf, cudaStream
   }
   std::vector<int2> plan(S->grid);
   deal_folded_blocks(*S, plan);
-  S->out_grid = std::max(1, std::min(H->num_sms, S->mtiles * S->out_nkb / 4));
-  // CTAs that contribute to an output tile (the shares of k_few_out)
-  const long long total = (long long)S->mtiles * S->out_nkb;
-  std::vector<unsigned int> parts(S->mtiles, 0u);
-  for (int c = 0; c < S->out_grid; ++c) {
-    const long long b = total * c / S->out_grid, e = total * (c + 1) / S->out_grid;
-    for (long long m = b / S->out_nkb; m * S->out_nkb < e; ++m) parts[m] += 1u;
-  }
+  S->out_grid = std::max(1, std::min(S->grid, S->mtiles * S->out_nkb / 4));
   TARDIS_CUDA_TRY(cudaMemsetAsync(S->nfl, 0, sizeof(unsigned int) * (MAX_TOKENS + 2 * S->mtiles + S->ntiles), s));
-  TARDIS_CUDA_TRY(cudaMemcpyAsync(S->plan, plan.data(), sizeof(int2) * S->grid, cudaMemcpyHostToDevice, s));
-  TARDIS_CUDA_TRY(cudaMemcpyAsync(S->parts, parts.data(), sizeof(unsigned int) * S->mtiles, cudaMemcpyHostToDevice, s));
-  TARDIS_CUDA_TRY(cudaStreamSynchronize(s));           // (the host buffers go away with this call)
+  Shares shares;
+  for (int c = 0; c < S->grid; ++c) shares.end[c] = plan[c].y;
+  k_plan<<<1, 256, 0, s>>>(shares, S->plan, S->grid, S->parts, S->mtiles, S->out_nkb, S->out_grid);
   TARDIS_CUDA_TRY(cudaMemsetAsync(S->yacc, 0, sizeof(float) * MAX_TOKENS * d, s));
   k_pack<<<dim3(S->ntiles, 8), S->rows, 0, s>>>(H->codes, static_cast<const __nv_bfloat16*>(H->scale), H->zero, S->codes, S->meta, S->two_terms,
                                                 S->rows, d, h, H->G, S->nkb);

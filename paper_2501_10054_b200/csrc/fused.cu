@@ -30,7 +30,6 @@
 #include <stdio.h>
 
 #include <new>
-#include <vector>
 
 #include "common.cuh"
 #include "exact.cuh"
@@ -1034,6 +1033,12 @@ __global__ void k_pack_folded(const __nv_bfloat16* __restrict__ C, uint4* __rest
   }
 }
 
+// tiles spread evenly over the CTAs: first tile and number of tiles of each
+__global__ void k_even_plan(int2* plan, int tiles, int grid) {
+  const int q = tiles / grid, r = tiles % grid;
+  for (int c = threadIdx.x; c < grid; c += blockDim.x) plan[c] = make_int2(c * q + min(c, r), q + (c < r ? 1 : 0));
+}
+
 __global__ void k_max_scale(const __nv_bfloat16* __restrict__ scale, size_t count, float* out) {
   float m = 0.f;
   for (size_t e = size_t(blockIdx.x) * blockDim.x + threadIdx.x; e < count; e += size_t(gridDim.x) * blockDim.x)
@@ -1107,16 +1112,8 @@ tardis_status_t fused_prepare(Handle* H, cudaStream_t s) {
   if (e != cudaSuccess) { set_last_error(e, "cudaMalloc"); cudaGetLastError(); return fail(TARDIS_ERR_ALLOC); }
   S->bytes = tally;
 
-  // tiles spread evenly over the CTAs
-  std::vector<int2> plan(grid);
-  int tile_cum = 0;
-  for (int c = 0; c < grid; ++c) {
-    const int tc = NT / grid + (c < NT % grid ? 1 : 0);
-    plan[c] = make_int2(tile_cum, tc);
-    tile_cum += tc;
-  }
-  e = cudaMemcpyAsync(S->plan, plan.data(), sizeof(int2) * grid, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);   // plan.data() is a stack-owned host buffer
+  k_even_plan<<<1, 256, 0, s>>>(S->plan, NT, grid);
+  e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaMemsetAsync(S->smax, 0, 16, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(S->yacc, 0, yacc_bytes, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(S->ctl, 0, sizeof(unsigned int) * CTL_WORDS, s);

@@ -337,6 +337,15 @@ def test_build_predictor_matches_oracle(h, d, G, bits, dt):
     _build_and_compare(W0, _upper_factor(X), bits, G)
 
 
+@pytest.mark.parametrize("h,d,G", [(129, 576, 192), (17, 768, 256), (16, 640, 640), (255, 1152, 64), (130, 896, 448)])
+def test_build_predictor_groups_and_superblocks(h, d, G):
+    # groups that divide the superblock of 256 channels, that are one (192, 448), that are too large for one (640); the last
+    # superblock short; neurons one more and one less than the CTAs' tiles
+    g = torch.Generator().manual_seed(h)
+    W1 = (torch.randn(h, d, generator=g) * 0.02).cuda()
+    _build_and_compare(W1, _upper_factor(torch.randn(2 * d, d, generator=g).numpy()), 2, G)
+
+
 def test_build_predictor_full_size_sampled_rows_and_use_in_a_layer():
     """The 7B-class layer (16384 x 4096, groups of 128, 2 bits): sampled neurons against the oracle (neurons are independent
     given U), then the built predictor goes into tardis_fold and a forward is compared with the oracle run on those codes."""

@@ -530,3 +530,36 @@ def test_save_and_load_round_trip(tmp_path, dtype):
     assert lib.tardis_load(bad.encode(), None, ctypes.byref(out)) == 6 and out.value is None
     open(bad, "wb").write(raw[:len(raw) // 3])
     assert lib.tardis_load(bad.encode(), None, ctypes.byref(out)) == 6 and out.value is None
+
+
+def test_buffers_of_destroyed_layers_are_taken_over_by_new_ones():
+    """Freed buffers wait for the next allocation of their size: layers folded, used and destroyed in turn by two threads on
+    streams of their own give the results of a layer folded alone, and nothing stays registered as alive."""
+    import threading
+    cfgs = [W.LayerConfig("pool%d" % i, 512, 2048, n_calib=256, bias=bool(i)) for i in range(2)]
+    Ls = [_layer(c, i) for i, c in enumerate(cfgs)]
+    x = W.make_tokens(cfgs[0], 9, 5).cuda()
+    want, live0 = [], T.tardis_debug_live_allocations()
+    for L in Ls:
+        h = T.fold_layer(L)
+        want.append(T.tardis_ffn_forward(h, x, torch.empty_like(x)).clone())
+        torch.cuda.synchronize()
+        T.tardis_destroy(h)
+    bad = []
+
+    def work(i):
+        s = torch.cuda.Stream()
+        with torch.cuda.stream(s):
+            for _ in range(6):
+                h = T.fold_layer(Ls[i])
+                y = T.tardis_ffn_forward(h, x, torch.empty_like(x))
+                s.synchronize()
+                if not (y.float() - want[i].float()).abs().max() <= 2e-2 * want[i].float().abs().max() or T.tardis_stats(h)["device_error"]:
+                    bad.append(i)
+                T.tardis_destroy(h)
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad and T.tardis_debug_live_allocations() == live0

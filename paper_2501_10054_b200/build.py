@@ -11,7 +11,7 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libtardis.so")
 LIB_STAMPS = os.path.join(PKG, "libtardis_stamps.so")
-SOURCES = ["api.cu", "fold.cu", "generic.cu", "decode.cu", "fused.cu", "gemm.cu", "batched.cu", "few.cu", "calibrate.cu", "stack.cu", "gptq.cu"]
+SOURCES = ["api.cu", "fold.cu", "generic.cu", "decode.cu", "fused.cu", "gemm.cu", "batched.cu", "few.cu", "f32.cu", "calibrate.cu", "stack.cu", "gptq.cu"]
 
 
 def nvcc_path() -> str:

@@ -173,6 +173,7 @@ static tardis_status_t dev_alloc(T** p, size_t count, size_t* tally) {
 static void free_all(Handle* H) {
   fused_release(H);
   decode_release(H);
+  f32_release(H);
   few_release(H);
   batched_release(H);
   void* ptrs[] = {H->W1, H->W2T, H->C, H->bf, H->lo, H->hi, H->a, H->c, H->b1, H->codes, H->scale,
@@ -264,6 +265,7 @@ tardis_status_t tardis_fold(const tardis_fold_desc_t* desc, tardis_stream_t stre
   if (st == TARDIS_OK && bf16) st = fused_prepare(H, s);
   if (st == TARDIS_OK && bf16 && !H->fscratch) st = decode_prepare(H, s);   // wider layers: the older per-token kernel
   if (st == TARDIS_OK && bf16) st = batched_finish(H, desc->W2, s);
+  if (st == TARDIS_OK) st = f32_prepare(H, s);
   if (st != TARDIS_OK) { cudaStreamSynchronize(s); free_all(H); return st; }
   *out = reinterpret_cast<tardis_handle_t>(H);
   return TARDIS_OK;
@@ -297,7 +299,8 @@ tardis_status_t tardis_ffn_forward(tardis_handle_t handle, const void* x, void* 
     st = launch_batched_forward(H, x, y, n_tokens, s);
     H->last_path = 3;
   } else {
-    st = launch_generic_forward(H, x, y, n_tokens, s);
+    // fp32 layers have kernels of their own, which the choice of the generic ones (1) and the exact-range mode (4) leave aside
+    st = H->f32 && H->path_override != 1 && H->path_override != 4 ? launch_f32_forward(H, x, y, n_tokens, s) : launch_generic_forward(H, x, y, n_tokens, s);
     H->last_path = 1;
   }
   if (st == TARDIS_OK) { H->calls += 1; H->tokens += uint64_t(n_tokens); }
@@ -545,6 +548,7 @@ tardis_status_t tardis_load(const char* path, tardis_stream_t stream, tardis_han
   if (st == TARDIS_OK && bf16) st = fused_prepare(H, s);
   if (st == TARDIS_OK && bf16 && !H->fscratch) st = decode_prepare(H, s);
   if (st == TARDIS_OK && bf16) st = batched_finish(H, nullptr, s);
+  if (st == TARDIS_OK) st = f32_prepare(H, s);
   if (st != TARDIS_OK) { cudaStreamSynchronize(s); free_all(H); return st; }
   *out = reinterpret_cast<tardis_handle_t>(H);
   return TARDIS_OK;

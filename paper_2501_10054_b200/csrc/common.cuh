@@ -44,6 +44,7 @@ struct Handle {
   void* dscratch;        // fused decode scratch (see decode.cu)
   size_t dscratch_bytes;
   void* bstate;          // batched / prefill state and scratch (see batched.cu); null when not built
+  void* f32;             // state of the kernels for fp32 layers (see f32.cu); null for other layers
   void* few;             // state of the kernels for a few to 128 tokens (see few.cu); null when not built
   // debug capture (caller-owned)
   uint32_t* dbg_bitmap;
@@ -99,6 +100,9 @@ tardis_status_t few_prepare(Handle* H);                                       //
 tardis_status_t few_finish(Handle* H, const void* W2, const void* Wf, cudaStream_t s);   // fills its state (W2 [d, h], W_f [d, d] row-major)
 tardis_status_t launch_few_forward(Handle* H, const void* x, void* y, int n, const float* smaxrow, cudaStream_t s);
 void few_release(Handle* H);
+tardis_status_t f32_prepare(Handle* H, cudaStream_t s);                        // f32.cu (fp32 layers only)
+tardis_status_t launch_f32_forward(Handle* H, const void* x, void* y, int64_t n, cudaStream_t s);
+void f32_release(Handle* H);
 tardis_status_t launch_stack_forward(const tardis_stack_desc_t* desc, const void* x, void* y, void* work, void* keep, int64_t n,
                                      cudaStream_t s);   // stack.cu; arguments checked by the caller
 tardis_status_t launch_build_predictor(int h, int d, int dtype, const void* W1, const double* U, int bits, int G, uint32_t* codes,

@@ -3,21 +3,21 @@
 // Calls on such layers are small (256 / 1024 and 64 tokens: 50 MFLOP, 2.6 MB), so latency and launches are what counts; six
 // launches of the generic kernels, the predictor among them with the tokens one after the other, took 284 us there.
 //
-//   k_f32_in: a CTA takes 32 neurons and 16 (or 4) tokens: predictor scores from the packed codes, flags, and for the flagged
+//   k_f32_in: a CTA takes 32 neurons and 16 (or 8) tokens: predictor scores from the packed codes, flags, and for the flagged
 //     pairs the exact pre-activation and its correction, written to a dense [token][neuron] array (zero where not flagged).
 //   k_f32_out: y = b_f + [C ; W2^T]^T [x ; corrections], one product over d + h channels; its channel range is split over the
 //     CTAs, partial sums go to places of their own, and the CTA that finishes a tile last adds them in order and writes y.
 //
-// Both products: a warp holds the 32 outputs x 16 tokens of the CTA (a thread 4 x 4) for every eighth channel of the range, so
-// that four 128-bit reads of shared memory serve sixteen fp64 multiply-adds; the eight warps' sums meet in shared memory.
-// Bound by the fp64 pipe beyond a few hundred tokens of the larger layers.
+// Both products run on the fp64 matrix instruction (m16n8k8: 5 multiply-adds per value read; one output and all tokens per
+// thread, with the tokens broadcast from shared memory, is bound four times over by those reads).  A warp has 32 outputs and a
+// slice of 16 of the 128 channels of a pass; weights go from global memory into registers, which are the A operand; the tokens,
+// widened once, are read from shared memory as the B operand; the eight warps' sums meet in shared memory at the end.
 #include <string.h>
 
 #include <algorithm>
 #include <new>
 
 #include "common.cuh"
-#include "exact.cuh"
 
 namespace tardis {
 namespace f32 {
@@ -42,42 +42,48 @@ struct Params {
 struct State { float* delta; double* part; unsigned int* words; size_t ndone; };
 
 template <int TT> struct Smem {
-  double ws[KC][TM];                      // weights of a pass
-  double xs[KC][TT + 2];                  // tokens of a pass (two values of padding: the stores of a half-warp spread over the banks)
-  double red[NWARP][TT][TM];              // the warps' sums
+  union {
+    double xs[2][KC][TT + 4];             // tokens of a pass and the next (padded: four channels x eight tokens in different banks)
+    double red[NWARP][TT][TM];            // the warps' sums
+  };
 };
 
-template <int NTK> struct Acc { double v[4][NTK]; };
+// D += A B, A 16 x 8 (rows: outputs), B 8 x 8 (columns: tokens).  With g = lane / 4, t = lane % 4: a0..a3 = A[g][t], A[g + 8][t],
+// A[g][t + 4], A[g + 8][t + 4]; b0, b1 = B[t][g], B[t + 4][g]; c0..c3 = D[g][2t], D[g][2t + 1], D[g + 8][2t], D[g + 8][2t + 1].
+__device__ __forceinline__ void mma_f64(double (&c)[4], double a0, double a1, double a2, double a3, double b0, double b1) {
+  asm("mma.sync.aligned.m16n8k8.row.col.f64.f64.f64.f64 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+d"(c[0]), "+d"(c[1]), "+d"(c[2]), "+d"(c[3]) : "d"(a0), "d"(a1), "d"(a2), "d"(a3), "d"(b0), "d"(b1));
+}
 
-// one pass: every eighth channel (of nk) of the staged weights and tokens into the warp's 32 x 4 NTK outputs
-template <int NTK> __device__ __forceinline__ void accumulate(Acc<NTK>& acc, const Smem<4 * NTK>& sm, int nk, int warp, int lane) {
-  const int mo = (lane & 7) * 4, to = (lane >> 3) * NTK;
-#pragma unroll 4
-  for (int k = warp; k < nk; k += NWARP) {
-    const double2 w0 = *reinterpret_cast<const double2*>(&sm.ws[k][mo]), w1 = *reinterpret_cast<const double2*>(&sm.ws[k][mo + 2]);
-    const double w[4] = {w0.x, w0.y, w1.x, w1.y};
-    double x[NTK];
-    if (NTK == 4) {
-      const double2 x0 = *reinterpret_cast<const double2*>(&sm.xs[k][to]), x1 = *reinterpret_cast<const double2*>(&sm.xs[k][to + 2]);
-      x[0] = x0.x; x[1 % NTK] = x0.y; x[2 % NTK] = x1.x; x[3 % NTK] = x1.y;
-    } else {
-      x[0] = sm.xs[k][to];
-    }
+// A warp's 32 outputs x TT tokens.  Output 4 g + m of the CTA's 32 is row g (m even) or g + 8 (m odd) of row tile m / 2.
+template <int TT> struct Acc {
+  double c[2][TT / 8][4];
+  // channels of the slice: w[s][m] = weight of channel t + 4 s and output 4 g + m
+  __device__ __forceinline__ void multiply(const double (&w)[4][4], const double (*x)[TT + 4], int g, int t) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int k8 = 0; k8 < 2; ++k8)
 #pragma unroll
-      for (int t = 0; t < NTK; ++t) acc.v[i][t] += w[i] * x[t];
+      for (int nt = 0; nt < TT / 8; ++nt) {
+        const double b0 = x[k8 * 8 + t][nt * 8 + g], b1 = x[k8 * 8 + t + 4][nt * 8 + g];
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt)
+          mma_f64(c[mt][nt], w[2 * k8][2 * mt], w[2 * k8][2 * mt + 1], w[2 * k8 + 1][2 * mt], w[2 * k8 + 1][2 * mt + 1], b0, b1);
+      }
   }
-}
-
-// the eight warps' sums -> red; afterwards sum_of gives an output's total (after a barrier)
-template <int NTK> __device__ __forceinline__ void put(const Acc<NTK>& acc, Smem<4 * NTK>& sm, int warp, int lane) {
-  const int mo = (lane & 7) * 4, to = (lane >> 3) * NTK;
+  // the eight warps' sums of an output meet (sum_of after this)
+  __device__ __forceinline__ void put(Smem<TT>& sm, int warp, int g, int t) const {
+    __syncthreads();
 #pragma unroll
-  for (int t = 0; t < NTK; ++t)
+    for (int nt = 0; nt < TT / 8; ++nt)
 #pragma unroll
-    for (int i = 0; i < 4; i += 2) *reinterpret_cast<double2*>(&sm.red[warp][to + t][mo + i]) = make_double2(acc.v[i][t], acc.v[i + 1][t]);
-}
+      for (int e = 0; e < 2; ++e) {
+        double* const at = &sm.red[warp][nt * 8 + 2 * t + e][4 * g];
+        *reinterpret_cast<double2*>(at) = make_double2(c[0][nt][e], c[0][nt][2 + e]);
+        *reinterpret_cast<double2*>(at + 2) = make_double2(c[1][nt][e], c[1][nt][2 + e]);
+      }
+    __syncthreads();
+  }
+};
 template <int TT> __device__ __forceinline__ double sum_of(const Smem<TT>& sm, int t, int m) {
   double s = 0.0;
 #pragma unroll
@@ -85,17 +91,31 @@ template <int TT> __device__ __forceinline__ double sum_of(const Smem<TT>& sm, i
   return s;
 }
 
-// tokens t0 .. t0 + TT - 1 at channels k0 .. k0 + KC - 1 of a [n][ld] array (zero outside) -> xs
-template <int TT> __device__ __forceinline__ void stage_tokens(Smem<TT>& sm, const float* __restrict__ src, size_t ld, int n, int t0, int k0, int kend) {
-  for (int e = threadIdx.x; e < TT * KC; e += NT) {
-    const int kk = e & (KC - 1), t = e / KC;
-    sm.xs[kk][t] = (t0 + t < n && k0 + kk < kend) ? double(src[size_t(t0 + t) * ld + k0 + kk]) : 0.0;
+// Tokens t0 .. t0 + TT - 1 at channels k0 .. k0 + KC - 1 of a [n][ld] array (zero outside): loaded into registers while the pass
+// before is multiplied (a pass that waits for its own loads takes 3 us, mostly for them), then widened into xs.
+template <int TT> struct Tokens {
+  float4 v[TT * KC / 4 / NT];                              // token e % TT, channels 4 (e / TT) .. + 3
+  __device__ __forceinline__ void load(const float* __restrict__ src, size_t ld, int n, int t0, int k0, int kend) {
+#pragma unroll
+    for (int q = 0; q < TT * KC / 4 / NT; ++q) {
+      const int e = q * NT + threadIdx.x, t = e % TT, k = k0 + e / TT * 4;
+      v[q] = (t0 + t < n && k < kend) ? *reinterpret_cast<const float4*>(src + size_t(t0 + t) * ld + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
   }
-}
+  __device__ __forceinline__ void store(Smem<TT>& sm, int buffer) const {
+#pragma unroll
+    for (int q = 0; q < TT * KC / 4 / NT; ++q) {
+      const int e = q * NT + threadIdx.x, t = e % TT, k = e / TT * 4;
+      sm.xs[buffer][k][t] = double(v[q].x);
+      sm.xs[buffer][k + 1][t] = double(v[q].y);
+      sm.xs[buffer][k + 2][t] = double(v[q].z);
+      sm.xs[buffer][k + 3][t] = double(v[q].w);
+    }
+  }
+};
 
-template <int BITS, int NTK>
+template <int BITS, int TT>
 __global__ void __launch_bounds__(NT) k_f32_in(const Params p) {
-  constexpr int TT = 4 * NTK;
   extern __shared__ __align__(16) unsigned char raw[];
   Smem<TT>& sm = *reinterpret_cast<Smem<TT>*>(raw);
   __shared__ int pairs[TT * TM];
@@ -104,40 +124,58 @@ __global__ void __launch_bounds__(NT) k_f32_in(const Params p) {
   const int j0 = blockIdx.x * TM, t0 = blockIdx.y * TT, ng = p.d / p.G;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (threadIdx.x == 0) npairs = 0;
-  Acc<NTK> acc = {};
-  bool waited = false;
-  for (int k0 = 0; k0 < p.d; k0 += KC) {
-    __syncthreads();
-    {
-      // a thread expands 16 channels (one group: groups are multiples of 16) of neuron `lane`: s (q - zp), exact in fp64
-      const int j = j0 + lane, kb = k0 + warp * 16;
+  Acc<TT> acc = {};
+  Tokens<TT> x;
+  // a thread expands four channels of four neurons (all of one group: groups are multiples of 16): s (q - zp), exact in fp64
+  const int g = lane >> 2, t4 = lane & 3;
+  uint32_t w[4][BITS == 8 ? 4 : 2];
+  float sc[4], zp[4];
+  auto load_codes = [&](int k0) {
+    const int kb = k0 + warp * 16;
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      const size_t j = j0 + 4 * g + m;
+      sc[m] = zp[m] = 0.f;
       if (kb < p.d) {
-        const double s = double(p.scale[size_t(j) * ng + kb / p.G]), zp = 4503599627370496.0 + double(p.zero[size_t(j) * ng + kb / p.G]);
-        const uint32_t* row = p.codes + size_t(j) * (size_t(p.d) * BITS / 32);
-        uint32_t w[4] = {0u, 0u, 0u, 0u};
-        if (BITS != 3) {
+        sc[m] = p.scale[j * ng + kb / p.G];
+        zp[m] = float(p.zero[j * ng + kb / p.G]);
+        const uint32_t* const row = p.codes + j * (size_t(p.d) * BITS / 32);
+        if (BITS == 3) {                                   // 48 bits from a half-word on
+          const uint16_t* at = reinterpret_cast<const uint16_t*>(row) + kb * 3 / 16;
+          w[m][0] = uint32_t(at[0]) | uint32_t(at[1]) << 16;
+          w[m][1] = at[2];
+        } else {
 #pragma unroll
-          for (int q = 0; q < BITS / 2; ++q) w[q] = row[kb * BITS / 32 + q];
+          for (int q = 0; q < BITS / 2; ++q) w[m][q] = row[kb * BITS / 32 + q];
         }
-#pragma unroll
-        for (int c = 0; c < 16; ++c) {
-          const uint32_t q = BITS == 3 ? (kb + c < p.d ? stream_code(row, kb + c, 3) : 0u) : (w[c * BITS / 32] >> (c * BITS % 32)) & ((1u << BITS) - 1u);
-          // (2^52 + q) - (2^52 + zp): the code as a double without a conversion
-          const double v = __hiloint2double(0x43300000, int(q)) - zp;
-          sm.ws[warp * 16 + c][lane] = kb + c < p.d ? s * v : 0.0;
-        }
-      } else {
-#pragma unroll
-        for (int c = 0; c < 16; ++c) sm.ws[warp * 16 + c][lane] = 0.0;
       }
     }
-    if (!waited) { asm volatile("griddepcontrol.wait;" ::: "memory"); waited = true; }   // (x may come from the launch before)
-    stage_tokens<TT>(sm, p.x, p.d, p.n, t0, k0, p.d);
-    __syncthreads();
-    accumulate<NTK>(acc, sm, min(KC, p.d - k0), warp, lane);
+  };
+  load_codes(0);
+  asm volatile("griddepcontrol.wait;" ::: "memory");       // (x may come from the launch before)
+  x.load(p.x, p.d, p.n, t0, 0, p.d);
+  int buffer = 0;
+  for (int k0 = 0; k0 < p.d; k0 += KC, buffer ^= 1) {
+    x.store(sm, buffer);
+    double v[4][4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      const double s = double(sc[m]), z = 4503599627370496.0 + double(zp[m]);
+#pragma unroll
+      for (int q4 = 0; q4 < 4; ++q4) {
+        const int c = q4 * 4;                              // channel c + t4
+        uint32_t q;
+        if (BITS == 3) q = uint32_t((uint64_t(w[m][0]) | uint64_t(w[m][1]) << 32) >> (3 * (c + t4))) & 7u;
+        else q = (w[m][c * BITS / 32] >> ((c * BITS) % 32 + t4 * BITS)) & ((1u << BITS) - 1u);
+        // (2^52 + q) - (2^52 + zp): the code as a double without a conversion
+        v[q4][m] = s * (__hiloint2double(0x43300000, int(q)) - z);
+      }
+    }
+    __syncthreads();                                       // (a buffer is written again two passes on, behind this barrier)
+    if (k0 + KC < p.d) { load_codes(k0 + KC); x.load(p.x, p.d, p.n, t0, k0 + KC, p.d); }
+    acc.multiply(v, &sm.xs[buffer][warp * 16], g, t4);
   }
-  put<NTK>(acc, sm, warp, lane);
-  __syncthreads();
+  acc.put(sm, warp, g, t4);
   // scores -> flags; lane = neuron, a warp takes tokens warp, warp + 8, ...
   const int j = j0 + lane;
   const double lo = double(p.lo[j]), hi = double(p.hi[j]), b1 = double(p.b1[j]);
@@ -167,15 +205,16 @@ __global__ void __launch_bounds__(NT) k_f32_in(const Params p) {
     const int pr = pairs[min(e, np - 1)], jj = j0 + (pr & (TM - 1)), t = t0 + pr / TM;
     const float* row = p.W1 + size_t(jj) * p.d;
     const float* xt = p.x + size_t(t) * p.d;
-    double z = 0.0;
-#pragma unroll 4
+    double z0 = 0.0, z1 = 0.0, z2 = 0.0, z3 = 0.0;         // (four chains: the latency of one would be most of the time)
+#pragma unroll 8
     for (int k = sub * 4; k < p.d; k += 32) {              // (d is a multiple of 8, rows are 16-byte aligned)
       const float4 w = *reinterpret_cast<const float4*>(row + k), v = *reinterpret_cast<const float4*>(xt + k);
-      z += double(w.x) * double(v.x);
-      z += double(w.y) * double(v.y);
-      z += double(w.z) * double(v.z);
-      z += double(w.w) * double(v.w);
+      z0 += double(w.x) * double(v.x);
+      z1 += double(w.y) * double(v.y);
+      z2 += double(w.z) * double(v.z);
+      z3 += double(w.w) * double(v.w);
     }
+    double z = (z0 + z1) + (z2 + z3);
 #pragma unroll
     for (int o = 4; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
     if (sub == 0 && e < np) {
@@ -185,9 +224,8 @@ __global__ void __launch_bounds__(NT) k_f32_in(const Params p) {
   }
 }
 
-template <int NTK>
+template <int TT>
 __global__ void __launch_bounds__(NT) k_f32_out(const Params p) {
-  constexpr int TT = 4 * NTK;
   extern __shared__ __align__(16) unsigned char raw[];
   Smem<TT>& sm = *reinterpret_cast<Smem<TT>*>(raw);
   __shared__ bool last;
@@ -196,25 +234,38 @@ __global__ void __launch_bounds__(NT) k_f32_out(const Params p) {
   const int passes_d = (p.d + KC - 1) / KC, passes = passes_d + (p.h + KC - 1) / KC;   // C first, then W2^T
   const int from = int((long long)passes * z / p.splits), to = int((long long)passes * (z + 1) / p.splits);
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  Acc<NTK> acc = {};
-  bool waited = false;
-  for (int ps = from; ps < to; ++ps) {
+  Acc<TT> acc = {};
+  Tokens<TT> x;
+  const int g = lane >> 2, t4 = lane & 3;
+  float4 w[4];                                             // channels 16 warp + t4 + 4 s of outputs 4 g .. 4 g + 3
+  auto load_weights = [&](int ps) {
     const bool fold = ps < passes_d;
     const int k0 = (fold ? ps : ps - passes_d) * KC, kend = fold ? p.d : p.h;
-    const float* m = fold ? p.C : p.W2T;                   // both [channel][output]
-    __syncthreads();
-    for (int e = threadIdx.x; e < KC * TM; e += NT) {
-      const int i = e & (TM - 1), k = e / TM;
-      sm.ws[k][i] = (k0 + k < kend && i0 + i < p.d) ? double(m[size_t(k0 + k) * p.d + i0 + i]) : 0.0;
+    const float* m = (fold ? p.C : p.W2T) + i0 + 4 * g;    // both [channel][output]; d is a multiple of 8
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int k = k0 + warp * 16 + t4 + 4 * q;
+      w[q] = (k < kend && i0 + 4 * g < p.d) ? *reinterpret_cast<const float4*>(m + size_t(k) * p.d) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    if (!waited) { asm volatile("griddepcontrol.wait;" ::: "memory"); waited = true; }
-    stage_tokens<TT>(sm, fold ? p.x : p.delta, fold ? p.d : p.h, p.n, t0, k0, kend);
-    __syncthreads();
-    accumulate<NTK>(acc, sm, min(KC, kend - k0), warp, lane);
+  };
+  auto load_tokens = [&](int ps) {
+    const bool fold = ps < passes_d;
+    x.load(fold ? p.x : p.delta, fold ? p.d : p.h, p.n, t0, (fold ? ps : ps - passes_d) * KC, fold ? p.d : p.h);
+  };
+  load_weights(from);
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  load_tokens(from);
+  int buffer = 0;
+  for (int ps = from; ps < to; ++ps, buffer ^= 1) {
+    x.store(sm, buffer);
+    double v[4][4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) { v[q][0] = double(w[q].x); v[q][1] = double(w[q].y); v[q][2] = double(w[q].z); v[q][3] = double(w[q].w); }
+    __syncthreads();                                       // (a buffer is written again two passes on, behind this barrier)
+    if (ps + 1 < to) { load_weights(ps + 1); load_tokens(ps + 1); }
+    acc.multiply(v, &sm.xs[buffer][warp * 16], g, t4);
   }
-  if (!waited) asm volatile("griddepcontrol.wait;" ::: "memory");
-  put<NTK>(acc, sm, warp, lane);
-  __syncthreads();
+  acc.put(sm, warp, g, t4);
   const int i = i0 + lane;
   if (p.splits > 1) {
 #pragma unroll
@@ -253,6 +304,11 @@ __global__ void __launch_bounds__(NT) k_f32_out(const Params p) {
   }
 }
 
+using Kernel = void (*)(Params);
+template <int TT> static Kernel in_kernel(int bits) {
+  return bits == 2 ? k_f32_in<2, TT> : (bits == 3 ? k_f32_in<3, TT> : (bits == 4 ? k_f32_in<4, TT> : k_f32_in<8, TT>));
+}
+
 }  // namespace f32
 
 using namespace f32;
@@ -264,7 +320,7 @@ tardis_status_t f32_prepare(Handle* H, cudaStream_t s) {
   if (!S) return TARDIS_ERR_ALLOC;
   memset(S, 0, sizeof(*S));
   H->f32 = S;
-  S->ndone = size_t((H->d + TM - 1) / TM) * (MAX_CHUNK / 4);
+  S->ndone = size_t((H->d + TM - 1) / TM) * (MAX_CHUNK / 8);
   const size_t bytes[3] = {size_t(MAX_CHUNK) * H->h * 4, size_t(MAX_PARTS) * H->d * 8, (S->ndone + MAX_CHUNK) * 4};
   void** ptrs[3] = {reinterpret_cast<void**>(&S->delta), reinterpret_cast<void**>(&S->part), reinterpret_cast<void**>(&S->words)};
   for (int i = 0; i < 3; ++i) {
@@ -273,6 +329,11 @@ tardis_status_t f32_prepare(Handle* H, cudaStream_t s) {
     H->bytes_scratch += bytes[i];
   }
   TARDIS_CUDA_TRY(cudaMemsetAsync(S->words, 0, bytes[2], s));
+  const Kernel wide[2] = {in_kernel<16>(H->bits), k_f32_out<16>}, narrow[2] = {in_kernel<8>(H->bits), k_f32_out<8>};
+  for (int i = 0; i < 2; ++i) {
+    TARDIS_CUDA_TRY(cudaFuncSetAttribute(wide[i], cudaFuncAttributeMaxDynamicSharedMemorySize, int(sizeof(Smem<16>))));
+    TARDIS_CUDA_TRY(cudaFuncSetAttribute(narrow[i], cudaFuncAttributeMaxDynamicSharedMemorySize, int(sizeof(Smem<8>))));
+  }
   return TARDIS_OK;
 }
 
@@ -286,16 +347,13 @@ void f32_release(Handle* H) {
   H->f32 = nullptr;
 }
 
-template <int NTK> static tardis_status_t launch_chunk(const Handle* H, const Params& p, cudaStream_t s) {
-  using Kernel = void (*)(Params);
-  const Kernel in = H->bits == 2 ? k_f32_in<2, NTK> : (H->bits == 3 ? k_f32_in<3, NTK> : (H->bits == 4 ? k_f32_in<4, NTK> : k_f32_in<8, NTK>));
-  const int tiles = (p.n + 4 * NTK - 1) / (4 * NTK);
+template <int TT> static tardis_status_t launch_chunk(const Handle* H, const Params& p, cudaStream_t s) {
+  const int tiles = (p.n + TT - 1) / TT;
   const dim3 grids[2] = {dim3(p.h / TM, tiles), dim3((p.d + TM - 1) / TM, tiles, p.splits)};
-  const Kernel kernels[2] = {in, k_f32_out<NTK>};
+  const Kernel kernels[2] = {in_kernel<TT>(H->bits), k_f32_out<TT>};
   for (int i = 0; i < 2; ++i) {
-    TARDIS_CUDA_TRY(cudaFuncSetAttribute(kernels[i], cudaFuncAttributeMaxDynamicSharedMemorySize, int(sizeof(Smem<4 * NTK>))));
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grids[i]; cfg.blockDim = dim3(NT); cfg.dynamicSmemBytes = sizeof(Smem<4 * NTK>); cfg.stream = s;
+    cfg.gridDim = grids[i]; cfg.blockDim = dim3(NT); cfg.dynamicSmemBytes = sizeof(Smem<TT>); cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -318,10 +376,10 @@ tardis_status_t launch_f32_forward(Handle* H, const void* xv, void* yv, int64_t 
     p.dbg_bitmap = H->dbg_bitmap ? H->dbg_bitmap + size_t(t0) * (H->h / 32) : nullptr;
     p.dbg_scores = H->dbg_scores ? H->dbg_scores + size_t(t0) * H->h : nullptr;
     // parts of the split product: about two CTAs per SM, at least one pass of KC channels each, what the workspace holds
-    const int ntk = p.n <= 4 ? 1 : 4, tiles = ((p.d + TM - 1) / TM) * ((p.n + 4 * ntk - 1) / (4 * ntk));
+    const int tt = p.n <= 8 ? 8 : 16, tiles = ((p.d + TM - 1) / TM) * ((p.n + tt - 1) / tt);
     const int passes = (p.d + KC - 1) / KC + (p.h + KC - 1) / KC;
     p.splits = std::max(1, std::min({2 * H->num_sms / tiles, passes, MAX_PARTS / p.n, 64}));
-    const tardis_status_t st = ntk == 1 ? launch_chunk<1>(H, p, s) : launch_chunk<4>(H, p, s);
+    const tardis_status_t st = tt == 8 ? launch_chunk<8>(H, p, s) : launch_chunk<16>(H, p, s);
     if (st != TARDIS_OK) return st;
     H->launches += 2;
   }

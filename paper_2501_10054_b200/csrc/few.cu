@@ -60,8 +60,10 @@ struct OutParams {
 template <int N> struct InCfg {
   static constexpr int X_BYTES = N * BK * 2, STAGE = W_BYTES + X_BYTES;
   static constexpr int NS = N == 128 ? 5 : (N == 64 ? 4 : (N == 32 ? 5 : 6));
-  static constexpr int NBUF = 4;                                    // expanded predictor blocks in TMEM (32 columns each)
+  static constexpr int NBUF = N == 64 ? 2 : 4;                      // expanded predictor blocks in TMEM (32 columns each)
   static constexpr int COL_S = 0, COL_Z = N, COL_F = 2 * N, COL_A = 3 * N;
+  // A CTA that starts early must leave the columns that the launch before it still has to allocate on the same SM, or the two
+  // wait for each other: 256 of 512 up to 64 columns of tokens (k_few_out takes 128 at most).  With 128 it takes all, after the wait.
   static constexpr int TMEM = COL_A + NBUF * 32 <= 256 ? 256 : 512;
   static constexpr int SMEM = 1024 + NS * STAGE + 256 + MAX_NEAR * 16 + BM * ((N + 31) / 32) * 4 + N * 8 + 8 * 1024;
 };
@@ -232,8 +234,11 @@ k_few_in(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUten
   for (int i = threadIdx.x; i < BM * ((N + 31) / 32); i += NT_IN) settled[i] = 0u;
   if (threadIdx.x < N) tok_flagged[threadIdx.x] = 0u;
   __syncthreads();
-  // (warp 0 goes on with its copies: the allocation waits while the launch before holds too much of the SM's tensor memory)
-  if (warp == 1) tmem_alloc(tmem_slot, C::TMEM);
+  // (warp 0 goes on with its copies meanwhile)
+  if (warp == 1) {
+    if (C::TMEM > 256) pdl_wait();
+    tmem_alloc(tmem_slot, C::TMEM);
+  }
   if (warp != 0) {
     tc_fence_before();
     asm volatile("bar.sync 2, 352;" ::: "memory");
@@ -768,7 +773,7 @@ static void deal_folded_blocks(const State& S, std::vector<int2>& plan) {
     }
     return sum;
   };
-  double lo = 0.0, hi = per_tile * (S.ntiles / S.grid + 2) + blocks;
+  double lo = 0.0, hi = per_tile * (S.ntiles / S.grid + 2) + blocks + 8.0;      // (one CTA alone could take all)
   while (hi - lo > 1e-3) { const double mid = 0.5 * (lo + hi); (fill(mid) >= blocks ? hi : lo) = mid; }   // the level that holds all blocks
   const double sum = fill(hi);
   double cum = 0.0;
@@ -808,6 +813,12 @@ tardis_status_t few_prepare(Handle* H) {
     const cudaError_t e = dev_malloc(r.p, r.bytes);
     if (e != cudaSuccess) { set_last_error(e, "cudaMalloc"); cudaGetLastError(); few_release(H); return TARDIS_ERR_ALLOC; }
   }
+  auto room = [](auto kernel, int smem) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); };
+  const cudaError_t es[] = {room(k_few_in<16, 2>, InCfg<16>::SMEM), room(k_few_in<32, 1>, InCfg<32>::SMEM), room(k_few_in<64, 1>, InCfg<64>::SMEM),
+                            room(k_few_in<128, 1>, InCfg<128>::SMEM), room(k_few_out<32>, OutCfg<32>::SMEM), room(k_few_out<64>, OutCfg<64>::SMEM),
+                            room(k_few_out<128>, OutCfg<128>::SMEM)};
+  for (cudaError_t e : es)
+    if (e != cudaSuccess) { set_last_error(e, "cudaFuncSetAttribute"); few_release(H); return TARDIS_ERR_CUDA; }
   S->done = S->nfl + MAX_TOKENS;
   S->parts = S->done + S->mtiles;
   S->two_terms = S->parts + S->mtiles;
@@ -850,8 +861,6 @@ void few_release(Handle* H) {
 
 template <typename K, typename... Args>
 static cudaError_t launch_overlapped(K kernel, int grid, int threads, size_t smem, cudaStream_t s, const Args&... args) {
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid); cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = s;
   cudaLaunchAttribute attr[1];

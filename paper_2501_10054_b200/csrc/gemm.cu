@@ -367,14 +367,18 @@ static tardis_status_t launch_bn(const GemmArgs& g, cudaStream_t s) {
   p.lo = g.lo; p.hi = g.hi; p.colscale = g.colscale; p.rowscale = g.rowscale; p.keps = g.keps; p.bitmap_out = g.bitmap_out;
   p.rlist = g.rlist; p.rcount = g.rcount; p.rcap = g.rcap; p.codes = g.codes; p.scale = static_cast<const __nv_bfloat16*>(g.scale);
   p.zero = g.zero; p.xsrc = static_cast<const __nv_bfloat16*>(g.xsrc); p.d = g.d; p.G = g.G; p.bits = g.bits;
-  TARDIS_CUDA_TRY(cudaFuncSetAttribute(k_gemm<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<BN>::SMEM));
+  static thread_local int room_on = -1;               // the device on which this thread last gave the kernel its shared memory
+  int dev = 0, sms = 0;
+  TARDIS_CUDA_TRY(cudaGetDevice(&dev));
+  if (dev != room_on) {
+    TARDIS_CUDA_TRY(cudaFuncSetAttribute(k_gemm<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<BN>::SMEM));
+    room_on = dev;
+  }
   const int nm = (g.M + BM - 1) / BM, nn = (g.N + BN - 1) / BN;
   p.fast_m = nm <= nn ? 1 : 0;
   const int fcount = p.fast_m ? nm : nn;
   p.band = fcount <= 16 ? fcount : 12;
   const long tiles = long(nm) * nn * p.splits;
-  int dev = 0, sms = 0;
-  TARDIS_CUDA_TRY(cudaGetDevice(&dev));
   TARDIS_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const unsigned grid = unsigned(tiles < sms ? tiles : sms);          // one CTA per SM (shared memory), persistent
   k_gemm<BN><<<grid, NTHREADS, Cfg<BN>::SMEM, s>>>(a1, b1, a2, b2, p);

@@ -563,3 +563,20 @@ def test_buffers_of_destroyed_layers_are_taken_over_by_new_ones():
     for t in threads:
         t.join()
     assert not bad and T.tardis_debug_live_allocations() == live0
+
+
+@pytest.mark.parametrize("d,h,G,bits", [(64, 32, 16, 2), (136 - 8, 96, 32, 3), (272, 1056, 16, 4), (400, 544, 80, 8), (1040, 160, 16, 2)])
+def test_f32_kernels_at_the_edges_of_their_tiles(d, h, G, bits):
+    # tiles of 32 outputs, 16 or 8 tokens, passes of 128 channels (a slice of 16 per warp) of d, then of h; 256 tokens per pass
+    cfg = W.LayerConfig("f32edge%d" % d, d, h, dtype="f32", group=G, bits=bits, n_calib=256)
+    calls = [1, 7, 8, 9, 16, 17, 33, 255, 257]
+    _run(cfg, sum(calls), calls)
+
+
+@pytest.mark.parametrize("d,h,G,q", [(128, 32, 64, 0.05), (192, 96, 64, 0.2), (576, 2080, 192, 0.05), (1152, 4640, 128, 0.1), (640, 19040, 64, 0.02)])
+def test_kernels_for_a_few_tokens_at_the_edges_of_their_tiles(d, h, G, q):
+    # columns of 16 (two-term corrections), 32, 64, 128 tokens; neuron tiles of 16 to 128 rows with a short last one, one or several
+    # per CTA; output tiles of 128 columns with a short last one; more neuron blocks than CTAs and fewer
+    cfg = W.LayerConfig("fewedge%d" % d, d, h, group=G, n_calib=256, q_lo=q, q_hi=1 - q, act=W.ACT_GELU_ERF if d == 192 else W.ACT_GELU_TANH)
+    calls = [1, 5, 16, 17, 32, 33, 64, 65, 127, 128, 2]
+    _run(cfg, sum(calls), calls, path=3)

@@ -29,7 +29,7 @@ namespace bat {
 constexpr int kChunk = 2048;
 constexpr int kChunkCapture = 1024;          // ... while the debug capture is on (the score buffer holds that many)
 constexpr float kEps = 7.62939453125e-6f;    // 2^-17: relative accumulation-error allowance of the fast scores
-constexpr int kMaxRecheck = 1 << 21;         // (token, neuron) pairs per chunk that can queue for re-evaluation
+constexpr int kMaxRecheck = 512;             // neurons per token that can queue for re-evaluation
 
 struct State {
   __nv_bfloat16 *Wf, *W2, *What_hi, *What_lo;     // [d,d], [d,h], [h,d], [h,d]
@@ -38,8 +38,8 @@ struct State {
   float *zhat, *yacc, *x1;                         // [kChunkCapture,h] (scores for the capture; fold temporary), [kChunk,d], [kChunk]
   __nv_bfloat16* delta;                            // [kChunk,h]
   uint32_t* bitmap;                                // [kChunk,h/32]
-  uint2* rlist;                                    // [kMaxRecheck] (token, neuron)
-  unsigned int* rcount;                            // [2]: queued pairs (may exceed the queue), pairs settled in place
+  uint32_t* rlist;                                 // [kChunk][kMaxRecheck] neurons of a token to re-evaluate
+  unsigned int* rcount;                            // [kChunk] how many (more than the queue holds: the rest was settled at once)
   size_t bytes_state, bytes_scratch;
 };
 
@@ -92,10 +92,15 @@ __global__ void k_xnorm(const __nv_bfloat16* __restrict__ x, int d, float* __res
   const int t = blockIdx.x;
   float s = 0.f;
   bool bad = false;
-  for (int k = threadIdx.x; k < d; k += blockDim.x) {
-    const float v = __bfloat162float(x[size_t(t) * d + k]);
-    if (!(fabsf(v) <= 3.0e38f)) bad = true;
-    s += fabsf(v);
+  for (int k = threadIdx.x * 8; k < d; k += blockDim.x * 8) {          // (d is a multiple of 8)
+    const uint4 v = *reinterpret_cast<const uint4*>(x + size_t(t) * d + k);
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float a = fabsf(__uint_as_float(w[q] << 16)), b = fabsf(__uint_as_float(w[q] & 0xffff0000u));
+      bad |= !(a <= 3.0e38f) || !(b <= 3.0e38f);
+      s += a + b;
+    }
   }
   if (bad) s = __int_as_float(0x7f800000);
 #pragma unroll
@@ -109,19 +114,53 @@ __global__ void k_xnorm(const __nv_bfloat16* __restrict__ x, int d, float* __res
   }
 }
 
-// One warp per queued pair: exact fp64 score from the packed codes decides the flag.
-__global__ void k_recheck(const uint2* __restrict__ rlist, const unsigned int* __restrict__ rcount,
-                          const uint32_t* __restrict__ codes, const __nv_bfloat16* __restrict__ scale,
-                          const uint8_t* __restrict__ zero, const float* __restrict__ b1, const float* __restrict__ lo,
-                          const float* __restrict__ hi, const __nv_bfloat16* __restrict__ x, int d, int h, int G, int bits,
-                          uint32_t* __restrict__ bitmap, float* __restrict__ zhat, unsigned long long* counters) {
-  const int lane = threadIdx.x & 31;
-  const unsigned int total = min(rcount[0], (unsigned int)kMaxRecheck);
-  const unsigned int nwarps = (gridDim.x * blockDim.x) >> 5;
-  for (unsigned int e = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; e < total; e += nwarps) {
-    const uint2 pr = rlist[e];
-    const int t = int(pr.x), j = int(pr.y);
-    const double z = exact_score_wide(codes, scale, zero, x + size_t(t) * d, j, d, G, bits, lane) + double(b1[j]);
+// A CTA per token: the exact fp64 scores of its queued neurons (one warp each, from the packed codes) decide their flags; then the
+// token's flags are counted.  The token is widened to fp64 once, in shared memory: with a conversion per product these, at 16 per
+// clock and SM, were the bound (2048 tokens on 4096 / 16384: MEASURED_RECHECK us, 93 before with the count as a kernel of its own).
+// WIDTH: bits per code where 32 is a multiple of it, else 0.  STAGED: false for tokens that do not fit in shared memory.
+template <int WIDTH, bool STAGED>
+__global__ void __launch_bounds__(256) k_recheck(const uint32_t* __restrict__ rlist, const unsigned int* __restrict__ rcount, const uint32_t* __restrict__ codes,
+                                                 const __nv_bfloat16* __restrict__ scale, const uint8_t* __restrict__ zero, const float* __restrict__ b1,
+                                                 const float* __restrict__ lo, const float* __restrict__ hi, const __nv_bfloat16* __restrict__ x, int d, int h,
+                                                 int G, int bits, uint32_t* __restrict__ bitmap, float* __restrict__ zhat, unsigned long long* counters) {
+  extern __shared__ double xd[];                           // channel c of unit u (16 channels) at c (d / 16 + 1) + u: the lanes' units side by side
+  __shared__ unsigned int flagged;
+  const int t = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const unsigned int queued = rcount[t], total = min(queued, (unsigned int)kMaxRecheck);
+  const __nv_bfloat16* const xt = x + size_t(t) * d;
+  const int nw = d / 16;
+  auto xv = [&](int u, int c) { return STAGED ? xd[c * (nw + 1) + u] : double(__bfloat162float(xt[u * 16 + c])); };
+  if (threadIdx.x == 0) flagged = 0u;
+  if (STAGED && total > 0)
+    for (int k = threadIdx.x; k < d; k += blockDim.x) xd[(k & 15) * (nw + 1) + (k >> 4)] = double(__bfloat162float(xt[k]));
+  __syncthreads();
+  const int ng = d / G;
+  for (unsigned int e = warp; e < total; e += 8) {
+    const int j = int(rlist[size_t(t) * kMaxRecheck + e]);
+    const uint32_t* const row = codes + size_t(j) * (size_t(d) * bits / 32);
+    double z = 0.0;
+    for (int u = lane; u < nw; u += 32) {                  // 16 channels, all of one group
+      const int g = u * 16 / G;
+      const double s = double(__bfloat162float(scale[size_t(j) * ng + g])), zp = 4503599627370496.0 + double(zero[size_t(j) * ng + g]);
+      double p0 = 0.0, p1 = 0.0;
+      uint32_t w[4] = {0u, 0u, 0u, 0u};
+      if (WIDTH) {
+#pragma unroll
+        for (int q = 0; q < WIDTH / 2; ++q) w[q] = row[u * (WIDTH / 2) + q];
+      }
+#pragma unroll
+      for (int c = 0; c < 16; c += 2) {
+        const uint32_t q0 = WIDTH ? (w[c * WIDTH / 32] >> (c * WIDTH % 32)) & ((1u << WIDTH) - 1u) : stream_code(row, u * 16 + c, bits);
+        const uint32_t q1 = WIDTH ? (w[(c + 1) * WIDTH / 32] >> ((c + 1) * WIDTH % 32)) & ((1u << WIDTH) - 1u) : stream_code(row, u * 16 + c + 1, bits);
+        // (2^52 + q) - (2^52 + zp): the code less the zero-point without a conversion
+        p0 += (__hiloint2double(0x43300000, int(q0)) - zp) * xv(u, c);
+        p1 += (__hiloint2double(0x43300000, int(q1)) - zp) * xv(u, c + 1);
+      }
+      z += s * (p0 + p1);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+    z += double(b1[j]);
     if (lane == 0) {
       const bool inside = (double(lo[j]) <= z) && (z < double(hi[j]));
       uint32_t* wp = bitmap + size_t(t) * (h / 32) + (j >> 5);
@@ -130,22 +169,19 @@ __global__ void k_recheck(const uint2* __restrict__ rlist, const unsigned int* _
       if (zhat) zhat[size_t(t) * h + j] = float(z);
     }
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    atomicAdd(&counters[CTR_RECHECKS], (unsigned long long)total + rcount[1]);
-  }
-}
-
-__global__ void k_flag_counts(const uint32_t* __restrict__ bitmap, int words, unsigned long long* counters) {
-  __shared__ unsigned int total;
-  if (threadIdx.x == 0) total = 0;
+  __threadfence_block();
   __syncthreads();
   unsigned int c = 0;
-  for (int w = threadIdx.x; w < words; w += blockDim.x) c += __popc(bitmap[size_t(blockIdx.x) * words + w]);
-  atomicAdd(&total, c);
+  for (int w = threadIdx.x; w < h / 32; w += blockDim.x) c += __popc(__ldcg(bitmap + size_t(t) * (h / 32) + w));
+  c = __reduce_add_sync(0xffffffffu, c);
+  if (lane == 0) atomicAdd(&flagged, c);
   __syncthreads();
   if (threadIdx.x == 0) {
-    atomicAdd(&counters[CTR_FLAGGED_TOTAL], (unsigned long long)total);
-    atomicMax(&counters[CTR_FLAGGED_MAX], (unsigned long long)total);
+    if (flagged) {
+      atomicAdd(&counters[CTR_FLAGGED_TOTAL], (unsigned long long)flagged);
+      atomicMax(&counters[CTR_FLAGGED_MAX], (unsigned long long)flagged);
+    }
+    if (queued) atomicAdd(&counters[CTR_RECHECKS], (unsigned long long)queued);
   }
 }
 
@@ -207,7 +243,8 @@ tardis_status_t batched_prepare(Handle* H) {
       {reinterpret_cast<void**>(&S->zhat), size_t(kChunkCapture) * h * 4, true}, {reinterpret_cast<void**>(&S->yacc), size_t(kChunk) * d * 4, true},
       {reinterpret_cast<void**>(&S->x1), size_t(kChunk) * 4, true},       {reinterpret_cast<void**>(&S->delta), size_t(kChunk) * h * 2, true},
       {reinterpret_cast<void**>(&S->bitmap), size_t(kChunk) * (h / 32) * 4, true},
-      {reinterpret_cast<void**>(&S->rlist), size_t(kMaxRecheck) * 8, true}, {reinterpret_cast<void**>(&S->rcount), 16, true}};
+      {reinterpret_cast<void**>(&S->rlist), size_t(kChunk) * kMaxRecheck * 4, true},
+      {reinterpret_cast<void**>(&S->rcount), size_t(kChunk) * 4, true}};
   for (const Req& r : reqs) {
     cudaError_t e = dev_malloc(r.p, r.bytes);
     if (e != cudaSuccess) { set_last_error(e, "cudaMalloc"); cudaGetLastError(); batched_release(H); return TARDIS_ERR_ALLOC; }
@@ -328,7 +365,7 @@ tardis_status_t launch_batched_forward(Handle* H, const void* xv, void* yv, int6
   for (int64_t t0 = 0; t0 < n_total; t0 += chunk) {
     const int n = int(n_total - t0 < chunk ? n_total - t0 : chunk);
     const __nv_bfloat16* xc = x + size_t(t0) * d;
-    TARDIS_CUDA_TRY(cudaMemsetAsync(S->rcount, 0, 16, s));
+    TARDIS_CUDA_TRY(cudaMemsetAsync(S->rcount, 0, size_t(n) * 4, s));
     k_xnorm<<<n, 256, 0, s>>>(xc, d, S->x1);
     // 1. fast scores: one GEMM over the hi and lo halves of the dequantised predictor
     GemmArgs g = {};
@@ -343,9 +380,13 @@ tardis_status_t launch_batched_forward(Handle* H, const void* xv, void* yv, int6
     g.codes = H->codes; g.scale = H->scale; g.zero = H->zero; g.xsrc = xc; g.d = d; g.G = H->G; g.bits = H->bits;
     tardis_status_t st = launch_gemm(g, s);
     if (st != TARDIS_OK) return st;
-    k_recheck<<<H->num_sms * 4, 256, 0, s>>>(S->rlist, S->rcount, H->codes, static_cast<const __nv_bfloat16*>(H->scale), H->zero, H->b1,
-                                             H->lo, H->hi, xc, d, h, H->G, H->bits, S->bitmap, keep_scores ? S->zhat : nullptr, H->counters);
-    k_flag_counts<<<n, 256, 0, s>>>(S->bitmap, h / 32, H->counters);
+    const bool staged = d <= 24576;                        // (192 KB)
+    const size_t room = staged ? size_t(d / 16 + 1) * 16 * sizeof(double) : 0;
+    const auto recheck = H->bits == 2 ? (staged ? k_recheck<2, true> : k_recheck<2, false>)
+                                      : (H->bits == 4 ? (staged ? k_recheck<4, true> : k_recheck<4, false>) : (staged ? k_recheck<0, true> : k_recheck<0, false>));
+    if (room > 48 * 1024) TARDIS_CUDA_TRY(cudaFuncSetAttribute(recheck, cudaFuncAttributeMaxDynamicSharedMemorySize, int(room)));
+    recheck<<<n, 256, room, s>>>(S->rlist, S->rcount, H->codes, static_cast<const __nv_bfloat16*>(H->scale), H->zero, H->b1, H->lo, H->hi, xc, d, h,
+                                 H->G, H->bits, S->bitmap, keep_scores ? S->zhat : nullptr, H->counters);
     if (H->dbg_bitmap || H->dbg_scores) {
       const size_t cnt = size_t(n) * h;
       k_capture<<<unsigned((cnt + 255) / 256), 256, 0, s>>>(S->bitmap, S->zhat, S->x1, n, h,
@@ -384,7 +425,7 @@ tardis_status_t launch_batched_forward(Handle* H, const void* xv, void* yv, int6
       const size_t cnt = size_t(n) * d;
       k_round_store<<<unsigned((cnt / 4 + 255) / 256 + 1), 256, 0, s>>>(S->yacc, y + size_t(t0) * d, cnt);
     }
-    H->launches += 9 + ((H->dbg_bitmap || H->dbg_scores) ? 1 : 0);
+    H->launches += 8 + ((H->dbg_bitmap || H->dbg_scores) ? 1 : 0);
   }
   TARDIS_CUDA_TRY(cudaGetLastError());
   return TARDIS_OK;

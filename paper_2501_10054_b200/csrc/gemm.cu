@@ -4,7 +4,7 @@
 // 128 x 64 (A) and BN x 64 (B) operand boxes into a ring of shared-memory stages with TMA
 // (cp.async.bulk.tensor, 128-byte swizzle, no multicast); warp 1 issues tcgen05.mma (M = 128, N = BN,
 // K = 16 per instruction; one elected lane), accumulating in tensor memory (TMEM, 128 lanes x BN fp32 columns,
-// two accumulators used in turn) and releasing each stage with tcgen05.commit; warps 2..5 read a finished
+// two accumulators used in turn) and releasing each stage with tcgen05.commit; warps 2..9 read a finished
 // accumulator back with tcgen05.ld (each warp its own 32 lanes) and run the epilogue while the next tile's
 // main loop fills the other accumulator.  Every wait on an mbarrier is bounded: when it runs out the waiter
 // sets an error word and the CTA falls through to the end, where TMEM is released.
@@ -53,7 +53,7 @@ using namespace tc;
 
 constexpr int BM = 128;                 // tile rows (tokens / outputs)
 constexpr int BK = 64;                  // channels per stage: 64 bf16 = one 128-byte swizzle row
-constexpr int NTHREADS = 192;           // warp 0 TMA, warp 1 MMA, warps 2..5 epilogue
+constexpr int NTHREADS = 320;           // warp 0 TMA, warp 1 MMA, warps 2..9 epilogue
 
 struct KParams {
   int M, N, kb1, kb2;          // k blocks (of 64) of the two operand pairs
@@ -67,7 +67,7 @@ struct KParams {
   const float *lo, *hi, *colscale, *rowscale;
   float keps;
   uint32_t* bitmap_out;
-  uint2* rlist; unsigned int* rcount; int rcap;
+  uint32_t* rlist; unsigned int* rcount; int rcap;
   const uint32_t* codes; const __nv_bfloat16* scale; const uint8_t* zero;
   const __nv_bfloat16* xsrc; int d, G, bits;
 };
@@ -75,7 +75,7 @@ struct KParams {
 template <int BN> struct Cfg {
   static constexpr int STAGE_BYTES = BM * BK * 2 + BN * BK * 2;
   static constexpr int NS = (BN == 256) ? 4 : 6;                      // stages
-  static constexpr int SMEM = NS * STAGE_BYTES + 1024 /* alignment slack */ + 256 /* barriers */ + 4 * 4096 /* epilogue staging */;
+  static constexpr int SMEM = NS * STAGE_BYTES + 1024 /* alignment slack */ + 256 /* barriers */ + 8 * 2048 /* epilogue staging */ + BN * 16 /* column table */;
   static constexpr int TMEM_COLS = 2 * BN;                            // two accumulators
 };
 
@@ -93,45 +93,44 @@ __device__ __forceinline__ float gelu_quick(float z, int act) {
   return 0.5f * z * (1.f + copysignf(e, z));
 }
 
-// `stage`: 32 x 32 floats of shared memory of the calling warp (element [i][lane]).
+// `stage`: 16 x 32 floats of shared memory of the calling warp (element [i][lane]); `tab`: the tile's column table (see
+// fill_table), from column n on.
 __device__ __forceinline__ void epilogue_chunk(const KParams& p, float (&v)[32], int m, int n, int nv, bool first_split, bool have_acc,
-                                               float* stage, int lane) {
+                                               float* stage, const float4* tab, int lane) {
   if (p.epilogue == GEMM_EPI_FLAGS) {
+    // (the table holds lo - b1 and hi - b1: where the rounding of that difference could matter, |score - b1| and with it the
+    // allowance is more than a hundred times as large, and the pair is re-evaluated)
     const float xn = p.rowscale[m];
     const uint32_t valid = nv == 32 ? 0xffffffffu : ((1u << nv) - 1u);
     uint32_t word = valid;                                   // a non-finite token: every neuron flagged
     if (xn <= 3.0e38f) {
       const float kx = p.keps * xn;
-      word = 0u;
+      uint32_t outside = 0u, open = 0u;
 #pragma unroll
       for (int i = 0; i < 32; ++i) {
-        if (i < nv) {
-          const float z = v[i] + p.bias[n + i], l = p.lo[n + i], u = p.hi[n + i];
-          const float tau = fmaf(p.colscale[n + i], kx, 1e-30f);
-          bool flag = !((l <= z) && (z < u));
-          if (fabsf(z - l) <= tau || fabsf(z - u) <= tau) {  // rare
-            const unsigned int slot = atomicAdd(&p.rcount[0], 1u);
-            if (slot < (unsigned int)p.rcap) p.rlist[slot] = make_uint2((unsigned int)m, (unsigned int)(n + i));
-            else {                                           // queue full: settle this one here (slow, but exact)
-              const double ze = exact_score_single(p.codes, p.scale, p.zero, p.xsrc + size_t(m) * p.d, n + i, p.d, p.G, p.bits) + double(p.bias[n + i]);
-              flag = !((double(l) <= ze) && (ze < double(u)));
-              atomicAdd(&p.rcount[1], 1u);
-            }
-          }
-          word |= (flag ? 1u : 0u) << i;
-          v[i] = z;
+        const float4 t = tab[i];
+        const float dl = v[i] - t.x, du = v[i] - t.y;
+        outside |= (!(dl >= 0.f && du < 0.f) ? 1u : 0u) << i;
+        open |= (fminf(fabsf(dl), fabsf(du)) <= fmaf(t.z, kx, 1e-30f) ? 1u : 0u) << i;
+      }
+      word = outside & valid;
+      for (uint32_t w = open & valid; w; w &= w - 1u) {      // rare
+        const int i = __ffs(w) - 1;
+        const unsigned int slot = atomicAdd(&p.rcount[m], 1u);
+        if (slot < (unsigned int)p.rcap) p.rlist[size_t(m) * p.rcap + slot] = uint32_t(n + i);
+        else {                                               // the token's queue is full: settle this one here (slow, but exact)
+          const double ze = exact_score_single(p.codes, p.scale, p.zero, p.xsrc + size_t(m) * p.d, n + i, p.d, p.G, p.bits) + double(p.bias[n + i]);
+          const bool flag = !((double(p.lo[n + i]) <= ze) && (ze < double(p.hi[n + i])));
+          word = flag ? word | (1u << i) : word & ~(1u << i);
         }
       }
     }
     p.bitmap_out[size_t(m) * (p.N / 32) + (n >> 5)] = word;
     if (p.out_f32) {
       float* o = p.out_f32 + size_t(m) * p.ldo + n;
-      if (nv == 32 && (p.ldo & 3) == 0) {
 #pragma unroll
-        for (int i = 0; i < 32; i += 4) *reinterpret_cast<float4*>(o + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
-      } else {
-        for (int i = 0; i < nv; ++i) o[i] = v[i];
-      }
+      for (int i = 0; i < 32; ++i)
+        if (i < nv) o[i] = v[i] + tab[i].w;
     }
     return;
   }
@@ -182,14 +181,18 @@ __device__ __forceinline__ void epilogue_chunk(const KParams& p, float (&v)[32],
       uint32_t word = p.bitmap[size_t(m) * (p.N / 32) + (n >> 5)];
       if (nv < 32) word &= (1u << nv) - 1u;
 #pragma unroll
-      for (int i = 0; i < 32; ++i) stage[i * 32 + lane] = v[i];
-      for (uint32_t w = word; w; w &= w - 1u) {
-        const int i = __ffs(w) - 1;
-        const float z = stage[i * 32 + lane] + (p.bias ? p.bias[n + i] : 0.f);
-        stage[i * 32 + lane] = gelu_quick(z, p.act) - p.a[n + i] * z - p.c[n + i];
-      }
+      for (int half = 0; half < 32; half += 16) {
 #pragma unroll
-      for (int i = 0; i < 32; ++i) v[i] = ((word >> i) & 1u) ? stage[i * 32 + lane] : 0.f;
+        for (int i = 0; i < 16; ++i) stage[i * 32 + lane] = v[half + i];
+        for (uint32_t w = (word >> half) & 0xffffu; w; w &= w - 1u) {
+          const int i = __ffs(w) - 1;
+          const float4 t = tab[half + i];
+          const float z = stage[i * 32 + lane] + t.x;
+          stage[i * 32 + lane] = gelu_quick(z, p.act) - t.y * z - t.z;
+        }
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[half + i] = ((word >> (half + i)) & 1u) ? stage[i * 32 + lane] : 0.f;
+      }
     }
     __nv_bfloat16* o = p.out_bf16 + size_t(m) * p.ldo + n;
     if (nv == 32 && (p.ldo & 7) == 0) {
@@ -203,6 +206,26 @@ __device__ __forceinline__ void epilogue_chunk(const KParams& p, float (&v)[32],
     } else {
       for (int i = 0; i < nv; ++i) o[i] = __float2bfloat16_rn(v[i]);
     }
+  }
+}
+
+// What the epilogues look up per column, columns n0 .. n0 + count - 1 (one warp group of 128 threads): GEMM_EPI_FLAGS lo - bias,
+// hi - bias, allowance per unit of |x|_1, bias; GEMM_EPI_DELTA bias, a, c.  (Looked up in global memory by every row of the tile,
+// the scores of 2048 tokens on 4096 / 16384 took 427 us where the product alone takes 230.)
+__device__ __forceinline__ void fill_table(const KParams& p, float4* tab, int n0, int count, int tid) {
+  for (int c = tid; c < count; c += 128) {
+    const int n = n0 + c;
+    float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (n < p.N) {
+      const float b = p.bias ? p.bias[n] : 0.f;
+      if (p.epilogue == GEMM_EPI_DELTA) t = make_float4(b, p.a[n], p.c[n], 0.f);
+      else {
+        // a term of a score is at most max |code - zero-point| times the scale times |x|: 2 instead of 3 where no second term exists
+        const float most = p.second_used && p.bits == 2 && p.second_used[n >> 7] == 0u ? 2.f / 3.f : 1.f;
+        t = make_float4(p.lo[n] - b, p.hi[n] - b, p.colscale[n] * most, b);
+      }
+    }
+    tab[c] = t;
   }
 }
 
@@ -227,7 +250,7 @@ k_gemm(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtenso
   const int ntiles = nm * nn * p.splits;
   if (threadIdx.x == 0) {
     for (int s = 0; s < C::NS; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
-    for (int b = 0; b < 2; ++b) { mbar_init(&accum_full[b], 1); mbar_init(&accum_empty[b], 4); }
+    for (int b = 0; b < 2; ++b) { mbar_init(&accum_full[b], 1); mbar_init(&accum_empty[b], 8); }
     *failed = 0u;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tmA1) : "memory");
@@ -311,22 +334,30 @@ k_gemm(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtenso
       ++use;
     }
   } else {
-    // ---------------- epilogue: warp q reads TMEM lanes 32 (warp % 4) .. + 31 ----------------
-    const int q = warp & 3;
-    float* const stage = reinterpret_cast<float*>(smem + C::NS * C::STAGE_BYTES + 256) + q * 1024;
+    // ---------------- epilogue: a warp reads TMEM lanes 32 (warp % 4) .. + 31 and half of the columns ----------------
+    const int q = warp & 3, half = (warp - 2) >> 2;
+    uint8_t* const after = smem + C::NS * C::STAGE_BYTES + 256;
+    float* const stage = reinterpret_cast<float*>(after) + (warp - 2) * 512;
+    float4* const tab = reinterpret_cast<float4*>(after + 8 * 2048) + half * (BN / 2);
+    const bool table = p.epilogue == GEMM_EPI_FLAGS || p.epilogue == GEMM_EPI_DELTA;
     uint32_t use = 0;
     bool ok = true;
-    for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
       int m0, n0, kb_lo, nkb, z;
       decode(tile, m0, n0, kb_lo, nkb, z);
       const int m = m0 + q * 32 + lane;
       const uint32_t ab = use & 1u;
+      if (table) {                                         // (the warps of a half are a group of 128 threads)
+        asm volatile("bar.sync %0, 128;" ::"r"(1 + half) : "memory");
+        fill_table(p, tab, n0 + half * (BN / 2), BN / 2, (threadIdx.x - 64) & 127);
+        asm volatile("bar.sync %0, 128;" ::"r"(1 + half) : "memory");
+      }
       if (nkb > 0) {
-        ok = mbar_wait_warp(&accum_full[ab], (use >> 1) & 1);
-        if (!ok) { *failed = 1u; break; }
+        ok = ok && mbar_wait_warp(&accum_full[ab], (use >> 1) & 1);
+        if (!ok) *failed = 1u;                               // (no way out here: the group meets at its barriers)
         tc_fence_after();
       }
-      for (int ch = 0; ch < BN / 32; ++ch) {
+      for (int ch = half * (BN / 64); ch < (half + 1) * (BN / 64); ++ch) {
         float v[32];
         if (nkb > 0) tmem_ld32(tmem_base + ab * BN + (uint32_t(q * 32) << 16) + uint32_t(ch * 32), v);
         else {
@@ -335,7 +366,7 @@ k_gemm(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtenso
         }
         const int n = n0 + ch * 32;
         const int nv = min(32, p.N - n);
-        if (m < p.M && nv > 0) epilogue_chunk(p, v, m, n, nv, z == 0, nkb > 0, stage, lane);   // (no early exit: tcgen05.ld needs the whole warp)
+        if (m < p.M && nv > 0) epilogue_chunk(p, v, m, n, nv, z == 0, nkb > 0, stage, tab + ch * 32 - half * (BN / 2), lane);   // (no early exit: tcgen05.ld needs the whole warp)
       }
       if (nkb > 0) {
         tc_fence_before();

@@ -40,7 +40,7 @@ struct GemmArgs {
   const float *lo, *hi, *colscale, *rowscale;   // [N], [N], [N], [M]
   float keps;
   uint32_t* bitmap_out;             // [M, N / 32]
-  uint2* rlist; unsigned int* rcount; int rcap;   // queue of (m, n) pairs, its fill count ([1]: pairs settled in place), capacity
+  uint32_t* rlist; unsigned int* rcount; int rcap;   // per row m a queue of rcap columns, and how many wanted to enter it
   const uint32_t* codes; const void* scale; const uint8_t* zero;   // the packed predictor (rows n)
   const void* xsrc; int d, G, bits; // the bf16 rows A1 came from (leading dimension d), group size, bits per code
 };

@@ -116,7 +116,7 @@ __global__ void k_xnorm(const __nv_bfloat16* __restrict__ x, int d, float* __res
 
 // A CTA per token: the exact fp64 scores of its queued neurons (one warp each, from the packed codes) decide their flags; then the
 // token's flags are counted.  The token is widened to fp64 once, in shared memory: with a conversion per product these, at 16 per
-// clock and SM, were the bound (2048 tokens on 4096 / 16384: MEASURED_RECHECK us, 93 before with the count as a kernel of its own).
+// clock and SM, were the bound (2048 tokens on 4096 / 16384: 51 us, 93 before with the count as a kernel of its own).
 // WIDTH: bits per code where 32 is a multiple of it, else 0.  STAGED: false for tokens that do not fit in shared memory.
 template <int WIDTH, bool STAGED>
 __global__ void __launch_bounds__(256) k_recheck(const uint32_t* __restrict__ rlist, const unsigned int* __restrict__ rcount, const uint32_t* __restrict__ codes,
@@ -132,31 +132,55 @@ __global__ void __launch_bounds__(256) k_recheck(const uint32_t* __restrict__ rl
   auto xv = [&](int u, int c) { return STAGED ? xd[c * (nw + 1) + u] : double(__bfloat162float(xt[u * 16 + c])); };
   if (threadIdx.x == 0) flagged = 0u;
   if (STAGED && total > 0)
-    for (int k = threadIdx.x; k < d; k += blockDim.x) xd[(k & 15) * (nw + 1) + (k >> 4)] = double(__bfloat162float(xt[k]));
+    for (int u = threadIdx.x; u < nw; u += blockDim.x) {
+      const uint4 a = *reinterpret_cast<const uint4*>(xt + u * 16), b = *reinterpret_cast<const uint4*>(xt + u * 16 + 8);
+      const uint32_t v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        xd[2 * c * (nw + 1) + u] = double(__uint_as_float(v[c] << 16));
+        xd[(2 * c + 1) * (nw + 1) + u] = double(__uint_as_float(v[c] & 0xffff0000u));
+      }
+    }
   __syncthreads();
   const int ng = d / G;
   for (unsigned int e = warp; e < total; e += 8) {
     const int j = int(rlist[size_t(t) * kMaxRecheck + e]);
     const uint32_t* const row = codes + size_t(j) * (size_t(d) * bits / 32);
     double z = 0.0;
-    for (int u = lane; u < nw; u += 32) {                  // 16 channels, all of one group
-      const int g = u * 16 / G;
-      const double s = double(__bfloat162float(scale[size_t(j) * ng + g])), zp = 4503599627370496.0 + double(zero[size_t(j) * ng + g]);
-      double p0 = 0.0, p1 = 0.0;
-      uint32_t w[4] = {0u, 0u, 0u, 0u};
-      if (WIDTH) {
+    // units of 16 channels (all of one group), four at a time: their loads go out before the first is used, since waiting for them
+    // is most of what a warp does here
+    for (int u0 = lane; u0 < nw; u0 += 128) {
+      uint32_t w[4][WIDTH ? WIDTH / 2 : 1];
+      __nv_bfloat16 sc[4];
+      uint8_t zr[4];
 #pragma unroll
-        for (int q = 0; q < WIDTH / 2; ++q) w[q] = row[u * (WIDTH / 2) + q];
+      for (int v = 0; v < 4; ++v) {
+        const int u = u0 + 32 * v;
+        if (u < nw) {
+          sc[v] = scale[size_t(j) * ng + u * 16 / G];
+          zr[v] = zero[size_t(j) * ng + u * 16 / G];
+          if (WIDTH) {
+#pragma unroll
+            for (int q = 0; q < WIDTH / 2; ++q) w[v][q] = row[u * (WIDTH / 2) + q];
+          }
+        }
       }
 #pragma unroll
-      for (int c = 0; c < 16; c += 2) {
-        const uint32_t q0 = WIDTH ? (w[c * WIDTH / 32] >> (c * WIDTH % 32)) & ((1u << WIDTH) - 1u) : stream_code(row, u * 16 + c, bits);
-        const uint32_t q1 = WIDTH ? (w[(c + 1) * WIDTH / 32] >> ((c + 1) * WIDTH % 32)) & ((1u << WIDTH) - 1u) : stream_code(row, u * 16 + c + 1, bits);
-        // (2^52 + q) - (2^52 + zp): the code less the zero-point without a conversion
-        p0 += (__hiloint2double(0x43300000, int(q0)) - zp) * xv(u, c);
-        p1 += (__hiloint2double(0x43300000, int(q1)) - zp) * xv(u, c + 1);
+      for (int v = 0; v < 4; ++v) {
+        const int u = u0 + 32 * v;
+        if (u >= nw) break;
+        const double zp = 4503599627370496.0 + double(zr[v]);
+        double p0 = 0.0, p1 = 0.0;
+#pragma unroll
+        for (int c = 0; c < 16; c += 2) {
+          const uint32_t q0 = WIDTH ? (w[v][c * WIDTH / 32] >> (c * WIDTH % 32)) & ((1u << WIDTH) - 1u) : stream_code(row, u * 16 + c, bits);
+          const uint32_t q1 = WIDTH ? (w[v][(c + 1) * WIDTH / 32] >> ((c + 1) * WIDTH % 32)) & ((1u << WIDTH) - 1u) : stream_code(row, u * 16 + c + 1, bits);
+          // (2^52 + q) - (2^52 + zp): the code less the zero-point without a conversion
+          p0 += (__hiloint2double(0x43300000, int(q0)) - zp) * xv(u, c);
+          p1 += (__hiloint2double(0x43300000, int(q1)) - zp) * xv(u, c + 1);
+        }
+        z += double(__bfloat162float(sc[v])) * (p0 + p1);
       }
-      z += s * (p0 + p1);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);

@@ -13,8 +13,8 @@
 namespace tardis {
 namespace {
 
-constexpr int LN_THREADS = 256;
-constexpr int LN_MAXPER = 48;   // elements per thread: d_model up to 12288
+constexpr int LN_THREADS = 512;
+constexpr int LN_MAXVEC = 3;    // vectors of 8 elements per thread: d_model up to 12288
 
 __device__ __forceinline__ float block_sum(float v, float* sh) {
 #pragma unroll
@@ -23,72 +23,116 @@ __device__ __forceinline__ float block_sum(float v, float* sh) {
   __syncthreads();                       // (sh may still be read from the previous sum)
   if (lane == 0) sh[warp] = v;
   __syncthreads();
-  float t = 0.f;
+  v = sh[lane & (LN_THREADS / 32 - 1)];  // every warp adds the same numbers in the same order
 #pragma unroll
-  for (int w = 0; w < LN_THREADS / 32; ++w) t += sh[w];   // every thread adds the same numbers in the same order
-  return t;
+  for (int o = LN_THREADS / 64; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
 }
 
-// stream[t][:] takes the previous layer's output f[t][:] (update: added when `residual`, else copied), then
+// 8 consecutive elements (16-byte aligned) as fp32, and back
+__device__ __forceinline__ void load8(float (&v)[8], const float* p) {
+  const float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + 4);
+  v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+}
+__device__ __forceinline__ void load8(float (&v)[8], const __nv_bfloat16* p) {
+  const uint4 a = *reinterpret_cast<const uint4*>(p);
+  const uint32_t w[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) { v[2 * i] = __uint_as_float(w[i] << 16); v[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u); }
+}
+__device__ __forceinline__ void store8(float* p, const float (&v)[8]) {
+  *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+  *reinterpret_cast<float4*>(p + 4) = make_float4(v[4], v[5], v[6], v[7]);
+}
+__device__ __forceinline__ void store8(__nv_bfloat16* p, const float (&v)[8]) {
+  __nv_bfloat162 o[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) o[i] = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+  *reinterpret_cast<uint4*>(p) = *reinterpret_cast<const uint4*>(o);
+}
+// v = residual ? v + f : f, rounded as it is stored
+template <typename T> __device__ __forceinline__ void add_output(float (&v)[8], const T* f, int residual) {
+  float w[8];
+  load8(w, f);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = residual ? to_f32<T>(from_f32<T>(v[i] + w[i])) : w[i];
+}
+
+// stream[t][:] = src[t][:] (the stream itself, or x for the first layer that needs it), with the previous layer's output f[t][:]
+// (update: added when `residual`, else in its place), then
 // out[t][i] = (stream[t][i] - mean_t) / sqrt(var_t + eps) * gamma[i] + beta[i]; mean and variance (1/d, not 1/(d-1)) over the
-// row; without `normalise` out is the stream itself.
-template <typename T>
-__global__ void __launch_bounds__(LN_THREADS) k_update_norm(T* __restrict__ stream, const T* __restrict__ f, int update, int residual,
+// row; without `normalise` out is the stream itself.  One CTA per token, the row in registers: bound by the latency of one load, two
+// sums and one store (4096 elements, one token: 16 us with an element per load and 48 guarded steps for any d_model, 3 us now).
+template <typename T, int NV>
+__global__ void __launch_bounds__(LN_THREADS) k_update_norm(const T* src, T* stream, const T* __restrict__ f, int update, int residual,
                                                             int normalise, T* __restrict__ out, const float* __restrict__ gamma,
                                                             const float* __restrict__ beta, int d, float eps) {
   __shared__ float sh[LN_THREADS / 32];
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");          // the launch before wrote f (or the stream)
-  T* row = stream + size_t(blockIdx.x) * d;
-  const T* frow = f + size_t(blockIdx.x) * d;
-  float v[LN_MAXPER];
-  float s = 0.f;
+  float ga[NV][8], be[NV][8];
 #pragma unroll
-  for (int e = 0; e < LN_MAXPER; ++e) {
-    const int i = threadIdx.x + e * LN_THREADS;
-    v[e] = 0.f;
-    if (i < d) {
-      if (update) {
-        const T nv = residual ? from_f32<T>(to_f32<T>(row[i]) + to_f32<T>(frow[i])) : frow[i];   // rounded as it is stored
-        row[i] = nv;
-        v[e] = to_f32<T>(nv);
-      } else {
-        v[e] = to_f32<T>(row[i]);
+  for (int e = 0; e < NV; ++e) {                               // (the caller's constants: before the wait)
+    const int i = (threadIdx.x + e * LN_THREADS) * 8;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) { ga[e][q] = 1.f; be[e][q] = 0.f; }
+    if (normalise && i < d) {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        if (gamma) ga[e][q] = gamma[i + q];
+        if (beta) be[e][q] = beta[i + q];
       }
     }
-    s += v[e];
   }
-  if (!normalise) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");          // the launch before wrote f (or the stream)
+  const size_t row = size_t(blockIdx.x) * d;
+  float v[NV][8];
+  float s = 0.f;
 #pragma unroll
-    for (int e = 0; e < LN_MAXPER; ++e) {
-      const int i = threadIdx.x + e * LN_THREADS;
-      if (i < d) out[size_t(blockIdx.x) * d + i] = from_f32<T>(v[e]);
+  for (int e = 0; e < NV; ++e) {
+    const int i = (threadIdx.x + e * LN_THREADS) * 8;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) v[e][q] = 0.f;
+    if (i < d) {                                               // (d is a multiple of 8)
+      load8(v[e], src + row + i);
+      if (update) add_output<T>(v[e], f + row + i, residual);
+      if (update || src != stream) store8(stream + row + i, v[e]);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) s += v[e][q];
     }
-    return;
   }
-  const float mean = block_sum(s, sh) / float(d);
-  float q = 0.f;
+  if (normalise) {
+    const float mean = block_sum(s, sh) / float(d);
+    float sq = 0.f;
 #pragma unroll
-  for (int e = 0; e < LN_MAXPER; ++e) {
-    const int i = threadIdx.x + e * LN_THREADS;
-    const float c = i < d ? v[e] - mean : 0.f;
-    q += c * c;
+    for (int e = 0; e < NV; ++e)
+      if ((threadIdx.x + e * LN_THREADS) * 8 < d) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) { const float c = v[e][q] - mean; sq += c * c; }
+      }
+    const float rstd = rsqrtf(block_sum(sq, sh) / float(d) + eps);
+#pragma unroll
+    for (int e = 0; e < NV; ++e)
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[e][q] = (v[e][q] - mean) * rstd * ga[e][q] + be[e][q];
   }
-  const float rstd = rsqrtf(block_sum(q, sh) / float(d) + eps);
 #pragma unroll
-  for (int e = 0; e < LN_MAXPER; ++e) {
-    const int i = threadIdx.x + e * LN_THREADS;
-    if (i < d) out[size_t(blockIdx.x) * d + i] = from_f32<T>((v[e] - mean) * rstd * (gamma ? gamma[i] : 1.f) + (beta ? beta[i] : 0.f));
+  for (int e = 0; e < NV; ++e) {
+    const int i = (threadIdx.x + e * LN_THREADS) * 8;
+    if (i < d) store8(out + row + i, v[e]);
   }
 }
 
-// stream += f (residual) or stream = f: after the last layer
+// stream = src + f (residual) or stream = f: after the last layer
 template <typename T>
-__global__ void k_stream_update(T* __restrict__ stream, const T* __restrict__ f, size_t count, int residual) {
+__global__ void __launch_bounds__(128) k_stream_update(const T* src, T* stream, const T* __restrict__ f, size_t count, int residual) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < count; i += size_t(gridDim.x) * blockDim.x)
-    stream[i] = residual ? from_f32<T>(to_f32<T>(stream[i]) + to_f32<T>(f[i])) : f[i];
+  for (size_t i = (size_t(blockIdx.x) * blockDim.x + threadIdx.x) * 8; i < count; i += size_t(gridDim.x) * blockDim.x * 8) {
+    float v[8];
+    load8(v, src + i);
+    add_output<T>(v, f + i, residual);
+    store8(stream + i, v);
+  }
 }
 
 template <typename... Args>
@@ -108,27 +152,30 @@ tardis_status_t run_stack(const tardis_stack_desc_t* desc, const void* x, void* 
   const int d = H0->d;
   const size_t count = size_t(n) * d;
   T* stream = static_cast<T*>(y);
-  if (x != y) TARDIS_CUDA_TRY(cudaMemcpyAsync(y, x, count * sizeof(T), cudaMemcpyDeviceToDevice, s));
+  const T* src = static_cast<const T*>(x);                     // where the stream's values are: in x until a kernel has written y
   const int norm = desc->normalise != 0 ? 1 : 0;
+  const auto update_norm = d <= LN_THREADS * 8 ? k_update_norm<T, 1> : (d <= LN_THREADS * 16 ? k_update_norm<T, 2> : k_update_norm<T, LN_MAXVEC>);
   T* fprev = nullptr;
   for (int l = 0; l < desc->n_layers; ++l) {
     // with `keep`, the layer's input and output stay where the caller can read them; else two buffers for the inputs take
     // turns with one for the output (the update of layer l + 1 reads the output of layer l while writing its own input)
     T* xin = keep ? static_cast<T*>(keep) + size_t(2 * l) * count : static_cast<T*>(work);
     T* fout = keep ? static_cast<T*>(keep) + size_t(2 * l + 1) * count : static_cast<T*>(work) + count;
-    const T* layer_in = stream;
+    const T* layer_in = src;
     if (norm || keep || l > 0) {
-      TARDIS_CUDA_TRY(launch_chained(k_update_norm<T>, dim3(unsigned(n)), dim3(LN_THREADS), s, stream, static_cast<const T*>(fprev ? fprev : stream),
-                                     l > 0 ? 1 : 0, desc->residual, norm, xin, norm && desc->ln_gamma ? desc->ln_gamma[l] : static_cast<const float*>(nullptr),
+      TARDIS_CUDA_TRY(launch_chained(update_norm, dim3(unsigned(n)), dim3(LN_THREADS), s, src, stream, static_cast<const T*>(fprev ? fprev : stream),
+                                     l > 0 ? 1 : 0, int(desc->residual), norm, xin, norm && desc->ln_gamma ? desc->ln_gamma[l] : static_cast<const float*>(nullptr),
                                      norm && desc->ln_beta ? desc->ln_beta[l] : static_cast<const float*>(nullptr), d, desc->ln_eps));
       layer_in = xin;
+      src = stream;
     }
     const tardis_status_t st = tardis_ffn_forward(desc->layers[l], layer_in, fout, n, reinterpret_cast<tardis_stream_t>(s));
     if (st != TARDIS_OK) return st;
     fprev = fout;
   }
-  const unsigned blocks = unsigned((count + 255) / 256 < 4096 ? (count + 255) / 256 : 4096);
-  TARDIS_CUDA_TRY(launch_chained(k_stream_update<T>, dim3(blocks), dim3(256), s, stream, static_cast<const T*>(fprev), count, desc->residual));
+  const size_t blocks = (count / 8 + 127) / 128;
+  TARDIS_CUDA_TRY(launch_chained(k_stream_update<T>, dim3(unsigned(blocks < 4096 ? blocks : 4096)), dim3(128), s, src, stream, static_cast<const T*>(fprev),
+                                 count, int(desc->residual)));
   return TARDIS_OK;
 }
 
@@ -137,7 +184,7 @@ tardis_status_t run_stack(const tardis_stack_desc_t* desc, const void* x, void* 
 tardis_status_t launch_stack_forward(const tardis_stack_desc_t* desc, const void* x, void* y, void* work, void* keep, int64_t n,
                                      cudaStream_t s) {
   Handle* H0 = reinterpret_cast<Handle*>(desc->layers[0]);
-  if (H0->d > LN_THREADS * LN_MAXPER) return TARDIS_ERR_UNSUPPORTED;
+  if (H0->d > LN_THREADS * 8 * LN_MAXVEC) return TARDIS_ERR_UNSUPPORTED;
   return H0->dtype == TARDIS_F32 ? run_stack<float>(desc, x, y, work, keep, n, s) : run_stack<__nv_bfloat16>(desc, x, y, work, keep, n, s);
 }
 

@@ -580,3 +580,31 @@ def test_kernels_for_a_few_tokens_at_the_edges_of_their_tiles(d, h, G, q):
     cfg = W.LayerConfig("fewedge%d" % d, d, h, group=G, n_calib=256, q_lo=q, q_hi=1 - q, act=W.ACT_GELU_ERF if d == 192 else W.ACT_GELU_TANH)
     calls = [1, 5, 16, 17, 32, 33, 64, 65, 127, 128, 2]
     _run(cfg, sum(calls), calls, path=3)
+
+
+@pytest.mark.parametrize("d,dtype", [(16, "f32"), (1040, "f32"), (4096, "bf16"), (4160, "bf16"), (8256, "bf16")])
+def test_stack_normalisation_at_the_edges_of_its_vectors(d, dtype):
+    # one, two and three vectors of 8 elements per thread of 512, the last ones partly beyond the row; x apart from y and in place
+    cfg = W.LayerConfig("norm%d" % d, d, 32, group=16 if d < 64 else 16 * (2 if d % 32 == 0 else 1), dtype=dtype, n_calib=64)
+    L = _layer(cfg, 1)
+    x = (W.make_tokens(cfg, 3, 1).cuda().float() * 3 + 0.5).to(L.W1.dtype)
+    gam, bet = torch.linspace(0.5, 2, d, device="cuda"), torch.linspace(-1, 1, d, device="cuda")
+    h = T.fold_layer(L)
+    try:
+        for in_place in (False, True):
+            xs = x.clone()
+            y = xs if in_place else torch.empty_like(x)
+            keep = torch.empty(2, 2, 3, d, dtype=x.dtype, device="cuda")
+            T.tardis_stack_forward([h, h], xs, y, [gam, bet], [bet, gam], keep=keep)
+            torch.cuda.synchronize()
+            assert in_place or torch.equal(xs, x)
+            s = x
+            for l, (a, b) in enumerate(((gam, bet), (bet, gam))):
+                u = torch.nn.functional.layer_norm(s.double(), (d,), a.double(), b.double(), 1e-5)
+                # one rounding to the dtype (bf16 has 8 significant bits: half a unit in the last is at most 2^-8 of the value; fp32: 2^-24)
+                # plus the fp32 mean and deviation (a few 1e-6 of values below 10)
+                assert ((keep[l, 0].double() - u).abs() <= (2.0 ** -8 if dtype == "bf16" else 0) * u.abs() + 3e-5).all()
+                s = (s.float() + keep[l, 1].float()).to(x.dtype)
+            assert torch.equal(y, s)
+    finally:
+        T.tardis_destroy(h)

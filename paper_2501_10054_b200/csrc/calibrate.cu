@@ -187,19 +187,24 @@ k_calibrate(const float* __restrict__ z, long long ldz, const float* __restrict_
 //
 // Neither the densities nor the errors are needed as numbers, only which one is the largest / smaller, so both are screened
 // by cheap values with a bound on what these can be off by, and evaluated as defined only where the bound leaves it open:
-//   * density: value F and slope F' at every 16th sample in fp32.  |F''| <= N per squared kernel width, so
-//     F(x) <= F(c) + F'(c) t + N t^2 / 2 at a distance of t widths; only samples whose bound reaches the largest value seen
-//     (about 150 of 2048) are evaluated in fp32, and of those only the ones within the fp32 error of the best (a handful) in
-//     fp64.  All N^2 exponentials in fp64 took 95 % of the time before.
-//   * candidate errors: from moments that grow with the range (fp64 sums over the samples of each step, made for all steps
-//     at once, a thread each).  One warp then walks the steps, half of its lanes with the left candidate, half with the right.
-//     Two errors closer than the rounding bound of the moments (or moments that cancel) are evaluated by the definition;
-//     exact zeros of piecewise-linear activations, on which the tie rule depends, thus stay exact.
-// 16384 neurons x 2048 samples: 4.3 ms (133 ms with every density and error evaluated as defined).
+//   * density: the samples fall into bins of a quarter of the kernel width (only those that hold any are kept: some 130 of 260
+//     possible ones); from the moments of the bins around it, each bin gets the Taylor polynomial of the density about its
+//     centre (Hermite polynomials, order 4 on both sides), which gives all samples' densities to 1e-5 N.  Only the samples within
+//     that of the best (some 30 of 2048) are evaluated as sums of exponentials in fp32, and of those only the ones that these
+//     cannot tell apart (a handful) in fp64.  All N^2 exponentials in fp64 took 95 % of the time at first; values and slopes at
+//     every 16th sample, with |F''| <= N, still left 300 samples' worth of exponentials.
+//   * candidate errors: from moments of the samples that the steps on either side add (fp64, made for all steps at once and summed
+//     up by scans).  One warp walks the steps; its lanes hold the errors of all ranges that the next six steps can lead to, so
+//     that the chain of dependent fp64 instructions is paid once per six steps.  Two errors closer than the rounding bound of
+//     the moments (or moments that cancel) are evaluated by the definition; exact zeros of piecewise-linear activations, on
+//     which the tie rule depends, thus stay exact.
+// 16384 neurons x 2048 samples: 2.4 ms (133 ms with every density and error evaluated as defined).
 constexpr int kMaxSearchSamples = 2048;
-constexpr int kMaxSteps = 160;           // steps on one side whose moments are made ahead (later ones: when they are reached)
-constexpr int kCoarse = 16;              // samples per coarse density point
-constexpr int kMaxCoarse = kMaxSearchSamples / kCoarse;
+constexpr int kMaxSteps = 160;           // steps on one side whose moments are made at once
+constexpr int kAhead = 6;                // steps that a warp looks ahead: 28 ranges
+// Bins: samples within 5 standard deviations fill at most 10 / (0.25 * 1.06 N^-0.2) = 174 of them at N = 2048 (fewer below), and at
+// most N / 25 samples lie beyond.
+constexpr int kMaxBins = 272;
 
 __device__ __forceinline__ float ex2f(float x) { float y; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
 __device__ __forceinline__ double warp_sum(double v) {
@@ -208,76 +213,149 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// Position of the highest density among the sorted samples keys[0 .. n - 1] (the smallest position among equals); the whole
-// CTA, every thread gets it.  bw: kernel width (> 0).  list: room for n positions.
-__device__ __forceinline__ int densest_sample(const float* keys, int n, double bw, int* list) {
-  __shared__ float cf[kMaxCoarse], cs[kMaxCoarse];
+struct Bins {
+  float centre[kMaxBins];
+  float m[5][kMaxBins];                  // sum of offset^n / n! of the bin's samples, offsets from the centre in kernel widths
+  float l[5][kMaxBins];                  // Taylor coefficients of the density about the centre
+};
+struct Steps {
+  double m[2][5][kMaxSteps + 1];         // [side][moment][k]: what the first k steps add
+  int end[2][kMaxSteps + 1];             // position of the range's end after k steps
+};
+
+// Position of the highest density among the sorted samples (the smallest position among equals); the whole CTA, every thread gets
+// it.  v: the thread's samples (positions tid E ...), keys: all of them; bw: kernel width (> 0); list: room for n positions.
+template <int E> __device__ __forceinline__ int densest_sample(const float (&v)[E], const float* keys, int n, double bw, Bins& bins, int* list) {
   __shared__ float wmax[NT / 32];
+  __shared__ int wcnt[NT / 32];
   __shared__ double bestv[NT / 32];
   __shared__ int besti[NT / 32];
   __shared__ int count;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const float scale = float(0.8493218002880191 / bw);       // sqrt(log2(e) / 2) / width: e^(-u^2/2) = 2^-(scale (zk - zi))^2
-  const bool screen = bw > 1e-30 && bw < 1e30 && double(keys[n - 1]) - double(keys[0]) < 1e30;
+  const float zmin = keys[0], zmax = keys[n - 1], inv = float(1.0 / bw), width = float(0.25 * bw);
+  bool screen = bw > 1e-30 && bw < 1e30 && double(zmax) - double(zmin) < 1e30;
+  // bins: a sample opens one where its predecessor is in another
+  auto bin_of = [&](float z) { return floorf((z - zmin) * (4.f * inv)); };
+  int first[E], nopen = 0;               // ordinal of the bin within the thread's samples
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const int i = tid * E + e;
+    if (i < n && (i == 0 || bin_of(v[e]) != bin_of(e ? v[e > 0 ? e - 1 : 0] : keys[i - 1]))) ++nopen;
+    first[e] = nopen;
+  }
+  int scan = nopen;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(0xffffffffu, scan, o); if (lane >= o) scan += t; }
+  if (lane == 31) wcnt[warp] = scan;
   if (tid == 0) count = 0;
   __syncthreads();
+  int before = scan - nopen, nbins = 0;
+#pragma unroll
+  for (int w = 0; w < NT / 32; ++w) { if (w < warp) before += wcnt[w]; nbins += wcnt[w]; }
+  screen = screen && nbins <= kMaxBins;
   if (screen) {
-    const int nc = (n + kCoarse - 1) / kCoarse;             // coarse points: samples 8, 24, 40, ...
-    auto point = [&](int c) { return min(c * kCoarse + kCoarse / 2, n - 1); };
-    // a pair of lanes per point, each half of the samples
-    for (int c0 = 0; c0 < nc; c0 += NT / 2) {
-      const int ci = c0 + (tid >> 1);
-      const float zi = keys[point(min(ci, nc - 1))];
-      float f = 0.f, s = 0.f;
-      const int half = (n + 1) >> 1, k0 = (tid & 1) * half, k1 = min(n, k0 + half);
-#pragma unroll 8
-      for (int k = k0; k < k1; ++k) {
-        const float t = (keys[k] - zi) * scale, w = ex2f(-t * t);
-        f += w;
-        s = fmaf(t, w, s);
+    for (int e = tid; e < 5 * nbins; e += NT) bins.m[e / nbins][e % nbins] = 0.f;
+    __syncthreads();
+    // moments: a thread adds up the run of its samples in one bin before it adds to the bin
+    float sum[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const int i = tid * E + e;
+      if (i < n) {
+        const int b = before + first[e] - 1;
+        const float c = zmin + (bin_of(v[e]) + 0.5f) * width, o = (v[e] - c) * inv;
+        if (e == 0 || first[e] != first[e > 0 ? e - 1 : 0]) bins.centre[b] = c;   // (neighbours in other threads write the same)
+        const float o2 = o * o;
+        sum[0] += 1.f; sum[1] += o; sum[2] += 0.5f * o2; sum[3] += o2 * o * (1.f / 6.f); sum[4] += o2 * o2 * (1.f / 24.f);
+        if (e == E - 1 || i == n - 1 || first[e + 1 < E ? e + 1 : e] != first[e]) {
+#pragma unroll
+          for (int q = 0; q < 5; ++q) { atomicAdd(&bins.m[q][b], sum[q]); sum[q] = 0.f; }
+        }
       }
-      f += __shfl_xor_sync(0xffffffffu, f, 1);
-      s += __shfl_xor_sync(0xffffffffu, s, 1);
-      if (!(tid & 1) && ci < nc) { cf[ci] = f; cs[ci] = s * 1.1774100225f; }   // slope per kernel width
     }
     __syncthreads();
-    float best = 0.f;
-    for (int c = tid; c < nc; c += NT) best = fmaxf(best, cf[c]);
+    // Taylor coefficients: e^(-(D + t - o)^2 / 2) = e^(-D^2 / 2) sum He_(n + m)(D) o^n / n! (-t)^m / m!; bins further than 6 widths
+    // away do not count (1.5e-8 N).  A pair of lanes per bin, one for the bins below it and itself, one for those above.
+    for (int b0 = 0; b0 < nbins; b0 += NT / 2) {
+      const int b = b0 + (tid >> 1), dir = (tid & 1) ? 1 : -1;
+      float l[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+      if (b < nbins) {
+        const float c = bins.centre[b];
+        for (int j = dir > 0 ? b + 1 : b; j >= 0 && j < nbins; j += dir) {
+          const float D = (c - bins.centre[j]) * inv;
+          if (fabsf(D) > 6.f) break;
+          float he[9];
+          he[0] = ex2f(-0.7213475204f * D * D);
+          he[1] = D * he[0];
+#pragma unroll
+          for (int q = 2; q < 9; ++q) he[q] = fmaf(D, he[q - 1], -float(q - 1) * he[q - 2]);
+#pragma unroll
+          for (int q = 0; q < 5; ++q) {
+            const float m = bins.m[q][j];
+#pragma unroll
+            for (int r = 0; r < 5; ++r) l[r] = fmaf(he[q + r], m, l[r]);
+          }
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < 5; ++r) l[r] += __shfl_xor_sync(0xffffffffu, l[r], 1);
+      if (b < nbins && !(tid & 1)) {
+        bins.l[0][b] = l[0]; bins.l[1][b] = -l[1]; bins.l[2][b] = 0.5f * l[2]; bins.l[3][b] = l[3] * (-1.f / 6.f); bins.l[4][b] = l[4] * (1.f / 24.f);
+      }
+    }
+    __syncthreads();
+    float f[E], best = 0.f;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const int i = tid * E + e;
+      f[e] = -1.f;
+      if (i < n && !(i > 0 && v[e] == (e ? v[e > 0 ? e - 1 : 0] : keys[i - 1]))) {   // (else the same density as its predecessor)
+        const int b = before + first[e] - 1;
+        const float t = (v[e] - bins.centre[b]) * inv;
+        f[e] = fmaf(t, fmaf(t, fmaf(t, fmaf(t, bins.l[4][b], bins.l[3][b]), bins.l[2][b]), bins.l[1][b]), bins.l[0][b]);
+        best = fmaxf(best, f[e]);
+      }
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, o));
     if (lane == 0) wmax[warp] = best;
     __syncthreads();
 #pragma unroll
     for (int w = 0; w < NT / 32; ++w) best = fmaxf(best, wmax[w]);
-    // What an fp32 density can be off by: the exponent (two roundings of t, squared) by 4e-7 of itself, which changes a term by
-    // less than 2e-7; the additions by 2^-24 of the sum each, 69 in a row for the listed samples (5e-6 N in all, once for each
-    // of two values compared), 1024 in a row for the coarse ones (6e-5 of the sum, 6e-5 N per width for the slope).
-    const float slack = 1e-5f * float(n), N2 = 0.5f * float(n), inv = float(1.0 / bw);
-    for (int i = tid; i < n; i += NT) {
-      if (i > 0 && keys[i] == keys[i - 1]) continue;        // the same density as its neighbour, which comes first
-      const int c = i / kCoarse;
-      const float t = (keys[i] - keys[point(c)]) * inv;
-      const float bound = fmaf(t, fmaf(t, N2, cs[c]), cf[c]);
-      if (bound * 1.0003f + slack * (1.f + 8.f * fabsf(t)) >= best) list[atomicAdd(&count, 1)] = i;
-    }
+    // What a value can be off by: the terms of order 5 left out on either side (|He_5 e^(-D^2/2)| < 6, 8^-5 / 120: 1.5e-6 N each), the
+    // rounding of the offsets (1e-6 N), of the bins' sums (n 2^-24) and of the 45 x 5 products (together 7e-6 N): below 1.2e-5 N, twice for
+    // two values compared.
+    const float slack = 3e-5f * float(n);
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+      if (f[e] >= 0.f && f[e] + slack >= best) list[atomicAdd(&count, 1)] = tid * E + e;
     __syncthreads();
     const int m = count;
-    // fp32 densities of the listed samples, two per warp at a time
-    float* dens = reinterpret_cast<float*>(list + n);
+    // sums of exponentials of the listed samples, two per warp at a time; eight terms at a time in fp32, those sums in fp64
+    const float scale = float(0.8493218002880191 / bw);     // sqrt(log2(e) / 2) / width: e^(-u^2/2) = 2^-(scale (zk - zi))^2
+    float* const dens = reinterpret_cast<float*>(list + n);
     float top = 0.f;
     for (int e = warp * 2; e < m; e += (NT / 32) * 2) {
       const float za = keys[list[e]], zb = keys[list[min(e + 1, m - 1)]];
-      float fa = 0.f, fb = 0.f;
-#pragma unroll 4
-      for (int k = lane; k < n; k += 32) {
-        const float x = keys[k], ta = (x - za) * scale, tb = (x - zb) * scale;
-        fa += ex2f(-ta * ta);
-        fb += ex2f(-tb * tb);
-      }
+      double fa = 0.0, fb = 0.0;
+      for (int k0 = lane; k0 < n; k0 += 256) {
+        float pa = 0.f, pb = 0.f;
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) { fa += __shfl_xor_sync(0xffffffffu, fa, o); fb += __shfl_xor_sync(0xffffffffu, fb, o); }
-      if (lane == 0) { dens[e] = fa; if (e + 1 < m) dens[e + 1] = fb; }
-      top = fmaxf(top, fmaxf(fa, fb));
+        for (int q = 0; q < 8; ++q) {
+          const int k = k0 + 32 * q;
+          if (k < n) {
+            const float x = keys[k], ta = (x - za) * scale, tb = (x - zb) * scale;
+            pa += ex2f(-ta * ta);
+            pb += ex2f(-tb * tb);
+          }
+        }
+        fa += double(pa);
+        fb += double(pb);
+      }
+      fa = warp_sum(fa);
+      fb = warp_sum(fb);
+      if (lane == 0) { dens[e] = float(fa); if (e + 1 < m) dens[e + 1] = float(fb); }
+      top = fmaxf(top, fmaxf(float(fa), float(fb)));
     }
     __syncthreads();                                        // (count and wmax have been read)
     if (tid == 0) count = 0;
@@ -285,11 +363,14 @@ __device__ __forceinline__ int densest_sample(const float* keys, int n, double b
     __syncthreads();
 #pragma unroll
     for (int w = 0; w < NT / 32; ++w) top = fmaxf(top, wmax[w]);
+    // What these can be off by: the exponent (seven roundings) by 4.2e-7 of itself, which changes a term by at most 1.6e-7; the
+    // exponential by 2^-22, the sums of eight terms and the last rounding by 10 2^-24 of the sum; twice for two values compared.
+    const float slack2 = 3.2e-7f * float(n) + 1.8e-6f * top;
     int keep[(kMaxSearchSamples + NT - 1) / NT], nk = 0;
 #pragma unroll
     for (int r = 0; r < (kMaxSearchSamples + NT - 1) / NT; ++r) {
       const int e = r * NT + tid;
-      keep[r] = (e < m && dens[e] + slack >= top) ? list[e] : -1;
+      keep[r] = (e < m && dens[e] + slack2 >= top) ? list[e] : -1;
       nk += keep[r] >= 0;
     }
     __syncthreads();
@@ -304,17 +385,18 @@ __device__ __forceinline__ int densest_sample(const float* keys, int n, double b
   __syncthreads();
   // fp64 densities of what is left, one warp per sample
   const int m = count;
-  const double inv = 1.0 / bw;
+  const double inv64 = 1.0 / bw;
   double bv = -1.0;
   int bi = 0x7fffffff;
-  for (int e = warp; e < m; e += NT / 32) {
+  for (int e = warp; e < m && m > 1; e += NT / 32) {
     const int i = list[e];
     const double zi = double(keys[i]);
     double dsum = 0.0;
-    for (int k = lane; k < n; k += 32) { const double u = (double(keys[k]) - zi) * inv; dsum += exp(-0.5 * u * u); }
+    for (int k = lane; k < n; k += 32) { const double u = (double(keys[k]) - zi) * inv64; dsum += exp(-0.5 * u * u); }
     dsum = warp_sum(dsum);
     if (dsum > bv || (dsum == bv && i < bi)) { bv = dsum; bi = i; }
   }
+  if (m == 1) bi = list[0];
   if (lane == 0) { bestv[warp] = bv; besti[warp] = bi; }
   __syncthreads();
 #pragma unroll
@@ -322,10 +404,6 @@ __device__ __forceinline__ int densest_sample(const float* keys, int n, double b
     if (bestv[w] > bv || (bestv[w] == bv && besti[w] < bi)) { bv = bestv[w]; bi = besti[w]; }
   return bi;
 }
-
-// Moments of some samples about the centroid (y = z - centroid, g = activation - activation at the centroid)
-struct Moments { double y, g, yy, yg, gg; };
-__device__ __forceinline__ Moments operator+(const Moments& p, const Moments& q) { return {p.y + q.y, p.g + q.g, p.yy + q.yy, p.yg + q.yg, p.gg + q.gg}; }
 
 template <int E> __global__ void __launch_bounds__(NT, 4)
 k_range_search(const float* __restrict__ z, long long ldz, const float* __restrict__ b1, int n,
@@ -336,8 +414,9 @@ k_range_search(const float* __restrict__ z, long long ldz, const float* __restri
   float* keys = reinterpret_cast<float*>(gs + NT * E);             // [NT E] sorted samples
   __shared__ double red[1][NT / 32];
   __shared__ float range_s[2];
-  __shared__ Moments ahead[2][kMaxSteps];
-  __shared__ int ends[2][kMaxSteps];
+  __shared__ union Scratch { Bins bins; Steps steps; __device__ Scratch() {} } scratch;
+  __shared__ double base_m[5];                                     // moments of the range so far (the walk starts anew from time to time)
+  __shared__ int base_k[2], base_end[2], total_steps, finished;
   const int j = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
   float v[E];
   load_samples<E>(v, z, ldz, b1, j, n);
@@ -354,120 +433,145 @@ k_range_search(const float* __restrict__ z, long long ldz, const float* __restri
   for (int e = 0; e < E; ++e) if (tid * E + e < n) { const double dz = double(v[e]) - mean; s2[0] += dz * dz; }
   block_sums<1>(s2, red);
   const double bw = n > 1 ? 1.06 * sqrt(s2[0] / double(n - 1)) * pow(double(n), -0.2) : 0.0;
-  const int ic = bw > 0.0 ? densest_sample(keys, n, bw, reinterpret_cast<int*>(gs)) : 0;
+  const int ic = bw > 0.0 ? densest_sample<E>(v, keys, n, bw, scratch.bins, reinterpret_cast<int*>(gs)) : 0;
   const double cen = double(keys[ic]);
   __syncthreads();                                                 // (the list in the place of gs has been read)
 #pragma unroll
   for (int e = 0; e < E; ++e) gs[tid * E + e] = tid * E + e < n ? gelu_f64(double(v[e]), act) : 0.0;
   __syncthreads();
-  // what every step on either side adds to the range: the samples between two successive bounds
-  const double gc = gs[ic];
-  auto lower = [&](double v) {                            // number of samples below v
+  // number of samples below x
+  auto lower = [&](double x) {
     int l = 0, r = n;
-    while (l < r) { const int m = (l + r) >> 1; if (double(keys[m]) < v) l = m + 1; else r = m; }
+    while (l < r) { const int m = (l + r) >> 1; if (double(keys[m]) < x) l = m + 1; else r = m; }
     return l;
   };
-  // position of the range's end on a side (0 left, 1 right) after k steps; what the step from k to k + 1 adds there
-  auto edge = [&](int side, int k) { return lower(side ? cen + k * step : cen - k * step); };
-  auto added = [&](int side, int k, int& next) {
-    const int p = edge(side, k);
-    next = edge(side, k + 1);
-    Moments m = {0.0, 0.0, 0.0, 0.0, 0.0};
-    for (int i = side ? p : next; i < (side ? next : p); ++i) {
-      const double y = double(keys[i]) - cen, q = gs[i] - gc;
-      m.y += y; m.g += q; m.yy += y * y; m.yg += y * q; m.gg += q * q;
-    }
-    return m;
-  };
-  for (int e = tid; e < 2 * kMaxSteps; e += NT) {
-    const int side = e & 1, k = e >> 1;
-    if (k > 0 && (side ? cen + k * step > double(keys[n - 1]) : cen - k * step <= double(keys[0]))) continue;   // nothing beyond
-    int next;
-    ahead[side][k] = added(side, k, next);
-    ends[side][k] = next;
+  const double gc = gs[ic], zmin = double(keys[0]), zmax = double(keys[n - 1]);
+  const double t = thr ? double(thr[j]) : t_all;
+  const int cap = 4 + 2 * int(fmin(1.0e7, (zmax - zmin) / step + 2.0));   // the loop ends long before; a guard against a bad step
+  Steps& st = scratch.steps;
+  if (tid < 5) base_m[tid] = 0.0;
+  if (tid == 0) {
+    base_k[0] = base_k[1] = total_steps = finished = 0;
+    base_end[0] = base_end[1] = lower(cen);                        // samples inside: none yet
   }
-  __syncthreads();
-  if (tid < 32) {
-    // the greedy loop, one warp: lanes 0 .. 15 look at the left side, lanes 16 .. 31 at the right one
-    const double t = thr ? double(thr[j]) : t_all;
-    const double zmin = double(keys[0]), zmax = double(keys[n - 1]);
-    const int side = lane >> 4;
-    // mean squared residual of the least-squares line over the sorted samples i0 .. i1 - 1, as it is defined
-    auto mse = [&](int i0, int i1) -> double {
-      const int cnt = i1 - i0;
-      if (cnt < 2) return 0.0;
-      const double q = 1.0 / double(cnt);
-      double sz = 0.0, sg = 0.0;
-      for (int i = i0 + lane; i < i1; i += 32) { sz += double(keys[i]); sg += gs[i]; }
-      const double mz = warp_sum(sz) * q, mg = warp_sum(sg) * q;
-      double vzz = 0.0, vzg = 0.0;
-      for (int i = i0 + lane; i < i1; i += 32) { const double dz = double(keys[i]) - mz; vzz += dz * dz; vzg += dz * (gs[i] - mg); }
-      vzz = warp_sum(vzz) * q; vzg = warp_sum(vzg) * q;
-      if (!(vzz > 1e-30)) return 0.0;
-      const double sl = vzg / vzz;
-      double rr = 0.0;
-      for (int i = i0 + lane; i < i1; i += 32) { const double r = (gs[i] - mg) - sl * (double(keys[i]) - mz); rr += r * r; }
-      return warp_sum(rr) * q;
-    };
-    // the same from the moments of the range (times its number of samples, and so on, to have one division), and what it
-    // can be off by (infinite where the moments cancel)
-    auto quick = [&](const Moments& m, int i0, int i1, float& off) -> double {
-      const int cnt = i1 - i0;
-      off = 0.f;
-      if (cnt < 2) return 0.0;
-      if (act == TARDIS_ACT_RELU && (keys[i0] > 0.f || keys[i1 - 1] <= 0.f)) return 0.0;   // one straight piece: exactly zero
-      const double q = double(cnt), yy = m.yy * q, gg = m.gg * q;
-      const double vyy = yy - m.y * m.y, vyg = m.yg * q - m.y * m.g, vgg = gg - m.g * m.g;
-      // every moment is off by less than 1e-13 of the sum of its terms' sizes (2 n 2^-53); |yg| <= sqrt(yy gg)
-      const float k = 1.f + __fdividef(float(yy), float(vyy)), iq = __fdividef(1.f, float(q));
-      off = fmaxf(1e-12f * float(gg) * iq * iq * k * k, 1e-37f);
-      if (!(vyy > 1e-8 * yy && vyy > 1e-25 * q * q)) off = __int_as_float(0x7f800000);
-      return (vgg * vyy - vyg * vyg) / (vyy * q * q);
-    };
-    int kl = 0, kr = 0, nsteps = 0;
-    int i0 = edge(0, 0), i1 = i0;                                  // samples inside: i0 .. i1 - 1 (none yet)
-    Moments in = {0.0, 0.0, 0.0, 0.0, 0.0};
-    const int cap = 4 + 2 * int(fmin(1.0e7, (zmax - zmin) / step + 2.0));   // the loop ends long before; a guard against a bad step
-    for (; nsteps < cap; ++nsteps) {
-      const double l = cen - kl * step, u = cen + kr * step;
-      const int inside = i1 - i0;
-      if (double(inside) >= t * double(n) || inside == n) break;
-      const bool right_done = u > zmax, left_done = l <= zmin;     // (not both: every sample would be inside)
-      // the range grown on the lane's side, if there is anything left on it
-      int end = side ? i1 : i0;
-      Moments m = in;
-      if (side ? !right_done : !left_done) {
-        const int k = side ? kr : kl;
-        if (k < kMaxSteps) { m = in + ahead[side][k]; end = ends[side][k]; }
-        else m = in + added(side, k, end);
+  do {
+    __syncthreads();                                               // (the bins, or the steps before, have been read)
+    // (1) where the next kMaxSteps steps on either side end, (2) what each adds about the centroid (y = z - centroid, g = activation -
+    // activation at the centroid; sums of y, g, y y, y g, g g), (3) running sums
+    for (int e = tid; e < 2 * (kMaxSteps + 1); e += NT) {
+      const int side = e & 1, k = e >> 1;
+      st.end[side][k] = k == 0 ? base_end[side] : lower(side ? cen + (base_k[1] + k) * step : cen - (base_k[0] + k) * step);
+    }
+    __syncthreads();
+    for (int e = tid; e < 2 * kMaxSteps; e += NT) {
+      const int side = e & 1, k = e >> 1;
+      const int p0 = side ? st.end[1][k] : st.end[0][k + 1], p1 = side ? st.end[1][k + 1] : st.end[0][k];
+      double m0 = 0.0, m1 = 0.0, m2 = 0.0, m3 = 0.0, m4 = 0.0;
+      for (int i = p0; i < p1; ++i) {
+        const double y = double(keys[i]) - cen, q = gs[i] - gc;
+        m0 += y; m1 += q; m2 += y * y; m3 += y * q; m4 += q * q;
       }
-      bool go_left;
-      if (right_done) go_left = true;
-      else if (left_done) go_left = false;
-      else {
-        float off;
-        const double e = quick(m, side ? i0 : end, side ? end : i1, off);
-        const double eo = __shfl_xor_sync(0xffffffffu, e, 16);
-        const float oo = __shfl_xor_sync(0xffffffffu, off, 16);
-        const double gap = side ? e - eo : eo - e;                 // right minus left
-        go_left = gap > 0.0;
-        const bool open = !(fabs(gap) > double(off + oo)) && off + oo != 0.f;
-        if (__any_sync(0xffffffffu, open)) {                       // (every lane agrees; the vote makes the branch a uniform one)
-          const int l0 = __shfl_sync(0xffffffffu, end, 0), r1 = __shfl_sync(0xffffffffu, end, 16);
-          go_left = mse(l0, i1) < mse(i0, r1);
+      st.m[side][0][k + 1] = m0; st.m[side][1][k + 1] = m1; st.m[side][2][k + 1] = m2; st.m[side][3][k + 1] = m3; st.m[side][4][k + 1] = m4;
+    }
+    __syncthreads();
+    for (int q = tid >> 5; q < 10; q += NT / 32) {
+      double* const m = st.m[q & 1][q >> 1];
+      double carry = 0.0;
+      if (lane == 0) m[0] = 0.0;
+      for (int k0 = 1; k0 <= kMaxSteps; k0 += 32) {                // (kMaxSteps is a multiple of 32)
+        double x = m[k0 + lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const double up = __shfl_up_sync(0xffffffffu, x, o); if (lane >= o) x += up; }
+        x += carry;
+        m[k0 + lane] = x;
+        carry = __shfl_sync(0xffffffffu, x, 31);
+      }
+    }
+    __syncthreads();
+    if (tid < 32) {
+      // mean squared residual of the least-squares line over the sorted samples i0 .. i1 - 1, as it is defined
+      auto mse = [&](int i0, int i1) -> double {
+        const int cnt = i1 - i0;
+        if (cnt < 2) return 0.0;
+        const double q = 1.0 / double(cnt);
+        double sz = 0.0, sg = 0.0;
+        for (int i = i0 + lane; i < i1; i += 32) { sz += double(keys[i]); sg += gs[i]; }
+        const double mz = warp_sum(sz) * q, mg = warp_sum(sg) * q;
+        double vzz = 0.0, vzg = 0.0;
+        for (int i = i0 + lane; i < i1; i += 32) { const double dz = double(keys[i]) - mz; vzz += dz * dz; vzg += dz * (gs[i] - mg); }
+        vzz = warp_sum(vzz) * q; vzg = warp_sum(vzg) * q;
+        if (!(vzz > 1e-30)) return 0.0;
+        const double sl = vzg / vzz;
+        double rr = 0.0;
+        for (int i = i0 + lane; i < i1; i += 32) { const double r = (gs[i] - mg) - sl * (double(keys[i]) - mz); rr += r * r; }
+        return warp_sum(rr) * q;
+      };
+      // lane = range after i steps to the left and jr to the right, i + jr <= kAhead: lanes s (s + 1) / 2 + jr, s = i + jr
+      auto lane_of = [](int i, int jr) { const int s = i + jr; return s * (s + 1) / 2 + jr; };
+      int s_mine = 0;
+      while ((s_mine + 1) * (s_mine + 2) / 2 <= lane) ++s_mine;
+      const int j_mine = min(lane - s_mine * (s_mine + 1) / 2, kAhead), i_mine = max(0, min(s_mine, kAhead) - j_mine);
+      int kl = 0, kr = 0, nsteps = total_steps;
+      bool done = false;
+      while (!done && kl + kAhead <= kMaxSteps && kr + kAhead <= kMaxSteps) {
+        // the lane's range: error from the moments (times its number of samples, and so on, to have one division), and what it can be
+        // off by (infinite where the moments cancel)
+        const int e0 = st.end[0][kl + i_mine], e1 = st.end[1][kr + j_mine], cnt = e1 - e0;
+        double err = 0.0;
+        float off = 0.f;
+        if (cnt >= 2 && !(act == TARDIS_ACT_RELU && (keys[e0] > 0.f || keys[e1 - 1] <= 0.f))) {   // (one straight piece: exactly zero)
+          double m[5];
+#pragma unroll
+          for (int q = 0; q < 5; ++q) m[q] = base_m[q] + (st.m[0][q][kl + i_mine] + st.m[1][q][kr + j_mine]);
+          const double q = double(cnt), yy = m[2] * q, gg = m[4] * q;
+          const double vyy = yy - m[0] * m[0], vyg = m[3] * q - m[0] * m[1], vgg = gg - m[1] * m[1];
+          // every moment is off by less than 1e-13 of the sum of its terms' sizes (2 n 2^-53); |yg| <= sqrt(yy gg)
+          const float k = 1.f + __fdividef(float(yy), float(vyy)), iq = __fdividef(1.f, float(q));
+          off = fmaxf(1e-12f * float(gg) * iq * iq * k * k, 1e-37f);
+          if (!(vyy > 1e-8 * yy && vyy > 1e-25 * q * q)) off = __int_as_float(0x7f800000);
+          else err = (vgg * vyy - vyg * vyg) / (vyy * q * q);
         }
+        int i = 0, jr = 0;
+        while (i + jr < kAhead) {                                  // (the same for all lanes)
+          const double l = cen - (base_k[0] + kl + i) * step, u = cen + (base_k[1] + kr + jr) * step;
+          const int here = lane_of(i, jr), p0 = __shfl_sync(0xffffffffu, e0, here), p1 = __shfl_sync(0xffffffffu, e1, here);
+          const int inside = p1 - p0;
+          done = double(inside) >= t * double(n) || inside == n || nsteps >= cap;
+          if (done) break;
+          bool go_left;
+          if (u > zmax) go_left = true;                            // (not both sides: every sample would be inside)
+          else if (l <= zmin) go_left = false;
+          else {
+            const int ll = lane_of(i + 1, jr), lr = lane_of(i, jr + 1);
+            const double el = __shfl_sync(0xffffffffu, err, ll), er = __shfl_sync(0xffffffffu, err, lr);
+            const float o = __shfl_sync(0xffffffffu, off, ll) + __shfl_sync(0xffffffffu, off, lr);
+            go_left = el < er;
+            const bool open = !(fabs(el - er) > double(o)) && o != 0.f;
+            if (__any_sync(0xffffffffu, open)) {                   // (every lane agrees; the vote makes the branch a uniform one)
+              const int l0 = __shfl_sync(0xffffffffu, e0, ll), r1 = __shfl_sync(0xffffffffu, e1, lr);
+              go_left = mse(l0, p1) < mse(p0, r1);
+            }
+          }
+          if (go_left) ++i; else ++jr;
+          ++nsteps;
+        }
+        kl += i;
+        kr += jr;
       }
-      const int from = go_left ? 0 : 16;
-      in.y = __shfl_sync(0xffffffffu, m.y, from); in.g = __shfl_sync(0xffffffffu, m.g, from); in.yy = __shfl_sync(0xffffffffu, m.yy, from);
-      in.yg = __shfl_sync(0xffffffffu, m.yg, from); in.gg = __shfl_sync(0xffffffffu, m.gg, from);
-      const int at = __shfl_sync(0xffffffffu, end, from);
-      if (go_left) { ++kl; i0 = at; } else { ++kr; i1 = at; }
+      if (lane < 5) base_m[lane] += st.m[0][lane][kl] + st.m[1][lane][kr];
+      if (lane == 0) {
+        base_k[0] += kl; base_k[1] += kr;
+        base_end[0] = st.end[0][kl]; base_end[1] = st.end[1][kr];
+        total_steps = nsteps;
+        finished = done;
+      }
     }
-    if (lane == 0) {
-      range_s[0] = float(cen - kl * step);
-      range_s[1] = float(cen + kr * step);
-      if (steps_out) steps_out[j] = nsteps;
-    }
+    __syncthreads();
+  } while (!finished);
+  if (tid == 0) {
+    range_s[0] = float(cen - base_k[0] * step);
+    range_s[1] = float(cen + base_k[1] * step);
+    if (steps_out) steps_out[j] = total_steps;
   }
   __syncthreads();
   double g[E];

@@ -41,6 +41,19 @@ def test_ranges_and_fits_match_oracle(shape, act):
     _check(z, None, 0.4, 0.4, act)                              # empty range: every neuron takes the tangent
 
 
+@pytest.mark.parametrize("n", [2, 255, 256, 1500, 4097])
+@pytest.mark.parametrize("q", [(0.0, 1.0), (0.05, 0.95), (0.5, 0.5)])
+def test_quantiles_picked_without_sorting_and_where_that_is_left_to_the_sort(n, q):
+    # samples far out that put all others into one step of the histogram, many equal ones, all equal, an ordinary row, two heaps
+    g = torch.Generator().manual_seed(n)
+    z = torch.randn(5, n, generator=g)
+    z[0, 0], z[0, -1] = 1e6, -3e5
+    z[1] = (z[1] * 3).round() / 3
+    z[2] = 0.25
+    z[4] += torch.where(torch.rand(n, generator=g) < 0.5, 50.0, -50.0)
+    _check(z.cuda(), None, q[0], q[1], W.ACT_GELU_TANH)
+
+
 def test_padded_rows_ties_and_degenerate_neurons():
     # leading dimension larger than n, many equal samples, constant neurons
     g = torch.Generator().manual_seed(7)

@@ -318,34 +318,34 @@ k_few_in(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUten
     // ---------------- token norms sum |x|, read beside the MMAs while the first tile passes by ----------------
     const int total = Walk(p, wf).total;
     const bool any_tile = int(blockIdx.x) < p.ntiles;
-    float sum[2] = {0.f, 0.f};
-    bool bad[2] = {false, false};
-    const int tk = (warp - 2) * 32 + lane;
+    // A stage goes back only when they have read it, so they must not take longer than the MMAs: LPT lanes per token, each with its
+    // 16-byte pieces of a 128-byte row, four sums side by side (one lane per token and one chain of additions: 5 us per call).
+    constexpr int LPT = N >= 64 ? 1 : 64 / N, TPL = N > 64 ? N / 64 : 1, PIECES = 8 / LPT;
+    float sum[TPL][4] = {};
+    const int me = (warp - 2) * 32 + lane;
     for (int i = 0, s = 0, parity = 0; i < total; ++i) {
       if (!mbar_wait_warp(&full[s], parity)) { *failed = 1u; break; }
       if (any_tile && i < nkb) {
         const uint8_t* xt = smem + s * C::STAGE + W_BYTES;
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
-          const int t = tk + 64 * r;
-          if (t < N) {
+        for (int r = 0; r < TPL; ++r) {
+          const int t = me / LPT + 64 * r;
 #pragma unroll
-            for (int c = 0; c < 8; ++c) {
-              const uint4 v = *reinterpret_cast<const uint4*>(xt + t * 128 + ((c ^ (t & 7)) << 4));
-              const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+          for (int c = 0; c < PIECES; ++c) {
+            const uint4 v = *reinterpret_cast<const uint4*>(xt + t * 128 + (((c * LPT + me % LPT) ^ (t & 7)) << 4));
+            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-              for (int q = 0; q < 4; ++q) {
-                const float lo = fabsf(__uint_as_float(w[q] << 16)), hi = fabsf(__uint_as_float(w[q] & 0xffff0000u));
-                bad[r] |= !(lo <= 3.0e38f) || !(hi <= 3.0e38f);
-                sum[r] += lo + hi;
-              }
-            }
+            for (int q = 0; q < 4; ++q) sum[r][q] += fabsf(__uint_as_float(w[q] << 16)) + fabsf(__uint_as_float(w[q] & 0xffff0000u));
           }
         }
         if (i == nkb - 1) {
 #pragma unroll
-          for (int r = 0; r < 2; ++r)
-            if (tk + 64 * r < N) x1[tk + 64 * r] = bad[r] ? __int_as_float(0x7f800000) : sum[r];
+          for (int r = 0; r < TPL; ++r) {
+            float tot = (sum[r][0] + sum[r][1]) + (sum[r][2] + sum[r][3]);   // (inf or NaN where the token holds one)
+#pragma unroll
+            for (int o = LPT / 2; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+            if (me % LPT == 0) x1[me / LPT + 64 * r] = tot <= 3.0e38f ? tot : __int_as_float(0x7f800000);
+          }
         }
       }
       __syncwarp();

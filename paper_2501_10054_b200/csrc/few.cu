@@ -34,6 +34,7 @@ constexpr int W_BYTES = BM * BK * 2;
 constexpr int NT_IN = 384;                // warp 0 TMA, 1 MMA, 2..3 token norms, 4..11 predictor expansion and epilogues
 constexpr int NT_OUT = 192;               // warp 0 TMA, 1 MMA, 2..5 epilogue
 constexpr int MAX_TOKENS = 128;
+constexpr int BARS = 512;                 // bytes for barriers and a few words behind the stages
 constexpr int MAX_NEAR = 256;             // scores near a range end per tile that can queue (further ones are settled in place)
 constexpr float kEps = 7.62939453125e-6f; // 2^-17: accumulation-error allowance of the fast scores, relative to 3 max s |x|_1
 
@@ -59,19 +60,23 @@ struct OutParams {
 
 template <int N> struct InCfg {
   static constexpr int X_BYTES = N * BK * 2, STAGE = W_BYTES + X_BYTES;
-  static constexpr int NS = N == 128 ? 5 : (N == 64 ? 4 : (N == 32 ? 5 : 6));
+  static constexpr int NS = N == 128 ? 6 : (N == 64 ? 8 : (N == 32 ? 10 : 11));
   static constexpr int NBUF = N == 64 ? 2 : 4;                      // expanded predictor blocks in TMEM (32 columns each)
   static constexpr int COL_S = 0, COL_Z = N, COL_F = 2 * N, COL_A = 3 * N;
   // A CTA that starts early must leave the columns that the launch before it still has to allocate on the same SM, or the two
   // wait for each other: 256 of 512 up to 64 columns of tokens (k_few_out takes 128 at most).  With 128 it takes all, after the wait.
   static constexpr int TMEM = COL_A + NBUF * 32 <= 256 ? 256 : 512;
-  static constexpr int SMEM = 1024 + NS * STAGE + 256 + MAX_NEAR * 16 + BM * ((N + 31) / 32) * 4 + N * 8 + 8 * 1024;
+  static constexpr int SMEM = 1024 + NS * STAGE + BARS + MAX_NEAR * 16 + BM * ((N + 31) / 32) * 4 + N * 8 + 8 * 1024;
+  static_assert((2 * NS + 2 * NBUF + 5) * 8 + 16 <= BARS, "barriers");
+  static_assert(SMEM <= 232448, "shared memory");
 };
 template <int N> struct OutCfg {
   static constexpr int X_BYTES = N * BK * 2, STAGE = W_BYTES + X_BYTES;
-  static constexpr int NS = N == 128 ? 4 : (N == 64 ? 4 : 5);
+  static constexpr int NS = N == 128 ? 6 : (N == 64 ? 9 : 10);
   static constexpr int TMEM = N < 32 ? 32 : N;
-  static constexpr int SMEM = 1024 + NS * STAGE + 256;
+  static constexpr int SMEM = 1024 + NS * STAGE + BARS;
+  static_assert((2 * NS + 2) * 8 + 16 <= BARS, "barriers");
+  static_assert(SMEM <= 232448, "shared memory");
 };
 
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
@@ -213,7 +218,7 @@ k_few_in(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUten
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(norm_ready + 1);
   volatile uint32_t* failed = tmem_slot + 1;
   uint32_t* near_count = tmem_slot + 2;
-  uint4* near = reinterpret_cast<uint4*>(smem + C::NS * C::STAGE + 256);          // [MAX_NEAR] row << 8 | token, lo, hi, b1
+  uint4* near = reinterpret_cast<uint4*>(smem + C::NS * C::STAGE + BARS);         // [MAX_NEAR] row << 8 | token, lo, hi, b1
   uint32_t* settled = reinterpret_cast<uint32_t*>(near + MAX_NEAR);               // [BM][(N + 31) / 32] re-evaluated scores that are outside
   float* x1 = reinterpret_cast<float*>(settled + BM * ((N + 31) / 32));           // [N] sum |x|
   unsigned int* tok_flagged = reinterpret_cast<unsigned int*>(x1 + N);            // [N]
@@ -556,7 +561,7 @@ k_few_in(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUten
 // Corrections times W2.  N: columns (tokens rounded up, times the terms of a correction).  CTA c works on the pairs
 // [c total / grid, (c + 1) total / grid) of (output tile, neuron block).
 template <int N>
-__global__ void __maxnreg__(80)                        // (NT_OUT threads beside NT_IN of k_few_in: 64512 of 65536 registers)
+__global__ void __maxnreg__(64)                        // (a quarter of the SM then holds three warps of k_few_in and two of these)
 k_few_out(const __grid_constant__ CUtensorMap tmW2, const __grid_constant__ CUtensorMap tmD, const OutParams p) {
   using C = OutCfg<N>;
   extern __shared__ uint8_t smem_raw[];
@@ -674,13 +679,13 @@ k_few_out(const __grid_constant__ CUtensorMap tmW2, const __grid_constant__ CUte
           if (i4 < p.d) {
             const float4 bf = *reinterpret_cast<const float4*>(p.bf + i4);
 #pragma unroll 1
-            for (int t0 = q; t0 < p.n; t0 += 32) {
-              float4 v[8];
+            for (int t0 = q; t0 < p.n; t0 += 16) {
+              float4 v[4];
 #pragma unroll
-              for (int r = 0; r < 8; ++r)
+              for (int r = 0; r < 4; ++r)
                 if (t0 + 4 * r < p.n) v[r] = __ldcg(reinterpret_cast<const float4*>(p.yacc + size_t(t0 + 4 * r) * p.d + i4));
 #pragma unroll
-              for (int r = 0; r < 8; ++r)
+              for (int r = 0; r < 4; ++r)
                 if (t0 + 4 * r < p.n) {
                   const size_t at = size_t(t0 + 4 * r) * p.d + i4;
                   const __nv_bfloat162 o[2] = {__floats2bfloat162_rn(v[r].x + bf.x, v[r].y + bf.y), __floats2bfloat162_rn(v[r].z + bf.z, v[r].w + bf.w)};
@@ -813,7 +818,11 @@ tardis_status_t few_prepare(Handle* H) {
     const cudaError_t e = dev_malloc(r.p, r.bytes);
     if (e != cudaSuccess) { set_last_error(e, "cudaMalloc"); cudaGetLastError(); few_release(H); return TARDIS_ERR_ALLOC; }
   }
-  auto room = [](auto kernel, int smem) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); };
+  // (all of an SM's shared memory, so that both kernels fit on it side by side: the share is fixed while a kernel runs there)
+  auto room = [](auto kernel, int smem) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    return e != cudaSuccess ? e : cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  };
   const cudaError_t es[] = {room(k_few_in<16, 2>, InCfg<16>::SMEM), room(k_few_in<32, 1>, InCfg<32>::SMEM), room(k_few_in<64, 1>, InCfg<64>::SMEM),
                             room(k_few_in<128, 1>, InCfg<128>::SMEM), room(k_few_out<32>, OutCfg<32>::SMEM), room(k_few_out<64>, OutCfg<64>::SMEM),
                             room(k_few_out<128>, OutCfg<128>::SMEM)};

@@ -23,14 +23,13 @@
 //     one channel chunk at a time and draws output tiles from a global ticket of that chunk, so the
 //     units spread over all CTAs however busy each one is.
 //   * All 16 warps meet; flags are compacted by ballot + prefix sum into the CTA's ascending list.
-//   * Result fixing: the predictor buffers are free by now and become row slots.  The W1 rows of the
+//   * Result fixing: the predictor's shared memory is free by now and becomes row slots.  The W1 rows of the
 //     CTA's flagged neurons, then their W2T rows, are fetched by one bulk copy per row, all slots at once
 //     (a ring of slot groups when there are more rows than slots).  W1 rows give z_j (the warps split
 //     the channels) and delta_j = GELU(z_j) - a_j z_j - c_j; then every thread owns 8 output columns
 //     (per slot of 512 vectors) and adds delta_j times its slice of the W2T rows.
-//   * All partial outputs are added (red.global) into one of a few replicas of an fp32 accumulator
-//     (the replicas keep the number of reductions per address small).  CTAs count themselves when
-//     done; the last one sums the replicas, adds b_f, rounds to bf16, and re-zeroes the scratch.
+//   * All partial outputs are added (red.global) into an fp32 accumulator.  CTAs count themselves when
+//     done; the last one adds b_f, rounds to bf16, and re-zeroes the scratch.
 #include <stdio.h>
 
 #include <vector>
@@ -52,7 +51,6 @@ constexpr int MAXBUF = 8;         // predictor unit buffers in shared memory
 constexpr int MAXSLOTS = 16;      // rows of W1 / W2T held in shared memory at once by the result fixing
 constexpr int MAXGROUPS = 8;      // slot groups (one barrier each) of the result fixing
 constexpr int kBadRow = 0x40000000;   // row whose group scales do not fit the integer form: always re-evaluated
-constexpr int NREP = 4;           // replicas of the output accumulator
 constexpr int XVR = 2;            // 8-channel vectors of x per thread (padded d <= 8192)
 // control words (unsigned int) in global scratch; all zero between calls
 constexpr int CTL_TICKET = 0;     // [32] stride 32: next output tile of a channel chunk of the folded matrix
@@ -71,7 +69,7 @@ struct Params {
   const int* rowexp;       // per neuron: power of two its integer group scales are expressed in (kBadRow: none)
   const int2* plan;        // per CTA: first tile, tile count
   const __nv_bfloat16* x; __nv_bfloat16* y;
-  float* yacc;             // [NREP][dacc] fp32
+  float* yacc;             // [dacc] fp32
   unsigned int* ctl; unsigned long long* counters;
   uint32_t* dbg_bitmap; double* dbg_scores;
   int d, dpad, dacc, h, ngroups, act;
@@ -90,22 +88,19 @@ struct Scratch {           // handle-owned device memory of the fused path
 };
 
 // ---- shared-memory carve-up (host and device agree through this) -----------------------------------
+// Small tables first, then what only the predictor needs: everything from pbuf on becomes the row slots of the result fixing.
+// (8192 / 32768, one token: with the predictor buffers alone there was room for two rows per CTA, too few in flight to keep
+// the memory busy.)
 struct SmemLayout {
-  size_t pbuf_bytes, pbuf, xq, zeros, xh, sxi, zpart, wpart, score, tab, fl_j, fl_delta, rc, flagbits, wred, bars, misc, total;
+  size_t pbuf, xq, zeros, xh, sxi, zpart, wpart, score, tab, fl_j, fl_delta, rc, flagbits, wred, bars, misc, total;
   __host__ __device__ SmemLayout(int dpad, int ngroups, int tiles_max, int nbuf, int unit_bytes) {
     size_t o = 0;
     auto take = [&](size_t bytes, size_t align) { o = (o + align - 1) / align * align; size_t r = o; o += bytes; return r; };
     const size_t rows = size_t(tiles_max) * 16;
-    pbuf_bytes = size_t(nbuf) * unit_bytes;
-    if (pbuf_bytes < size_t(4) * dpad) pbuf_bytes = size_t(4) * dpad;   // room for two rows of the result fixing
-    pbuf = take(pbuf_bytes, 128);
-    xq = take(size_t(4) * (dpad + 64), 128);
     zeros = take(256, 16);                    // what the lanes that feed unused operand columns read
     xh = take(size_t(dpad + 16) * 2, 16);     // + 16 zeros: the B operand of lanes that feed the unused columns
     sxi = take(size_t(ngroups + 16) * sizeof(int), 8);
-    zpart = take(rows * NW * sizeof(double), 8);
     wpart = take(size_t(2) * MAXSLOTS * NW * sizeof(float), 4);
-    score = take(rows * sizeof(double), 8);
     tab = take(6 * rows * sizeof(float), 4);
     fl_j = take(rows * sizeof(int), 4);
     fl_delta = take(rows * sizeof(float), 4);
@@ -114,6 +109,10 @@ struct SmemLayout {
     wred = take(size_t(3) * NW * sizeof(float), 4);
     bars = take(size_t(MAXBUF + MAXGROUPS) * sizeof(uint64_t), 8);
     misc = take(48 * sizeof(int), 8);
+    pbuf = take(size_t(nbuf) * unit_bytes, 128);
+    xq = take(size_t(4) * (dpad + 64), 128);
+    zpart = take(rows * NW * sizeof(double), 8);
+    score = take(rows * sizeof(double), 8);
     total = o;
   }
 };
@@ -251,9 +250,8 @@ __global__ void __launch_bounds__(NTH, 2) k_decode(const Params p) {
   // A-fragment order).  A warp works on channel chunks first, first + step, ... and draws the output tiles from
   // the global ticket of the chunk; it streams a unit as four blocks of four 128-bit loads per lane (one
   // block ahead of the one being multiplied), multiplies it with x (the B operand: column 0 = x, other
-  // columns zero) in two independent accumulators, and adds the 16 partial outputs to the accumulator
-  // replica of its CTA.
-  float* const rep = p.yacc + size_t(blockIdx.x % NREP) * p.dacc;
+  // columns zero) in two independent accumulators, and adds the 16 partial outputs to the accumulator.
+  float* const rep = p.yacc;
   auto stream_c = [&](int first, int step) {
     unsigned int* ticket = p.ctl + CTL_TICKET;
     auto issue = [&]() -> unsigned int {        // lane 0 draws; the value is looked at one unit later
@@ -596,7 +594,7 @@ __global__ void __launch_bounds__(NTH, 2) k_decode(const Params p) {
   TARDIS_STAMP(tid == 0, ST_FLAGS);
   TARDIS_STAMP_VALUE(tid == 0, ST_NFL, nfl);
   // ---- result fixing ----
-  // The predictor buffers are free now and take the rows the fixing needs, one bulk copy per row: item i < nfl
+  // The predictor's shared memory is free now and takes the rows the fixing needs, one bulk copy per row: item i < nfl
   // is the W1 row of the i-th flagged neuron, item nfl + i its W2T row.  The row slots form a ring of groups
   // with one barrier each; all groups are filled at once (for a typical token that is every row the CTA
   // needs, so the fixing costs one trip to memory), and a group is filled again as soon as its rows have been
@@ -706,43 +704,38 @@ __global__ void __launch_bounds__(NTH, 2) k_decode(const Params p) {
   TARDIS_STAMP(tid == 0, ST_COUNTED);
   if (misc[MS_LAST] == int(gridDim.x) - 1) {
     __threadfence();
-    for (int vec = tid; vec < p.nvec; vec += NTH) {
-      const int c0 = vec * 8;
-      float4 a0[NREP + 1], a1[NREP + 1];
-      a0[NREP] = *reinterpret_cast<const float4*>(p.bf + c0);
-      a1[NREP] = *reinterpret_cast<const float4*>(p.bf + c0 + 4);
-#pragma unroll
-      for (int rp = 0; rp < NREP; ++rp) {
-        const float* q = p.yacc + size_t(rp) * p.dacc + c0;
-        a0[rp] = __ldcg(reinterpret_cast<const float4*>(q));
-        a1[rp] = __ldcg(reinterpret_cast<const float4*>(q + 4));
-      }
-      float4 s0 = a0[NREP], s1 = a1[NREP];
-#pragma unroll
-      for (int rp = 0; rp < NREP; ++rp) {
-        s0.x += a0[rp].x; s0.y += a0[rp].y; s0.z += a0[rp].z; s0.w += a0[rp].w;
-        s1.x += a1[rp].x; s1.y += a1[rp].y; s1.z += a1[rp].z; s1.w += a1[rp].w;
-        float* q = p.yacc + size_t(rp) * p.dacc + c0;
-        *reinterpret_cast<float4*>(q) = make_float4(0.f, 0.f, 0.f, 0.f);
-        *reinterpret_cast<float4*>(q + 4) = make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-      __nv_bfloat162 o[4];
-      o[0] = __floats2bfloat162_rn(s0.x, s0.y);
-      o[1] = __floats2bfloat162_rn(s0.z, s0.w);
-      o[2] = __floats2bfloat162_rn(s1.x, s1.y);
-      o[3] = __floats2bfloat162_rn(s1.z, s1.w);
-      *reinterpret_cast<uint4*>(p.y + c0) = *reinterpret_cast<const uint4*>(o);
-    }
-    TARDIS_STAMP(tid == 0, ST_FINAL);
-    if (lane == 0) {
-      for (int kc = warp; kc < p.nkc; kc += NW) p.ctl[CTL_TICKET + kc * 32] = 0u;
-      if (warp == 0) {   // every CTA has arrived, so every CTA's flagged count is in
+    // Nothing else runs any more, so this is latency from here to the end: the counts go to the handle beside the sums, and a thread
+    // has all its loads in flight at once.
+    if (warp == NW - 1) {
+      for (int kc = lane; kc < p.nkc; kc += 32) p.ctl[CTL_TICKET + kc * 32] = 0u;
+      if (lane == 0) {   // every CTA has arrived, so every CTA's flagged count is in
         p.ctl[CTL_DONE] = 0u;
         const unsigned int tot = atomicExch(&p.ctl[CTL_NFL], 0u);
         atomicAdd(&p.counters[CTR_FLAGGED_TOTAL], (unsigned long long)tot);
         atomicMax(&p.counters[CTR_FLAGGED_MAX], (unsigned long long)tot);
       }
     }
+    float4 sum[2 * VPT], add[2 * VPT];                              // vectors of 4 columns
+#pragma unroll
+    for (int k = 0; k < 2 * VPT; ++k) {
+      const int c0 = (k * NTH + tid) * 4;
+      if (c0 < d) {
+        sum[k] = __ldcg(reinterpret_cast<const float4*>(p.yacc + c0));
+        add[k] = *reinterpret_cast<const float4*>(p.bf + c0);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 2 * VPT; ++k) {
+      const int c0 = (k * NTH + tid) * 4;
+      if (c0 < d) {
+        *reinterpret_cast<float4*>(p.yacc + c0) = make_float4(0.f, 0.f, 0.f, 0.f);
+        __nv_bfloat162 o[2];
+        o[0] = __floats2bfloat162_rn(add[k].x + sum[k].x, add[k].y + sum[k].y);
+        o[1] = __floats2bfloat162_rn(add[k].z + sum[k].z, add[k].w + sum[k].w);
+        *reinterpret_cast<uint2*>(p.y + c0) = *reinterpret_cast<const uint2*>(o);
+      }
+    }
+    TARDIS_STAMP(tid == 0, ST_FINAL);
   }
 }
 
@@ -881,9 +874,10 @@ tardis_status_t decode_prepare(Handle* H, cudaStream_t s) {
     const int nbuf_lo = units < 2 ? units : 2;
     for (int nbuf = nbuf_hi; nbuf >= nbuf_lo && nbuf >= 1; --nbuf) {
       const size_t need = SmemLayout(dpad, p.ngroups, tiles_max, nbuf, p.unit_bytes).total;
-      if (need <= budget && need <= size_t(max_smem)) {
-        S->grid = grid; p.tiles_max = tiles_max; p.nbuf = nbuf; S->smem_bytes = need;
-        size_t slots = SmemLayout(dpad, p.ngroups, tiles_max, nbuf, p.unit_bytes).pbuf_bytes / (size_t(dpad) * 2);
+      if (need <= budget && need <= size_t(max_smem)) {   // (x alone, four bytes per channel, leaves room for two rows)
+        S->grid = grid; p.tiles_max = tiles_max; p.nbuf = nbuf;
+        S->smem_bytes = budget < size_t(max_smem) ? budget : size_t(max_smem);
+        size_t slots = (S->smem_bytes - SmemLayout(dpad, p.ngroups, tiles_max, nbuf, p.unit_bytes).pbuf) / (size_t(dpad) * 2);
         if (slots > size_t(MAXSLOTS)) slots = MAXSLOTS;
         p.fix_gs = slots >= 6 ? int(slots) / 3 : 1;
         p.fix_ng = int(slots) / p.fix_gs;
@@ -899,7 +893,7 @@ tardis_status_t decode_prepare(Handle* H, cudaStream_t s) {
   auto fail = [&](tardis_status_t st) { H->dscratch = S; decode_release(H); return st; };
   size_t tally = 0;
   const size_t pb_bytes = size_t(NT) * p.nkc * p.pbs;
-  const size_t yacc_bytes = sizeof(float) * NREP * p.dacc;
+  const size_t yacc_bytes = sizeof(float) * p.dacc;
   cudaError_t e = dev_malloc(&S->pblocks, pb_bytes); tally += pb_bytes;
   if (e == cudaSuccess) { e = dev_malloc(&S->plan, sizeof(int2) * grid); tally += sizeof(int2) * grid; }
   if (e == cudaSuccess) { e = dev_malloc(&S->smax, 16); tally += 16; }

@@ -24,9 +24,8 @@
 //     for the tokens that flagged the neuron, else 0.  Outputs: A = the W2^T rows transposed by
 //     ldmatrix.trans (16 output columns x 16 neurons), B = delta split into two bf16 terms, accumulators
 //     for all output columns stay in registers over all steps.
-//   * All partial outputs are added (red.global) into one of a few replicas of the fp32 accumulator; CTAs
-//     count themselves when done; the last one sums the replicas, adds b_f, rounds to bf16, writes y and
-//     re-zeroes the scratch.
+//   * All partial outputs are added (red.global) into an fp32 accumulator; CTAs count themselves when done; the
+//     last one adds b_f, rounds to bf16, writes y and re-zeroes the scratch.
 #include <stdio.h>
 
 #include <new>
@@ -50,8 +49,6 @@ constexpr int MAXRC = 64;         // exact re-checks per CTA and pass before the
 constexpr int MAXBUF = 10;        // predictor tile buffers in shared memory
 constexpr int MAXGROUPS = 4;      // slot groups (one barrier each, one buffer of partial sums each) of the result fixing
 constexpr int MAXGS = 16;         // rows per slot group (one MMA tile)
-constexpr int NREP = 1;           // replicas of the output accumulator (more replicas spread the reductions, but the last CTA
-                                  // reads them all: one measured fastest)
 constexpr int CTMAX = 9;          // 16-column output tiles per warp (d <= 32 * 16 * CTMAX = 4608)
 // control words (unsigned int) in global scratch; all zero between calls
 constexpr int CTL_TICKET = 0;     // next unit of the folded matrix
@@ -70,7 +67,7 @@ struct Params {
   const float* smax;       // largest group scale of the layer
   const int2* plan;        // per CTA: first tile, tile count
   const __nv_bfloat16* x; __nv_bfloat16* y;
-  float* yacc;             // [NREP][MAXT][dacc] fp32
+  float* yacc;             // [MAXT][dacc] fp32 (replicas, which spread the reductions, measured no faster)
   float* dpart;            // deterministic mode: [nkc + grid][MAXT][dacc] partial outputs, each written by one owner; else null
   unsigned int* ctl; unsigned long long* counters;
   uint32_t* dbg_bitmap; double* dbg_scores;
@@ -405,8 +402,8 @@ __global__ void __launch_bounds__(NTH, 1) k_fused(const Params p) {
   // order), unit u = (output tile u / nkc, channel chunk u % nkc).  A warp draws units from one global ticket
   // (one draw ahead), streams a unit as four blocks of four 128-bit loads per lane (one block ahead of the one
   // being multiplied), multiplies it with x (the B operand: column t = token t, other columns zero) in two
-  // independent accumulators, and adds the 16 x n partial outputs to the accumulator replica of its CTA.
-  float* const rep = p.yacc + size_t(blockIdx.x % NREP) * MAXT * p.dacc;
+  // independent accumulators, and adds the 16 x n partial outputs to the accumulator.
+  float* const rep = p.yacc;
   auto stream_c = [&]() {
     unsigned int* ticket = p.ctl + CTL_TICKET;
     auto issue = [&]() -> unsigned int {        // lane 0 draws; the value is looked at one unit later
@@ -907,7 +904,7 @@ __global__ void __launch_bounds__(NTH, 1) k_fused(const Params p) {
     }
   }
   // The accumulators hold 16 output columns x (leading | remaining term of 4 tokens) per tile: add the two terms,
-  // stage the sums in shared memory (the row slots are free) and add them to this CTA's replica with 128-bit reductions.
+  // stage the sums in shared memory (the row slots are free) and add them to the accumulator with 128-bit reductions.
   if (nun > 0 || p.dpart) {                                         // (deterministic mode: every CTA writes its part, zeros too)
     __syncthreads();
     float* const yst = reinterpret_cast<float*>(slots);           // [n][dpad]
@@ -942,44 +939,43 @@ __global__ void __launch_bounds__(NTH, 1) k_fused(const Params p) {
   FZ_STAMP(tid == 0, ST_COUNTED);
   if (misc[MS_LAST] == int(gridDim.x) - 1) {
     __threadfence();
-    for (int i = tid; i < (p.dpart ? 0 : n * p.nvec); i += NTH) {    // (deterministic mode: k_ordered_sum writes y)
-      const int t = i / p.nvec, c0 = (i - t * p.nvec) * 8;
-      float4 a0[NREP + 1], a1[NREP + 1];
-      a0[NREP] = *reinterpret_cast<const float4*>(p.bf + c0);
-      a1[NREP] = *reinterpret_cast<const float4*>(p.bf + c0 + 4);
-#pragma unroll
-      for (int rp = 0; rp < NREP; ++rp) {
-        const float* q = p.yacc + (size_t(rp) * MAXT + t) * p.dacc + c0;
-        a0[rp] = __ldcg(reinterpret_cast<const float4*>(q));
-        a1[rp] = __ldcg(reinterpret_cast<const float4*>(q + 4));
-      }
-      float4 s0 = a0[NREP], s1 = a1[NREP];
-#pragma unroll
-      for (int rp = 0; rp < NREP; ++rp) {
-        s0.x += a0[rp].x; s0.y += a0[rp].y; s0.z += a0[rp].z; s0.w += a0[rp].w;
-        s1.x += a1[rp].x; s1.y += a1[rp].y; s1.z += a1[rp].z; s1.w += a1[rp].w;
-        float* q = p.yacc + (size_t(rp) * MAXT + t) * p.dacc + c0;
-        *reinterpret_cast<float4*>(q) = make_float4(0.f, 0.f, 0.f, 0.f);
-        *reinterpret_cast<float4*>(q + 4) = make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-      __nv_bfloat162 o[4];
-      o[0] = __floats2bfloat162_rn(s0.x, s0.y);
-      o[1] = __floats2bfloat162_rn(s0.z, s0.w);
-      o[2] = __floats2bfloat162_rn(s1.x, s1.y);
-      o[3] = __floats2bfloat162_rn(s1.z, s1.w);
-      *reinterpret_cast<uint4*>(p.y + size_t(t) * d + c0) = *reinterpret_cast<const uint4*>(o);
-    }
-    FZ_STAMP(tid == 0, ST_FINAL);
-    if (tid == 0) {   // every CTA has arrived, so every CTA's counts are in
-      p.ctl[CTL_TICKET] = 0u;
-      p.ctl[CTL_DONE] = 0u;
-      for (int t = 0; t < n; ++t) {
-        const unsigned int tot = atomicExch(&p.ctl[CTL_NFL + t], 0u);
+    // Nothing else runs any more, so this is latency from here to the end: the call's counts go to the handle beside the sums, one
+    // lane each (one after the other behind the sums: 2 us per call of one token, 9 us per call of four), and a thread has all
+    // its loads in flight at once.
+    if (warp == NW - 1 && lane <= n) {                              // every CTA has arrived, so every CTA's counts are in
+      const unsigned int tot = atomicExch(&p.ctl[lane < n ? CTL_NFL + lane : CTL_UNION], 0u);
+      if (lane < n) {
         atomicAdd(&p.counters[CTR_FLAGGED_TOTAL], (unsigned long long)tot);
         atomicMax(&p.counters[CTR_FLAGGED_MAX], (unsigned long long)tot);
+      } else {
+        p.counters[CTR_LAST_UNION] = (unsigned long long)tot;
+        p.ctl[CTL_TICKET] = 0u;
+        p.ctl[CTL_DONE] = 0u;
       }
-      p.counters[CTR_LAST_UNION] = (unsigned long long)atomicExch(&p.ctl[CTL_UNION], 0u);
     }
+    constexpr int ITEMS = ((NTK == 1 ? 1 : MAXT) * CTMAX * NW * 4 + NTH - 1) / NTH;   // vectors of 4 columns per thread
+    const int nq = d >> 2, nitems = p.dpart ? 0 : n * nq;           // (deterministic mode: k_ordered_sum writes y)
+    float4 sum[ITEMS], add[ITEMS];
+#pragma unroll
+    for (int k = 0; k < ITEMS; ++k) {
+      const int i = k * NTH + tid;
+      if (i < nitems) {
+        const int t = i / nq, c0 = (i - t * nq) * 4;
+        sum[k] = __ldcg(reinterpret_cast<const float4*>(p.yacc + size_t(t) * p.dacc + c0));
+        add[k] = *reinterpret_cast<const float4*>(p.bf + c0);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < ITEMS; ++k) {
+      const int i = k * NTH + tid;
+      if (i < nitems) {
+        const int t = i / nq, c0 = (i - t * nq) * 4;
+        *reinterpret_cast<float4*>(p.yacc + size_t(t) * p.dacc + c0) = make_float4(0.f, 0.f, 0.f, 0.f);
+        const uint32_t o0 = pack_bf16(add[k].x + sum[k].x, add[k].y + sum[k].y), o1 = pack_bf16(add[k].z + sum[k].z, add[k].w + sum[k].w);
+        *reinterpret_cast<uint2*>(p.y + size_t(t) * d + c0) = make_uint2(o0, o1);
+      }
+    }
+    FZ_STAMP(tid == 0, ST_FINAL);
   }
 }
 
@@ -1101,7 +1097,7 @@ tardis_status_t fused_prepare(Handle* H, cudaStream_t s) {
   auto fail = [&](tardis_status_t st) { H->fscratch = S; fused_release(H); return st; };
   size_t tally = 0;
   const size_t pb_bytes = size_t(NT) * p.nkc * p.pbs;
-  const size_t yacc_bytes = sizeof(float) * NREP * MAXT * p.dacc;
+  const size_t yacc_bytes = sizeof(float) * MAXT * p.dacc;
   const size_t cp_bytes = size_t(p.nunits) * 8192;
   cudaError_t e = dev_malloc(&S->pblocks, pb_bytes); tally += pb_bytes;
   if (e == cudaSuccess) { e = dev_malloc(&S->plan, sizeof(int2) * grid); tally += sizeof(int2) * grid; }

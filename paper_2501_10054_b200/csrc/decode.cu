@@ -49,7 +49,6 @@ constexpr int MAXTILES = 16;      // predictor tiles (of 16 neurons) per CTA
 constexpr int MAXRC = 64;         // exact re-checks per CTA before the list overflows (rest handled in place)
 constexpr int MAXBUF = 8;         // predictor unit buffers in shared memory
 constexpr int MAXSLOTS = 16;      // rows of W1 / W2T held in shared memory at once by the result fixing
-constexpr int MAXGROUPS = 8;      // slot groups (one barrier each) of the result fixing
 constexpr int kBadRow = 0x40000000;   // row whose group scales do not fit the integer form: always re-evaluated
 constexpr int XVR = 2;            // 8-channel vectors of x per thread (padded d <= 8192)
 // control words (unsigned int) in global scratch; all zero between calls
@@ -77,7 +76,7 @@ struct Params {
   int nbuf, unit_bytes;    // unit buffers in shared memory and their size
   int tiles_max;
   int nvec;                // 8-column vectors in a row
-  int fix_gs, fix_ng;      // result fixing: row slots per group, groups (fix_gs * fix_ng rows fit in the predictor buffers)
+  int fix_slots;           // row slots of the result fixing
   int nunits;              // folded-matrix units in all
   int ntk;                 // output tiles of the folded matrix (16 outputs each)
 };
@@ -100,14 +99,14 @@ struct SmemLayout {
     zeros = take(256, 16);                    // what the lanes that feed unused operand columns read
     xh = take(size_t(dpad + 16) * 2, 16);     // + 16 zeros: the B operand of lanes that feed the unused columns
     sxi = take(size_t(ngroups + 16) * sizeof(int), 8);
-    wpart = take(size_t(2) * MAXSLOTS * NW * sizeof(float), 4);
+    wpart = take(rows * (NW + 1) * sizeof(float), 4);   // (+ 1: a thread reads the sums of its row without bank conflicts)
     tab = take(6 * rows * sizeof(float), 4);
     fl_j = take(rows * sizeof(int), 4);
     fl_delta = take(rows * sizeof(float), 4);
     rc = take(MAXRC * sizeof(int), 4);
     flagbits = take(rows * sizeof(int), 4);
     wred = take(size_t(3) * NW * sizeof(float), 4);
-    bars = take(size_t(MAXBUF + MAXGROUPS) * sizeof(uint64_t), 8);
+    bars = take(size_t(MAXBUF + 2 * MAXSLOTS) * sizeof(uint64_t), 8);
     misc = take(48 * sizeof(int), 8);
     pbuf = take(size_t(nbuf) * unit_bytes, 128);
     xq = take(size_t(4) * (dpad + 64), 128);
@@ -188,7 +187,7 @@ __global__ void __launch_bounds__(NTH, 2) k_decode(const Params p) {
 
   if (tid == 0) {
     for (int b = 0; b < p.nbuf; ++b) mbar_init(&full[b], 1);
-    for (int b = 0; b < MAXGROUPS; ++b) mbar_init(&full[MAXBUF + b], 1);
+    for (int b = 0; b < MAXSLOTS; ++b) { mbar_init(&full[MAXBUF + b], 1); mbar_init(&full[MAXBUF + MAXSLOTS + b], NW); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (tid < 48) misc[tid] = 0;
@@ -595,92 +594,91 @@ __global__ void __launch_bounds__(NTH, 2) k_decode(const Params p) {
   TARDIS_STAMP_VALUE(tid == 0, ST_NFL, nfl);
   // ---- result fixing ----
   // The predictor's shared memory is free now and takes the rows the fixing needs, one bulk copy per row: item i < nfl
-  // is the W1 row of the i-th flagged neuron, item nfl + i its W2T row.  The row slots form a ring of groups
-  // with one barrier each; all groups are filled at once (for a typical token that is every row the CTA
-  // needs, so the fixing costs one trip to memory), and a group is filled again as soon as its rows have been
-  // used.  W1 rows: the warps split the channels, partial dot products meet in shared memory and give
-  // delta_j = GELU(z_j) - a_j z_j - c_j.  W2T rows: a thread owns VPT vectors of 8 output columns and adds
-  // delta_j times its slice of the row.
+  // is the W1 row of the i-th flagged neuron, item nfl + i its W2T row.  The slots form a ring with two barriers
+  // each (row landed; row used by every warp), and all of them are filled at once.  W1 rows: the warps split the
+  // channels, and leave their partial dot products for the end of the W1 rows, where every delta_j = GELU(z_j) - a_j z_j - c_j
+  // is formed at once.  W2T rows: a thread owns VPT vectors of 8 output columns and adds delta_j times its slice of
+  // the row.  The warps meet nowhere else: with a meeting and a delta per row, the latency of a step (0.9 us), not the
+  // memory, set the pace.
   float acc[VPT][8];
 #pragma unroll
   for (int m = 0; m < VPT; ++m)
 #pragma unroll
     for (int i = 0; i < 8; ++i) acc[m][i] = 0.f;
   {
-    uint64_t* fixbar = &full[MAXBUF];
+    uint64_t* const landed_bar = &full[MAXBUF];
+    uint64_t* const used_bar = landed_bar + MAXSLOTS;
     const uint32_t rowbytes = uint32_t(d) * 2u;
-    const size_t slot_bytes = size_t(p.dpad) * 2;
-    const int nitems = 2 * nfl;
-    const int GS = p.fix_gs, NG = p.fix_ng;
+    const int slot_bytes = p.dpad * 2;
+    const int nitems = 2 * nfl, NS = p.fix_slots;
     const int kw = p.dpad / NW;                                   // channels per warp (a multiple of 16)
-    // fills group gr with the items of step st (all threads call it; thread 0 arms the barrier, lane 0 of
-    // warp k issues the copy of the k-th item)
-    auto fill = [&](int gr, int st) {
-      const int i0 = st * GS, cnt = min(GS, nitems - i0);
-      if (cnt <= 0) return;
-      if (tid == 0) mbar_expect_tx(&fixbar[gr], uint32_t(cnt) * rowbytes);
-      if (lane == 0) {
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the slots were read with ordinary loads
-        for (int k = warp; k < cnt; k += NW) {
-          const int i = i0 + k;
-          const __nv_bfloat16* src = i < nfl ? p.W1 + size_t(fl_j[i]) * d : p.W2T + size_t(fl_j[i - nfl]) * d;
-          bulk_g2s(pbuf + size_t(gr * GS + k) * slot_bytes, src, rowbytes, &fixbar[gr]);
-        }
-      }
+    auto fill = [&](int i, int slot) {                            // (one thread)
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the slots were read (and written) with ordinary accesses
+      const __nv_bfloat16* src = i < nfl ? p.W1 + size_t(fl_j[i]) * d : p.W2T + size_t(fl_j[i - nfl]) * d;
+      mbar_expect_tx(&landed_bar[slot], rowbytes);
+      bulk_g2s(pbuf + size_t(slot) * slot_bytes, src, rowbytes, &landed_bar[slot]);
     };
-    const int nsteps = (nitems + GS - 1) / GS;
-    for (int gr = 0; gr < NG; ++gr) fill(gr, gr);
-    int gr = 0;
-    uint32_t par = 0u;
-    for (int st = 0; st < nsteps; ++st) {
-      const int i0 = st * GS, cnt = min(GS, nitems - i0);
-      bool landed = mbar_wait(&fixbar[gr], par);
+    if (lane == 0 && warp < min(NS, nitems)) fill(warp, warp);    // (NS <= MAXSLOTS = NW)
+    uint4 xr[VPT];                                                // x of this lane's channels
+#pragma unroll
+    for (int m = 0; m < VPT; ++m) {
+      const int c0 = lane * 8 + m * 256;
+      xr[m] = make_uint4(0u, 0u, 0u, 0u);
+      if (c0 < kw && warp * kw + c0 < d) xr[m] = *reinterpret_cast<const uint4*>(xh + warp * kw + c0);
+    }
+    int slot = 0, prev = 0;
+    uint32_t par = 0u, prev_par = 0u;
+    for (int i = 0; i < nitems; ++i) {
+      bool landed = mbar_wait_warp(&landed_bar[slot], par);
       if (!landed) {
         if (lane == 0) { atomicExch(&p.counters[CTR_ERROR], 1ull); misc[MS_ERR] = 1; }
-        landed = mbar_wait(&fixbar[gr], par);
+        landed = mbar_wait_warp(&landed_bar[slot], par);
       }
-      const int nw1 = max(0, min(cnt, nfl - i0));                 // items of this step that are W1 rows
-      float* wp = wpart + (st & 1) * MAXSLOTS * NW;
-      for (int k = 0; k < nw1; ++k) {
-        const __nv_bfloat16* row = reinterpret_cast<const __nv_bfloat16*>(pbuf + size_t(gr * GS + k) * slot_bytes);
+      if (i == nfl) {
+        __syncthreads();                                          // partial dot products complete
+        if (tid < nfl) {
+          const int rowi = fl_j[tid] - plan.x * 16;
+          float z = 0.f;
+#pragma unroll
+          for (int ww = 0; ww < NW; ++ww) z += wpart[tid * (NW + 1) + ww];
+          z += tab[2 * TR + rowi];
+          fl_delta[tid] = gelu_f32(z, p.act) - tab[3 * TR + rowi] * z - tab[4 * TR + rowi];
+        }
+        __syncthreads();
+      }
+      const __nv_bfloat16* row = reinterpret_cast<const __nv_bfloat16*>(pbuf + size_t(slot) * slot_bytes);
+      if (i < nfl) {
         float part = 0.f;
-        for (int c0 = warp * kw + lane * 8; c0 < (warp + 1) * kw; c0 += 256) {
-          if (c0 < d && landed) {
+#pragma unroll
+        for (int m = 0; m < VPT; ++m) {
+          const int c0 = lane * 8 + m * 256;
+          if (c0 < kw && warp * kw + c0 < d && landed) {
             float xv[8];
-            unpack8(xv, *reinterpret_cast<const uint4*>(xh + c0));
-            part += dot8(*reinterpret_cast<const uint4*>(row + c0), xv);
+            unpack8(xv, xr[m]);
+            part += dot8(*reinterpret_cast<const uint4*>(row + warp * kw + c0), xv);
           }
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-        if (lane == 0) wp[k * NW + warp] = part;
-      }
-      if (nw1 > 0) {
-        __syncthreads();
-        if (tid < nw1) {
-          const int rowi = fl_j[i0 + tid] - plan.x * 16;
-          float z = 0.f;
-#pragma unroll
-          for (int ww = 0; ww < NW; ++ww) z += wp[tid * NW + ww];
-          z += tab[2 * TR + rowi];
-          fl_delta[i0 + tid] = gelu_f32(z, p.act) - tab[3 * TR + rowi] * z - tab[4 * TR + rowi];
-        }
-        if (nw1 < cnt) __syncthreads();                           // W2T rows of the same step need these deltas
-      }
-      for (int k = nw1; k < cnt; ++k) {
-        const __nv_bfloat16* row = reinterpret_cast<const __nv_bfloat16*>(pbuf + size_t(gr * GS + k) * slot_bytes);
-        const float dl = fl_delta[i0 + k - nfl];
+        if (lane == 0) wpart[i * (NW + 1) + warp] = part;
+      } else {
+        const float dl = fl_delta[i - nfl];
 #pragma unroll
         for (int m = 0; m < VPT; ++m) {
           const int vec = m * NTH + tid;
           if (vec < p.nvec && landed) fma8(acc[m], dl, *reinterpret_cast<const uint4*>(row + vec * 8));
         }
+        __syncwarp();
       }
-      if (st + 1 < nsteps) {
-        __syncthreads();                                          // rows used, deltas visible
-        fill(gr, st + NG);
+      if (lane == 0) mbar_arrive(&used_bar[slot]);
+      // the slot of the item before is filled again by one warp, in turn: the others have most likely used it by now
+      if (i > 0 && i - 1 + NS < nitems && lane == 0 && warp == (i & (NW - 1))) {
+        if (mbar_wait(&used_bar[prev], prev_par)) fill(i - 1 + NS, prev);
+        else atomicExch(&p.counters[CTR_ERROR], 1ull);
       }
-      if (++gr == NG) { gr = 0; par ^= 1u; }
+      prev = slot;
+      prev_par = par;
+      if (++slot == NS) { slot = 0; par ^= 1u; }
     }
   }
   if (nfl > 0) {
@@ -878,10 +876,7 @@ tardis_status_t decode_prepare(Handle* H, cudaStream_t s) {
         S->grid = grid; p.tiles_max = tiles_max; p.nbuf = nbuf;
         S->smem_bytes = budget < size_t(max_smem) ? budget : size_t(max_smem);
         size_t slots = (S->smem_bytes - SmemLayout(dpad, p.ngroups, tiles_max, nbuf, p.unit_bytes).pbuf) / (size_t(dpad) * 2);
-        if (slots > size_t(MAXSLOTS)) slots = MAXSLOTS;
-        p.fix_gs = slots >= 6 ? int(slots) / 3 : 1;
-        p.fix_ng = int(slots) / p.fix_gs;
-        if (p.fix_ng > MAXGROUPS) p.fix_ng = MAXGROUPS;
+        p.fix_slots = int(slots < size_t(MAXSLOTS) ? slots : size_t(MAXSLOTS));
         placed = true;
         break;
       }

@@ -114,15 +114,31 @@ __global__ void __launch_bounds__(BROWS * NL) k_block(double* __restrict__ Wd, c
   if (real) *reinterpret_cast<unsigned long long*>(q + size_t(r) * d + b0 + l * 8) = codes;
 }
 
-// W[r][j] <- W[r][j] - e[r][i] U[k0 + i][j], i = 0 .. nk - 1 in this order (nk a multiple of 32), for the channels j0 <= j < j1 (both
-// multiples of 64).  Per i a thread reads 12 values from shared memory for 64 fp64 instructions.
-constexpr int SK = 32;            // channels k per pass through shared memory
+// W[r][j] <- W[r][j] - e[r][i] U[k0 + i][j], i = 0 .. nk - 1 in this order (nk a multiple of 16), for the channels j0 <= j < j1 (both
+// multiples of 64).  Bound by the fp64 units: per i a thread reads 12 values from shared memory for 64 fp64 instructions.  The next
+// pass's values arrive by asynchronous copies meanwhile.
+constexpr int SK = 16;            // channels k per pass through shared memory
+__device__ __forceinline__ void copy_8_async(double* dst, const double* src, bool valid) {      // (zero where not valid)
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(uint32_t(__cvta_generic_to_shared(dst))), "l"(src), "r"(valid ? 8 : 0) : "memory");
+}
 __global__ void __launch_bounds__(256, 2) k_spread(double* __restrict__ Wd, const double* __restrict__ U, const double* __restrict__ E,
                                                    int h, int d, int k0, int nk, int j0) {
-  __shared__ double Es[SK][SROWS];
-  __shared__ double Ut[SK / 2][SCOLS];      // (half a pass at a time: 48 KB in all)
+  __shared__ __align__(16) double Es[2][SK][SROWS];
+  __shared__ __align__(16) double Ut[2][SK][SCOLS];
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   const int jb = j0 + blockIdx.x * SCOLS, r0 = blockIdx.y * SROWS;
+  auto fetch = [&](int kb, int stage) {
+    const int rr = threadIdx.x & (SROWS - 1), cc = threadIdx.x & (SCOLS - 1);
+    const bool valid = r0 + rr < h;
+    const double* es = E + size_t(kb + threadIdx.x / SROWS) * h + (valid ? r0 + rr : 0);
+    const double* us = U + size_t(k0 + kb + threadIdx.x / SCOLS) * d + jb + cc;
+#pragma unroll
+    for (int i = 0; i < SK; i += 256 / SROWS, es += size_t(256 / SROWS) * h) copy_8_async(&Es[stage][i + threadIdx.x / SROWS][rr], es, valid);
+#pragma unroll
+    for (int i = 0; i < SK; i += 256 / SCOLS, us += size_t(256 / SCOLS) * d) copy_8_async(&Ut[stage][i + threadIdx.x / SCOLS][cc], us, true);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  fetch(0, 0);
   double w[8][4];
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
@@ -135,31 +151,21 @@ __global__ void __launch_bounds__(256, 2) k_spread(double* __restrict__ Wd, cons
     }
     w[k][0] = a.x; w[k][1] = a.y; w[k][2] = b.x; w[k][3] = b.y;
   }
-  for (int kb = 0; kb < nk; kb += SK) {
-    __syncthreads();
-    for (int e = threadIdx.x; e < SK * SROWS; e += 256) {
-      const int i = e / SROWS, rr = e - i * SROWS;
-      Es[i][rr] = r0 + rr < h ? E[size_t(kb + i) * h + r0 + rr] : 0.0;
-    }
-    for (int half = 0; half < 2; ++half) {
-      if (half) __syncthreads();
-      for (int e = threadIdx.x; e < SK / 2 * SCOLS; e += 256) {
-        const int i = e / SCOLS, c = e - i * SCOLS;
-        Ut[i][c] = U[size_t(k0 + kb + half * (SK / 2) + i) * d + jb + c];
-      }
-      __syncthreads();
+  for (int kb = 0, stage = 0; kb < nk; kb += SK, stage ^= 1) {
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();                                   // this pass's values are in place, the other stage has been read
+    if (kb + SK < nk) fetch(kb + SK, stage ^ 1);
 #pragma unroll 2
-      for (int i = 0; i < SK / 2; ++i) {
-        const double2 ua = *reinterpret_cast<const double2*>(&Ut[i][tx * 4]), ub = *reinterpret_cast<const double2*>(&Ut[i][tx * 4 + 2]);
-        const double u[4] = {ua.x, ua.y, ub.x, ub.y};
+    for (int i = 0; i < SK; ++i) {
+      const double2 ua = *reinterpret_cast<const double2*>(&Ut[stage][i][tx * 4]), ub = *reinterpret_cast<const double2*>(&Ut[stage][i][tx * 4 + 2]);
+      const double u[4] = {ua.x, ua.y, ub.x, ub.y};
 #pragma unroll
-        for (int k = 0; k < 8; k += 2) {
-          const double2 e2 = *reinterpret_cast<const double2*>(&Es[half * (SK / 2) + i][ty * 8 + k]);
+      for (int k = 0; k < 8; k += 2) {
+        const double2 e2 = *reinterpret_cast<const double2*>(&Es[stage][i][ty * 8 + k]);
 #pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            w[k][c] = __dsub_rn(w[k][c], __dmul_rn(e2.x, u[c]));
-            w[k + 1][c] = __dsub_rn(w[k + 1][c], __dmul_rn(e2.y, u[c]));
-          }
+        for (int c = 0; c < 4; ++c) {
+          w[k][c] = __dsub_rn(w[k][c], __dmul_rn(e2.x, u[c]));
+          w[k + 1][c] = __dsub_rn(w[k + 1][c], __dmul_rn(e2.y, u[c]));
         }
       }
     }

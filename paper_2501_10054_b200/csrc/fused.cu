@@ -7,7 +7,7 @@
 //     the CTA owns a few 16-neuron tiles; their predictor blocks (packed 2-bit codes + one word per
 //     neuron and group) are fetched with bulk async copies into shared memory.
 //   * x of every token is loaded once: a bf16 copy in shared memory, and a 4-limb signed base-256 fixed-point
-//     copy (of two tokens at a time) in tensor-core operand order.
+//     copy in tensor-core operand order.
 //   * Warps 16..31 then stream the folded matrix (stored in A-fragment order, 8 KB units drawn from one
 //     global ticket) through mma.m16n8k16.bf16 with the tokens as operand columns, straight from global
 //     memory into registers, and add the partial outputs to an fp32 accumulator in global memory.
@@ -16,7 +16,8 @@
 //     undoes); the 8 operand columns are the 4 limbs of two tokens.  The integer group sums are exact; they are
 //     scaled by the bf16 group scales and added up in fp32.  The fp32 steps and the truncation of tiny x
 //     elements have a bound tau; a score within tau of a range end is re-evaluated in fp64 from the codes, so
-//     the flags are the exact ones.  Calls of 3 or 4 tokens run this pass twice.
+//     the flags are the exact ones.  Calls of 3 or 4 tokens take the masked codes as bf16 instead (mma.m16n8k16.bf16, a
+//     column per token, no limbs), with a wider tau.
 //   * Result fixing, all 32 warps: W1 rows, then W2^T rows of the union of the flagged neurons arrive by one
 //     bulk copy per row in a ring of row slots (the predictor buffers, free by then).  A step of the ring holds
 //     up to 16 rows.  Pre-activations: one mma.m16n8k16 chain per warp over its share of the channels (A = 16
@@ -29,6 +30,7 @@
 #include <stdio.h>
 
 #include <new>
+#include <type_traits>
 
 #include "common.cuh"
 #include "exact.cuh"
@@ -84,7 +86,7 @@ struct Params {
 
 struct Scratch {           // handle-owned device memory of this path
   uint8_t* pblocks; int2* plan; float* smax; float* yacc; unsigned int* ctl; uint4* Cp;
-  Params base; size_t smem_bytes; size_t bytes; int grid; const void* kernels[2][2]; bool pairs_fit;
+  Params base; size_t smem_bytes; size_t bytes; int grid; const void* kernels[3][2]; bool pairs_fit;
   float* dpart;            // partial outputs of the deterministic mode (allocated when the mode is first switched on)
   int nbuf_n[MAXT + 1];    // tile buffers in shared memory for a call of n tokens
   int gs_cap_n[MAXT + 1];  // ... and the most neurons of a step of its result fixing
@@ -97,6 +99,9 @@ struct Scratch {           // handle-owned device memory of this path
 struct SmemLayout {
   size_t zeros, sx2, tab, fl_j, fl_mask, fl_delta, rc, flagbits, red, bars, misc, xh, wz, wz_end, pbuf, xq, zpart, pred_end, slots_end;
   int xstride, xq_stride, wz_groups, ztok;
+  // elements between tokens of the re-ordered bf16 copy (16 bytes more than a multiple of 128: the lanes that read two tokens' vectors
+  // at once hit different banks)
+  static __host__ __device__ int xp_stride(int dpad) { return dpad + 8; }
   __host__ __device__ SmemLayout(int dpad, int ngroups, int tiles_max, int nbuf, int buf_bytes, int ntok, size_t total_bytes, int gs_cap) {
     size_t o = 0;
     auto take = [&](size_t bytes, size_t align) { o = (o + align - 1) / align * align; size_t r = o; o += bytes; return r; };
@@ -116,8 +121,9 @@ struct SmemLayout {
     misc = take(64 * sizeof(int), 8);
     xh = take(size_t(ntok) * xstride * 2, 16);
     pbuf = take(size_t(nbuf) * buf_bytes, 128);
-    ztok = ntok < 2 ? ntok : 2;                            // tokens of a predictor pass
-    xq = take(size_t(ztok) * 4 * xq_stride, 128);          // limbs of the tokens of a pass
+    ztok = ntok;
+    // limbs of one or two tokens; of three or four, bf16 values in the order of the codes' fields
+    xq = take(ntok <= 2 ? size_t(ntok) * 4 * xq_stride : size_t(ntok) * xp_stride(dpad) * 2, 128);
     zpart = take(size_t(tiles_max) * NWP * ztok * 16 * sizeof(float), 16);
     pred_end = o;
     // the partial pre-activations of the result fixing sit at the very end: they are not needed while the predictor runs,
@@ -187,13 +193,17 @@ __device__ __forceinline__ double exact_from_blocks(const uint8_t* ubase, int pb
   return acc;
 }
 __device__ __forceinline__ void bar_sync_pred() { asm volatile("bar.sync 2, %0;" ::"n"(NTP) : "memory"); }
+__device__ __forceinline__ uint32_t mul_bf16x2(uint32_t a, uint32_t b) {
+  const __nv_bfloat162 r = __hmul2(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));
+  return *reinterpret_cast<const uint32_t*>(&r);
+}
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   return uint32_t(__bfloat16_as_ushort(__float2bfloat16_rn(lo))) | (uint32_t(__bfloat16_as_ushort(__float2bfloat16_rn(hi))) << 16);
 }
 
 // ---- the kernel ---------------------------------------------------------------------------------------
-// G: predictor group size; CT: 16-column output tiles per warp; NTK: 1 = the call has one token (most of the token loops
-// fold away), 4 = up to four; FAST: every tile of the CTA has its own buffer and a warp has the same one or two channel
+// G: predictor group size; CT: 16-column output tiles per warp; NTK: tokens of the call (4: three or four; the others' token loops
+// fold away); FAST: every tile of the CTA has its own buffer and a warp has the same one or two channel
 // pairs in every tile (their x operands stay in registers), else the general loop over a ring of tile buffers.
 template <int G, int CT, int NTK, bool FAST>
 __global__ void __launch_bounds__(NTH, 1) k_fused(const Params p) {
@@ -216,13 +226,11 @@ __global__ void __launch_bounds__(NTH, 1) k_fused(const Params p) {
   volatile int* misc = reinterpret_cast<volatile int*>(smem + L.misc);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int d = p.d, n = NTK == 1 ? 1 : p.n;
+  const int d = p.d, n = NTK <= 2 ? NTK : p.n;
   const int TR = p.tiles_max * 16;
   const int XS = L.xstride, xq_stride = L.xq_stride;
   const int2 plan = p.plan[blockIdx.x];
   const int NU = plan.y;                           // predictor units (tiles) of this CTA
-  const int NP = (n + 1) >> 1;                     // predictor passes (two tokens each)
-  const int NQ = NU * NP;                          // units in the order they are consumed
   const bool resident = FAST || NU <= p.nbuf;      // every tile has its own buffer: nothing is fetched twice
   const int g = lane >> 2, t4 = lane & 3;
   const int nv = p.dpad >> 3;                      // 8-channel vectors per token (padded)
@@ -257,7 +265,7 @@ __global__ void __launch_bounds__(NTH, 1) k_fused(const Params p) {
     if (tid == 0) mbar_expect_tx(&full[0], uint32_t(NU) * uint32_t(p.unit_bytes));
     if (lane == 0 && warp < NU)
       bulk_g2s(pbuf + size_t(warp) * p.buf_bytes, p.pblocks + size_t(plan.x + warp) * p.unit_bytes, uint32_t(p.unit_bytes), &full[0]);
-  } else if (lane == 0 && warp < p.nbuf && warp < NQ) {
+  } else if (lane == 0 && warp < p.nbuf && warp < NU) {
     issue_unit(warp % NU, warp);
   }
   // tiles that have to wait for a buffer are asked into L2 meanwhile: their copies then do not queue behind the folded matrix
@@ -314,19 +322,18 @@ __global__ void __launch_bounds__(NTH, 1) k_fused(const Params p) {
     return max(int((__float_as_uint(am) >> 23) & 0xff) - 127 - 21, -100);
   };
 
-  // ---- fixed-point limbs of two tokens in tensor-core operand order; group sums; truncation residual ----
+  // ---- fixed-point limbs of the tokens in tensor-core operand order; group sums; truncation residual ----
   // A thread takes 8 channels = half of a 16-channel unit; the two halves meet through one shuffle.  X = round(x 2^-E)
   // is pre-scaled by 4^(3 - channel mod 4) (the predictor masks code fields in place, which weights them by 4^field)
   // and split into four signed base-256 digits.
-  auto build_limbs = [&](int t0, int ptid, int nthreads) {
-    const int ntk = min(2, n - t0);
+  if constexpr (NTK <= 2) {
     constexpr int lpg = G / 8;                                        // lanes per predictor group
     constexpr int g_log2 = G == 64 ? 6 : 7;
     const bool odd = lane & 1;
-    for (int base = 0; base < ntk * nv; base += nthreads) {
-      const int i = base + ptid;
-      if (i >= ntk * nv) break;                                       // uniform over a warp
-      const int tl = i / nv, v = i - tl * nv, t = t0 + tl;
+    for (int base = 0; base < n * nv; base += NTH) {
+      const int i = base + tid;
+      if (i >= n * nv) break;                                         // uniform over a warp
+      const int t = i / nv, v = i - t * nv;
       const int E = token_exp(t);
       const bool dead = misc[MS_NONFIN + t] != 0;
       const float inv = __uint_as_float(uint32_t(127 - E) << 23);    // 2^-E
@@ -379,7 +386,7 @@ __global__ void __launch_bounds__(NTH, 1) k_fused(const Params p) {
             wv[2 * q] = __byte_perm(lo, hi, 0x5410);
             wv[2 * q + 1] = __byte_perm(lo, hi, 0x7632);
           }
-          *reinterpret_cast<uint4*>(xq + size_t(tl * 4 + l) * xq_stride + size_t(kb) * 64 + tt * 16) = make_uint4(wv[0], wv[1], wv[2], wv[3]);
+          *reinterpret_cast<uint4*>(xq + size_t(t * 4 + l) * xq_stride + size_t(kb) * 64 + tt * 16) = make_uint4(wv[0], wv[1], wv[2], wv[3]);
         }
       }
       // group sums of the integer x (exact); stored as 64 sum = hi 65536 + lo for the two halves of the limbs
@@ -387,14 +394,44 @@ __global__ void __launch_bounds__(NTH, 1) k_fused(const Params p) {
       for (int o = 1; o < lpg; o <<= 1) sx += __shfl_xor_sync(0xffffffffu, sx, o);
       if ((lane & (lpg - 1)) == 0) {
         const long long S = 64ll * sx;
-        sx2[tl * (p.ngroups + 16) + ((v * 8) >> g_log2)] = make_int2(int(S & 0xffff), int(S >> 16));
+        sx2[t * (p.ngroups + 16) + ((v * 8) >> g_log2)] = make_int2(int(S & 0xffff), int(S >> 16));
       }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) resid += __shfl_xor_sync(0xffffffffu, resid, o);
       if (lane == 0) red[(n + t) * 40 + (v >> 5)] = resid;
     }
-  };
-  build_limbs(0, tid, NTH);
+  } else {
+    // Calls of three or four tokens: per 16 channels the pairs (c, c + 8), c = 0 .. 7, times 2^96 over 4^(c mod 4).  A code word holds
+    // the codes of c and c + 8 sixteen bits apart, and they are masked where they are: an integer below 256 in the low bits of a
+    // bf16 is that many times 2^-133 (denormal, or the first normal binade), and the MMA takes it as such.  Group sums of x in the
+    // same unit of 2^-37.
+    __nv_bfloat16* const xp = reinterpret_cast<__nv_bfloat16*>(xq);
+    float* const sxf = reinterpret_cast<float*>(sx2);
+    const int nw = p.dpad >> 4;
+    for (int base = 0; base < n * nw; base += NTH) {
+      const int i = min(base + tid, n * nw - 1);
+      const int t = i / nw, w = i - t * nw;
+      const uint4* const src = reinterpret_cast<const uint4*>(xh + t * XS + w * 16);
+      const uint4 lo = src[0], hi = src[1];
+      const uint32_t a[4] = {lo.x, lo.y, lo.z, lo.w}, b[4] = {hi.x, hi.y, hi.z, hi.w};
+      uint32_t o[8];
+      float sum = 0.f;
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        const uint32_t pair = __byte_perm(a[c >> 1], b[c >> 1], (c & 1) ? 0x7632 : 0x5410);
+        sum += __uint_as_float(pair << 16) + __uint_as_float(pair & 0xffff0000u);
+        o[c] = mul_bf16x2(pair, (0x6f80u - uint32_t(c & 3) * 0x100u) * 0x10001u);   // 2^96, 2^94, 2^92, 2^90
+      }
+#pragma unroll
+      for (int q = 1; q < G / 16; q <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, q);
+      if (base + tid < n * nw) {
+        uint4* const dst = reinterpret_cast<uint4*>(xp + t * L.xp_stride(p.dpad) + w * 16);
+        dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
+        dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
+        if (w % (G / 16) == 0) sxf[t * (p.ngroups + 16) + w / (G / 16)] = sum * 7.2759576141834259e-12f;   // 2^-37
+      }
+    }
+  }
   FZ_STAMP(tid == 0, ST_LIMBS);
 
   // ---- speculative folded product on the tensor cores (warps NWP..NW-1) ----
@@ -481,24 +518,17 @@ __global__ void __launch_bounds__(NTH, 1) k_fused(const Params p) {
     FZ_STAMP(tid == NTP, ST_STREAM);
   } else {
     asm volatile("bar.sync 1, %0;" ::"n"(NTH) : "memory");
-    // ---- predictor: two tokens per pass; within tile u the warp takes the 128-channel pairs with
-    //      (u npairs + pair) mod NWP = warp, so that the pairs of all tiles spread evenly ----
+    // ---- predictor: within tile u the warp takes the 128-channel pairs with (u npairs + pair) mod NWP = warp, so that the pairs
+    //      of all tiles spread evenly ----
     constexpr int GPC = KC / G;                              // groups per chunk: 4 or 2
     const int npairs = p.nkc * 2;
     const double smax = double(smax_f);
-    int q = 0;                                               // units consumed so far (over all passes)
-    for (int pass = 0; pass < NP; ++pass) {
-      const int t0 = pass * 2, ntk = min(2, n - t0);
-      if (pass > 0) {                                        // limbs of the next two tokens replace the old ones
-        bar_sync_pred();
-        build_limbs(t0, tid, NTP);
-        bar_sync_pred();
-      }
-      // operand side: column g = limb g & 3 of token t0 + (g >> 2); columns of a missing token read zeros
-      const bool bcol = (g >> 2) < ntk;
+    {
+      // operand side: column g = limb g & 3 of token g >> 2; columns of a missing token read zeros
+      const bool bcol = (g >> 2) < n;
       const uint8_t* const xql = bcol ? xq + size_t(g) * xq_stride + t4 * 16 : smem + L.zeros + t4 * 16;
       const int xon = bcol ? 1 : 0;
-      // result side: this lane holds limbs 2 (t4 & 1), 2 (t4 & 1) + 1 of token t0 + (t4 >> 1)
+      // result side: this lane holds limbs 2 (t4 & 1), 2 (t4 & 1) + 1 of token t4 >> 1
       const int* const sxl = reinterpret_cast<const int*>(sx2 + (t4 >> 1) * (p.ngroups + 16)) + (t4 & 1);
       // one item: 128 channels (pair) x the 16 neurons of a tile.  A group done: integer sums (exact) -> minus zero-point
       // times the sum of x -> times the bf16 scale, accumulated in fp32 (rows g and g + 8 of the tile)
@@ -535,6 +565,47 @@ __global__ void __launch_bounds__(NTH, 1) k_fused(const Params p) {
           float* zp = zpart + size_t((u * NWP + warp) * L.ztok + (t4 >> 1)) * 16;
           zp[g] = fmaf(65536.f, o0, fa0);
           zp[g + 8] = fmaf(65536.f, o1, fa1);
+        }
+      };
+      // The same for three or four tokens, a column per token: the codes as bf16 where they are, group sums in fp32, minus zero-point
+      // times the sum of x.  fa: rows g (first two) and g + 8, tokens 2 t4 and 2 t4 + 1.
+      const __nv_bfloat16* const xpl = g < n ? reinterpret_cast<const __nv_bfloat16*>(xq) + g * L.xp_stride(p.dpad) + t4 * 16
+                                             : reinterpret_cast<const __nv_bfloat16*>(smem + L.zeros) + t4 * 16;
+      const int xpon = g < n ? 1 : 0;
+      const float* const sxf = reinterpret_cast<const float*>(sx2) + (t4 == 1 ? 2 : 0) * (p.ngroups + 16);
+      const int sx_next = t4 == 1 && n == 3 ? 0 : p.ngroups + 16;
+      auto item_of_four = [&](const uint8_t* ubase, int pair, float (&fa)[4]) {
+        const int kc = pair >> 1, half = pair & 1;
+        const uint8_t* const blk = ubase + kc * p.pbs;
+        const uint4 cw = reinterpret_cast<const uint4*>(blk)[half * 32 + lane];
+        const uint4* const xs = reinterpret_cast<const uint4*>(xpl + (kc * KC + half * 128) * xpon);
+        auto multiply = [&](float (&c)[4], uint32_t r0, uint32_t r1, const uint4& xa, const uint4& xb) {   // 64 channels
+          const uint32_t x[8] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w};
+          const uint32_t h0 = r0 >> 8, h1 = r1 >> 8;
+          c[0] = c[1] = c[2] = c[3] = 0.f;
+#pragma unroll
+          for (int m = 0; m < 8; m += 2) {
+            const uint32_t k0 = 0x00030003u << (2 * (m & 3)), k1 = k0 << 2, w0 = m < 4 ? r0 : h0, w1 = m < 4 ? r1 : h1;
+            mma_bf16(c, w0 & k0, w1 & k0, w0 & k1, w1 & k1, x[m], x[m + 1]);
+          }
+        };
+        auto scale_group = [&](const float (&c)[4], int gl, int grp) {
+          const uint2 mw = reinterpret_cast<const uint2*>(blk + 1024)[gl * 8 + g];
+          const float s0 = __uint_as_float(mw.x & 0xffff0000u), s1 = __uint_as_float(mw.y & 0xffff0000u);
+          const float z0 = float(mw.x & 3u), z1 = float(mw.y & 3u), sa = sxf[grp], sb = sxf[grp + sx_next];
+          fa[0] = fmaf(s0, fmaf(-z0, sa, c[0]), fa[0]); fa[1] = fmaf(s0, fmaf(-z0, sb, c[1]), fa[1]);
+          fa[2] = fmaf(s1, fmaf(-z1, sa, c[2]), fa[2]); fa[3] = fmaf(s1, fmaf(-z1, sb, c[3]), fa[3]);
+        };
+        float ca[4], cb[4];
+        multiply(ca, cw.x, cw.y, xs[0], xs[1]);
+        multiply(cb, cw.z, cw.w, xs[8 * xpon], xs[8 * xpon + 1]);
+        if (G == 64) {
+          scale_group(ca, half * 2, kc * GPC + half * 2);
+          scale_group(cb, half * 2 + 1, kc * GPC + half * 2 + 1);
+        } else {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) ca[e] += cb[e];
+          scale_group(ca, half, kc * GPC + half);
         }
       };
       auto wait_unit = [&](int b, uint32_t par) -> bool {
@@ -578,26 +649,34 @@ __global__ void __launch_bounds__(NTH, 1) k_fused(const Params p) {
             }
           store_partial(u, fa0 + fc0, fa1 + fc1);
         }
-        q += NU;
       } else {
         // within tile u the warp takes the pairs with (u npairs + pair) mod NWP = warp, so that the pairs of all tiles
         // spread evenly over the warps
-        for (int u = 0; u < NU; ++u, ++q) {
-          const int b = resident ? 0 : q % p.nbuf;
-          const bool usable = wait_unit(b, resident ? 0u : uint32_t((q / p.nbuf) & 1));
+        for (int u = 0; u < NU; ++u) {
+          const int b = resident ? 0 : u % p.nbuf;
+          const bool usable = wait_unit(b, resident ? 0u : uint32_t((u / p.nbuf) & 1));
           const uint8_t* const ubase = pbuf + size_t(resident ? u : b) * p.buf_bytes;
-          float fa0 = 0.f, fa1 = 0.f;
           int first = (warp - u * npairs) % NWP;
           if (first < 0) first += NWP;
-          for (int pair = first; pair < npairs && usable; pair += NWP) {
+          float fa0 = 0.f, fa1 = 0.f;
+          if constexpr (NTK > 2) {
+            float fa[4] = {0.f, 0.f, 0.f, 0.f};
+            for (int pair = first; pair < npairs && usable; pair += NWP) item_of_four(ubase, pair, fa);
+            if (2 * t4 < n) {                              // (lanes t4 = 0, 1)
+              float* const zp = zpart + size_t((u * NWP + warp) * L.ztok + 2 * t4) * 16 + g;
+              zp[0] = fa[0]; zp[8] = fa[2];
+              if (2 * t4 + 1 < n) { zp[16] = fa[1]; zp[24] = fa[3]; }
+            }
+          }
+          for (int pair = first; NTK <= 2 && pair < npairs && usable; pair += NWP) {
             uint4 xb0, xb1;
             int sxa, sxb;
             load_x(pair, xb0, xb1, sxa, sxb);
             item(ubase, pair, xb0, xb1, sxa, sxb, fa0, fa1);
           }
-          store_partial(u, fa0, fa1);
+          if (NTK <= 2) store_partial(u, fa0, fa1);
           // hand the buffer back: the last warp to leave it starts the copy of the unit that reuses it
-          if (!resident && q + p.nbuf < NQ) {
+          if (!resident && u + p.nbuf < NU) {
             __threadfence_block();
             __syncwarp();
             if (lane == 0) {
@@ -605,42 +684,45 @@ __global__ void __launch_bounds__(NTH, 1) k_fused(const Params p) {
               if (old == NWP - 1) {
                 misc[MS_BUFCNT + b] = 0;
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                issue_unit((q + p.nbuf) % NU, b);
+                issue_unit(u + p.nbuf, b);
               }
             }
           }
         }
       }
       bar_sync_pred();
-      FZ_STAMP(tid == 0 && pass == 0, ST_PRED);
-      // ---- scores and flags of this pass ----
+      FZ_STAMP(tid == 0, ST_PRED);
+      // ---- scores and flags ----
       // tau bounds what the fast score can be off by: the rounding residuals of x (each at most 1/2 unit of 2^E)
       // times |code - zero| <= 3 times the scale, plus the fp32 roundings (one per conversion, product-sum and
-      // combination: at most 12 per partial score, each at most 2^-24 of 3 smax sum |x|).
-      if (tid < ntk * nrow) {
-        const int tl = tid / nrow, r = tid - tl * nrow, t = t0 + tl;
+      // combination: at most 12 per partial score, each at most 2^-24 of 3 smax sum |x|).  Three or four tokens: no residuals, but the
+      // group sums come from chains of four MMAs that add 17 numbers each, with as many roundings, and the sums of x have
+      // eight (x too small for 2^-37 of it to count: the last term).
+      for (int i = tid; i < n * nrow; i += NTP) {
+        const int t = i / nrow, r = i - t * nrow;
         const int tile = r >> 4, rr = r & 15;
         const int j = plan.x * 16 + r;
         const int E = token_exp(t);
         float rs = 0.f, l1 = 0.f;
         for (int w = 0; w < (nv >> 5); ++w) { l1 += red[t * 40 + w]; rs += red[(n + t) * 40 + w]; }
         const double unit = __longlong_as_double((long long)(1023 + E) << 52);   // 2^E
-        const double tau = 1.01 * 3.0 * smax * (double(rs) * unit + 12.0 * 5.9604644775390625e-08 * (double(l1) + double(rs) * unit));
+        const double roundings = NTK > 2 ? 12.0 + 17.0 * 4 + 8.0 : 12.0;
+        const double tau = 1.01 * 3.0 * smax * (double(rs) * unit + roundings * 5.9604644775390625e-08 * (double(l1) + double(rs) * unit)) +
+                           (NTK > 2 ? 1e-30 : 0.0);
         double s = 0.0;
 #pragma unroll
-        for (int w = 0; w < NWP; ++w) s += double(zpart[size_t((tile * NWP + w) * L.ztok + tl) * 16 + rr]);
+        for (int w = 0; w < NWP; ++w) s += double(zpart[size_t((tile * NWP + w) * L.ztok + t) * 16 + rr]);
         const double b1 = double(tab[2 * TR + r]);
-        double zhat = b1 + s * (unit * 0.015625);
+        double zhat = b1 + s * (NTK > 2 ? 137438953472.0 : unit * 0.015625);   // (2^37)
         const double lo = double(tab[r]), hi = double(tab[TR + r]);
         int f = ((lo <= zhat) && (zhat < hi)) ? 0 : 1;
         if (misc[MS_NONFIN + t]) { f = 1; zhat = __longlong_as_double(0x7ff8000000000000ll); }
-        else if (fabs(zhat - lo) <= tau || fabs(zhat - hi) <= tau) {
+        else if (fabs(zhat - lo) <= tau || fabs(zhat - hi) <= tau || (NTK > 2 && !(fabs(zhat) < 1e37))) {
           const int e = atomicAdd(const_cast<int*>(&misc[MS_NRC]), 1);
-          if (e < MAXRC) { rc[e] = (tl << 16) | r; f = -1; }
+          if (e < MAXRC) { rc[e] = (t << 16) | r; f = -1; }
           else {                                        // list full: this thread re-evaluates its neuron alone
-            const int qu = pass * NU + tile;            // the tile's blocks are still in shared memory unless its buffer was refilled
-            const bool here = resident || qu + p.nbuf >= NQ;
-            zhat = b1 + (here ? exact_from_blocks(pbuf + size_t(resident ? tile : qu % p.nbuf) * p.buf_bytes, p.pbs, G, rr, xh + t * XS, d, 0, 1)
+            const bool here = resident || tile + p.nbuf >= NU;   // the tile's blocks are still in shared memory: its buffer was not refilled
+            zhat = b1 + (here ? exact_from_blocks(pbuf + size_t(resident ? tile : tile % p.nbuf) * p.buf_bytes, p.pbs, G, rr, xh + t * XS, d, 0, 1)
                               : exact_score_single(p.codes, p.scale, p.zero, xh + t * XS, j, d, G, 2));
             f = ((lo <= zhat) && (zhat < hi)) ? 0 : 1;
           }
@@ -653,12 +735,12 @@ __global__ void __launch_bounds__(NTH, 1) k_fused(const Params p) {
       {
         const int nrc = min(int(misc[MS_NRC]), MAXRC);
         for (int e = warp; e < nrc; e += NWP) {
-          const int tl = rc[e] >> 16, r = rc[e] & 0xffff, t = t0 + tl;
+          const int t = rc[e] >> 16, r = rc[e] & 0xffff;
           const int j = plan.x * 16 + r;
           double ex;
-          const int qu = pass * NU + (r >> 4);
-          if (resident || qu + p.nbuf >= NQ) {  // the tile's blocks are still in shared memory (its buffer was not refilled)
-            ex = exact_from_blocks(pbuf + size_t(resident ? (r >> 4) : qu % p.nbuf) * p.buf_bytes, p.pbs, G, r & 15, xh + t * XS, d, lane, 32);
+          const int tile = r >> 4;
+          if (resident || tile + p.nbuf >= NU) {  // the tile's blocks are still in shared memory (its buffer was not refilled)
+            ex = exact_from_blocks(pbuf + size_t(resident ? tile : tile % p.nbuf) * p.buf_bytes, p.pbs, G, r & 15, xh + t * XS, d, lane, 32);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) ex += __shfl_xor_sync(0xffffffffu, ex, o);
           } else {
@@ -953,7 +1035,7 @@ __global__ void __launch_bounds__(NTH, 1) k_fused(const Params p) {
         p.ctl[CTL_DONE] = 0u;
       }
     }
-    constexpr int ITEMS = ((NTK == 1 ? 1 : MAXT) * CTMAX * NW * 4 + NTH - 1) / NTH;   // vectors of 4 columns per thread
+    constexpr int ITEMS = (NTK * CTMAX * NW * 4 + NTH - 1) / NTH;   // vectors of 4 columns per thread
     const int nq = d >> 2, nitems = p.dpart ? 0 : n * nq;           // (deterministic mode: k_ordered_sum writes y)
     float4 sum[ITEMS], add[ITEMS];
 #pragma unroll
@@ -1120,16 +1202,19 @@ tardis_status_t fused_prepare(Handle* H, cudaStream_t s) {
   k_max_scale<<<64, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(H->scale), size_t(h) * H->ngroups, S->smax);
   e = cudaGetLastError();
   const bool wide = dpad > 32 * 16 * 8;
-  // kernels[one token or more][ring or fast]
-  if (G == 64 && wide) { S->kernels[0][0] = (const void*)k_fused<64, 9, 1, false>; S->kernels[0][1] = (const void*)k_fused<64, 9, 1, true>;
-                         S->kernels[1][0] = (const void*)k_fused<64, 9, 4, false>; S->kernels[1][1] = (const void*)k_fused<64, 9, 4, true>; }
-  else if (G == 64) { S->kernels[0][0] = (const void*)k_fused<64, 8, 1, false>; S->kernels[0][1] = (const void*)k_fused<64, 8, 1, true>;
-                      S->kernels[1][0] = (const void*)k_fused<64, 8, 4, false>; S->kernels[1][1] = (const void*)k_fused<64, 8, 4, true>; }
-  else if (wide) { S->kernels[0][0] = (const void*)k_fused<128, 9, 1, false>; S->kernels[0][1] = (const void*)k_fused<128, 9, 1, true>;
-                   S->kernels[1][0] = (const void*)k_fused<128, 9, 4, false>; S->kernels[1][1] = (const void*)k_fused<128, 9, 4, true>; }
-  else { S->kernels[0][0] = (const void*)k_fused<128, 8, 1, false>; S->kernels[0][1] = (const void*)k_fused<128, 8, 1, true>;
-         S->kernels[1][0] = (const void*)k_fused<128, 8, 4, false>; S->kernels[1][1] = (const void*)k_fused<128, 8, 4, true>; }
-  for (int a = 0; a < 2 && e == cudaSuccess; ++a)
+  // kernels[one token, two, three or four][ring or fast]
+  auto choose = [&](auto g, auto ct) {
+    constexpr int GG = decltype(g)::value, CC = decltype(ct)::value;
+    S->kernels[0][0] = (const void*)k_fused<GG, CC, 1, false>; S->kernels[0][1] = (const void*)k_fused<GG, CC, 1, true>;
+    S->kernels[1][0] = (const void*)k_fused<GG, CC, 2, false>; S->kernels[1][1] = (const void*)k_fused<GG, CC, 2, true>;
+    S->kernels[2][0] = S->kernels[2][1] = (const void*)k_fused<GG, CC, 4, false>;
+  };
+  using std::integral_constant;
+  if (G == 64 && wide) choose(integral_constant<int, 64>(), integral_constant<int, 9>());
+  else if (G == 64) choose(integral_constant<int, 64>(), integral_constant<int, 8>());
+  else if (wide) choose(integral_constant<int, 128>(), integral_constant<int, 9>());
+  else choose(integral_constant<int, 128>(), integral_constant<int, 8>());
+  for (int a = 0; a < 3 && e == cudaSuccess; ++a)
     for (int b = 0; b < 2 && e == cudaSuccess; ++b)
       e = cudaFuncSetAttribute(S->kernels[a][b], cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
   S->pairs_fit = (p.nkc * 2 == NWP || (p.nkc * 2 >= 2 * NWP && p.nkc * 2 < 3 * NWP));
@@ -1214,7 +1299,7 @@ tardis_status_t launch_fused_forward(Handle* H, const void* x, void* y, int n, c
     cfg.attrs = attr; cfg.numAttrs = 1;
     void* args[] = {&p};
     const bool fast = S->pairs_fit && S->nbuf_n[nt] >= p.tiles_max;
-    TARDIS_CUDA_TRY(cudaLaunchKernelExC(&cfg, S->kernels[nt == 1 ? 0 : 1][fast ? 1 : 0], args));
+    TARDIS_CUDA_TRY(cudaLaunchKernelExC(&cfg, S->kernels[nt <= 2 ? nt - 1 : 2][fast ? 1 : 0], args));
     H->launches += 1;
     if (det) {
       const int work = nt * (H->d >> 2);                    // warps

@@ -57,56 +57,6 @@ __device__ inline double exact_score(const uint32_t* __restrict__ codes, const _
   return acc;
 }
 
-// The same sums for a kernel that does nothing else (k_recheck): with 2-bit codes the 16 channels of a word come in as two
-// 128-bit loads and the loads of four words go out before the first is used; same terms in the same order as exact_score.
-// (Kept apart from exact_score: inside the fused kernels its registers would spill.)
-__device__ inline double exact_score_wide(const uint32_t* __restrict__ codes, const __nv_bfloat16* __restrict__ scale,
-                                          const uint8_t* __restrict__ zero, const __nv_bfloat16* __restrict__ xt, int j, int d, int G,
-                                          int bits, int lane) {
-  if (bits != 2 || (reinterpret_cast<uintptr_t>(xt) & 15u) != 0) return exact_score(codes, scale, zero, xt, j, d, G, bits, lane);
-  const int nwords = d / 16, ng = d / G;
-  double acc = 0.0;
-  {
-    // the 16 channels of a word come in as two 128-bit loads, and the loads of four words go out before the first is used
-    // (same terms in the same order as the general loop below)
-    for (int w0 = lane; w0 < nwords; w0 += 128) {
-      uint32_t word[4];
-      uint8_t zr[4];
-      __nv_bfloat16 sr[4];
-      uint4 xa[4], xb[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int w = w0 + 32 * u;
-        if (w < nwords) {
-          const int g = (w * 16) / G;
-          word[u] = codes[size_t(j) * nwords + w];
-          zr[u] = zero[size_t(j) * ng + g];
-          sr[u] = scale[size_t(j) * ng + g];
-          xa[u] = *reinterpret_cast<const uint4*>(xt + w * 16);
-          xb[u] = *reinterpret_cast<const uint4*>(xt + w * 16 + 8);
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        if (w0 + 32 * u < nwords) {
-          const double zp = double(zr[u]);
-          const uint32_t xw[8] = {xa[u].x, xa[u].y, xa[u].z, xa[u].w, xb[u].x, xb[u].y, xb[u].z, xb[u].w};
-          double inner = 0.0;
-#pragma unroll
-          for (int q = 0; q < 16; ++q) {
-            const float xf = __uint_as_float((q & 1) ? (xw[q >> 1] & 0xffff0000u) : (xw[q >> 1] << 16));
-            inner += (double((word[u] >> (2 * q)) & 3u) - zp) * double(xf);
-          }
-          acc += double(__bfloat162float(sr[u])) * inner;
-        }
-      }
-    }
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  return acc;
-}
-
 __device__ inline double exact_score_single(const uint32_t* __restrict__ codes, const __nv_bfloat16* __restrict__ scale,
                                      const uint8_t* __restrict__ zero, const __nv_bfloat16* __restrict__ xt, int j, int d, int G, int bits) {
   if (32 % bits) return exact_score_stream(codes, scale, zero, xt, j, d, G, bits, 0, 1);

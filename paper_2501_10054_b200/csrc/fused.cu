@@ -33,7 +33,6 @@
 #include <type_traits>
 
 #include "common.cuh"
-#include "exact.cuh"
 #include "ptx.cuh"
 
 namespace tardis {
@@ -47,7 +46,7 @@ constexpr int NTP = NWP * 32;     // threads of the predictor warps
 constexpr int KC = 256;           // channels per predictor block
 constexpr int MAXT = 4;           // tokens per launch
 constexpr int MAXTILES = 10;      // predictor tiles (of 16 neurons) per CTA
-constexpr int MAXRC = 64;         // exact re-checks per CTA and pass before the list overflows (rest handled in place)
+constexpr int MAXRC = 64;         // exact re-checks per CTA before the list overflows (rest handled in place)
 constexpr int MAXBUF = 10;        // predictor tile buffers in shared memory
 constexpr int MAXGROUPS = 4;      // slot groups (one barrier each, one buffer of partial sums each) of the result fixing
 constexpr int MAXGS = 16;         // rows per slot group (one MMA tile)
@@ -65,7 +64,6 @@ struct Params {
   const __nv_bfloat16 *W1, *W2T;
   const uint4* Cp;         // folded matrix in tensor-core fragment order
   const float *bf, *lo, *hi, *a, *c, *b1;
-  const uint32_t* codes; const __nv_bfloat16* scale; const uint8_t* zero;   // originals (exact re-check)
   const float* smax;       // largest group scale of the layer
   const int2* plan;        // per CTA: first tile, tile count
   const __nv_bfloat16* x; __nv_bfloat16* y;
@@ -117,7 +115,7 @@ struct SmemLayout {
     rc = take(MAXRC * sizeof(int), 4);
     flagbits = take(rows * sizeof(int), 4);
     red = take(size_t(2) * ntok * 40 * sizeof(float), 4);  // per token and warp round: sum |x|, rounding residual
-    bars = take(size_t(MAXBUF + MAXGROUPS) * sizeof(uint64_t), 8);
+    bars = take(size_t(2 * MAXBUF + MAXGROUPS) * sizeof(uint64_t), 8);
     misc = take(64 * sizeof(int), 8);
     xh = take(size_t(ntok) * xstride * 2, 16);
     pbuf = take(size_t(nbuf) * buf_bytes, 128);
@@ -140,7 +138,7 @@ struct SmemLayout {
     slots_end = wz;
   }
 };
-enum { MS_NRC = 1, MS_ERR = 2, MS_LAST = 3, MS_NUN = 4, MS_AMAX = 8, MS_NONFIN = 12, MS_TOKCNT = 16, MS_WCNT = 24, MS_BUFCNT = 32 };
+enum { MS_NRC = 1, MS_ERR = 2, MS_LAST = 3, MS_NUN = 4, MS_AMAX = 8, MS_NONFIN = 12, MS_TOKCNT = 16, MS_WCNT = 24 };
 
 // ---- phase stamps (compiled in with -DTARDIS_PHASE_STAMPS only) -----------------------------------------
 // Thread 0 of every CTA (and lane 0 of the first streaming warp) writes the global timer at the phase
@@ -171,8 +169,8 @@ __device__ __forceinline__ void ldmatrix_x4(uint32_t& r0, uint32_t& r1, uint32_t
 __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3, uint32_t addr) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(addr) : "memory");
 }
-// Exact fp64 predictor sum of one neuron (row r of a tile) from the tile's predictor blocks in shared memory: the same
-// terms in the same order as exact_score, which reads the original arrays in global memory.  Lane `lane` of `nl` takes
+// Exact fp64 predictor sum of one neuron (row r of a tile) from the tile's predictor blocks: the same
+// terms as exact_score, which reads the original arrays.  Lane `lane` of `nl` takes
 // the code words lane, lane + nl, ...; the caller adds the lanes up.
 __device__ __forceinline__ double exact_from_blocks(const uint8_t* ubase, int pbs, int G, int r, const __nv_bfloat16* xt, int d,
                                                     int lane, int nl) {
@@ -223,6 +221,7 @@ __global__ void __launch_bounds__(NTH, 1) k_fused(const Params p) {
   int* flagbits = reinterpret_cast<int*>(smem + L.flagbits);
   float* red = reinterpret_cast<float*>(smem + L.red);    // [3][MAXT][40]
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + L.bars);
+  uint64_t* used = full + MAXBUF + MAXGROUPS;             // tile buffer read by every predictor warp
   volatile int* misc = reinterpret_cast<volatile int*>(smem + L.misc);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -253,6 +252,7 @@ __global__ void __launch_bounds__(NTH, 1) k_fused(const Params p) {
   }
   if (tid == 0) {
     for (int b = 0; b < MAXBUF + MAXGROUPS; ++b) mbar_init(&full[b], 1);
+    for (int b = 0; b < MAXBUF; ++b) mbar_init(&used[b], NWP);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (tid < 64) misc[tid] = 0;
@@ -675,16 +675,21 @@ __global__ void __launch_bounds__(NTH, 1) k_fused(const Params p) {
             item(ubase, pair, xb0, xb1, sxa, sxb, fa0, fa1);
           }
           if (NTK <= 2) store_partial(u, fa0, fa1);
-          // hand the buffer back: the last warp to leave it starts the copy of the unit that reuses it
-          if (!resident && u + p.nbuf < NU) {
-            __threadfence_block();
+          // hand the buffer back; the one of the tile before is filled again by one warp, in turn: the others have most likely read
+          // it by now (a single buffer: the one of this tile)
+          if (!resident) {
             __syncwarp();
             if (lane == 0) {
-              const int old = atomicAdd(const_cast<int*>(&misc[MS_BUFCNT + b]), 1);
-              if (old == NWP - 1) {
-                misc[MS_BUFCNT + b] = 0;
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                issue_unit(u + p.nbuf, b);
+              mbar_arrive(&used[b]);
+              const int v = p.nbuf > 1 ? u - 1 : u, vb = v % p.nbuf;
+              if (v >= 0 && v + p.nbuf < NU && warp == (u & (NWP - 1))) {
+                if (mbar_wait(&used[vb], uint32_t((v / p.nbuf) & 1))) {
+                  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                  issue_unit(v + p.nbuf, vb);
+                } else {
+                  atomicExch(&p.counters[CTR_ERROR], 1ull);
+                  misc[MS_ERR] = 1;
+                }
               }
             }
           }
@@ -698,6 +703,11 @@ __global__ void __launch_bounds__(NTH, 1) k_fused(const Params p) {
       // combination: at most 12 per partial score, each at most 2^-24 of 3 smax sum |x|).  Three or four tokens: no residuals, but the
       // group sums come from chains of four MMAs that add 17 numbers each, with as many roundings, and the sums of x have
       // eight (x too small for 2^-37 of it to count: the last term).
+      // a tile's blocks: still in shared memory unless its buffer was filled again
+      auto blocks_of = [&](int tile) -> const uint8_t* {
+        if (resident || tile + p.nbuf >= NU) return pbuf + size_t(resident ? tile : tile % p.nbuf) * p.buf_bytes;
+        return p.pblocks + size_t(plan.x + tile) * p.unit_bytes;
+      };
       for (int i = tid; i < n * nrow; i += NTP) {
         const int t = i / nrow, r = i - t * nrow;
         const int tile = r >> 4, rr = r & 15;
@@ -721,9 +731,7 @@ __global__ void __launch_bounds__(NTH, 1) k_fused(const Params p) {
           const int e = atomicAdd(const_cast<int*>(&misc[MS_NRC]), 1);
           if (e < MAXRC) { rc[e] = (t << 16) | r; f = -1; }
           else {                                        // list full: this thread re-evaluates its neuron alone
-            const bool here = resident || tile + p.nbuf >= NU;   // the tile's blocks are still in shared memory: its buffer was not refilled
-            zhat = b1 + (here ? exact_from_blocks(pbuf + size_t(resident ? tile : tile % p.nbuf) * p.buf_bytes, p.pbs, G, rr, xh + t * XS, d, 0, 1)
-                              : exact_score_single(p.codes, p.scale, p.zero, xh + t * XS, j, d, G, 2));
+            zhat = b1 + exact_from_blocks(blocks_of(tile), p.pbs, G, rr, xh + t * XS, d, 0, 1);
             f = ((lo <= zhat) && (zhat < hi)) ? 0 : 1;
           }
         }
@@ -731,26 +739,31 @@ __global__ void __launch_bounds__(NTH, 1) k_fused(const Params p) {
         if (p.dbg_scores && f >= 0) p.dbg_scores[size_t(t) * p.h + j] = zhat;
       }
       bar_sync_pred();
-      // exact re-evaluation from the original codes (rare): one warp per listed (token, neuron)
+      // exact re-evaluation of the listed (token, neuron) pairs (rare): all predictor warps share a pair's code words, the partial sums
+      // meet where the partial scores were.  (A warp per pair: 6 to 9 us, which the whole call waited for.)
       {
         const int nrc = min(int(misc[MS_NRC]), MAXRC);
-        for (int e = warp; e < nrc; e += NWP) {
-          const int t = rc[e] >> 16, r = rc[e] & 0xffff;
-          const int j = plan.x * 16 + r;
-          double ex;
-          const int tile = r >> 4;
-          if (resident || tile + p.nbuf >= NU) {  // the tile's blocks are still in shared memory (its buffer was not refilled)
-            ex = exact_from_blocks(pbuf + size_t(resident ? tile : tile % p.nbuf) * p.buf_bytes, p.pbs, G, r & 15, xh + t * XS, d, lane, 32);
+        double* const part = reinterpret_cast<double*>(zpart);
+        const int batch = p.tiles_max * L.ztok * 8;       // pairs whose partial sums fit there
+        for (int e0 = 0; e0 < nrc; e0 += batch) {
+          const int e1 = min(nrc, e0 + batch);
+          for (int e = e0; e < e1; ++e) {
+            const int t = rc[e] >> 16, r = rc[e] & 0xffff;
+            double ex = exact_from_blocks(blocks_of(r >> 4), p.pbs, G, r & 15, xh + t * XS, d, tid, NTP);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) ex += __shfl_xor_sync(0xffffffffu, ex, o);
-          } else {
-            ex = exact_score(p.codes, p.scale, p.zero, xh + t * XS, j, d, G, 2, lane);
+            if (lane == 0) part[(e - e0) * NWP + warp] = ex;
           }
-          const double zhat = double(tab[2 * TR + r]) + ex;
-          if (lane == 0) {
+          bar_sync_pred();
+          if (tid < e1 - e0) {
+            const int t = rc[e0 + tid] >> 16, r = rc[e0 + tid] & 0xffff;
+            double ex = 0.0;
+            for (int w = 0; w < NWP; ++w) ex += part[tid * NWP + w];
+            const double zhat = double(tab[2 * TR + r]) + ex;
             if (!((double(tab[r]) <= zhat) && (zhat < double(tab[TR + r])))) atomicOr(&flagbits[r], 1 << t);
-            if (p.dbg_scores) p.dbg_scores[size_t(t) * p.h + j] = zhat;
+            if (p.dbg_scores) p.dbg_scores[size_t(t) * p.h + plan.x * 16 + r] = zhat;
           }
+          if (e1 < nrc) bar_sync_pred();
         }
         if (nrc > 0) {                                  // (uniform over the predictor warps)
           bar_sync_pred();
@@ -1223,7 +1236,6 @@ tardis_status_t fused_prepare(Handle* H, cudaStream_t s) {
   p.pblocks = S->pblocks; p.plan = S->plan; p.smax = S->smax; p.yacc = S->yacc; p.ctl = S->ctl;
   p.W1 = static_cast<const __nv_bfloat16*>(H->W1); p.W2T = static_cast<const __nv_bfloat16*>(H->W2T);
   p.Cp = S->Cp; p.bf = H->bf; p.lo = H->lo; p.hi = H->hi; p.a = H->a; p.c = H->c; p.b1 = H->b1;
-  p.codes = H->codes; p.scale = static_cast<const __nv_bfloat16*>(H->scale); p.zero = H->zero;
   p.counters = H->counters;
   H->fscratch = S;
   // beyond this many tokens the batched tensor-core path is faster (decode_7b: 208 against 212 us at 16 tokens, 245 against

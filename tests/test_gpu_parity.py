@@ -582,6 +582,16 @@ def test_kernels_for_a_few_tokens_at_the_edges_of_their_tiles(d, h, G, q):
     _run(cfg, sum(calls), calls, path=3)
 
 
+@pytest.mark.parametrize("d,h,G,q", [(64, 32, 64, 0.4), (320, 2400, 64, 0.2), (4096, 16384, 128, 0.05), (4608, 18944, 64, 0.1),
+                                     (4672, 4768, 64, 0.1), (8192, 2400, 128, 0.4)])
+def test_fused_kernels_at_the_edges_of_their_rings(d, h, G, q):
+    # one to four tokens in one launch (three and four: the codes as bf16), one tile in all, tiles that all have a buffer and tiles that
+    # share them, as many channels as fit; wider layers: one token per launch, more flagged rows than row slots, CTAs with none
+    cfg = W.LayerConfig("fusededge%d" % d, d, h, group=G, n_calib=256, q_lo=q, q_hi=1 - q)
+    calls = [1, 3, 4, 2, 3]
+    _run(cfg, sum(calls), calls, path=2)
+
+
 @pytest.mark.parametrize("d,dtype", [(16, "f32"), (1040, "f32"), (4096, "bf16"), (4160, "bf16"), (8256, "bf16")])
 def test_stack_normalisation_at_the_edges_of_its_vectors(d, dtype):
     # one, two and three vectors of 8 elements per thread of 512, the last ones partly beyond the row; x apart from y and in place

@@ -1,4 +1,4 @@
-// The online path (Section 5.4) for calls of a few to 128 tokens on bf16 layers with 2-bit codes, sm_100a.
+// The online path (Section 5.4) for calls of a few to 128 tokens on bf16 layers with 2-bit or 4-bit codes, sm_100a.
 //
 // With that many tokens nearly every neuron is flagged by some token, so all of W1, W2, W_f and the predictor has to be read,
 // once: the bound is HBM (4096 / 16384: 320 MB = 49 us).  Two launches do the whole call; weights are the 128-row A operand
@@ -15,6 +15,8 @@
 //     added to the fp32 accumulator, and the last CTA to contribute to an output tile rounds it to y and clears it.
 //   Both take part in the programmatic hand-over: k_few_out fills its stages with W2 while k_few_in finishes, k_few_in its
 //     stages with W1 while the launch before it finishes (both fit on an SM side by side up to 64 tokens).
+//   4-bit codes take the same way with two bf16 terms per weight: 4096 / 16384, caches cold, 95 us for one token and 130 for 64, where
+//     the dense products over a dequantised predictor took 200 and 181.
 #include <string.h>
 
 #include <algorithm>
@@ -90,7 +92,7 @@ __device__ __forceinline__ uint32_t pair_of(float v) { return as_u32(__float2bfl
 // weights them by 1, 4 and 16), the offset (128 + weight zp) is subtracted and the scale over the weight multiplied: every step
 // is exact in bf16 when |q - zp| <= 2.  TERM 0 / 1: the two terms of values with |q - zp| = 3 (clamped to 2, and the rest).
 template <int TERM> __device__ __forceinline__ void expand(const uint4& code, uint32_t meta, uint32_t (&out)[32]) {
-  const float s = __uint_as_float(meta & 0xffff0000u), zp = float(meta & 3u);
+  const float s = __uint_as_float(meta & 0xffff0000u), zp = float(meta & 15u);
   const uint32_t words[4] = {code.x, code.y, code.z, code.w};
   __nv_bfloat162 off[3], sc[3], lim[3];
 #pragma unroll
@@ -115,36 +117,53 @@ template <int TERM> __device__ __forceinline__ void expand(const uint4& code, ui
     }
 }
 
+// The same with 4-bit codes, one field at a time into the low mantissa bits: s (q - zp) has up to 12 significant bits, so there are
+// always two terms, the rounded product and what it leaves (both exact: one fused multiply-add).
+template <int TERM> __device__ __forceinline__ void expand_4bit(const uint4 (&code)[2], uint32_t meta, uint32_t (&out)[32]) {
+  const __nv_bfloat162 off = as_bf2(pair_of(128.f + float(meta & 15u))), s = as_bf2(pair_of(__uint_as_float(meta & 0xffff0000u)));
+  const uint32_t words[8] = {code[0].x, code[0].y, code[0].z, code[0].w, code[1].x, code[1].y, code[1].z, code[1].w};
+#pragma unroll
+  for (int k = 0; k < 8; ++k)
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+      const __nv_bfloat162 v = __hsub2(as_bf2(((words[k] >> (4 * p)) & 0x000f000fu) | 0x43004300u), off), hi = __hmul2(v, s);
+      out[k * 4 + p] = as_u32(TERM == 0 ? hi : __hfma2(v, s, __hneg2(hi)));
+    }
+}
+
 // Exact fp64 predictor sum of one neuron and token over the code words first, first + step, ..., from the packed blocks the CTA
 // has just read (`rows` apart).  A lone warp waits for its loads and for its instructions, nothing else (8 us per pair with the
 // words read one after the other): four words' loads go out before the first is used, and the code is kept short.
-__device__ __noinline__ double exact_from_packed(const uint4* __restrict__ codes, const uint32_t* __restrict__ meta, const __nv_bfloat16* __restrict__ x,
+template <int BITS> __device__ __noinline__ double exact_from_packed(const uint4* __restrict__ codes, const uint32_t* __restrict__ meta, const __nv_bfloat16* __restrict__ x,
                                                  int nwords, int kpg, int rows, int first, int step) {
+  constexpr int PER = 32 / BITS, VEC = BITS / 2;           // codes of a word, 16-byte vectors of a block's neuron
+  constexpr uint32_t MASK = (1u << BITS) - 1u;
   double acc = 0.0;
 #pragma unroll 1
   for (int w0 = first; w0 < nwords; w0 += 4 * step) {
     uint32_t code[4], m[4];
-    uint4 xv[4][2];
+    uint4 xv[4][PER / 8];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      const int w = w0 + u * step, kb = w >> 2;
+      const int w = w0 + u * step;
       if (w < nwords) {
-        code[u] = reinterpret_cast<const uint32_t*>(codes + size_t(kb) * rows)[w & 3];
-        m[u] = meta[size_t(kb / kpg) * rows];
-        xv[u][0] = *reinterpret_cast<const uint4*>(x + w * 16);
-        xv[u][1] = *reinterpret_cast<const uint4*>(x + w * 16 + 8);
+        code[u] = reinterpret_cast<const uint32_t*>(codes + size_t(w >> 2) * rows)[w & 3];
+        m[u] = meta[size_t(w / (4 * VEC) / kpg) * rows];
+#pragma unroll
+        for (int q = 0; q < PER / 8; ++q) xv[u][q] = *reinterpret_cast<const uint4*>(x + w * PER + q * 8);
       }
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       if (w0 + u * step >= nwords) break;
-      const float zp = float(m[u] & 3u);
-      const uint32_t xw[8] = {xv[u][0].x, xv[u][0].y, xv[u][0].z, xv[u][0].w, xv[u][1].x, xv[u][1].y, xv[u][1].z, xv[u][1].w};
+      const float zp = float(m[u] & 15u);
       double p0 = 0.0, p1 = 0.0;
 #pragma unroll
-      for (int p = 0; p < 8; ++p) {                        // (q - zp) x is exact in fp32
-        p0 += double((float((code[u] >> (2 * p)) & 3u) - zp) * __uint_as_float(xw[p] << 16));
-        p1 += double((float((code[u] >> (16 + 2 * p)) & 3u) - zp) * __uint_as_float(xw[p] & 0xffff0000u));
+      for (int p = 0; p < PER / 2; ++p) {                  // (q - zp) x is exact in fp32
+        const uint4& xq = xv[u][p >> 2];
+        const uint32_t xw = (p & 3) == 0 ? xq.x : ((p & 3) == 1 ? xq.y : ((p & 3) == 2 ? xq.z : xq.w));
+        p0 += double((float((code[u] >> (BITS * p)) & MASK) - zp) * __uint_as_float(xw << 16));
+        p1 += double((float((code[u] >> (16 + BITS * p)) & MASK) - zp) * __uint_as_float(xw & 0xffff0000u));
       }
       acc += double(__uint_as_float(m[u] & 0xffff0000u)) * (p0 + p1);
     }
@@ -195,12 +214,14 @@ struct Walk {
   }
 };
 
-// N: token columns (the call's tokens rounded up); TERMS: bf16 terms of a correction (2 keeps 16 significant bits of it)
-template <int N, int TERMS>
+// N: token columns (the call's tokens rounded up); TERMS: bf16 terms of a correction (2 keeps 16 significant bits of it); BITS: of a
+// code
+template <int N, int TERMS, int BITS>
 __global__ void __maxnreg__(128)                       // (NT_IN threads; leaves room for k_few_out on the SM)
 k_few_in(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUtensorMap tmWf, const __grid_constant__ CUtensorMap tmX,
          const InParams p) {
   using C = InCfg<N>;
+  constexpr int VEC = BITS / 2, AHEAD = BITS == 2 ? 4 : 2;   // 16-byte vectors of a block's neuron; blocks fetched ahead (in registers)
   constexpr int RING = C::NBUF / 2;                    // expanded blocks per group of four warps
   constexpr int HALF = N / 2;                          // token columns per epilogue thread
   constexpr int MW = (HALF + 31) / 32;                 // flag words of a thread
@@ -275,7 +296,7 @@ k_few_in(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUten
     int s = 0, parity = 0, ati = 0, own0 = 0, own1 = 0;    // stage and its phase; tiles; expanded blocks used of either group
     auto next_stage = [&]() { if (++s == C::NS) { s = 0; parity ^= 1; } };
     for (int tile = blockIdx.x; tile < p.ntiles; tile += gridDim.x, ++ati) {
-      const int terms = p.two_terms[tile] ? 2 : 1;
+      const int terms = BITS > 2 || p.two_terms[tile] ? 2 : 1;
       bool ok = mbar_wait_issue(acc_free, (ati & 1) ^ 1, failed);
       for (int kb = 0; kb < nkb; ++kb) {
         ok = mbar_wait_issue(&full[s], parity, failed);
@@ -372,39 +393,44 @@ k_few_in(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUten
     bool ok = true;
     // (after a wait that ran out the flow stays the same, without further waits: the warps meet at named barriers)
     for (int tile = blockIdx.x; tile < p.ntiles; tile += gridDim.x, ++ati) {
-      // -- this group's channel blocks gi, gi + 2, ...: codes fetched four blocks ahead --
-      const int terms = p.two_terms[tile] ? 2 : 1;
-      const uint4* const tile_codes = p.codes + size_t(tile) * nkb * rows;
+      // -- this group's channel blocks gi, gi + 2, ...: codes fetched some blocks ahead --
+      const int terms = BITS > 2 || p.two_terms[tile] ? 2 : 1;
+      const uint4* const tile_codes = p.codes + size_t(tile) * nkb * VEC * rows;
       const uint32_t* const tile_meta = p.meta + size_t(tile) * (p.d / p.G) * rows;
       const int mine = (nkb - gi + 1) / 2;
-      uint4 code[4] = {};
-      uint32_t meta[4] = {};
-      auto fetch = [&](int kb, uint4& cd, uint32_t& mt) {
+      uint4 code[AHEAD][VEC] = {};
+      uint32_t meta[AHEAD] = {};
+      auto fetch = [&](int kb, uint4 (&cd)[VEC], uint32_t& mt) {
         if (row < rows) {
-          cd = __ldg(tile_codes + size_t(kb) * rows + row);
+#pragma unroll
+          for (int q = 0; q < VEC; ++q) cd[q] = __ldg(tile_codes + size_t(kb * VEC + q) * rows + row);
           mt = __ldg(tile_meta + size_t(kb / kpg) * rows + row);
         }
       };
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
+      for (int u = 0; u < AHEAD; ++u)
         if (u < mine) fetch(gi + 2 * u, code[u], meta[u]);
       const int j = tile * rows + row;
       const bool real = row < rows && j < p.h;
       float lo = 0.f, hi = 0.f, b1 = 0.f, fa = 0.f, fc = 0.f;
       if (real) { lo = p.lo[j]; hi = p.hi[j]; b1 = p.b1[j]; fa = p.a[j]; fc = p.c[j]; }
       const float smax = real ? p.smax[j] : 0.f;
-      for (int i0 = 0; i0 < mine && ok; i0 += 4) {
+      for (int i0 = 0; i0 < mine && ok; i0 += AHEAD) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < AHEAD; ++u) {
           const int i = i0 + u;
           if (i < mine && ok) {
             uint32_t w[32];
             for (int term = 0; term < terms && ok; ++term) {
               if (!holds) {}
-              else if (terms == 1) expand<-1>(code[u], meta[u], w);
-              else if (term == 0) expand<0>(code[u], meta[u], w);
-              else expand<1>(code[u], meta[u], w);
-              if (term == terms - 1 && i + 4 < mine) fetch(gi + 2 * (i + 4), code[u], meta[u]);
+              else if constexpr (BITS == 4) {
+                if (term == 0) expand_4bit<0>(code[u], meta[u], w);
+                else expand_4bit<1>(code[u], meta[u], w);
+              }
+              else if (terms == 1) expand<-1>(code[u][0], meta[u], w);
+              else if (term == 0) expand<0>(code[u][0], meta[u], w);
+              else expand<1>(code[u][0], meta[u], w);
+              if (term == terms - 1 && i + AHEAD < mine) fetch(gi + 2 * (i + AHEAD), code[u], meta[u]);
               const int b = gi + 2 * (own % RING);
               ok = mbar_wait_warp(&a_empty[b], ((own / RING) & 1) ^ 1);
               if (!ok) { *failed = 1u; break; }
@@ -426,7 +452,7 @@ k_few_in(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUten
       // (loops over columns stay rolled: unrolled, their code outgrows the instruction cache and costs 20 us)
       uint64_t flags = 0, open = 0;                        // bit c: token column gi HALF + c; open: too close to a range end to tell
       // the terms of a score are at most (largest |q - zp|) smax |x| each: 3 only where a tile has such codes
-      const float tau1 = (terms == 2 ? 3.f : 2.f) * kEps * smax;
+      const float tau1 = (BITS > 2 ? 15.f : (terms == 2 ? 3.f : 2.f)) * kEps * smax;
       const int cols = real ? min(HALF, p.n - gi * HALF) : 0;   // (may be negative)
 #pragma unroll 1
       for (int c0 = 0; c0 < HALF; c0 += 8) {
@@ -455,7 +481,7 @@ k_few_in(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUten
         const uint32_t slot = atomicAdd(near_count, 1u);
         if (slot < MAX_NEAR) near[slot] = make_uint4(uint32_t(row) << 8 | uint32_t(t), __float_as_uint(lo), __float_as_uint(hi), __float_as_uint(b1));
         else {                                             // list full: this thread settles the pair alone
-          const double ze = exact_from_packed(tile_codes + row, tile_meta + row, p.x + size_t(t) * p.d, nkb * 4, kpg, rows, 0, 1) + double(b1);
+          const double ze = exact_from_packed<BITS>(tile_codes + row, tile_meta + row, p.x + size_t(t) * p.d, nkb * 4 * VEC, kpg, rows, 0, 1) + double(b1);
           if (!(double(lo) <= ze && ze < double(hi))) flags |= 1ull << (t - gi * HALF);
         }
       }
@@ -466,7 +492,7 @@ k_few_in(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUten
           const uint4 pair = near[e];
           const int r = int(pair.x >> 8), t = int(pair.x & 255u);
           const float rl = __uint_as_float(pair.y), rh = __uint_as_float(pair.z), rb = __uint_as_float(pair.w);
-          double z = exact_from_packed(tile_codes + r, tile_meta + r, p.x + size_t(t) * p.d, nkb * 4, kpg, rows, lane, 32);
+          double z = exact_from_packed<BITS>(tile_codes + r, tile_meta + r, p.x + size_t(t) * p.d, nkb * 4 * VEC, kpg, rows, lane, 32);
 #pragma unroll
           for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
           z += double(rb);
@@ -708,34 +734,39 @@ k_few_out(const __grid_constant__ CUtensorMap tmW2, const __grid_constant__ CUte
 }
 
 // ---- set-up ---------------------------------------------------------------------------------------------
-// Packed predictor: block (tile of `rows` neurons, 64 channels) = rows x 16 bytes, a neuron's four code words each with its even
-// channels' codes in the lower half and the odd ones' in the upper half; per (tile, group) `rows` words, bf16 scale above,
-// zero-point below.  two_terms: the tile has a value with |q - zp| = 3.
+// Packed predictor: block (tile of `rows` neurons, 64 channels) = rows x 16 bytes (4-bit codes: twice, 32 channels each), a neuron's
+// four code words each with its even channels' codes in the lower half and the odd ones' in the upper half; per (tile, group)
+// `rows` words, bf16 scale above, zero-point below.  two_terms (2-bit codes): the tile has a value with |q - zp| = 3.
+template <int BITS>
 __global__ void k_pack(const uint32_t* __restrict__ codes, const __nv_bfloat16* __restrict__ scale, const uint8_t* __restrict__ zero,
                        uint4* __restrict__ out, uint32_t* __restrict__ meta, uint32_t* __restrict__ two_terms, int rows, int d, int h, int G, int nkb) {
+  constexpr int PER = 32 / BITS, VEC = BITS / 2;
+  constexpr uint32_t MASK = (1u << BITS) - 1u;
   const int tile = blockIdx.x, r = threadIdx.x, j = tile * rows + r, ng = d / G;
   bool two = false;
-  for (int kb = blockIdx.y; kb < nkb; kb += gridDim.y) {
+  for (int v = blockIdx.y; v < nkb * VEC; v += gridDim.y) {
     uint32_t w[4] = {0u, 0u, 0u, 0u};
     if (j < h) {
-      const uint4 src = *reinterpret_cast<const uint4*>(codes + size_t(j) * (d / 16) + kb * 4);
+      const uint4 src = *reinterpret_cast<const uint4*>(codes + size_t(j) * (d / PER) + v * 4);
       const uint32_t s[4] = {src.x, src.y, src.z, src.w};
-      const uint32_t zp = zero[size_t(j) * ng + kb * BK / G] & 3u;
+      const uint32_t zp = zero[size_t(j) * ng + v / VEC * BK / G] & MASK;
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
 #pragma unroll
-        for (int p = 0; p < 8; ++p)
-          w[k] |= ((s[k] >> (4 * p)) & 3u) << (2 * p) | ((s[k] >> (4 * p + 2)) & 3u) << (16 + 2 * p);
-        const uint32_t lo = s[k] & 0x55555555u, hi = (s[k] >> 1) & 0x55555555u;   // bits of the codes
-        two |= (zp == 0u && (lo & hi)) || (zp == 3u && (~(lo | hi) & 0x55555555u));
+        for (int p = 0; p < PER / 2; ++p)
+          w[k] |= ((s[k] >> (2 * BITS * p)) & MASK) << (BITS * p) | ((s[k] >> (2 * BITS * p + BITS)) & MASK) << (16 + BITS * p);
+        if (BITS == 2) {
+          const uint32_t lo = s[k] & 0x55555555u, hi = (s[k] >> 1) & 0x55555555u;   // bits of the codes
+          two |= (zp == 0u && (lo & hi)) || (zp == 3u && (~(lo | hi) & 0x55555555u));
+        }
       }
     }
-    out[(size_t(tile) * nkb + kb) * rows + r] = make_uint4(w[0], w[1], w[2], w[3]);
+    out[(size_t(tile) * nkb * VEC + v) * rows + r] = make_uint4(w[0], w[1], w[2], w[3]);
   }
   if (two) two_terms[tile] = 1u;
   for (int g = blockIdx.y; g < ng; g += gridDim.y)
     meta[(size_t(tile) * ng + g) * rows + r] =
-        j < h ? (uint32_t(__bfloat16_as_ushort(scale[size_t(j) * ng + g])) << 16) | (zero[size_t(j) * ng + g] & 3u) : 0u;
+        j < h ? (uint32_t(__bfloat16_as_ushort(scale[size_t(j) * ng + g])) << 16) | (zero[size_t(j) * ng + g] & MASK) : 0u;
 }
 
 // The shares of the folded product (end of each CTA's) and, per output tile, how many CTAs of k_few_out contribute to it (those that
@@ -795,11 +826,11 @@ static void deal_folded_blocks(const State& S, std::vector<int2>& plan) {
 
 using namespace few;
 
-// Serves bf16 layers with 2-bit codes in groups of a multiple of 64 channels (every channel block lies in one group).
+// Serves bf16 layers with 2-bit or 4-bit codes in groups of a multiple of 64 channels (every channel block lies in one group).
 tardis_status_t few_prepare(Handle* H) {
   H->few = nullptr;
   const int d = H->d, h = H->h, G = H->G;
-  if (H->dtype != TARDIS_BF16 || H->bits != 2 || G % BK || !tensor_maps_available()) return TARDIS_OK;
+  if (H->dtype != TARDIS_BF16 || (H->bits != 2 && H->bits != 4) || G % BK || !tensor_maps_available()) return TARDIS_OK;
   State* S = new (std::nothrow) State();
   if (!S) return TARDIS_ERR_ALLOC;
   memset(S, 0, sizeof(*S));
@@ -808,7 +839,7 @@ tardis_status_t few_prepare(Handle* H) {
   const int rounds = (h + S->grid * BM - 1) / (S->grid * BM), share = (h + S->grid * rounds - 1) / (S->grid * rounds);
   S->rows = std::min(BM, std::max(16, (share + 7) / 8 * 8));          // every CTA gets the same number of tiles, or one less
   S->nkb = d / BK; S->ntiles = (h + S->rows - 1) / S->rows; S->mtiles = (d + BM - 1) / BM; S->out_nkb = (h + BK - 1) / BK;
-  const size_t code_bytes = size_t(S->ntiles) * S->nkb * S->rows * 16, meta_bytes = size_t(S->ntiles) * (d / G) * S->rows * 4;
+  const size_t code_bytes = size_t(S->ntiles) * S->nkb * S->rows * 8 * H->bits, meta_bytes = size_t(S->ntiles) * (d / G) * S->rows * 4;
   struct Req { void** p; size_t bytes; };
   Req reqs[] = {{reinterpret_cast<void**>(&S->codes), code_bytes}, {reinterpret_cast<void**>(&S->meta), meta_bytes},
                 {reinterpret_cast<void**>(&S->plan), sizeof(int2) * S->grid}, {reinterpret_cast<void**>(&S->yacc), sizeof(float) * MAX_TOKENS * d},
@@ -823,9 +854,10 @@ tardis_status_t few_prepare(Handle* H) {
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     return e != cudaSuccess ? e : cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   };
-  const cudaError_t es[] = {room(k_few_in<16, 2>, InCfg<16>::SMEM), room(k_few_in<32, 1>, InCfg<32>::SMEM), room(k_few_in<64, 1>, InCfg<64>::SMEM),
-                            room(k_few_in<128, 1>, InCfg<128>::SMEM), room(k_few_out<32>, OutCfg<32>::SMEM), room(k_few_out<64>, OutCfg<64>::SMEM),
-                            room(k_few_out<128>, OutCfg<128>::SMEM)};
+  const cudaError_t es[] = {room(k_few_in<16, 2, 2>, InCfg<16>::SMEM), room(k_few_in<32, 1, 2>, InCfg<32>::SMEM), room(k_few_in<64, 1, 2>, InCfg<64>::SMEM),
+                            room(k_few_in<128, 1, 2>, InCfg<128>::SMEM), room(k_few_in<16, 2, 4>, InCfg<16>::SMEM), room(k_few_in<32, 1, 4>, InCfg<32>::SMEM),
+                            room(k_few_in<64, 1, 4>, InCfg<64>::SMEM), room(k_few_in<128, 1, 4>, InCfg<128>::SMEM), room(k_few_out<32>, OutCfg<32>::SMEM),
+                            room(k_few_out<64>, OutCfg<64>::SMEM), room(k_few_out<128>, OutCfg<128>::SMEM)};
   for (cudaError_t e : es)
     if (e != cudaSuccess) { set_last_error(e, "cudaFuncSetAttribute"); few_release(H); return TARDIS_ERR_CUDA; }
   S->done = S->nfl + MAX_TOKENS;
@@ -852,8 +884,9 @@ tardis_status_t few_finish(Handle* H, const void* W2, const void* Wf, cudaStream
   for (int c = 0; c < S->grid; ++c) shares.end[c] = plan[c].y;
   k_plan<<<1, 256, 0, s>>>(shares, S->plan, S->grid, S->parts, S->mtiles, S->out_nkb, S->out_grid);
   TARDIS_CUDA_TRY(cudaMemsetAsync(S->yacc, 0, sizeof(float) * MAX_TOKENS * d, s));
-  k_pack<<<dim3(S->ntiles, 8), S->rows, 0, s>>>(H->codes, static_cast<const __nv_bfloat16*>(H->scale), H->zero, S->codes, S->meta, S->two_terms,
-                                                S->rows, d, h, H->G, S->nkb);
+  auto pack = H->bits == 2 ? k_pack<2> : k_pack<4>;
+  pack<<<dim3(S->ntiles, 8), S->rows, 0, s>>>(H->codes, static_cast<const __nv_bfloat16*>(H->scale), H->zero, S->codes, S->meta, S->two_terms,
+                                              S->rows, d, h, H->G, S->nkb);
   TARDIS_CUDA_TRY(cudaGetLastError());
   return TARDIS_OK;
 }
@@ -891,7 +924,7 @@ static tardis_status_t launch_n(Handle* H, const __nv_bfloat16* x, __nv_bfloat16
   a.wf_plan = S->plan; a.delta = S->delta; a.yacc = S->yacc; a.nfl = S->nfl; a.counters = H->counters;
   a.dbg_bitmap = H->dbg_bitmap; a.dbg_scores = H->dbg_scores;
   if (H->dbg_bitmap) TARDIS_CUDA_TRY(cudaMemsetAsync(H->dbg_bitmap, 0, size_t(n) * (H->h / 32) * 4, s));
-  TARDIS_CUDA_TRY(launch_overlapped(k_few_in<N, TERMS>, S->grid, NT_IN, InCfg<N>::SMEM, s, S->w1, S->wf, tmx, a));
+  TARDIS_CUDA_TRY(launch_overlapped(H->bits == 2 ? k_few_in<N, TERMS, 2> : k_few_in<N, TERMS, 4>, S->grid, NT_IN, InCfg<N>::SMEM, s, S->w1, S->wf, tmx, a));
   OutParams o = {};
   o.n = n; o.d = H->d; o.h = H->h; o.nkb = S->out_nkb; o.total = S->mtiles * S->out_nkb; o.terms = TERMS;
   o.bf = H->bf; o.yacc = S->yacc; o.y = y; o.done = S->done; o.parts = S->parts; o.nfl = S->nfl; o.counters = H->counters;

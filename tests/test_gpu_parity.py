@@ -582,6 +582,14 @@ def test_kernels_for_a_few_tokens_at_the_edges_of_their_tiles(d, h, G, q):
     _run(cfg, sum(calls), calls, path=3)
 
 
+@pytest.mark.parametrize("d,h,G,q", [(64, 32, 64, 0.4), (192, 160, 64, 0.2), (1088, 4640, 64, 0.05), (1024, 4096, 128, 0.1)])
+def test_kernels_for_a_few_tokens_with_4_bit_codes(d, h, G, q):
+    # one channel block and several, an odd number of them, tiles with a short last one, every width of the token columns
+    cfg = W.LayerConfig("few4bit%d" % d, d, h, group=G, n_calib=256, q_lo=q, q_hi=1 - q, bits=4)
+    calls = [1, 3, 16, 17, 33, 64, 65, 128]
+    _run(cfg, sum(calls), calls)
+
+
 @pytest.mark.parametrize("d,h,G,q", [(64, 32, 64, 0.4), (320, 2400, 64, 0.2), (4096, 16384, 128, 0.05), (4608, 18944, 64, 0.1),
                                      (4672, 4768, 64, 0.1), (8192, 2400, 128, 0.4)])
 def test_fused_kernels_at_the_edges_of_their_rings(d, h, G, q):

@@ -98,7 +98,8 @@ typedef struct {
   uint64_t tokens;              /* tokens processed                                        */
   uint64_t flagged_total;       /* sum over tokens of flagged neurons                      */
   uint64_t flagged_max;         /* largest flagged count of a single token                 */
-  uint64_t last_path;           /* 0 none, 1 generic kernels, 2 fused decode kernel, 3 batched/prefill,
+  uint64_t last_path;           /* 0 none, 1 generic kernels (fp32 layers: their own), 2 fused decode
+                                   kernel, 3 batched/prefill (up to 128 tokens: the few-token kernels),
                                    5 generic kernels on the library's built-in scratch
                                    (tardis_ffn_forward_static)                              */
   uint64_t bytes_folded;        /* W_f and b_f                                             */

@@ -46,6 +46,15 @@ __device__ __forceinline__ double gelu_slope_f64(double z, int act) {
   return 0.5 * (1.0 + erf(z * 0.7071067811865476)) + z * exp(-0.5 * z * z) * 0.3989422804014327;
 }
 
+// The activation by the formula that defines it, for decisions that rest on its exact values: where tanh is -1 (+1) to the last bit it
+// is 0 (z), so that the errors of two ranges out there are both exactly 0 and the tie rule of the search applies.  (gelu_f64 keeps
+// values of 1e-37 there: more exact, but another side then wins.)
+__device__ __forceinline__ double activation_f64(double z, int act) {
+  if (act != TARDIS_ACT_GELU_TANH) return gelu_f64(z, act);
+  const double u = 0.7978845608028654 * (z + 0.044715 * z * z * z);
+  return 0.5 * z * (1.0 + tanh(u));
+}
+
 // The n samples of neuron j plus its bias, NT E values over the CTA (+inf beyond n): thread t gets samples e NT + t.
 template <int E> __device__ __forceinline__ void load_samples(float (&v)[E], const float* __restrict__ z, long long ldz,
                                                               const float* __restrict__ b1, int j, int n) {
@@ -526,7 +535,7 @@ k_range_search(const float* __restrict__ z, long long ldz, const float* __restri
   const double cen = double(keys[ic]);
   __syncthreads();                                                 // (the list in the place of gs has been read)
 #pragma unroll
-  for (int e = 0; e < E; ++e) gs[tid * E + e] = tid * E + e < n ? gelu_f64(double(v[e]), act) : 0.0;
+  for (int e = 0; e < E; ++e) gs[tid * E + e] = tid * E + e < n ? activation_f64(double(v[e]), act) : 0.0;
   __syncthreads();
   // number of samples below x
   auto lower = [&](double x) {
@@ -688,7 +697,7 @@ k_neuron_error(const float* __restrict__ z, long long ldz, const float* __restri
   for (int e = 0; e < E; ++e) {
     const double x = double(v[e]);
     const bool in = e * NT + threadIdx.x < n && x >= l && x < u;
-    g[e] = in ? gelu_f64(x, act) : 0.0;
+    g[e] = in ? activation_f64(x, act) : 0.0;
     if (in) { s[0] += 1.0; s[1] += x; s[2] += g[e]; }
     else v[e] = __int_as_float(0x7f800000);
   }

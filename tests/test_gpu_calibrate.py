@@ -201,6 +201,18 @@ def test_range_search_screening_falls_back_where_it_must(kind, n, step):
         assert _check_search(z.cuda(), None, 0.9, step, act) <= 3
 
 
+@pytest.mark.parametrize("mean,spread", [(-10.0, 0.3), (-20.0, 1.0), (-9.0, 0.2), (9.5, 0.3)])
+def test_range_search_of_saturated_neurons(mean, spread):
+    # far out the tanh form of GELU is exactly 0 (z): every error is exactly 0, every choice a tie, and the right side is grown
+    g = torch.Generator().manual_seed(3)
+    z = mean + spread * torch.randn(24, 300, generator=g)
+    for t in (0.3, 0.6):
+        assert _check_search(z.cuda(), None, t, spread / 10, W.ACT_GELU_TANH) == 0
+    if mean < 0:
+        err, _ = T.tardis_neuron_thresholds(z.cuda(), None, z.min(1).values.cuda(), z.max(1).values.cuda(), W.ACT_GELU_TANH, 0.8, 0.7, 0.9)
+        assert (err == 0).all()
+
+
 def test_greedy_range_search_edge_cases_and_errors():
     lib = T.load_library()
     # all samples equal, a single sample, threshold 0 (empty range at the centroid) and 1 (every sample)

@@ -587,22 +587,27 @@ k_range_search(const float* __restrict__ z, long long ldz, const float* __restri
     }
     __syncthreads();
     if (tid < 32) {
-      // mean squared residual of the least-squares line over the sorted samples i0 .. i1 - 1, as it is defined
+      // Mean squared residual of the least-squares line over the sorted samples i0 .. i1 - 1, as it is defined.  Where both errors are
+      // zero but for rounding (two distinct values inside, a straight stretch of the activation) the order of the additions decides,
+      // so it is a fixed one: 256 running sums, sample i0 + s + 256 k to sum s, added up in trees of 32, those in ascending order.
       auto mse = [&](int i0, int i1) -> double {
         const int cnt = i1 - i0;
         if (cnt < 2) return 0.0;
+        auto total = [&](auto term) {
+          double t = 0.0;
+          for (int s0 = 0; s0 < NT && s0 < cnt; s0 += 32) {        // (what is left out adds zeros)
+            double sum = 0.0;
+            for (int i = i0 + s0 + lane; i < i1; i += NT) sum += term(i);
+            t += warp_sum(sum);
+          }
+          return t;
+        };
         const double q = 1.0 / double(cnt);
-        double sz = 0.0, sg = 0.0;
-        for (int i = i0 + lane; i < i1; i += 32) { sz += double(keys[i]); sg += gs[i]; }
-        const double mz = warp_sum(sz) * q, mg = warp_sum(sg) * q;
-        double vzz = 0.0, vzg = 0.0;
-        for (int i = i0 + lane; i < i1; i += 32) { const double dz = double(keys[i]) - mz; vzz += dz * dz; vzg += dz * (gs[i] - mg); }
-        vzz = warp_sum(vzz) * q; vzg = warp_sum(vzg) * q;
+        const double mz = total([&](int i) { return double(keys[i]); }) * q, mg = total([&](int i) { return gs[i]; }) * q;
+        const double vzz = total([&](int i) { const double dz = double(keys[i]) - mz; return dz * dz; }) * q;
         if (!(vzz > 1e-30)) return 0.0;
-        const double sl = vzg / vzz;
-        double rr = 0.0;
-        for (int i = i0 + lane; i < i1; i += 32) { const double r = (gs[i] - mg) - sl * (double(keys[i]) - mz); rr += r * r; }
-        return warp_sum(rr) * q;
+        const double sl = total([&](int i) { return (double(keys[i]) - mz) * (gs[i] - mg); }) * q / vzz;
+        return total([&](int i) { const double r = (gs[i] - mg) - sl * (double(keys[i]) - mz); return r * r; }) * q;
       };
       // lane = range after i steps to the left and jr to the right, i + jr <= kAhead: lanes s (s + 1) / 2 + jr, s = i + jr
       auto lane_of = [](int i, int jr) { const int s = i + jr; return s * (s + 1) / 2 + jr; };

@@ -213,6 +213,16 @@ def test_range_search_of_saturated_neurons(mean, spread):
         assert (err == 0).all()
 
 
+def test_range_search_choices_that_rest_on_rounding_are_fixed():
+    # samples on a coarse grid: a range of two distinct values has no error but rounding, and the order of the additions in the error's
+    # definition (256 running sums, trees of 32) decides.  The step counts are pinned as that order gives them.
+    pinned = [15, 20, 17, 15, 12, 15, 28, 24, 17, 22, 17, 15, 22, 36, 25, 17, 20, 24, 15, 15, 20, 15, 15, 15, 17, 15, 20, 20, 15, 30, 17,
+              15, 15, 18, 17, 17, 15, 18, 31, 31, 15, 20, 22, 21, 20, 23, 25, 12]
+    z = (torch.randn(48, 200, generator=torch.Generator().manual_seed(5)) * 4).round() / 4
+    steps = T.tardis_range_search(z.cuda(), None, 0.5, 0.1, W.ACT_GELU_ERF, want_steps=True)[4]
+    assert steps.tolist() == pinned
+
+
 def test_greedy_range_search_edge_cases_and_errors():
     lib = T.load_library()
     # all samples equal, a single sample, threshold 0 (empty range at the centroid) and 1 (every sample)

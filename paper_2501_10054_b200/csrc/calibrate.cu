@@ -312,7 +312,7 @@ __device__ __forceinline__ double warp_sum(double v) {
 }
 
 struct Bins {
-  float centre[kMaxBins];
+  float centre[kMaxBins];                // from the smallest sample on
   float m[5][kMaxBins];                  // sum of offset^n / n! of the bin's samples, offsets from the centre in kernel widths
   float l[5][kMaxBins];                  // Taylor coefficients of the density about the centre
 };
@@ -361,7 +361,9 @@ template <int E> __device__ __forceinline__ int densest_sample(const float (&v)[
       const int i = tid * E + e;
       if (i < n) {
         const int b = before + first[e] - 1;
-        const float c = zmin + (bin_of(v[e]) + 0.5f) * width, o = (v[e] - c) * inv;
+        // (distances from the smallest sample, which are exact or rounded to 2^-24 of themselves: a centre in the samples' own
+        // coordinates would be off by an ulp of them, a fifth of the kernel width where the samples lie 4 ulps apart)
+        const float c = (bin_of(v[e]) + 0.5f) * width, o = ((v[e] - zmin) - c) * inv;
         if (e == 0 || first[e] != first[e > 0 ? e - 1 : 0]) bins.centre[b] = c;   // (neighbours in other threads write the same)
         const float o2 = o * o;
         sum[0] += 1.f; sum[1] += o; sum[2] += 0.5f * o2; sum[3] += o2 * o * (1.f / 6.f); sum[4] += o2 * o2 * (1.f / 24.f);
@@ -409,7 +411,7 @@ template <int E> __device__ __forceinline__ int densest_sample(const float (&v)[
       f[e] = -1.f;
       if (i < n && !(i > 0 && v[e] == (e ? v[e > 0 ? e - 1 : 0] : keys[i - 1]))) {   // (else the same density as its predecessor)
         const int b = before + first[e] - 1;
-        const float t = (v[e] - bins.centre[b]) * inv;
+        const float t = ((v[e] - zmin) - bins.centre[b]) * inv;
         f[e] = fmaf(t, fmaf(t, fmaf(t, fmaf(t, bins.l[4][b], bins.l[3][b]), bins.l[2][b]), bins.l[1][b]), bins.l[0][b]);
         best = fmaxf(best, f[e]);
       }
@@ -628,7 +630,9 @@ k_range_search(const float* __restrict__ z, long long ldz, const float* __restri
           for (int q = 0; q < 5; ++q) m[q] = base_m[q] + (st.m[0][q][kl + i_mine] + st.m[1][q][kr + j_mine]);
           const double q = double(cnt), yy = m[2] * q, gg = m[4] * q;
           const double vyy = yy - m[0] * m[0], vyg = m[3] * q - m[0] * m[1], vgg = gg - m[1] * m[1];
-          // every moment is off by less than 1e-13 of the sum of its terms' sizes (2 n 2^-53); |yg| <= sqrt(yy gg)
+          // Every moment is off by less than c = (n + 20) 2^-53 = 2.3e-13 of the sum of its terms' sizes (n additions, a few roundings
+          // in a term and in joining the parts), and |yg| <= sqrt(yy gg): vyy by 3 c yy, vyg by 3 c sqrt(yy gg), vgg by 3 c gg, so
+          // err q^2 by 3 c gg (1 + sqrt(yy / vyy))^2 <= 7e-13 gg k^2.
           const float k = 1.f + __fdividef(float(yy), float(vyy)), iq = __fdividef(1.f, float(q));
           off = fmaxf(1e-12f * float(gg) * iq * iq * k * k, 1e-37f);
           if (!(vyy > 1e-8 * yy && vyy > 1e-25 * q * q)) off = __int_as_float(0x7f800000);

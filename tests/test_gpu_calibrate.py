@@ -213,6 +213,18 @@ def test_range_search_of_saturated_neurons(mean, spread):
         assert (err == 0).all()
 
 
+@pytest.mark.parametrize("n,ulps", [(300, 3), (2048, 12), (2048, 17), (2048, 21), (2047, 30), (1000, 100), (2048, 3000)])
+def test_range_search_of_samples_few_ulps_apart(n, ulps):
+    # a large mean and a spread of few units in the last place: the densities are screened in distances from the smallest sample, and
+    # the bins' centres must not be rounded to the samples' own grid
+    g = torch.Generator().manual_seed(n + ulps)
+    z = 2.0 ** 23 + 4e6 + (torch.randn(16, n, generator=g, dtype=torch.float64) * ulps).round()
+    z[:4] = 2.0 ** 23 + torch.tensor([4., 7., 13., 32., 36., 48., 51.], dtype=torch.float64)[
+        torch.multinomial(torch.tensor([708., 327., 297., 99., 131., 182., 304.]), 4 * n, replacement=True, generator=g).view(4, n)]
+    for t in (0.0, 0.6):
+        assert _check_search(z.float().cuda(), None, t, ulps / 4, W.ACT_RELU) == 0
+
+
 def test_range_search_choices_that_rest_on_rounding_are_fixed():
     # samples on a coarse grid: a range of two distinct values has no error but rounding, and the order of the additions in the error's
     # definition (256 running sums, trees of 32) decides.  The step counts are pinned as that order gives them.

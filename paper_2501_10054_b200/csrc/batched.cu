@@ -39,7 +39,7 @@ struct State {
   __nv_bfloat16* delta;                            // [kChunk,h]
   uint32_t* bitmap;                                // [kChunk,h/32]
   uint32_t* rlist;                                 // [kChunk][kMaxRecheck] neurons of a token to re-evaluate
-  unsigned int* rcount;                            // [kChunk] how many (more than the queue holds: the rest was settled at once)
+  unsigned int* rcount;                            // [kChunk] how many (more than the queue holds: every neuron is re-evaluated)
   size_t bytes_state, bytes_scratch;
 };
 
@@ -115,7 +115,8 @@ __global__ void k_xnorm(const __nv_bfloat16* __restrict__ x, int d, float* __res
 }
 
 // A CTA per token: the exact fp64 scores of its queued neurons (one warp each, from the packed codes) decide their flags; then the
-// token's flags are counted.  The token is widened to fp64 once, in shared memory: with a conversion per product these, at 16 per
+// token's flags are counted.  Where more neurons wanted to queue than fit, all are re-evaluated (4096 / 16384: 3 ms for such a token;
+// each settled by the thread that met it, in the product's epilogue: 18 to 46 ms).  The token is widened to fp64 once, in shared memory: with a conversion per product these, at 16 per
 // clock and SM, were the bound (2048 tokens on 4096 / 16384: 51 us, 93 before with the count as a kernel of its own).
 // WIDTH: bits per code where 32 is a multiple of it, else 0.  STAGED: false for tokens that do not fit in shared memory.
 template <int WIDTH, bool STAGED>
@@ -126,7 +127,9 @@ __global__ void __launch_bounds__(256) k_recheck(const uint32_t* __restrict__ rl
   extern __shared__ double xd[];                           // channel c of unit u (16 channels) at c (d / 16 + 1) + u: the lanes' units side by side
   __shared__ unsigned int flagged;
   const int t = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const unsigned int queued = rcount[t], total = min(queued, (unsigned int)kMaxRecheck);
+  const unsigned int queued = rcount[t];
+  const bool all = queued > (unsigned int)kMaxRecheck;
+  const unsigned int total = all ? (unsigned int)h : queued;
   const __nv_bfloat16* const xt = x + size_t(t) * d;
   const int nw = d / 16;
   auto xv = [&](int u, int c) { return STAGED ? xd[c * (nw + 1) + u] : double(__bfloat162float(xt[u * 16 + c])); };
@@ -144,7 +147,7 @@ __global__ void __launch_bounds__(256) k_recheck(const uint32_t* __restrict__ rl
   __syncthreads();
   const int ng = d / G;
   for (unsigned int e = warp; e < total; e += 8) {
-    const int j = int(rlist[size_t(t) * kMaxRecheck + e]);
+    const int j = all ? int(e) : int(rlist[size_t(t) * kMaxRecheck + e]);
     const uint32_t* const row = codes + size_t(j) * (size_t(d) * bits / 32);
     double z = 0.0;
     // units of 16 channels (all of one group), four at a time: their loads go out before the first is used, since waiting for them
@@ -205,7 +208,7 @@ __global__ void __launch_bounds__(256) k_recheck(const uint32_t* __restrict__ rl
       atomicAdd(&counters[CTR_FLAGGED_TOTAL], (unsigned long long)flagged);
       atomicMax(&counters[CTR_FLAGGED_MAX], (unsigned long long)flagged);
     }
-    if (queued) atomicAdd(&counters[CTR_RECHECKS], (unsigned long long)queued);
+    if (total) atomicAdd(&counters[CTR_RECHECKS], (unsigned long long)total);
   }
 }
 
@@ -401,7 +404,7 @@ tardis_status_t launch_batched_forward(Handle* H, const void* xv, void* yv, int6
     g.error_word = &H->counters[CTR_ERROR];
     g.lo = H->lo; g.hi = H->hi; g.colscale = S->smaxrow; g.rowscale = S->x1; g.keps = kEps * float((1 << H->bits) - 1);
     g.bitmap_out = S->bitmap; g.rlist = S->rlist; g.rcount = S->rcount; g.rcap = kMaxRecheck;
-    g.codes = H->codes; g.scale = H->scale; g.zero = H->zero; g.xsrc = xc; g.d = d; g.G = H->G; g.bits = H->bits;
+    g.bits = H->bits;
     tardis_status_t st = launch_gemm(g, s);
     if (st != TARDIS_OK) return st;
     const bool staged = d <= 24576;                        // (192 KB)

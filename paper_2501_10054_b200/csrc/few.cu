@@ -463,7 +463,8 @@ k_few_in(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUten
         for (int e = 0; e < 8; ++e) {
           const float xn = x1[gi * HALF + c0 + e], z = v[e] + b1, tau = fmaf(tau1, xn, 1e-30f);
           const bool finite = xn <= 3.0e38f;               // (a non-finite token: every neuron flagged)
-          const bool near_end = finite && (fabsf(z - lo) <= tau || fabsf(z - hi) <= tau);
+          // (a token of zeros has no error, and its scores, the biases, may well lie on range ends)
+          const bool near_end = finite && xn > 0.f && (fabsf(z - lo) <= tau || fabsf(z - hi) <= tau);
           fl |= uint32_t(!near_end && !(finite && lo <= z && z < hi)) << e;
           op |= uint32_t(near_end) << e;
           v[e] = finite ? z : __int_as_float(0x7fc00000);

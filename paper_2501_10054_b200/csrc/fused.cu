@@ -169,8 +169,8 @@ __device__ __forceinline__ void ldmatrix_x4(uint32_t& r0, uint32_t& r1, uint32_t
 __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3, uint32_t addr) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(addr) : "memory");
 }
-// Exact fp64 predictor sum of one neuron (row r of a tile) from the tile's predictor blocks: the same
-// terms as exact_score, which reads the original arrays.  Lane `lane` of `nl` takes
+// Exact fp64 predictor sum of one neuron (row r of a tile) from the tile's predictor blocks: s[j,g] (q - zp) x over its
+// channels, without the bias.  Lane `lane` of `nl` takes
 // the code words lane, lane + nl, ...; the caller adds the lanes up.
 __device__ __forceinline__ double exact_from_blocks(const uint8_t* ubase, int pbs, int G, int r, const __nv_bfloat16* xt, int d,
                                                     int lane, int nl) {
@@ -727,7 +727,8 @@ __global__ void __launch_bounds__(NTH, 1) k_fused(const Params p) {
         const double lo = double(tab[r]), hi = double(tab[TR + r]);
         int f = ((lo <= zhat) && (zhat < hi)) ? 0 : 1;
         if (misc[MS_NONFIN + t]) { f = 1; zhat = __longlong_as_double(0x7ff8000000000000ll); }
-        else if (fabs(zhat - lo) <= tau || fabs(zhat - hi) <= tau || (NTK > 2 && !(fabs(zhat) < 1e37))) {
+        // (a token of zeros has no error, and its scores, the biases, may well lie on range ends)
+        else if (l1 > 0.f && (fabs(zhat - lo) <= tau || fabs(zhat - hi) <= tau || (NTK > 2 && !(fabs(zhat) < 1e37)))) {
           const int e = atomicAdd(const_cast<int*>(&misc[MS_NRC]), 1);
           if (e < MAXRC) { rc[e] = (t << 16) | r; f = -1; }
           else {                                        // list full: this thread re-evaluates its neuron alone

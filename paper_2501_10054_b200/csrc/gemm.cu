@@ -15,7 +15,6 @@
 #include <stdio.h>
 
 #include "common.cuh"
-#include "exact.cuh"
 #include "tc.cuh"
 
 namespace tardis {
@@ -67,9 +66,7 @@ struct KParams {
   const float *lo, *hi, *colscale, *rowscale;
   float keps;
   uint32_t* bitmap_out;
-  uint32_t* rlist; unsigned int* rcount; int rcap;
-  const uint32_t* codes; const __nv_bfloat16* scale; const uint8_t* zero;
-  const __nv_bfloat16* xsrc; int d, G, bits;
+  uint32_t* rlist; unsigned int* rcount; int rcap, bits;
 };
 
 template <int BN> struct Cfg {
@@ -114,15 +111,10 @@ __device__ __forceinline__ void epilogue_chunk(const KParams& p, float (&v)[32],
         open |= (fminf(fabsf(dl), fabsf(du)) <= fmaf(t.z, kx, 1e-30f) ? 1u : 0u) << i;
       }
       word = outside & valid;
-      for (uint32_t w = open & valid; w; w &= w - 1u) {      // rare
-        const int i = __ffs(w) - 1;
+      // (a token of zeros has no error, and its scores, the biases, may well lie on range ends)
+      for (uint32_t w = xn > 0.f ? open & valid : 0u; w; w &= w - 1u) {      // rare
         const unsigned int slot = atomicAdd(&p.rcount[m], 1u);
-        if (slot < (unsigned int)p.rcap) p.rlist[size_t(m) * p.rcap + slot] = uint32_t(n + i);
-        else {                                               // the token's queue is full: settle this one here (slow, but exact)
-          const double ze = exact_score_single(p.codes, p.scale, p.zero, p.xsrc + size_t(m) * p.d, n + i, p.d, p.G, p.bits) + double(p.bias[n + i]);
-          const bool flag = !((double(p.lo[n + i]) <= ze) && (ze < double(p.hi[n + i])));
-          word = flag ? word | (1u << i) : word & ~(1u << i);
-        }
+        if (slot < (unsigned int)p.rcap) p.rlist[size_t(m) * p.rcap + slot] = uint32_t(n + __ffs(w) - 1);
       }
     }
     p.bitmap_out[size_t(m) * (p.N / 32) + (n >> 5)] = word;
@@ -396,8 +388,7 @@ static tardis_status_t launch_bn(const GemmArgs& g, cudaStream_t s) {
   p.out_f32 = g.out_f32; p.out_bf16 = static_cast<__nv_bfloat16*>(g.out_bf16);
   p.bias = g.bias; p.addend = g.addend; p.a = g.a; p.c = g.c; p.bitmap = g.bitmap; p.error_word = g.error_word;
   p.lo = g.lo; p.hi = g.hi; p.colscale = g.colscale; p.rowscale = g.rowscale; p.keps = g.keps; p.bitmap_out = g.bitmap_out;
-  p.rlist = g.rlist; p.rcount = g.rcount; p.rcap = g.rcap; p.codes = g.codes; p.scale = static_cast<const __nv_bfloat16*>(g.scale);
-  p.zero = g.zero; p.xsrc = static_cast<const __nv_bfloat16*>(g.xsrc); p.d = g.d; p.G = g.G; p.bits = g.bits;
+  p.rlist = g.rlist; p.rcount = g.rcount; p.rcap = g.rcap; p.bits = g.bits;
   static thread_local int room_on = -1;               // the device on which this thread last gave the kernel its shared memory
   int dev = 0, sms = 0;
   TARDIS_CUDA_TRY(cudaGetDevice(&dev));
@@ -427,8 +418,7 @@ tardis_status_t launch_gemm(const GemmArgs& g, cudaStream_t s) {
   if (bad(g.A1, g.lda1, g.K1) || bad(g.B1, g.ldb1, g.K1)) return TARDIS_ERR_INVALID_ARG;
   if (g.K2 > 0 && (bad(g.A2, g.lda2, g.K2) || bad(g.B2, g.ldb2, g.K2))) return TARDIS_ERR_INVALID_ARG;
   if ((g.epilogue == GEMM_EPI_DELTA || g.epilogue == GEMM_EPI_FLAGS) && (g.N % 32)) return TARDIS_ERR_INVALID_ARG;
-  if (g.epilogue == GEMM_EPI_FLAGS && !(g.bias && g.lo && g.hi && g.colscale && g.rowscale && g.bitmap_out && g.rlist && g.rcount &&
-                                         g.codes && g.scale && g.zero && g.xsrc))
+  if (g.epilogue == GEMM_EPI_FLAGS && !(g.bias && g.lo && g.hi && g.colscale && g.rowscale && g.bitmap_out && g.rlist && g.rcount))
     return TARDIS_ERR_INVALID_ARG;
   if (g.splits > 1 && g.epilogue != GEMM_EPI_F32) return TARDIS_ERR_INVALID_ARG;
   // the epilogues store (or reduce) 16 bytes at a time

@@ -16,8 +16,9 @@ enum GemmEpilogue {
   GEMM_EPI_DELTA = 2,      // z = acc + bias[n]; out_bf16[m, n] = flagged(m, n) ? GELU(z) - a[n] z - c[n] : 0
   GEMM_EPI_FLAGS = 3       // z = acc + bias[n]; bit (m, n) of bitmap_out = !(lo[n] <= z < hi[n]); a z within
                            // keps * colscale[n] * rowscale[m] of lo[n] or hi[n] is queued in rlist for exact
-                           // re-evaluation (settled in place from the codes when the queue is full); a row whose
-                           // rowscale is not finite is flagged throughout; z is also stored when out_f32 is given
+                           // re-evaluation (rcount[m] above rcap: some were not); a row whose rowscale is not finite
+                           // is flagged throughout, one whose rowscale is 0 queues nothing (its z are the biases);
+                           // z is also stored when out_f32 is given
 };
 
 struct GemmArgs {
@@ -41,8 +42,7 @@ struct GemmArgs {
   float keps;
   uint32_t* bitmap_out;             // [M, N / 32]
   uint32_t* rlist; unsigned int* rcount; int rcap;   // per row m a queue of rcap columns, and how many wanted to enter it
-  const uint32_t* codes; const void* scale; const uint8_t* zero;   // the packed predictor (rows n)
-  const void* xsrc; int d, G, bits; // the bf16 rows A1 came from (leading dimension d), group size, bits per code
+  int bits;                         // bits per predictor code
 };
 
 // Enqueues the GEMM on `s`.  Returns UNSUPPORTED when the tensor-map entry point of the driver is not

@@ -626,3 +626,56 @@ def test_stack_normalisation_at_the_edges_of_its_vectors(d, dtype):
             assert torch.equal(y, s)
     finally:
         T.tardis_destroy(h)
+
+
+def _at_range_ends(d, h, bits, group, seed):
+    """A ReLU layer without biases whose ranges all end at 0."""
+    L = _layer(W.LayerConfig("ends%d" % bits, d, h, bits=bits, group=group, n_calib=128, act=W.ACT_RELU, bias=False), seed)
+    L.lo.fill_(float("-inf"))
+    L.hi.zero_()
+    L.a.zero_()
+    L.c.zero_()
+    return L
+
+
+@pytest.mark.parametrize("d,bits,group", [(512, 2, 64), (512, 4, 64), (512, 3, 64), (512, 2, 16), (4672, 2, 64)])
+def test_tokens_of_zeros_on_range_ends_need_no_re_evaluation(d, bits, group):
+    # such a token's scores are the biases, here exactly the range ends: nothing is uncertain about them
+    L = _at_range_ends(d, 2080, bits, group, 7)
+    h = T.fold_layer(L)
+    try:
+        for path in (0, 3):
+            T.tardis_set_path(h, path)
+            for n in (1, 2, 4, 9, 60, 150):
+                y, F, S = Hp.gpu_forward(h, L, torch.zeros(n, d, dtype=L.W1.dtype, device="cuda"))
+                assert F.all() and (S == 0).all() and T.tardis_stats(h)["exact_rechecks"] == 0
+                assert (y == (0 if L.b2 is None else L.b2.to(y.dtype))).all()
+    finally:
+        T.tardis_destroy(h)
+
+
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("n", [3, 40, 150])
+def test_more_scores_on_range_ends_than_are_queued(bits, n):
+    # every neuron has the same predictor row, and the ranges end at token 0's score: one neuron below the next above it
+    L = _layer(W.LayerConfig("crowd%d" % bits, 512, 2080, bits=bits, group=64, n_calib=128), 9)
+    for v in (L.codes, L.scale, L.zero):
+        v[:] = v[:1].clone()
+    L.b1.zero_()
+    s = L.numpy64()
+    x = W.make_tokens(L.cfg, n, 9).cuda()
+    z = np.float32(O.predictor_score(x[:1].double().cpu().numpy(), s["codes"], s["scale"], s["zero"], s["group"], s["b1"], s["bits"])[0, 0])
+    L.lo.fill_(float(z) - 1.0)
+    ends = [z, np.nextafter(z, np.float32(np.inf)), np.nextafter(z, np.float32(-np.inf))]
+    L.hi[:] = torch.tensor([ends[j % 3] for j in range(2080)], device="cuda")
+    s = L.numpy64()
+    h = T.fold_layer(L)
+    try:
+        for path in (0, 3):
+            T.tardis_set_path(h, path)
+            _, F, _ = Hp.gpu_forward(h, L, x)
+            zhat = O.predictor_score(x.double().cpu().numpy(), s["codes"], s["scale"], s["zero"], s["group"], s["b1"], s["bits"])
+            sure = np.abs(zhat - s["hi"]) > 1e-9 * np.abs(zhat)      # (fp64 sums in another order: 512 2^-53 of the terms)
+            assert (F == O.flags_from_score(zhat, s["lo"], s["hi"]))[sure].all() and sure.mean() > 0.6
+    finally:
+        T.tardis_destroy(h)

@@ -34,7 +34,7 @@ constexpr int kMaxRecheck = 512;             // neurons per token that can queue
 struct State {
   __nv_bfloat16 *Wf, *W2, *What_hi, *What_lo;     // [d,d], [d,h], [h,d], [h,d]
   float* smaxrow;                                  // [h] largest group scale of a neuron
-  uint32_t* lo_used;                               // [h / 128 rounded up] 0 where What_lo is zero in those rows
+  uint32_t* lo_used;                               // [h / 128 rounded up] bit 0: What_lo is not zero in those rows; bit 1: some |q - zp| > 2
   float *zhat, *yacc, *x1;                         // [kChunkCapture,h] (scores for the capture; fold temporary), [kChunk,d], [kChunk]
   __nv_bfloat16* delta;                            // [kChunk,h]
   uint32_t* bitmap;                                // [kChunk,h/32]
@@ -50,7 +50,7 @@ __global__ void k_dequant_split(const uint32_t* __restrict__ codes, const __nv_b
                                 const uint8_t* __restrict__ zero, __nv_bfloat16* __restrict__ hi,
                                 __nv_bfloat16* __restrict__ lo, float* __restrict__ smaxrow, uint32_t* __restrict__ lo_used, int d, int G, int bits) {
   __shared__ float wmax[8];
-  bool rest = false;                            // any of this thread's values has a second term
+  uint32_t notes = 0u;                          // of this thread's values: 1 one has a second term, 2 one has |q - zp| > 2 (3 s may well be a bf16 value)
   float smax = 0.f;
   const int j = blockIdx.x, ng = d / G;
   const uint32_t* row = codes + size_t(j) * (size_t(d) * bits / 32);
@@ -64,9 +64,10 @@ __global__ void k_dequant_split(const uint32_t* __restrict__ codes, const __nv_b
       float v[2], t[2];
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
-        v[e] = s * (float(stream_code(row, k0 + 2 * q + e, bits)) - zp);   // exact: 8-bit significand times |int| <= 15
+        const float m = float(stream_code(row, k0 + 2 * q + e, bits)) - zp;
+        v[e] = s * m;                                                      // exact: 8-bit significand times |int| <= 15
         t[e] = __bfloat162float(__float2bfloat16_rn(v[e]));
-        rest |= v[e] != t[e];
+        notes |= (v[e] != t[e] ? 1u : 0u) | (fabsf(m) > 2.f ? 2u : 0u);
       }
       h[q] = __floats2bfloat162_rn(t[0], t[1]);
       l[q] = __floats2bfloat162_rn(v[0] - t[0], v[1] - t[1]);
@@ -74,7 +75,8 @@ __global__ void k_dequant_split(const uint32_t* __restrict__ codes, const __nv_b
     *reinterpret_cast<uint4*>(hi + size_t(j) * d + k0) = *reinterpret_cast<const uint4*>(h);
     *reinterpret_cast<uint4*>(lo + size_t(j) * d + k0) = *reinterpret_cast<const uint4*>(l);
   }
-  if (rest) lo_used[j >> 7] = 1u;
+  notes = __reduce_or_sync(0xffffffffu, notes);
+  if (notes && (threadIdx.x & 31) == 0) atomicOr(&lo_used[j >> 7], notes);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) smax = fmaxf(smax, __shfl_xor_sync(0xffffffffu, smax, o));
   if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = smax;
@@ -115,8 +117,8 @@ __global__ void k_xnorm(const __nv_bfloat16* __restrict__ x, int d, float* __res
 }
 
 // A CTA per token: the exact fp64 scores of its queued neurons (one warp each, from the packed codes) decide their flags; then the
-// token's flags are counted.  Where more neurons wanted to queue than fit, all are re-evaluated (4096 / 16384: 3 ms for such a token;
-// each settled by the thread that met it, in the product's epilogue: 18 to 46 ms).  The token is widened to fp64 once, in shared memory: with a conversion per product these, at 16 per
+// token's flags are counted.  Where more neurons wanted to queue than fit, all are re-evaluated (one such token among 200 of
+// 4096 / 16384: 9 ms; each settled by the thread that met it, in the product's epilogue: 19 ms).  The token is widened to fp64 once, in shared memory: with a conversion per product these, at 16 per
 // clock and SM, were the bound (2048 tokens on 4096 / 16384: 51 us, 93 before with the count as a kernel of its own).
 // WIDTH: bits per code where 32 is a multiple of it, else 0.  STAGED: false for tokens that do not fit in shared memory.
 template <int WIDTH, bool STAGED>

@@ -56,7 +56,7 @@ constexpr int NTHREADS = 320;           // warp 0 TMA, warp 1 MMA, warps 2..9 ep
 
 struct KParams {
   int M, N, kb1, kb2;          // k blocks (of 64) of the two operand pairs
-  const uint32_t* second_used; // per 128 rows n: 0 = the second pair adds nothing (null: it always counts)
+  const uint32_t* second_used; // per 128 rows n: bit 0 = the second pair adds something (null: it always counts), bit 1 = see fill_table
   int epilogue, ldo, act, splits;
   int fast_m, band;            // tile raster (see decode() in the kernel)
   float* out_f32; __nv_bfloat16* out_bf16;
@@ -212,8 +212,8 @@ __device__ __forceinline__ void fill_table(const KParams& p, float4* tab, int n0
       const float b = p.bias ? p.bias[n] : 0.f;
       if (p.epilogue == GEMM_EPI_DELTA) t = make_float4(b, p.a[n], p.c[n], 0.f);
       else {
-        // a term of a score is at most max |code - zero-point| times the scale times |x|: 2 instead of 3 where no second term exists
-        const float most = p.second_used && p.bits == 2 && p.second_used[n >> 7] == 0u ? 2.f / 3.f : 1.f;
+        // a term of a score is at most max |code - zero-point| times the scale times |x|: 2 instead of 3 where the fold has found no 3
+        const float most = p.second_used && p.bits == 2 && (p.second_used[n >> 7] & 2u) == 0u ? 2.f / 3.f : 1.f;
         t = make_float4(p.lo[n] - b, p.hi[n] - b, p.colscale[n] * most, b);
       }
     }
@@ -269,7 +269,7 @@ k_gemm(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtenso
     int nkb_all = p.kb1;
     if (p.kb2 > 0) {
       bool used = p.second_used == nullptr;
-      for (int r = n0; r < min(p.N, n0 + BN) && !used; r += 128) used = __ldg(p.second_used + (r >> 7)) != 0u;
+      for (int r = n0; r < min(p.N, n0 + BN) && !used; r += 128) used = (__ldg(p.second_used + (r >> 7)) & 1u) != 0u;
       if (used) nkb_all += p.kb2;
     }
     const int per = (nkb_all + p.splits - 1) / p.splits;   // k blocks per split of the channel range

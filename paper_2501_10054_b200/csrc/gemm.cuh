@@ -25,7 +25,8 @@ struct GemmArgs {
   int M, N, K1, K2;                 // K2 = 0: one operand pair only.  K1, K2 multiples of 8.
   const void *A1, *B1, *A2, *B2;    // device bf16; leading dimensions lda1 ... in elements (multiples of 8)
   int lda1, ldb1, lda2, ldb2;
-  const uint32_t* second_used;      // null, or one word per 128 rows n: 0 where B2 is zero throughout (its k blocks are then skipped)
+  const uint32_t* second_used;      // null, or one word per 128 rows n: bit 0 clear where B2 is zero throughout (its k blocks are then
+                                    // skipped), bit 1 clear where no |code - zero-point| is above 2 (GEMM_EPI_FLAGS, 2-bit codes)
   int epilogue;                     // GemmEpilogue
   int splits;                       // > 1 (GEMM_EPI_F32 only): the channel range is split over that many CTAs per tile, which
                                     // ADD their parts to out_f32 (the caller zeroes it first); the bias is added once

@@ -679,3 +679,26 @@ def test_more_scores_on_range_ends_than_are_queued(bits, n):
             assert (F == O.flags_from_score(zhat, s["lo"], s["hi"]))[sure].all() and sure.mean() > 0.6
     finally:
         T.tardis_destroy(h)
+
+
+@pytest.mark.parametrize("n", [20, 130])
+def test_allowance_of_scores_whose_values_of_three_scales_are_bf16_values(n):
+    # scales that are powers of two: 3 s needs no second bf16 term, and yet a term of a score may be 3 s |x|; range ends at 0.8 of the
+    # allowance 3 2^-17 max s |x|_1 from the scores of the call's (equal) tokens have to be re-evaluated
+    L = _layer(W.LayerConfig("pow2", 512, 2048, group=64, n_calib=128, bias=False), 4)
+    L.scale[:] = torch.exp2(torch.floor(torch.log2(L.scale.float()))).to(L.scale.dtype)
+    L.zero[:] = torch.where(torch.arange(8, device="cuda") % 2 == 0, 0, 3).to(torch.uint8)
+    s = L.numpy64()
+    x = W.make_tokens(L.cfg, 1, 4).cuda().expand(n, 512).contiguous()
+    z = O.predictor_score(x[:1].double().cpu().numpy(), s["codes"], s["scale"], s["zero"], s["group"], s["b1"], s["bits"])[0]
+    tau = 3 * 2.0 ** -17 * np.abs(s["scale"]).max(axis=1) * float(x[0].double().abs().sum())
+    L.lo.fill_(float("-inf"))
+    L.hi.fill_(float("inf"))
+    L.hi[:100] = torch.tensor((z + 0.8 * tau)[:100], dtype=torch.float32, device="cuda")
+    h = T.fold_layer(L)
+    try:
+        T.tardis_set_path(h, 3)
+        _, F, _ = Hp.gpu_forward(h, L, x)
+        assert not F.any() and T.tardis_stats(h)["exact_rechecks"] == 100 * n
+    finally:
+        T.tardis_destroy(h)

@@ -29,7 +29,9 @@ namespace bat {
 constexpr int kChunk = 2048;
 constexpr int kChunkCapture = 1024;          // ... while the debug capture is on (the score buffer holds that many)
 constexpr float kEps = 7.62939453125e-6f;    // 2^-17: relative accumulation-error allowance of the fast scores
-constexpr int kMaxRecheck = 512;             // neurons per token that can queue for re-evaluation
+// neurons per token that can queue for re-evaluation: a sixteenth, some ten times what narrow ranges of a 4096 / 16384 layer need (the
+// allowance grows with d, the spread of the scores with its root: a fixed number would be too small for the widest layers)
+__host__ __device__ constexpr int max_recheck(int h) { return h / 16 > 512 ? h / 16 : 512; }
 
 struct State {
   __nv_bfloat16 *Wf, *W2, *What_hi, *What_lo;     // [d,d], [d,h], [h,d], [h,d]
@@ -38,7 +40,7 @@ struct State {
   float *zhat, *yacc, *x1;                         // [kChunkCapture,h] (scores for the capture; fold temporary), [kChunk,d], [kChunk]
   __nv_bfloat16* delta;                            // [kChunk,h]
   uint32_t* bitmap;                                // [kChunk,h/32]
-  uint32_t* rlist;                                 // [kChunk][kMaxRecheck] neurons of a token to re-evaluate
+  uint32_t* rlist;                                 // [kChunk][max_recheck(h)] neurons of a token to re-evaluate
   unsigned int* rcount;                            // [kChunk] how many (more than the queue holds: every neuron is re-evaluated)
   size_t bytes_state, bytes_scratch;
 };
@@ -130,7 +132,8 @@ __global__ void __launch_bounds__(256) k_recheck(const uint32_t* __restrict__ rl
   __shared__ unsigned int flagged;
   const int t = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned int queued = rcount[t];
-  const bool all = queued > (unsigned int)kMaxRecheck;
+  const unsigned int most = max_recheck(h);
+  const bool all = queued > most;
   const unsigned int total = all ? (unsigned int)h : queued;
   const __nv_bfloat16* const xt = x + size_t(t) * d;
   const int nw = d / 16;
@@ -149,7 +152,7 @@ __global__ void __launch_bounds__(256) k_recheck(const uint32_t* __restrict__ rl
   __syncthreads();
   const int ng = d / G;
   for (unsigned int e = warp; e < total; e += 8) {
-    const int j = all ? int(e) : int(rlist[size_t(t) * kMaxRecheck + e]);
+    const int j = all ? int(e) : int(rlist[size_t(t) * most + e]);
     const uint32_t* const row = codes + size_t(j) * (size_t(d) * bits / 32);
     double z = 0.0;
     // units of 16 channels (all of one group), four at a time: their loads go out before the first is used, since waiting for them
@@ -272,7 +275,7 @@ tardis_status_t batched_prepare(Handle* H) {
       {reinterpret_cast<void**>(&S->zhat), size_t(kChunkCapture) * h * 4, true}, {reinterpret_cast<void**>(&S->yacc), size_t(kChunk) * d * 4, true},
       {reinterpret_cast<void**>(&S->x1), size_t(kChunk) * 4, true},       {reinterpret_cast<void**>(&S->delta), size_t(kChunk) * h * 2, true},
       {reinterpret_cast<void**>(&S->bitmap), size_t(kChunk) * (h / 32) * 4, true},
-      {reinterpret_cast<void**>(&S->rlist), size_t(kChunk) * kMaxRecheck * 4, true},
+      {reinterpret_cast<void**>(&S->rlist), size_t(kChunk) * max_recheck(h) * 4, true},
       {reinterpret_cast<void**>(&S->rcount), size_t(kChunk) * 4, true}};
   for (const Req& r : reqs) {
     cudaError_t e = dev_malloc(r.p, r.bytes);
@@ -405,7 +408,7 @@ tardis_status_t launch_batched_forward(Handle* H, const void* xv, void* yv, int6
     g.epilogue = GEMM_EPI_FLAGS; g.out_f32 = keep_scores ? S->zhat : nullptr; g.ldo = h; g.bias = H->b1;
     g.error_word = &H->counters[CTR_ERROR];
     g.lo = H->lo; g.hi = H->hi; g.colscale = S->smaxrow; g.rowscale = S->x1; g.keps = kEps * float((1 << H->bits) - 1);
-    g.bitmap_out = S->bitmap; g.rlist = S->rlist; g.rcount = S->rcount; g.rcap = kMaxRecheck;
+    g.bitmap_out = S->bitmap; g.rlist = S->rlist; g.rcount = S->rcount; g.rcap = max_recheck(h);
     g.bits = H->bits;
     tardis_status_t st = launch_gemm(g, s);
     if (st != TARDIS_OK) return st;

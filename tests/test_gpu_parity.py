@@ -702,3 +702,22 @@ def test_allowance_of_scores_whose_values_of_three_scales_are_bf16_values(n):
         assert not F.any() and T.tardis_stats(h)["exact_rechecks"] == 100 * n
     finally:
         T.tardis_destroy(h)
+
+
+def test_queue_for_re_evaluation_grows_with_the_layer():
+    # 800 of 16384 neurons with a range end on the score of the call's (equal) tokens: those are re-evaluated and no others
+    L = _layer(W.LayerConfig("queue", 64, 16384, group=64, n_calib=64), 2)
+    x = W.make_tokens(L.cfg, 1, 2).cuda().expand(130, 64).contiguous()
+    s = L.numpy64()
+    z = O.predictor_score(x[:1].double().cpu().numpy(), s["codes"], s["scale"], s["zero"], s["group"], s["b1"], s["bits"])[0]
+    L.lo.fill_(float("-inf"))
+    L.hi.fill_(float("inf"))
+    L.hi[::20] = torch.tensor(z[::20], dtype=torch.float32, device="cuda")
+    h = T.fold_layer(L)
+    try:
+        _, F, _ = Hp.gpu_forward(h, L, x)
+        hi = L.hi.double().cpu().numpy()
+        sure = np.abs(z - hi) > 1e-9 * np.abs(z)
+        assert (F == (z >= hi))[:, sure].all() and T.tardis_stats(h)["exact_rechecks"] == 820 * 130
+    finally:
+        T.tardis_destroy(h)

@@ -50,12 +50,16 @@ __device__ __forceinline__ void store8(__nv_bfloat16* p, const float (&v)[8]) {
   for (int i = 0; i < 4; ++i) o[i] = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
   *reinterpret_cast<uint4*>(p) = *reinterpret_cast<const uint4*>(o);
 }
-// v = residual ? v + f : f, rounded as it is stored
-template <typename T> __device__ __forceinline__ void add_output(float (&v)[8], const T* f, int residual) {
-  float w[8];
-  load8(w, f);
+// 8 consecutive values of a table of the caller's, which need not begin on a 16-byte boundary
+__device__ __forceinline__ void load_table(float (&v)[8], const float* p) {
+  if ((reinterpret_cast<uintptr_t>(p) & 15u) == 0) return load8(v, p);
 #pragma unroll
-  for (int i = 0; i < 8; ++i) v[i] = residual ? to_f32<T>(from_f32<T>(v[i] + w[i])) : w[i];
+  for (int q = 0; q < 8; ++q) v[q] = p[q];
+}
+// v = residual ? v + f : f, rounded as it is stored
+template <typename T> __device__ __forceinline__ void add_output(float (&v)[8], const float (&f)[8], int residual) {
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = residual ? to_f32<T>(from_f32<T>(v[i] + f[i])) : f[i];
 }
 
 // stream[t][:] = src[t][:] (the stream itself, or x for the first layer that needs it), with the previous layer's output f[t][:]
@@ -65,36 +69,43 @@ template <typename T> __device__ __forceinline__ void add_output(float (&v)[8], 
 // sums and one store (4096 elements, one token: 16 us with an element per load and 48 guarded steps for any d_model, 3 us now).
 template <typename T, int NV>
 __global__ void __launch_bounds__(LN_THREADS) k_update_norm(const T* src, T* stream, const T* __restrict__ f, int update, int residual,
-                                                            int normalise, T* __restrict__ out, const float* __restrict__ gamma,
-                                                            const float* __restrict__ beta, int d, float eps) {
+                                                            int normalise, T* __restrict__ out, const float* gamma, const float* beta, int d,
+                                                            float eps) {
   __shared__ float sh[LN_THREADS / 32];
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  float ga[NV][8], be[NV][8];
-#pragma unroll
-  for (int e = 0; e < NV; ++e) {                               // (the caller's constants: before the wait)
-    const int i = (threadIdx.x + e * LN_THREADS) * 8;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) { ga[e][q] = 1.f; be[e][q] = 0.f; }
-    if (normalise && i < d) {
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        if (gamma) ga[e][q] = gamma[i + q];
-        if (beta) be[e][q] = beta[i + q];
-      }
-    }
+  // gamma and beta may be written by a launch of the caller's that is still running: asked into L2 now, read behind the wait (read from
+  // memory behind it: 0.8 us more per layer)
+  for (int i = threadIdx.x * 32; i < d && normalise; i += LN_THREADS * 32) {
+    if (gamma) asm volatile("prefetch.global.L2 [%0];" ::"l"(gamma + i));
+    if (beta) asm volatile("prefetch.global.L2 [%0];" ::"l"(beta + i));
   }
   asm volatile("griddepcontrol.wait;" ::: "memory");          // the launch before wrote f (or the stream)
   const size_t row = size_t(blockIdx.x) * d;
-  float v[NV][8];
+  float v[NV][8], w[NV][8], ga[NV][8], be[NV][8];
+#pragma unroll
+  for (int e = 0; e < NV; ++e) {                               // (d is a multiple of 8)
+    const int i = (threadIdx.x + e * LN_THREADS) * 8;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) { v[e][q] = 0.f; ga[e][q] = 1.f; be[e][q] = 0.f; }
+    if (i < d) {
+      load8(v[e], src + row + i);
+      if (update) load8(w[e], f + row + i);
+    }
+  }
+#pragma unroll
+  for (int e = 0; e < NV; ++e) {                               // (behind the row's loads: these arrive while the row is summed up)
+    const int i = (threadIdx.x + e * LN_THREADS) * 8;
+    if (normalise && i < d) {
+      if (gamma) load_table(ga[e], gamma + i);
+      if (beta) load_table(be[e], beta + i);
+    }
+  }
   float s = 0.f;
 #pragma unroll
   for (int e = 0; e < NV; ++e) {
     const int i = (threadIdx.x + e * LN_THREADS) * 8;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) v[e][q] = 0.f;
-    if (i < d) {                                               // (d is a multiple of 8)
-      load8(v[e], src + row + i);
-      if (update) add_output<T>(v[e], f + row + i, residual);
+    if (i < d) {
+      if (update) add_output<T>(v[e], w[e], residual);
       if (update || src != stream) store8(stream + row + i, v[e]);
 #pragma unroll
       for (int q = 0; q < 8; ++q) s += v[e][q];
@@ -128,9 +139,10 @@ __global__ void __launch_bounds__(128) k_stream_update(const T* src, T* stream, 
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
   for (size_t i = (size_t(blockIdx.x) * blockDim.x + threadIdx.x) * 8; i < count; i += size_t(gridDim.x) * blockDim.x * 8) {
-    float v[8];
+    float v[8], w[8];
     load8(v, src + i);
-    add_output<T>(v, f + i, residual);
+    load8(w, f + i);
+    add_output<T>(v, w, residual);
     store8(stream + i, v);
   }
 }

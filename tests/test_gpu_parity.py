@@ -721,3 +721,62 @@ def test_queue_for_re_evaluation_grows_with_the_layer():
         assert (F == (z >= hi))[:, sure].all() and T.tardis_stats(h)["exact_rechecks"] == 820 * 130
     finally:
         T.tardis_destroy(h)
+
+
+LATE_WRITER = r"""
+#include <stddef.h>
+// lets the next launch of the stream start at once, writes dst = src only some time later (bounded)
+__global__ void k_late(float* dst, const float* src, size_t count, long long cycles) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const long long t0 = clock64();
+  while (clock64() - t0 < cycles) {}
+  for (size_t i = threadIdx.x; i < count; i += blockDim.x) dst[i] = src[i];
+}
+extern "C" int late_write(float* dst, const float* src, size_t count, long long cycles, void* stream) {
+  k_late<<<1, 256, 0, static_cast<cudaStream_t>(stream)>>>(dst, src, count, cycles);
+  return cudaGetLastError();
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def late_write(tmp_path_factory):
+    """late_write(dst, src, cycles): dst = src on the current stream, written by a kernel that has let the next launch start before."""
+    import subprocess
+    from paper_2501_10054_b200.build import nvcc_path
+    d = tmp_path_factory.mktemp("late")
+    (d / "late.cu").write_text(LATE_WRITER)
+    subprocess.run([nvcc_path(), "-gencode", "arch=compute_100a,code=sm_100a", "-O2", "-shared", "-Xcompiler", "-fPIC", "-o", str(d / "late.so"), str(d / "late.cu")],
+                   check=True)
+    fn = ctypes.CDLL(str(d / "late.so")).late_write
+    fn.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_size_t, ctypes.c_longlong, ctypes.c_void_p]
+
+    def call(dst, src, cycles):
+        n = src.numel() * src.element_size()
+        assert n % 4 == 0 and dst.numel() * dst.element_size() == n and 0 <= cycles <= 10 ** 9
+        assert fn(dst.data_ptr(), src.data_ptr(), n // 4, cycles, torch.cuda.current_stream().cuda_stream) == 0
+    return call
+
+
+def test_stack_reads_gamma_and_beta_behind_the_launch_that_writes_them(late_write):
+    cfg = W.LayerConfig("late", 512, 2048, n_calib=64)
+    L = _layer(cfg, 1)
+    x = W.make_tokens(cfg, 2, 1).cuda()
+    gam, bet = torch.linspace(0.5, 2, 512, device="cuda"), torch.linspace(-1, 1, 512, device="cuda")
+    g2, b2 = torch.zeros_like(gam), torch.zeros_like(bet)
+    keep, want = (torch.empty(2, 2, 2, 512, dtype=x.dtype, device="cuda") for _ in range(2))
+    y = torch.empty_like(x)
+    h = T.fold_layer(L)
+    try:
+        T.tardis_set_deterministic(h, True)
+        T.tardis_stack_forward([h, h], x, y, [gam, gam], [bet, bet], keep=want)
+        torch.cuda.synchronize()
+        for dst, src, ga, be in ((g2, gam, [g2, gam], [bet] * 2), (b2, bet, [gam] * 2, [b2, bet]), (g2, gam, [gam, g2], [bet] * 2), (b2, bet, [gam] * 2, [bet, b2])):
+            for cycles in (2000, 20000, 2000000):
+                dst.zero_()
+                late_write(dst, src, cycles)
+                T.tardis_stack_forward([h, h], x, y, ga, be, keep=keep)
+                torch.cuda.synchronize()
+                assert torch.equal(keep[:, 0], want[:, 0])
+    finally:
+        T.tardis_destroy(h)

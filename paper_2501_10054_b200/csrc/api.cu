@@ -6,8 +6,6 @@
 #include <new>
 
 #include <atomic>
-#include <chrono>
-#include <list>
 #include <mutex>
 #include <unordered_map>
 #include <vector>
@@ -38,78 +36,65 @@ static std::atomic<int> g_fail_alloc{-1};   // >= 0: that many allocations still
 // looks at the guards of the handle's allocations and reports TARDIS_ERR_CORRUPT when a kernel has written past an end.
 constexpr size_t kGuard = 256;
 constexpr int kGuardByte = 0xA5;
-struct Allocation { char* base; size_t bytes; const void* owner; int device; };
+// Allocations are carved out of blocks: an entry point asks for one that holds all it is going to need (dev_reserve), what does not fit
+// gets a block of its own, and a block goes back to the driver with the last allocation in it.  (A layer's 46 buffers one by one:
+// 7 ms of cudaMalloc and 7 ms of cudaFree for 4096 / 16384; 1 GB in one piece: 0.6 and 1.0 ms.)
+struct Block { char* base; size_t bytes, used; int live; };
+struct Allocation { char* base; size_t bytes; const void* owner; Block* block; };
 static std::mutex g_alloc_mutex;
 static std::unordered_map<const void*, Allocation> g_allocs;        // keyed by the pointer handed out
 static thread_local const void* g_alloc_owner = nullptr;            // the handle whose entry point is running on this thread
+static thread_local Block* g_block = nullptr;                       // ... and what is left of the block it has reserved
+
+static Block* new_block(size_t bytes, cudaError_t* e) {
+  Block* b = new (std::nothrow) Block{nullptr, bytes, 0, 0};
+  *e = b ? cudaMalloc(reinterpret_cast<void**>(&b->base), bytes) : cudaErrorMemoryAllocation;
+  if (*e == cudaSuccess) return b;
+  delete b;
+  return nullptr;
+}
+static void give_back(Block* b) {
+  cudaFree(b->base);
+  delete b;
+}
 struct OwnerScope {
   explicit OwnerScope(const void* o) { g_alloc_owner = o; }
-  ~OwnerScope() { g_alloc_owner = nullptr; }
+  ~OwnerScope() {
+    g_alloc_owner = nullptr;
+    Block* const b = g_block;
+    g_block = nullptr;
+    if (b && b->live == 0) give_back(b);                            // nothing was carved, or all of it is gone again
+  }
 };
 
-// Freed blocks wait here for the next allocation of exactly their size on their device: a layer's 46 buffers took 4 ms of
-// cudaMalloc and 3 ms of cudaFree (7 and 7 with the pages of a 4096 / 16384 layer), more than its fold on the GPU.  Whoever frees a
-// block has waited for the work that used it (tardis_destroy and the failure paths synchronise; tardis_build_predictor ends with
-// its stream), so any stream may take it next.  At most kPoolBytes wait per process; the oldest go back to the driver first, all of
-// them when an allocation fails, and those that have waited for kPoolSeconds whenever something is allocated or freed.
-constexpr size_t kPoolBytes = size_t(2) << 30;
-constexpr double kPoolSeconds = 10.0;
-struct Waiting { char* base; size_t bytes; int device; std::chrono::steady_clock::time_point since; };
-static std::list<Waiting> g_pool;                                   // oldest first; under g_alloc_mutex
-static size_t g_pool_bytes = 0;
+size_t dev_room(size_t bytes) { return (bytes + 255) / 256 * 256 + 2 * kGuard; }
 
-// Takes what has to go out of the pool (the caller gives it to the driver once the lock is gone).
-static void trim_pool(bool all, std::vector<char*>* out) {
-  const auto now = std::chrono::steady_clock::now();
-  while (!g_pool.empty() && (all || g_pool_bytes > kPoolBytes || std::chrono::duration<double>(now - g_pool.front().since).count() > kPoolSeconds)) {
-    out->push_back(g_pool.front().base);
-    g_pool_bytes -= g_pool.front().bytes;
-    g_pool.pop_front();
-  }
-}
-static void give_back(const std::vector<char*>& blocks) {
-  for (char* b : blocks) cudaFree(b);
+void dev_reserve(size_t bytes) {
+  cudaError_t e = cudaSuccess;
+  if (bytes && !g_block) g_block = new_block(bytes, &e);
+  if (e != cudaSuccess) cudaGetLastError();                         // (the allocations are then made one by one)
 }
 
 cudaError_t dev_malloc_raw(void** p, size_t bytes) {
   *p = nullptr;
   if (g_fail_alloc.load() >= 0 && g_fail_alloc.fetch_sub(1) == 0) return cudaErrorMemoryAllocation;
-  int dev = -1;
-  cudaGetDevice(&dev);
-  char* base = nullptr;
-  std::vector<char*> old;
-  {
-    std::lock_guard<std::mutex> lock(g_alloc_mutex);
-    for (auto it = g_pool.begin(); it != g_pool.end(); ++it)
-      if (it->bytes == bytes && it->device == dev) {
-        base = it->base;
-        g_pool_bytes -= bytes;
-        g_pool.erase(it);
-        break;
-      }
-    trim_pool(false, &old);
+  const size_t room = dev_room(bytes);
+  cudaError_t e = cudaSuccess;
+  Block* const b = g_block && g_block->bytes - g_block->used >= room ? g_block : new_block(room, &e);
+  if (!b) return e;
+  char* const base = b->base + b->used;
+  e = cudaMemset2D(base, kGuard + bytes, kGuardByte, kGuard, 2);    // both guards
+  if (e == cudaSuccess) {
+    try {
+      std::lock_guard<std::mutex> lock(g_alloc_mutex);
+      g_allocs[base + kGuard] = Allocation{base, bytes, g_alloc_owner, b};
+      b->used += room;
+      b->live += 1;
+    } catch (...) { e = cudaErrorMemoryAllocation; }
   }
-  give_back(old);
-  if (!base) {
-    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&base), bytes + 2 * kGuard);
-    if (e != cudaSuccess) {                                         // what waits in the pool may be what is missing
-      cudaGetLastError();
-      old.clear();
-      {
-        std::lock_guard<std::mutex> lock(g_alloc_mutex);
-        trim_pool(true, &old);
-      }
-      if (old.empty()) return e;
-      give_back(old);
-      e = cudaMalloc(reinterpret_cast<void**>(&base), bytes + 2 * kGuard);
-      if (e != cudaSuccess) return e;
-    }
-  }
-  const cudaError_t e = cudaMemset2D(base, kGuard + bytes, kGuardByte, kGuard, 2);   // both guards
-  if (e != cudaSuccess) { cudaFree(base); return e; }
-  {
-    std::lock_guard<std::mutex> lock(g_alloc_mutex);
-    g_allocs[base + kGuard] = Allocation{base, bytes, g_alloc_owner, dev};
+  if (e != cudaSuccess) {
+    if (b != g_block) give_back(b);
+    return e;
   }
   *p = base + kGuard;
   return cudaSuccess;
@@ -117,18 +102,16 @@ cudaError_t dev_malloc_raw(void** p, size_t bytes) {
 
 void dev_free(void* p) {
   if (!p) return;
-  std::vector<char*> old;
+  Block* b = nullptr;
   {
     std::lock_guard<std::mutex> lock(g_alloc_mutex);
     auto it = g_allocs.find(p);
-    if (it != g_allocs.end()) {
-      g_pool.push_back(Waiting{it->second.base, it->second.bytes, it->second.device, std::chrono::steady_clock::now()});
-      g_pool_bytes += it->second.bytes;
-      g_allocs.erase(it);
-    }
-    trim_pool(false, &old);
+    if (it == g_allocs.end()) return;
+    b = it->second.block;
+    g_allocs.erase(it);
+    if (--b->live > 0) return;
   }
-  give_back(old);
+  if (b != g_block) give_back(b);                                   // (a block still being carved goes with its entry point)
 }
 
 // Number of damaged guards among the allocations of `owner` (both guards of every allocation are read back); -1 on a CUDA error.
@@ -156,17 +139,14 @@ static bool on_handle_device(const Handle* H) {
   return cudaGetDevice(&cur) == cudaSuccess && cur == H->device;
 }
 
-template <typename T>
-static tardis_status_t dev_alloc(T** p, size_t count, size_t* tally) {
-  *p = nullptr;
-  size_t bytes = count * sizeof(T);
-  cudaError_t e = dev_malloc(reinterpret_cast<void**>(p), bytes ? bytes : 16);
+static tardis_status_t dev_alloc(void** p, size_t bytes, size_t* tally) {
+  const cudaError_t e = dev_malloc_raw(p, bytes ? bytes : 16);
   if (e != cudaSuccess) {
     set_last_error(e, "cudaMalloc");
     cudaGetLastError();
     return TARDIS_ERR_ALLOC;
   }
-  if (tally) *tally += bytes;
+  *tally += bytes;
   return TARDIS_OK;
 }
 
@@ -200,23 +180,22 @@ static tardis_status_t new_handle(int d, int h, int dtype, int act, int G, int b
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&H->num_sms, cudaDevAttrMultiProcessorCount, H->device);
   if (e != cudaSuccess) { set_last_error(e, "device query"); delete H; return TARDIS_ERR_CUDA; }
   const size_t hd = size_t(h) * d;
+  struct Req { void** p; size_t bytes; size_t* tally; };
+  auto V = [](auto** p) { return reinterpret_cast<void**>(p); };
+  const Req reqs[] = {{V(&H->W1), hd * H->esize, &H->bytes_w1}, {V(&H->W2T), hd * H->esize, &H->bytes_w2t},
+                      {V(&H->C), size_t(d) * d * H->esize, &H->bytes_folded}, {V(&H->bf), size_t(d) * 4, &H->bytes_folded},
+                      {V(&H->lo), size_t(h) * 4, &H->bytes_tables}, {V(&H->hi), size_t(h) * 4, &H->bytes_tables},
+                      {V(&H->a), size_t(h) * 4, &H->bytes_tables}, {V(&H->c), size_t(h) * 4, &H->bytes_tables},
+                      {V(&H->b1), size_t(h) * 4, &H->bytes_tables}, {V(&H->codes), hd * H->bits / 32 * 4, &H->bytes_predictor},
+                      {V(&H->scale), size_t(h) * H->ngroups * H->esize, &H->bytes_predictor}, {V(&H->zero), size_t(h) * H->ngroups, &H->bytes_predictor},
+                      {V(&H->yacc), size_t(kGenericChunk) * d * 4, &H->bytes_scratch}, {V(&H->bitmap), size_t(kGenericChunk) * (h / 32) * 4, &H->bytes_scratch},
+                      {V(&H->counters), size_t(CTR_COUNT) * 8, &H->bytes_scratch}};
+  size_t room = batched_room(H) + fused_room(H) + f32_room(H);
+  for (const Req& r : reqs) room += dev_room(r.bytes);
+  dev_reserve(room);
   tardis_status_t st = TARDIS_OK;
-  auto A = [&](auto** p, size_t count, size_t* tally) { if (st == TARDIS_OK) st = dev_alloc(p, count, tally); };
-  A(reinterpret_cast<char**>(&H->W1), hd * H->esize, &H->bytes_w1);
-  A(reinterpret_cast<char**>(&H->W2T), hd * H->esize, &H->bytes_w2t);
-  A(reinterpret_cast<char**>(&H->C), size_t(d) * d * H->esize, &H->bytes_folded);
-  A(&H->bf, size_t(d), &H->bytes_folded);
-  A(&H->lo, size_t(h), &H->bytes_tables);
-  A(&H->hi, size_t(h), &H->bytes_tables);
-  A(&H->a, size_t(h), &H->bytes_tables);
-  A(&H->c, size_t(h), &H->bytes_tables);
-  A(&H->b1, size_t(h), &H->bytes_tables);
-  A(&H->codes, hd * H->bits / 32, &H->bytes_predictor);
-  A(reinterpret_cast<char**>(&H->scale), size_t(h) * H->ngroups * H->esize, &H->bytes_predictor);
-  A(&H->zero, size_t(h) * H->ngroups, &H->bytes_predictor);
-  A(&H->yacc, size_t(kGenericChunk) * d, &H->bytes_scratch);
-  A(&H->bitmap, size_t(kGenericChunk) * (h / 32), &H->bytes_scratch);
-  A(&H->counters, size_t(CTR_COUNT), &H->bytes_scratch);
+  for (const Req& r : reqs)
+    if (st == TARDIS_OK) st = dev_alloc(r.p, r.bytes, r.tally);
   if (st != TARDIS_OK) { free_all(H); return st; }
   *out = H;
   return TARDIS_OK;
@@ -589,6 +568,7 @@ tardis_status_t tardis_build_predictor(int32_t d_ff, int32_t d_model, tardis_dty
   if (d_ff < 1 || d_model < 1 || !W1 || !codes || !scale || !zero) return TARDIS_ERR_INVALID_ARG;
   if (!(dtype == TARDIS_F32 || dtype == TARDIS_BF16) || !(bits == 2 || bits == 3 || bits == 4 || bits == 8)) return TARDIS_ERR_INVALID_ARG;
   if (group < 64 || group % 64 || d_model % group) return TARDIS_ERR_INVALID_ARG;
+  OwnerScope scope(nullptr);
   return launch_build_predictor(d_ff, d_model, dtype, W1, U, bits, group, codes, scale, zero, reinterpret_cast<cudaStream_t>(stream));
 }
 
@@ -639,8 +619,12 @@ tardis_status_t tardis_set_path(tardis_handle_t handle, int32_t path) {
 tardis_status_t tardis_destroy(tardis_handle_t handle) {
   Handle* H = check(handle);
   if (!H) return TARDIS_ERR_INVALID_ARG;
+  int cur = -1;                                        // the handle's work and memory are on its own device
+  const bool other = cudaGetDevice(&cur) == cudaSuccess && cur != H->device;
+  if (other) cudaSetDevice(H->device);
   cudaError_t e = cudaDeviceSynchronize();
   free_all(H);
+  if (other) cudaSetDevice(cur);
   if (e != cudaSuccess) { set_last_error(e, "cudaDeviceSynchronize"); return TARDIS_ERR_CUDA; }
   return TARDIS_OK;
 }

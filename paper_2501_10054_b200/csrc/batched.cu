@@ -257,18 +257,12 @@ template <typename T> __global__ void k_transpose_b(const T* __restrict__ in, T*
   }
 }
 
-tardis_status_t batched_prepare(Handle* H) {
-  H->bstate = nullptr;
-  if (H->dtype != TARDIS_BF16) return TARDIS_OK;
-  const int d = H->d, h = H->h;
-  if (d % 8 || h % 32) return TARDIS_OK;
-  State* S = new (std::nothrow) State();
-  if (!S) return TARDIS_ERR_ALLOC;
-  memset(S, 0, sizeof(*S));
-  H->bstate = S;
+namespace {
+struct Req { void** p; size_t bytes; bool scratch; };
+struct Requests { Req r[13]; };
+Requests requests(State* S, int d, int h) {
   const size_t hd = size_t(h) * d;
-  struct Req { void** p; size_t bytes; bool scratch; };
-  Req reqs[] = {
+  const Requests all = {{
       {reinterpret_cast<void**>(&S->Wf), size_t(d) * d * 2, false}, {reinterpret_cast<void**>(&S->W2), hd * 2, false},
       {reinterpret_cast<void**>(&S->What_hi), hd * 2, false},       {reinterpret_cast<void**>(&S->What_lo), hd * 2, false},
       {reinterpret_cast<void**>(&S->smaxrow), size_t(h) * 4, false}, {reinterpret_cast<void**>(&S->lo_used), size_t((h + 127) / 128) * 4, false},
@@ -276,8 +270,30 @@ tardis_status_t batched_prepare(Handle* H) {
       {reinterpret_cast<void**>(&S->x1), size_t(kChunk) * 4, true},       {reinterpret_cast<void**>(&S->delta), size_t(kChunk) * h * 2, true},
       {reinterpret_cast<void**>(&S->bitmap), size_t(kChunk) * (h / 32) * 4, true},
       {reinterpret_cast<void**>(&S->rlist), size_t(kChunk) * max_recheck(h) * 4, true},
-      {reinterpret_cast<void**>(&S->rcount), size_t(kChunk) * 4, true}};
-  for (const Req& r : reqs) {
+      {reinterpret_cast<void**>(&S->rcount), size_t(kChunk) * 4, true}}};
+  return all;
+}
+bool served(const Handle* H) { return H->dtype == TARDIS_BF16 && H->d % 8 == 0 && H->h % 32 == 0; }
+}  // namespace
+
+size_t batched_room(const Handle* H) {
+  if (!served(H)) return 0;
+  State S = {};
+  size_t room = few_room(H);
+  for (const Req& r : requests(&S, H->d, H->h).r) room += dev_room(r.bytes);
+  return room;
+}
+
+tardis_status_t batched_prepare(Handle* H) {
+  H->bstate = nullptr;
+  const int d = H->d, h = H->h;
+  if (!served(H)) return TARDIS_OK;
+  State* S = new (std::nothrow) State();
+  if (!S) return TARDIS_ERR_ALLOC;
+  memset(S, 0, sizeof(*S));
+  H->bstate = S;
+  const size_t hd = size_t(h) * d;
+  for (const Req& r : requests(S, d, h).r) {
     cudaError_t e = dev_malloc(r.p, r.bytes);
     if (e != cudaSuccess) { set_last_error(e, "cudaMalloc"); cudaGetLastError(); batched_release(H); return TARDIS_ERR_ALLOC; }
     (r.scratch ? S->bytes_scratch : S->bytes_state) += r.bytes;

@@ -66,6 +66,8 @@ void set_last_error(cudaError_t e, const char* where);
 cudaError_t dev_malloc_raw(void** p, size_t bytes);
 template <typename T> inline cudaError_t dev_malloc(T** p, size_t bytes) { return dev_malloc_raw(reinterpret_cast<void**>(p), bytes); }
 void dev_free(void* p);   // what dev_malloc gave (null is fine)
+size_t dev_room(size_t bytes);      // what an allocation takes of a block, guards included
+void dev_reserve(size_t bytes);     // one block for the allocations that the running entry point is going to make (the sum of their dev_room)
 
 #define TARDIS_CUDA_TRY(expr)                                  \
   do {                                                         \
@@ -86,20 +88,24 @@ tardis_status_t decode_prepare(Handle* H, cudaStream_t s);                 // bu
 tardis_status_t launch_decode_forward(Handle* H, const void* x, void* y, int n, cudaStream_t s);
 void decode_release(Handle* H);
 tardis_status_t decode_read_stamps(long long* out, int max_ctas);
+size_t fused_room(const Handle* H);                                        // what fused_prepare or decode_prepare will allocate
 tardis_status_t fused_prepare(Handle* H, cudaStream_t s);                  // builds the state of fused.cu (bf16, d_model <= 4608)
 tardis_status_t launch_fused_forward(Handle* H, const void* x, void* y, int n, cudaStream_t s);
 void fused_release(Handle* H);
 tardis_status_t fused_set_deterministic(Handle* H, bool on);               // allocates the partial-output buffer of the mode
 tardis_status_t fused_read_stamps(long long* out, int max_ctas);
 tardis_status_t launch_wait_that_runs_out(Handle* H, long long limit_cycles, cudaStream_t s);   // UNSUPPORTED unless built with TARDIS_PHASE_STAMPS
+size_t batched_room(const Handle* H);                                                         // what batched_prepare (and few_prepare) will allocate
 tardis_status_t batched_prepare(Handle* H);                                                   // bf16 only: allocations
 tardis_status_t batched_finish(Handle* H, const void* W2, cudaStream_t s);   // fills the batched state (W2 null: from W2T)
 tardis_status_t launch_batched_forward(Handle* H, const void* x, void* y, int64_t n, cudaStream_t s);
 void batched_release(Handle* H);
+size_t few_room(const Handle* H);
 tardis_status_t few_prepare(Handle* H);                                       // few.cu: allocations
 tardis_status_t few_finish(Handle* H, const void* W2, const void* Wf, cudaStream_t s);   // fills its state (W2 [d, h], W_f [d, d] row-major)
 tardis_status_t launch_few_forward(Handle* H, const void* x, void* y, int n, const float* smaxrow, cudaStream_t s);
 void few_release(Handle* H);
+size_t f32_room(const Handle* H);
 tardis_status_t f32_prepare(Handle* H, cudaStream_t s);                        // f32.cu (fp32 layers only)
 tardis_status_t launch_f32_forward(Handle* H, const void* x, void* y, int64_t n, cudaStream_t s);
 void f32_release(Handle* H);

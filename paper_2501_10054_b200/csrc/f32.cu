@@ -313,6 +313,19 @@ template <int TT> static Kernel in_kernel(int bits) {
 
 using namespace f32;
 
+namespace {
+// words per handle: finished parts per output tile, flagged neurons per token
+size_t done_words(const Handle* H) { return size_t((H->d + TM - 1) / TM) * (MAX_CHUNK / 8); }
+struct Sizes { size_t bytes[3]; };                         // delta, part, words
+Sizes sizes(const Handle* H) { return {{size_t(MAX_CHUNK) * H->h * 4, size_t(MAX_PARTS) * H->d * 8, (done_words(H) + MAX_CHUNK) * 4}}; }
+}  // namespace
+
+size_t f32_room(const Handle* H) {
+  size_t room = 0;
+  for (size_t b : sizes(H).bytes) room += dev_room(b);
+  return H->dtype == TARDIS_F32 ? room : 0;
+}
+
 tardis_status_t f32_prepare(Handle* H, cudaStream_t s) {
   H->f32 = nullptr;
   if (H->dtype != TARDIS_F32) return TARDIS_OK;
@@ -320,8 +333,9 @@ tardis_status_t f32_prepare(Handle* H, cudaStream_t s) {
   if (!S) return TARDIS_ERR_ALLOC;
   memset(S, 0, sizeof(*S));
   H->f32 = S;
-  S->ndone = size_t((H->d + TM - 1) / TM) * (MAX_CHUNK / 8);
-  const size_t bytes[3] = {size_t(MAX_CHUNK) * H->h * 4, size_t(MAX_PARTS) * H->d * 8, (S->ndone + MAX_CHUNK) * 4};
+  S->ndone = done_words(H);
+  const Sizes sz = sizes(H);
+  const size_t (&bytes)[3] = sz.bytes;
   void** ptrs[3] = {reinterpret_cast<void**>(&S->delta), reinterpret_cast<void**>(&S->part), reinterpret_cast<void**>(&S->words)};
   for (int i = 0; i < 3; ++i) {
     const cudaError_t e = dev_malloc(ptrs[i], bytes[i]);

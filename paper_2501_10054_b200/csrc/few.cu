@@ -21,7 +21,6 @@
 
 #include <algorithm>
 #include <new>
-#include <vector>
 
 #include "common.cuh"
 #include "tc.cuh"
@@ -797,10 +796,10 @@ struct State {
 // Shares of the folded product's blocks: a neuron tile's block costs its rows' share of a 128-row one plus a seventh (codes);
 // every CTA is filled up to the same total, and pieces of fewer than 8 blocks are not dealt (a piece costs one pass over a
 // 128-row accumulator at its end).
-static void deal_folded_blocks(const State& S, std::vector<int2>& plan) {
+static void deal_folded_blocks(const State& S, Shares& plan) {
   const double per_tile = 1.15 * S.rows / BM * S.nkb;
   const int blocks = S.mtiles * S.nkb;
-  std::vector<double> room(S.grid);
+  double room[MAX_GRID];
   auto fill = [&](double level) {
     double sum = 0.0;
     for (int c = 0; c < S.grid; ++c) {
@@ -814,12 +813,9 @@ static void deal_folded_blocks(const State& S, std::vector<int2>& plan) {
   while (hi - lo > 1e-3) { const double mid = 0.5 * (lo + hi); (fill(mid) >= blocks ? hi : lo) = mid; }   // the level that holds all blocks
   const double sum = fill(hi);
   double cum = 0.0;
-  int at = 0;
   for (int c = 0; c < S.grid; ++c) {
     cum += room[c];
-    const int to = c == S.grid - 1 ? blocks : std::min(blocks, int(cum / sum * blocks + 0.5));
-    plan[c] = make_int2(at, to);
-    at = to;
+    plan.end[c] = c == S.grid - 1 ? blocks : std::min(blocks, int(cum / sum * blocks + 0.5));
   }
 }
 
@@ -827,25 +823,46 @@ static void deal_folded_blocks(const State& S, std::vector<int2>& plan) {
 
 using namespace few;
 
+namespace {
 // Serves bf16 layers with 2-bit or 4-bit codes in groups of a multiple of 64 channels (every channel block lies in one group).
+bool served(const Handle* H) { return H->dtype == TARDIS_BF16 && (H->bits == 2 || H->bits == 4) && H->G % BK == 0 && tensor_maps_available(); }
+
+State shape(const Handle* H) {
+  State S = {};
+  const int d = H->d, h = H->h;
+  S.grid = std::min(H->num_sms, MAX_GRID);
+  const int rounds = (h + S.grid * BM - 1) / (S.grid * BM), share = (h + S.grid * rounds - 1) / (S.grid * rounds);
+  S.rows = std::min(BM, std::max(16, (share + 7) / 8 * 8));           // every CTA gets the same number of tiles, or one less
+  S.nkb = d / BK; S.ntiles = (h + S.rows - 1) / S.rows; S.mtiles = (d + BM - 1) / BM; S.out_nkb = (h + BK - 1) / BK;
+  return S;
+}
+struct Req { void** p; size_t bytes; };
+struct Requests { Req r[6]; };                             // codes and meta, then scratch
+Requests requests(const Handle* H, State* S) {
+  return {{{reinterpret_cast<void**>(&S->codes), size_t(S->ntiles) * S->nkb * S->rows * 8 * H->bits},
+           {reinterpret_cast<void**>(&S->meta), size_t(S->ntiles) * (H->d / H->G) * S->rows * 4},
+           {reinterpret_cast<void**>(&S->plan), sizeof(int2) * S->grid}, {reinterpret_cast<void**>(&S->yacc), sizeof(float) * MAX_TOKENS * H->d},
+           {reinterpret_cast<void**>(&S->nfl), sizeof(unsigned int) * (MAX_TOKENS + 2 * S->mtiles + S->ntiles)},
+           {reinterpret_cast<void**>(&S->delta), size_t(2) * MAX_TOKENS * H->h}}};
+}
+}  // namespace
+
+size_t few_room(const Handle* H) {
+  if (!served(H)) return 0;
+  State S = shape(H);
+  size_t room = 0;
+  for (const Req& r : requests(H, &S).r) room += dev_room(r.bytes);
+  return room;
+}
+
 tardis_status_t few_prepare(Handle* H) {
   H->few = nullptr;
-  const int d = H->d, h = H->h, G = H->G;
-  if (H->dtype != TARDIS_BF16 || (H->bits != 2 && H->bits != 4) || G % BK || !tensor_maps_available()) return TARDIS_OK;
-  State* S = new (std::nothrow) State();
+  if (!served(H)) return TARDIS_OK;
+  State* S = new (std::nothrow) State(shape(H));
   if (!S) return TARDIS_ERR_ALLOC;
-  memset(S, 0, sizeof(*S));
   H->few = S;
-  S->grid = std::min(H->num_sms, MAX_GRID);
-  const int rounds = (h + S->grid * BM - 1) / (S->grid * BM), share = (h + S->grid * rounds - 1) / (S->grid * rounds);
-  S->rows = std::min(BM, std::max(16, (share + 7) / 8 * 8));          // every CTA gets the same number of tiles, or one less
-  S->nkb = d / BK; S->ntiles = (h + S->rows - 1) / S->rows; S->mtiles = (d + BM - 1) / BM; S->out_nkb = (h + BK - 1) / BK;
-  const size_t code_bytes = size_t(S->ntiles) * S->nkb * S->rows * 8 * H->bits, meta_bytes = size_t(S->ntiles) * (d / G) * S->rows * 4;
-  struct Req { void** p; size_t bytes; };
-  Req reqs[] = {{reinterpret_cast<void**>(&S->codes), code_bytes}, {reinterpret_cast<void**>(&S->meta), meta_bytes},
-                {reinterpret_cast<void**>(&S->plan), sizeof(int2) * S->grid}, {reinterpret_cast<void**>(&S->yacc), sizeof(float) * MAX_TOKENS * d},
-                {reinterpret_cast<void**>(&S->nfl), sizeof(unsigned int) * (MAX_TOKENS + 2 * S->mtiles + S->ntiles)},
-                {reinterpret_cast<void**>(&S->delta), size_t(2) * MAX_TOKENS * h}};
+  const Requests all = requests(H, S);
+  const Req (&reqs)[6] = all.r;
   for (const Req& r : reqs) {
     const cudaError_t e = dev_malloc(r.p, r.bytes);
     if (e != cudaSuccess) { set_last_error(e, "cudaMalloc"); cudaGetLastError(); few_release(H); return TARDIS_ERR_ALLOC; }
@@ -864,7 +881,7 @@ tardis_status_t few_prepare(Handle* H) {
   S->done = S->nfl + MAX_TOKENS;
   S->parts = S->done + S->mtiles;
   S->two_terms = S->parts + S->mtiles;
-  H->bytes_predictor += code_bytes + meta_bytes;
+  H->bytes_predictor += reqs[0].bytes + reqs[1].bytes;
   for (int i = 2; i < 6; ++i) H->bytes_scratch += reqs[i].bytes;
   return TARDIS_OK;
 }
@@ -877,12 +894,10 @@ tardis_status_t few_finish(Handle* H, const void* W2, const void* Wf, cudaStream
     few_release(H);                                    // (not served: the other kernels take these calls)
     return TARDIS_OK;
   }
-  std::vector<int2> plan(S->grid);
-  deal_folded_blocks(*S, plan);
+  Shares shares;
+  deal_folded_blocks(*S, shares);
   S->out_grid = std::max(1, std::min(S->grid, S->mtiles * S->out_nkb / 4));
   TARDIS_CUDA_TRY(cudaMemsetAsync(S->nfl, 0, sizeof(unsigned int) * (MAX_TOKENS + 2 * S->mtiles + S->ntiles), s));
-  Shares shares;
-  for (int c = 0; c < S->grid; ++c) shares.end[c] = plan[c].y;
   k_plan<<<1, 256, 0, s>>>(shares, S->plan, S->grid, S->parts, S->mtiles, S->out_nkb, S->out_grid);
   TARDIS_CUDA_TRY(cudaMemsetAsync(S->yacc, 0, sizeof(float) * MAX_TOKENS * d, s));
   auto pack = H->bits == 2 ? k_pack<2> : k_pack<4>;

@@ -1144,6 +1144,14 @@ __global__ void k_max_scale(const __nv_bfloat16* __restrict__ scale, size_t coun
 
 using namespace fz;
 
+// The predictor's blocks, the folded matrix and the small arrays of this path or, for wider layers, of k_decode.
+size_t fused_room(const Handle* H) {
+  if (H->dtype != TARDIS_BF16 || H->bits != 2 || !(H->G == 64 || H->G == 128)) return 0;
+  const size_t nkc = (H->d + KC - 1) / KC, dacc = (H->d + 31) / 32 * 32;
+  return dev_room(size_t(H->h / 16) * nkc * (1024 + 64 * (KC / H->G))) + dev_room(size_t(H->d / 16) * nkc * 8192) + dev_room(size_t(H->num_sms) * 2 * sizeof(int2)) +
+         dev_room(16) + dev_room(sizeof(float) * MAXT * dacc) + dev_room(8192) + dev_room(sizeof(int) * H->h);
+}
+
 // Builds the state of this path for bf16 layers with 2-bit codes, group size 64 or 128 and d_model a multiple of 16
 // up to 4608; other layers are left to the other kernels (H->fscratch stays null).
 tardis_status_t fused_prepare(Handle* H, cudaStream_t s) {

@@ -218,6 +218,7 @@ tardis_status_t launch_build_predictor(int h, int d, int dtype, const void* W1, 
   auto release = [&]() {
     dev_free(Wd); dev_free(Eb); dev_free(scale64); dev_free(zero64); dev_free(q);
   };
+  dev_reserve(dev_room(size_t(h) * d * 8) + dev_room(size_t(h) * sb * 8) + 2 * dev_room(size_t(h) * ng * 8) + dev_room(size_t(h) * d));
   cudaError_t e = dev_malloc(&Wd, size_t(h) * d * sizeof(double));
   if (e == cudaSuccess) e = dev_malloc(&Eb, size_t(h) * sb * sizeof(double));
   if (e == cudaSuccess) e = dev_malloc(&scale64, size_t(h) * ng * sizeof(double));
@@ -245,7 +246,8 @@ tardis_status_t launch_build_predictor(int h, int d, int dtype, const void* W1, 
     else k_pack_out<__nv_bfloat16><<<1024, 256, 0, s>>>(q, scale64, zero64, h, d, G, bits, codes, static_cast<__nv_bfloat16*>(scale), zero);
     e = cudaGetLastError();
   }
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);      // the scratch goes away with this call
+  const cudaError_t es = cudaStreamSynchronize(s);         // the scratch goes away with this call, whatever has been launched
+  if (e == cudaSuccess) e = es;
   release();
   if (e != cudaSuccess) { set_last_error(e, "tardis_build_predictor"); return TARDIS_ERR_CUDA; }
   return TARDIS_OK;

@@ -780,3 +780,27 @@ def test_stack_reads_gamma_and_beta_behind_the_launch_that_writes_them(late_writ
                 assert torch.equal(keep[:, 0], want[:, 0])
     finally:
         T.tardis_destroy(h)
+
+
+@pytest.mark.parametrize("dtype,bits,d,h", [("bf16", 2, 1024, 8192), ("bf16", 4, 1024, 8192), ("bf16", 2, 4736, 2048), ("f32", 2, 1024, 8192)])
+def test_destroy_and_the_builder_give_device_memory_back(dtype, bits, d, h):
+    # a small layer first, so that kernels are loaded; then what a layer (over 100 MB) and the builder's scratch (8 d h bytes) take has
+    # to be free again when the calls return
+    for dd, hh in ((512, 2048), (d, h)):
+        L = _layer(W.LayerConfig("back", dd, hh, dtype=dtype, bits=bits, group=64, n_calib=64))
+        x = W.make_tokens(L.cfg, 150, 1).cuda()
+        y = torch.empty_like(x)
+        T.tardis_build_predictor(L.W1, None, bits, 64)
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        T.tardis_build_predictor(L.W1, None, bits, 64)
+        hd = T.fold_layer(L)
+        for n in (1, 4, 40, 150):
+            T.tardis_ffn_forward(hd, x[:n], y[:n])
+        torch.cuda.synchronize()
+        taken = free - torch.cuda.mem_get_info()[0]
+        st = T.tardis_stats(hd)
+        T.tardis_destroy(hd)
+        left = free - torch.cuda.mem_get_info()[0]
+    held = sum(v for k, v in st.items() if k.startswith("bytes_"))
+    assert taken >= 50 << 20 and held <= taken <= held + (8 << 20) and left <= 2 << 20, (taken, held, left)

@@ -270,6 +270,8 @@ k_few_in(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUten
     tc_fence_after();
   }
   const uint32_t tmem = *tmem_slot;
+  // The waits below are bounded, so none of them may begin before the launch before this one has ended: it may take any time.
+  InFlight flight;
 
   if (warp == 0) {
     // ---------------- TMA: W1 tiles, then the folded matrix's blocks; the tokens beside each ----------------
@@ -283,9 +285,11 @@ k_few_in(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUten
     pdl_wait();
     for (int s = 0; s < ahead; ++s, first.next())
       if (elect_one()) tokens(first, s);
+    flight.begin(ahead);
     for (int i = ahead, s = 0, parity = 0; i < w.total; ++i, w.next()) {
       const bool ok = mbar_wait_issue(&empty[s], parity, failed);
       if (elect_one() && ok) { mbar_expect_tx(&full[s], bytes(w)); weights(w, s); tokens(w, s); }
+      if (ok) flight.issued(s, parity ^ 1);
       if (++s == C::NS) { s = 0; parity ^= 1; }
     }
   } else if (warp == 1) {
@@ -294,6 +298,7 @@ k_few_in(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUten
     const uint64_t wdesc = smem_desc_k_major_sw128(smem_u32(smem)), xdesc = smem_desc_k_major_sw128(smem_u32(smem) + W_BYTES);
     int s = 0, parity = 0, ati = 0, own0 = 0, own1 = 0;    // stage and its phase; tiles; expanded blocks used of either group
     auto next_stage = [&]() { if (++s == C::NS) { s = 0; parity ^= 1; } };
+    pdl_wait();
     for (int tile = blockIdx.x; tile < p.ntiles; tile += gridDim.x, ++ati) {
       const int terms = BITS > 2 || p.two_terms[tile] ? 2 : 1;
       bool ok = mbar_wait_issue(acc_free, (ati & 1) ^ 1, failed);
@@ -348,6 +353,7 @@ k_few_in(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUten
     constexpr int LPT = N >= 64 ? 1 : 64 / N, TPL = N > 64 ? N / 64 : 1, PIECES = 8 / LPT;
     float sum[TPL][4] = {};
     const int me = (warp - 2) * 32 + lane;
+    pdl_wait();
     for (int i = 0, s = 0, parity = 0; i < total; ++i) {
       if (!mbar_wait_warp(&full[s], parity)) { *failed = 1u; break; }
       if (any_tile && i < nkb) {
@@ -431,6 +437,7 @@ k_few_in(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUten
               else expand<1>(code[u][0], meta[u], w);
               if (term == terms - 1 && i + AHEAD < mine) fetch(gi + 2 * (i + AHEAD), code[u], meta[u]);
               const int b = gi + 2 * (own % RING);
+              if (own == RING) pdl_wait();                 // (the first RING blocks find their places free)
               ok = mbar_wait_warp(&a_empty[b], ((own / RING) & 1) ^ 1);
               if (!ok) { *failed = 1u; break; }
               tc_fence_after();
@@ -581,6 +588,7 @@ k_few_in(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUten
   tc_fence_before();
   __syncthreads();
   if (threadIdx.x == 0 && *failed) atomicExch(&p.counters[CTR_ERROR], 1ull);
+  if (warp == 0 && *failed) flight.land(full);
   if (warp == 1) tmem_dealloc(tmem, C::TMEM);
 }
 
@@ -602,6 +610,7 @@ k_few_out(const __grid_constant__ CUtensorMap tmW2, const __grid_constant__ CUte
   const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // (warp: uniform, and known to be)
   auto begin_of = [&](int c) { return int((long long)p.total * c / int(gridDim.x)); };
   const int begin = begin_of(blockIdx.x), end = begin_of(blockIdx.x + 1), nkb = p.nkb;
+  InFlight flight;
   pdl_launch();
   if (threadIdx.x == 0) {
     for (int s = 0; s < C::NS; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
@@ -624,9 +633,11 @@ k_few_out(const __grid_constant__ CUtensorMap tmW2, const __grid_constant__ CUte
     pdl_wait();
     for (int s = 0; s < ahead; ++s, next_corrections())
       if (elect_one()) corrections(s);
+    flight.begin(ahead);
     for (int i = ahead, s = 0, parity = 0; i < total; ++i, next_weights(), next_corrections()) {
       const bool ok = mbar_wait_issue(&empty[s], parity, failed);
       if (elect_one() && ok) { mbar_expect_tx(&full[s], C::STAGE); weights(s); corrections(s); }
+      if (ok) flight.issued(s, parity ^ 1);
       if (++s == C::NS) { s = 0; parity ^= 1; }
     }
   } else {
@@ -731,6 +742,7 @@ k_few_out(const __grid_constant__ CUtensorMap tmW2, const __grid_constant__ CUte
   }
   __syncthreads();
   if (threadIdx.x == 0 && *failed) atomicExch(&p.counters[CTR_ERROR], 1ull);
+  if (warp == 0 && *failed) flight.land(full);
 }
 
 // ---- set-up ---------------------------------------------------------------------------------------------

@@ -277,6 +277,7 @@ k_gemm(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtenso
     nkb = max(0, min(nkb_all, kb_lo + per) - kb_lo);
   };
 
+  InFlight flight;
   if (warp == 0) {
     // ---------------- TMA producer ----------------
     int s = 0, parity = 1;                             // stage and the phase of its `empty` barrier to wait for
@@ -293,6 +294,7 @@ k_gemm(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtenso
           tma_load_2d(sa, second ? &tmA2 : &tmA1, kx, m0, &full[s]);
           tma_load_2d(sa + BM * BK * 2, second ? &tmB2 : &tmB1, kx, n0, &full[s]);
         }
+        if (ok) flight.issued(s, parity ^ 1);
         if (++s == C::NS) { s = 0; parity ^= 1; }
       }
     }
@@ -371,6 +373,7 @@ k_gemm(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtenso
   tc_fence_before();
   __syncthreads();
   if (threadIdx.x == 0 && *failed && p.error_word) atomicExch(p.error_word, 1ull);
+  if (warp == 0 && *failed) flight.land(full);
   if (warp == 1) tmem_dealloc(tmem_base, C::TMEM_COLS);
 }
 

@@ -804,3 +804,23 @@ def test_destroy_and_the_builder_give_device_memory_back(dtype, bits, d, h):
         left = free - torch.cuda.mem_get_info()[0]
     held = sum(v for k, v in st.items() if k.startswith("bytes_"))
     assert taken >= 50 << 20 and held <= taken <= held + (8 << 20) and left <= 2 << 20, (taken, held, left)
+
+
+@pytest.mark.parametrize("dtype,bits,d,calls", [("bf16", 2, 512, [1, 4, 16, 17, 64, 128, 130]), ("bf16", 4, 512, [1, 33, 128]), ("bf16", 2, 4736, [1, 5]), ("f32", 2, 512, [3])])
+def test_calls_behind_a_long_launch_that_lets_them_start_early(late_write, dtype, bits, d, calls):
+    # the launch before writes the tokens 0.3 s after it has let the call's kernels start: longer than the kernels' own waits may take
+    cfg = W.LayerConfig("patient", d, 2048, dtype=dtype, bits=bits, n_calib=64)
+    L = _layer(cfg, 1)
+    h = T.fold_layer(L)
+    try:
+        for n in calls:
+            x = W.make_tokens(cfg, n, n).cuda()
+            want, y = T.tardis_ffn_forward(h, x, torch.empty_like(x)), torch.empty_like(x)
+            late = torch.zeros_like(x)
+            torch.cuda.synchronize()
+            late_write(late, x, 600000000)
+            T.tardis_ffn_forward(h, late, y)
+            assert T.tardis_stats(h)["device_error"] == 0
+            assert ((y.float() - want.float()).abs() <= 2.0 ** -7 * want.float().abs() + 1e-3).all()   # (bf16 roundings of sums in another order)
+    finally:
+        T.tardis_destroy(h)

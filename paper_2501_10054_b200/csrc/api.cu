@@ -164,6 +164,16 @@ static void free_all(Handle* H) {
   delete H;
 }
 
+// Behind the set-up of a layer: an ordinary launch, which begins when all that the set-up has written is complete and visible.  The
+// kernels of the forward calls read a layer's state before their programmatic wait for the launch before them; without this that
+// launch could be the one that writes it.
+__global__ void k_settle() {}
+static tardis_status_t settle(cudaStream_t s) {
+  k_settle<<<1, 32, 0, s>>>();
+  TARDIS_CUDA_TRY(cudaGetLastError());
+  return TARDIS_OK;
+}
+
 // Allocates a handle and its device arrays for a layer of the given shape (nothing is filled in yet).
 static tardis_status_t new_handle(int d, int h, int dtype, int act, int G, int bits, cudaStream_t s, Handle** out) {
   *out = nullptr;
@@ -245,6 +255,7 @@ tardis_status_t tardis_fold(const tardis_fold_desc_t* desc, tardis_stream_t stre
   if (st == TARDIS_OK && bf16 && !H->fscratch) st = decode_prepare(H, s);   // wider layers: the older per-token kernel
   if (st == TARDIS_OK && bf16) st = batched_finish(H, desc->W2, s);
   if (st == TARDIS_OK) st = f32_prepare(H, s);
+  if (st == TARDIS_OK) st = settle(s);
   if (st != TARDIS_OK) { cudaStreamSynchronize(s); free_all(H); return st; }
   *out = reinterpret_cast<tardis_handle_t>(H);
   return TARDIS_OK;
@@ -528,6 +539,7 @@ tardis_status_t tardis_load(const char* path, tardis_stream_t stream, tardis_han
   if (st == TARDIS_OK && bf16 && !H->fscratch) st = decode_prepare(H, s);
   if (st == TARDIS_OK && bf16) st = batched_finish(H, nullptr, s);
   if (st == TARDIS_OK) st = f32_prepare(H, s);
+  if (st == TARDIS_OK) st = settle(s);
   if (st != TARDIS_OK) { cudaStreamSynchronize(s); free_all(H); return st; }
   *out = reinterpret_cast<tardis_handle_t>(H);
   return TARDIS_OK;

@@ -824,3 +824,21 @@ def test_calls_behind_a_long_launch_that_lets_them_start_early(late_write, dtype
             assert ((y.float() - want.float()).abs() <= 2.0 ** -7 * want.float().abs() + 1e-3).all()   # (bf16 roundings of sums in another order)
     finally:
         T.tardis_destroy(h)
+
+
+@pytest.mark.parametrize("dtype,bits,d,n", [("bf16", 2, 512, 1), ("bf16", 2, 512, 20), ("bf16", 4, 512, 3), ("bf16", 2, 4736, 2), ("f32", 2, 512, 5)])
+def test_first_call_right_behind_the_fold(dtype, bits, d, n):
+    # no wait in between, into memory that another layer's state has been in: the call has to find the new layer's state complete
+    cfg = W.LayerConfig("behind", d, 2048, dtype=dtype, bits=bits, n_calib=64)
+    layers = [_layer(cfg, seed) for seed in (1, 2)]
+    x = W.make_tokens(cfg, n, 1).cuda()
+    want = []
+    for i in range(8):
+        L = layers[i % 2]
+        h = T.fold_layer(L)
+        y = T.tardis_ffn_forward(h, x, torch.empty_like(x)).float()
+        torch.cuda.synchronize()
+        if i < 2:
+            want.append(T.tardis_ffn_forward(h, x, torch.empty_like(x)).float())
+        T.tardis_destroy(h)
+        assert ((y - want[i % 2]).abs() <= 2.0 ** -7 * want[i % 2].abs() + 1e-3).all()      # (bf16 roundings of sums in another order)

@@ -271,7 +271,7 @@ k_few_in(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUten
   }
   const uint32_t tmem = *tmem_slot;
   // The waits below are bounded, so none of them may begin before the launch before this one has ended: it may take any time.
-  InFlight flight;
+  int issued = 0;                                      // fills of a stage, by warp 0
 
   if (warp == 0) {
     // ---------------- TMA: W1 tiles, then the folded matrix's blocks; the tokens beside each ----------------
@@ -285,11 +285,10 @@ k_few_in(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUten
     pdl_wait();
     for (int s = 0; s < ahead; ++s, first.next())
       if (elect_one()) tokens(first, s);
-    flight.begin(ahead);
-    for (int i = ahead, s = 0, parity = 0; i < w.total; ++i, w.next()) {
-      const bool ok = mbar_wait_issue(&empty[s], parity, failed);
-      if (elect_one() && ok) { mbar_expect_tx(&full[s], bytes(w)); weights(w, s); tokens(w, s); }
-      if (ok) flight.issued(s, parity ^ 1);
+    issued = ahead;
+    for (int s = 0, parity = 0; issued < w.total; ++issued, w.next()) {
+      if (!mbar_wait_issue(&empty[s], parity, failed)) break;
+      if (elect_one()) { mbar_expect_tx(&full[s], bytes(w)); weights(w, s); tokens(w, s); }
       if (++s == C::NS) { s = 0; parity ^= 1; }
     }
   } else if (warp == 1) {
@@ -420,6 +419,7 @@ k_few_in(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUten
       float lo = 0.f, hi = 0.f, b1 = 0.f, fa = 0.f, fc = 0.f;
       if (real) { lo = p.lo[j]; hi = p.hi[j]; b1 = p.b1[j]; fa = p.a[j]; fc = p.c[j]; }
       const float smax = real ? p.smax[j] : 0.f;
+      if (terms == 2) pdl_wait();
       for (int i0 = 0; i0 < mine && ok; i0 += AHEAD) {
 #pragma unroll
         for (int u = 0; u < AHEAD; ++u) {
@@ -437,7 +437,7 @@ k_few_in(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUten
               else expand<1>(code[u][0], meta[u], w);
               if (term == terms - 1 && i + AHEAD < mine) fetch(gi + 2 * (i + AHEAD), code[u], meta[u]);
               const int b = gi + 2 * (own % RING);
-              if (own == RING) pdl_wait();                 // (the first RING blocks find their places free)
+              if (u == RING && i0 == 0) pdl_wait();        // (a tile's first RING blocks of one term find their places free)
               ok = mbar_wait_warp(&a_empty[b], ((own / RING) & 1) ^ 1);
               if (!ok) { *failed = 1u; break; }
               tc_fence_after();
@@ -588,7 +588,7 @@ k_few_in(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUten
   tc_fence_before();
   __syncthreads();
   if (threadIdx.x == 0 && *failed) atomicExch(&p.counters[CTR_ERROR], 1ull);
-  if (warp == 0 && *failed) flight.land(full);
+  if (warp == 0 && *failed) land_copies<C::NS>(full, issued);
   if (warp == 1) tmem_dealloc(tmem, C::TMEM);
 }
 
@@ -610,7 +610,7 @@ k_few_out(const __grid_constant__ CUtensorMap tmW2, const __grid_constant__ CUte
   const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // (warp: uniform, and known to be)
   auto begin_of = [&](int c) { return int((long long)p.total * c / int(gridDim.x)); };
   const int begin = begin_of(blockIdx.x), end = begin_of(blockIdx.x + 1), nkb = p.nkb;
-  InFlight flight;
+  int issued = 0;                                      // fills of a stage, by warp 0
   pdl_launch();
   if (threadIdx.x == 0) {
     for (int s = 0; s < C::NS; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
@@ -633,11 +633,10 @@ k_few_out(const __grid_constant__ CUtensorMap tmW2, const __grid_constant__ CUte
     pdl_wait();
     for (int s = 0; s < ahead; ++s, next_corrections())
       if (elect_one()) corrections(s);
-    flight.begin(ahead);
-    for (int i = ahead, s = 0, parity = 0; i < total; ++i, next_weights(), next_corrections()) {
-      const bool ok = mbar_wait_issue(&empty[s], parity, failed);
-      if (elect_one() && ok) { mbar_expect_tx(&full[s], C::STAGE); weights(s); corrections(s); }
-      if (ok) flight.issued(s, parity ^ 1);
+    issued = ahead;
+    for (int s = 0, parity = 0; issued < total; ++issued, next_weights(), next_corrections()) {
+      if (!mbar_wait_issue(&empty[s], parity, failed)) break;
+      if (elect_one()) { mbar_expect_tx(&full[s], C::STAGE); weights(s); corrections(s); }
       if (++s == C::NS) { s = 0; parity ^= 1; }
     }
   } else {
@@ -742,7 +741,7 @@ k_few_out(const __grid_constant__ CUtensorMap tmW2, const __grid_constant__ CUte
   }
   __syncthreads();
   if (threadIdx.x == 0 && *failed) atomicExch(&p.counters[CTR_ERROR], 1ull);
-  if (warp == 0 && *failed) flight.land(full);
+  if (warp == 0 && *failed) land_copies<C::NS>(full, issued);
 }
 
 // ---- set-up ---------------------------------------------------------------------------------------------

@@ -277,7 +277,7 @@ k_gemm(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtenso
     nkb = max(0, min(nkb_all, kb_lo + per) - kb_lo);
   };
 
-  InFlight flight;
+  int issued = 0;                                      // fills of a stage, by warp 0
   if (warp == 0) {
     // ---------------- TMA producer ----------------
     int s = 0, parity = 1;                             // stage and the phase of its `empty` barrier to wait for
@@ -285,16 +285,16 @@ k_gemm(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtenso
       int m0, n0, kb_lo, nkb, z;
       decode(tile, m0, n0, kb_lo, nkb, z);
       for (int kg = kb_lo; kg < kb_lo + nkb; ++kg) {   // k block in the whole channel range
-        const bool ok = mbar_wait_issue(&empty[s], parity, failed);
+        if (!mbar_wait_issue(&empty[s], parity, failed)) break;
+        ++issued;
         const bool second = kg >= p.kb1;
         const int kx = (second ? kg - p.kb1 : kg) * BK;
         uint8_t* sa = smem + s * C::STAGE_BYTES;
-        if (elect_one() && ok) {
+        if (elect_one()) {
           mbar_expect_tx(&full[s], C::STAGE_BYTES);
           tma_load_2d(sa, second ? &tmA2 : &tmA1, kx, m0, &full[s]);
           tma_load_2d(sa + BM * BK * 2, second ? &tmB2 : &tmB1, kx, n0, &full[s]);
         }
-        if (ok) flight.issued(s, parity ^ 1);
         if (++s == C::NS) { s = 0; parity ^= 1; }
       }
     }
@@ -373,7 +373,7 @@ k_gemm(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtenso
   tc_fence_before();
   __syncthreads();
   if (threadIdx.x == 0 && *failed && p.error_word) atomicExch(p.error_word, 1ull);
-  if (warp == 0 && *failed) flight.land(full);
+  if (warp == 0 && *failed) land_copies<C::NS>(full, issued);
   if (warp == 1) tmem_dealloc(tmem_base, C::TMEM_COLS);
 }
 

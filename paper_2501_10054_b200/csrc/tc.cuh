@@ -63,16 +63,11 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* b, uint32_t parity) {
   }
   return __shfl_sync(0xffffffffu, ok, 0) != 0;
 }
-// What the warp that issues copies has last sent to each stage, so that a CTA in which a wait has run out does not end before its copies
-// have: they would land in shared memory that is another CTA's by then.
-struct InFlight {
-  uint32_t stages = 0u, odd = 0u;                            // bit s: stage s has been filled; ... in an odd phase of its barrier
-  __device__ __forceinline__ void begin(int first) { stages = (1u << first) - 1u; }   // stages 0 .. first - 1 for the first time
-  __device__ __forceinline__ void issued(int s, int parity) { stages |= 1u << s; odd = (odd & ~(1u << s)) | uint32_t(parity) << s; }
-  __device__ __forceinline__ void land(uint64_t* full) const {   // (the whole warp; bounded)
-    for (uint32_t w = stages; w; w &= w - 1u) { const int s = __ffs(w) - 1; mbar_wait_warp(&full[s], (odd >> s) & 1u); }
-  }
-};
+// The whole warp waits (bounded) for the last of its copies in each of NS stages, after `issued` fills of them in turn: a CTA in which a
+// wait has run out must not end before its copies have, they would land in shared memory that is another CTA's by then.
+template <int NS> __device__ __forceinline__ void land_copies(uint64_t* full, int issued) {
+  for (int k = issued > NS ? issued - NS : 0; k < issued; ++k) mbar_wait_warp(&full[k % NS], (k / NS) & 1);
+}
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
   asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
                ::"r"(smem_u32(dst)), "l"(map), "r"(smem_u32(bar)), "r"(x), "r"(y) : "memory");

@@ -13,8 +13,9 @@
 //     X W_f^T needs only the tokens; its channel blocks are dealt to the CTAs so that all of them have about the same to do.
 //   k_few_out: the corrections times W2, the (output tile, neuron block) pairs dealt evenly to the CTAs; partial outputs are
 //     added to the fp32 accumulator, and the last CTA to contribute to an output tile rounds it to y and clears it.
-//   Both take part in the programmatic hand-over: k_few_out fills its stages with W2 while k_few_in finishes, k_few_in its
-//     stages with W1 while the launch before it finishes (both fit on an SM side by side up to 64 tokens).
+//   Both take part in the programmatic hand-over: a CTA of k_few_out fills its stages with W2, one of k_few_in its stages with W1, as
+//     soon as the launch before has left its SM, while other SMs still finish that one (two CTAs do not fit on an SM: the rings
+//     take 200 KB and more).
 //   4-bit codes take the same way with two bf16 terms per weight: 4096 / 16384, caches cold, 95 us for one token and 130 for 64, where
 //     the dense products over a dequantised predictor took 200 and 181.
 #include <string.h>
@@ -64,8 +65,7 @@ template <int N> struct InCfg {
   static constexpr int NS = N == 128 ? 6 : (N == 64 ? 8 : (N == 32 ? 10 : 11));
   static constexpr int NBUF = N == 64 ? 2 : 4;                      // expanded predictor blocks in TMEM (32 columns each)
   static constexpr int COL_S = 0, COL_Z = N, COL_F = 2 * N, COL_A = 3 * N;
-  // A CTA that starts early must leave the columns that the launch before it still has to allocate on the same SM, or the two
-  // wait for each other: 256 of 512 up to 64 columns of tokens (k_few_out takes 128 at most).  With 128 it takes all, after the wait.
+  // (an allocation is a power of two; a kernel that takes all 512 columns does so only behind the wait, they may be another's until then)
   static constexpr int TMEM = COL_A + NBUF * 32 <= 256 ? 256 : 512;
   static constexpr int SMEM = 1024 + NS * STAGE + BARS + MAX_NEAR * 16 + BM * ((N + 31) / 32) * 4 + N * 8 + 8 * 1024;
   static_assert((2 * NS + 2 * NBUF + 5) * 8 + 16 <= BARS, "barriers");
@@ -216,7 +216,7 @@ struct Walk {
 // N: token columns (the call's tokens rounded up); TERMS: bf16 terms of a correction (2 keeps 16 significant bits of it); BITS: of a
 // code
 template <int N, int TERMS, int BITS>
-__global__ void __maxnreg__(128)                       // (NT_IN threads; leaves room for k_few_out on the SM)
+__global__ void __launch_bounds__(NT_IN, 1)            // (one CTA per SM: its shared memory)
 k_few_in(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUtensorMap tmWf, const __grid_constant__ CUtensorMap tmX,
          const InParams p) {
   using C = InCfg<N>;
@@ -595,7 +595,7 @@ k_few_in(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUten
 // Corrections times W2.  N: columns (tokens rounded up, times the terms of a correction).  CTA c works on the pairs
 // [c total / grid, (c + 1) total / grid) of (output tile, neuron block).
 template <int N>
-__global__ void __maxnreg__(64)                        // (a quarter of the SM then holds three warps of k_few_in and two of these)
+__global__ void __launch_bounds__(NT_OUT, 1)
 k_few_out(const __grid_constant__ CUtensorMap tmW2, const __grid_constant__ CUtensorMap tmD, const OutParams p) {
   using C = OutCfg<N>;
   extern __shared__ uint8_t smem_raw[];
@@ -878,11 +878,7 @@ tardis_status_t few_prepare(Handle* H) {
     const cudaError_t e = dev_malloc(r.p, r.bytes);
     if (e != cudaSuccess) { set_last_error(e, "cudaMalloc"); cudaGetLastError(); few_release(H); return TARDIS_ERR_ALLOC; }
   }
-  // (all of an SM's shared memory, so that both kernels fit on it side by side: the share is fixed while a kernel runs there)
-  auto room = [](auto kernel, int smem) {
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-    return e != cudaSuccess ? e : cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  };
+  auto room = [](auto kernel, int smem) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); };
   const cudaError_t es[] = {room(k_few_in<16, 2, 2>, InCfg<16>::SMEM), room(k_few_in<32, 1, 2>, InCfg<32>::SMEM), room(k_few_in<64, 1, 2>, InCfg<64>::SMEM),
                             room(k_few_in<128, 1, 2>, InCfg<128>::SMEM), room(k_few_in<16, 2, 4>, InCfg<16>::SMEM), room(k_few_in<32, 1, 4>, InCfg<32>::SMEM),
                             room(k_few_in<64, 1, 4>, InCfg<64>::SMEM), room(k_few_in<128, 1, 4>, InCfg<128>::SMEM), room(k_few_out<32>, OutCfg<32>::SMEM),

@@ -274,10 +274,12 @@ tardis_status_t tardis_ffn_forward(tardis_handle_t handle, const void* x, void* 
   tardis_status_t st;
   // (deterministic mode: only the kernels of fused.cu and the tensor-core products without a split channel range qualify)
   const bool has_fused = H->fscratch != nullptr || (H->codes_mma != nullptr && !H->deterministic);
-  // One launch of the fused kernel (4 tokens) is faster than the kernels of few.cu (4096 / 16384: 52 us against 75), two are not;
-  // of the per-token kernel of wider layers two launches are the most (8192 / 32768: 87 us each against 255).  Where few.cu
-  // does not serve a layer the batched path takes over later.
-  const int most_fused = H->few && !H->deterministic ? (H->fscratch ? 4 : 2) : (H->fscratch ? H->fused_max_tokens : 8);
+  // One launch of the fused kernel (up to 4 tokens) is faster than the kernels of few.cu, two are not (4096 / 16384, a tenth of the
+  // neurons flagged: 4 tokens 49 us against 73, 5 tokens 76 against 73).  Of the per-token kernel of wider layers three launches are the
+  // most (8192 / 32768: 3 tokens 215 us against 247, 4 tokens 289 against 247; 5120 / 20480: 127 against 138 and 168 against 138; with a
+  // fifth flagged 3 tokens 270 against 246, with a twentieth 190 against 247).  Where few.cu does not serve a layer the batched path
+  // takes over later.
+  const int most_fused = H->few && !H->deterministic ? (H->fscratch ? 4 : 3) : (H->fscratch ? H->fused_max_tokens : 8);
   const bool fused = has_fused && ((H->path_override == 0 && n_tokens <= most_fused) || (H->path_override == 2 && n_tokens <= 4096));
   // (8-bit codes times a bf16 scale do not fit the exact two-term bf16 form the batched scores rely on)
   const bool batched = ((H->path_override == 0 && !fused) || H->path_override == 3) && H->bstate != nullptr && H->bits <= 4;

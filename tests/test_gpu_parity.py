@@ -842,3 +842,19 @@ def test_first_call_right_behind_the_fold(dtype, bits, d, n):
             want.append(T.tardis_ffn_forward(h, x, torch.empty_like(x)).float())
         T.tardis_destroy(h)
         assert ((y - want[i % 2]).abs() <= 2.0 ** -7 * want[i % 2].abs() + 1e-3).all()      # (bf16 roundings of sums in another order)
+
+
+@pytest.mark.parametrize("d,bits,most", [(512, 2, 4), (4736, 2, 3), (512, 4, 0)])
+def test_largest_call_that_goes_to_the_decode_kernels(d, bits, most):
+    cfg = W.LayerConfig("line%d" % d, d, 2048, bits=bits, n_calib=64)
+    L = _layer(cfg, 1)
+    s = L.numpy64()
+    x = W.make_tokens(cfg, 5, 1).cuda()
+    h = T.fold_layer(L)
+    try:
+        for n in range(1, 6):
+            y, F, S = Hp.gpu_forward(h, L, x[:n])
+            assert T.tardis_stats(h)["last_path"] == (2 if n <= most else 3)
+            Hp.assert_parity(L, s, x[:n], y, F, S, score_tol=3e-4, label="%d tokens" % n)
+    finally:
+        T.tardis_destroy(h)

@@ -296,7 +296,7 @@ k_calibrate(const float* __restrict__ z, long long ldz, const float* __restrict_
 //     that the chain of dependent fp64 instructions is paid once per six steps.  Two errors closer than the rounding bound of
 //     the moments (or moments that cancel) are evaluated by the definition; exact zeros of piecewise-linear activations, on
 //     which the tie rule depends, thus stay exact.
-// 16384 neurons x 2048 samples: 2.4 ms (133 ms with every density and error evaluated as defined).
+// 16384 neurons x 2048 samples: 2.5 ms (133 ms with every density and error evaluated as defined).
 constexpr int kMaxSearchSamples = 2048;
 constexpr int kMaxSteps = 160;           // steps on one side whose moments are made at once
 constexpr int kAhead = 6;                // steps that a warp looks ahead: 28 ranges

@@ -13,7 +13,7 @@
 // (neuron, channel) in ascending order of k.  A channel thus sees exactly the sequence of subtractions of the
 // channel-by-channel procedure, each a rounded product followed by a rounded difference in double precision (no fused
 // multiply-add), so the codes equal those of a plain double-precision implementation bit for bit.
-// Bound by the fp64 pipe: h d^2 separate products and differences (16384 x 4096, 2.7e11: 15 ms).  Measured 25 ms (53
+// Bound by the fp64 pipe: h d^2 separate products and differences (16384 x 4096, 2.7e11: 15 ms).  Measured 23 ms of kernels (53
 // before, with one thread per neuron and 16 x 1 outputs per thread, which read shared memory as often as they computed).
 #include "common.cuh"
 

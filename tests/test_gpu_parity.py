@@ -533,8 +533,7 @@ def test_save_and_load_round_trip(tmp_path, dtype):
 
 
 def test_buffers_of_destroyed_layers_are_taken_over_by_new_ones():
-    """Freed buffers wait for the next allocation of their size: layers folded, used and destroyed in turn by two threads on
-    streams of their own give the results of a layer folded alone, and nothing stays registered as alive."""
+    """Layers folded, used and destroyed in turn by two threads on streams of their own, the memory of one going to the next, give the results of a layer folded alone, and nothing stays registered as alive."""
     import threading
     cfgs = [W.LayerConfig("pool%d" % i, 512, 2048, n_calib=256, bias=bool(i)) for i in range(2)]
     Ls = [_layer(c, i) for i, c in enumerate(cfgs)]

@@ -69,9 +69,10 @@ struct KParams {
   uint32_t* rlist; unsigned int* rcount; int rcap, bits;
 };
 
-template <int BN> struct Cfg {
-  static constexpr int STAGE_BYTES = BM * BK * 2 + BN * BK * 2;
-  static constexpr int NS = (BN == 256) ? 4 : 6;                      // stages
+// CTAS: 1, or 2 for a pair of CTAs that works on 256 x BN tiles
+template <int BN, int CTAS> struct Cfg {
+  static constexpr int STAGE_BYTES = BM * BK * 2 + BN / CTAS * BK * 2;   // (of a CTA)
+  static constexpr int NS = (BN / CTAS == 256) ? 4 : 6;               // stages
   static constexpr int SMEM = NS * STAGE_BYTES + 1024 /* alignment slack */ + 256 /* barriers */ + 8 * 2048 /* epilogue staging */ + BN * 16 /* column table */;
   static constexpr int TMEM_COLS = 2 * BN;                            // two accumulators
 };
@@ -223,11 +224,19 @@ __device__ __forceinline__ void fill_table(const KParams& p, float4* tab, int n0
 
 // Persistent: CTA c works on tiles c, c + gridDim.x, ... of a banded raster.  Two accumulators in tensor memory:
 // while the epilogue warps drain one, the MMA warp is already filling the other with the next tile.
-template <int BN>
+//
+// With CTAS = 2 two CTAs on neighbouring SMs share a tile of 256 x BN: each holds 128 rows of A and of the accumulator and half of the
+// rows of B, and rank 0 issues the MMAs (M = 256) for both, so an operand row is written to and read from shared memory once
+// per 256 rows of the other operand instead of once per 128 (a CTA of its own reads and writes 192 bytes of shared memory per clock at the
+// MMAs' full rate, more than there are; 16384 prompt tokens of a 4096 / 16384 layer 7068 -> 6637 us, a calibration's product included
+// 519 -> 497).  Rank 0's `full` barrier counts the bytes of both; a stage and an
+// accumulator are handed back to both (multicast commit), and the accumulators of both have to be drained.
+template <int BN, int CTAS>
 __global__ void __launch_bounds__(NTHREADS, 1)
 k_gemm(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtensorMap tmB1,
        const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB2, const KParams p) {
-  using C = Cfg<BN>;
+  using C = Cfg<BN, CTAS>;
+  constexpr int TM = BM * CTAS, BROWS = BN / CTAS;      // rows of a tile; of B in this CTA
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + C::NS * C::STAGE_BYTES);
@@ -238,19 +247,24 @@ k_gemm(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtenso
   volatile uint32_t* failed = tmem_slot + 1;
 
   const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // (warp: uniform, and known to be)
-  const int nm = (p.M + BM - 1) / BM, nn = (p.N + BN - 1) / BN;
+  const int nm = (p.M + TM - 1) / TM, nn = (p.N + BN - 1) / BN;
   const int ntiles = nm * nn * p.splits;
+  const int rank = CTAS == 2 ? int(cluster_rank()) : 0, first_tile = blockIdx.x / CTAS, step = gridDim.x / CTAS;
   if (threadIdx.x == 0) {
     for (int s = 0; s < C::NS; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
-    for (int b = 0; b < 2; ++b) { mbar_init(&accum_full[b], 1); mbar_init(&accum_empty[b], 8); }
+    for (int b = 0; b < 2; ++b) { mbar_init(&accum_full[b], 1); mbar_init(&accum_empty[b], 8 * CTAS); }
     *failed = 0u;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tmA1) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tmB1) : "memory");
   }
-  if (warp == 1) tmem_alloc(tmem_slot, C::TMEM_COLS);  // the whole warp; a power of two >= 32 fp32 columns
+  if (warp == 1) {                                     // the whole warp; a power of two >= 32 fp32 columns
+    if (CTAS == 2) tmem_alloc_pair(tmem_slot, C::TMEM_COLS);
+    else tmem_alloc(tmem_slot, C::TMEM_COLS);
+  }
   tc_fence_before();
-  __syncthreads();
+  if (CTAS == 2) cluster_sync();                       // (the other CTA's barriers are reported to)
+  else __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
@@ -265,7 +279,7 @@ k_gemm(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtenso
     const int w = min(p.band, F - bi * p.band);
     const int slow = r2 / w, fast = bi * p.band + (r2 - slow * w);
     const int mi = p.fast_m ? fast : slow, ni = p.fast_m ? slow : fast;
-    m0 = mi * BM; n0 = ni * BN;
+    m0 = mi * TM + rank * BM; n0 = ni * BN;
     int nkb_all = p.kb1;
     if (p.kb2 > 0) {
       bool used = p.second_used == nullptr;
@@ -281,7 +295,7 @@ k_gemm(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtenso
   if (warp == 0) {
     // ---------------- TMA producer ----------------
     int s = 0, parity = 1;                             // stage and the phase of its `empty` barrier to wait for
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    for (int tile = first_tile; tile < ntiles; tile += step) {
       int m0, n0, kb_lo, nkb, z;
       decode(tile, m0, n0, kb_lo, nkb, z);
       for (int kg = kb_lo; kg < kb_lo + nkb; ++kg) {   // k block in the whole channel range
@@ -291,20 +305,26 @@ k_gemm(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtenso
         const int kx = (second ? kg - p.kb1 : kg) * BK;
         uint8_t* sa = smem + s * C::STAGE_BYTES;
         if (elect_one()) {
-          mbar_expect_tx(&full[s], C::STAGE_BYTES);
-          tma_load_2d(sa, second ? &tmA2 : &tmA1, kx, m0, &full[s]);
-          tma_load_2d(sa + BM * BK * 2, second ? &tmB2 : &tmB1, kx, n0, &full[s]);
+          if (rank == 0) mbar_expect_tx(&full[s], CTAS * C::STAGE_BYTES);
+          if (CTAS == 2) {
+            const uint32_t bar = in_rank_0(&full[s]);
+            tma_load_2d_pair(sa, second ? &tmA2 : &tmA1, kx, m0, bar);
+            tma_load_2d_pair(sa + BM * BK * 2, second ? &tmB2 : &tmB1, kx, n0 + rank * BROWS, bar);
+          } else {
+            tma_load_2d(sa, second ? &tmA2 : &tmA1, kx, m0, &full[s]);
+            tma_load_2d(sa + BM * BK * 2, second ? &tmB2 : &tmB1, kx, n0, &full[s]);
+          }
         }
         if (++s == C::NS) { s = 0; parity ^= 1; }
       }
     }
   } else if (warp == 1) {
-    // ---------------- MMA issuer ----------------
-    constexpr uint32_t idesc = instr_desc_bf16(BM, BN);
+    // ---------------- MMA issuer (of a pair: rank 0) ----------------
+    constexpr uint32_t idesc = instr_desc_bf16(TM, BN);
     const uint64_t adesc = smem_desc_k_major_sw128(smem_u32(smem)), bdesc = smem_desc_k_major_sw128(smem_u32(smem) + BM * BK * 2);
     int s = 0, parity = 0;
     uint32_t use = 0;                                  // accumulator uses so far
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    for (int tile = rank == 0 ? first_tile : ntiles; tile < ntiles; tile += step) {
       int m0, n0, kb_lo, nkb, z;
       decode(tile, m0, n0, kb_lo, nkb, z);
       if (nkb == 0) continue;                          // nothing to add: the epilogue takes zeros
@@ -319,12 +339,19 @@ k_gemm(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtenso
         const uint64_t da = adesc + uint32_t(s * (C::STAGE_BYTES >> 4)), db = bdesc + uint32_t(s * (C::STAGE_BYTES >> 4));
         if (elect_one() && ok) {
 #pragma unroll
-          for (int k = 0; k < BK / 16; ++k) umma_f16(tacc, da + k * 2, db + k * 2, idesc, (kb | k) != 0 ? 1u : 0u);
-          umma_commit(&empty[s]);                      // frees the stage when these MMAs have read it
+          for (int k = 0; k < BK / 16; ++k) {
+            if (CTAS == 2) umma_f16_pair(tacc, da + k * 2, db + k * 2, idesc, (kb | k) != 0 ? 1u : 0u);
+            else umma_f16(tacc, da + k * 2, db + k * 2, idesc, (kb | k) != 0 ? 1u : 0u);
+          }
+          if (CTAS == 2) umma_commit_pair(&empty[s]);  // frees the stage when these MMAs have read it
+          else umma_commit(&empty[s]);
         }
         if (++s == C::NS) { s = 0; parity ^= 1; }
       }
-      if (elect_one() && ok) umma_commit(&accum_full[ab]);   // accumulator complete
+      if (elect_one() && ok) {                         // accumulator complete
+        if (CTAS == 2) umma_commit_pair(&accum_full[ab]);
+        else umma_commit(&accum_full[ab]);
+      }
       ++use;
     }
   } else {
@@ -336,7 +363,7 @@ k_gemm(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtenso
     const bool table = p.epilogue == GEMM_EPI_FLAGS || p.epilogue == GEMM_EPI_DELTA;
     uint32_t use = 0;
     bool ok = true;
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    for (int tile = first_tile; tile < ntiles; tile += step) {
       int m0, n0, kb_lo, nkb, z;
       decode(tile, m0, n0, kb_lo, nkb, z);
       const int m = m0 + q * 32 + lane;
@@ -365,7 +392,10 @@ k_gemm(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtenso
       if (nkb > 0) {
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&accum_empty[ab]);  // this warp's lanes of the accumulator may be overwritten
+        if (lane == 0) {                               // this warp's lanes of the accumulator may be overwritten
+          if (CTAS == 2) mbar_arrive_cluster(in_rank_0(&accum_empty[ab]));
+          else mbar_arrive(&accum_empty[ab]);
+        }
         ++use;
       }
     }
@@ -373,17 +403,26 @@ k_gemm(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtenso
   tc_fence_before();
   __syncthreads();
   if (threadIdx.x == 0 && *failed && p.error_word) atomicExch(p.error_word, 1ull);
-  if (warp == 0 && *failed) land_copies<C::NS>(full, issued);
-  if (warp == 1) tmem_dealloc(tmem_base, C::TMEM_COLS);
+  if (CTAS == 2) {
+    // neither ends while the other may still report to it or its MMAs read it; copies of both report to rank 0
+    if (threadIdx.x == 0 && rank == 1 && *failed) asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(in_rank_0(const_cast<uint32_t*>(failed))), "r"(1u) : "memory");
+    cluster_sync();
+    if (rank == 0 && warp == 0 && *failed) land_copies<C::NS>(full, issued);
+    if (warp == 1) tmem_dealloc_pair(tmem_base, C::TMEM_COLS);
+    cluster_sync();
+  } else {
+    if (warp == 0 && *failed) land_copies<C::NS>(full, issued);
+    if (warp == 1) tmem_dealloc(tmem_base, C::TMEM_COLS);
+  }
 }
 
 // ---- host side ------------------------------------------------------------------------------------------
-template <int BN>
+template <int BN, int CTAS>
 static tardis_status_t launch_bn(const GemmArgs& g, cudaStream_t s) {
   CUtensorMap a1, b1, a2, b2;
-  if (!make_map(&a1, g.A1, g.M, g.K1, g.lda1, BM) || !make_map(&b1, g.B1, g.N, g.K1, g.ldb1, BN)) return TARDIS_ERR_INVALID_ARG;
+  if (!make_map(&a1, g.A1, g.M, g.K1, g.lda1, BM) || !make_map(&b1, g.B1, g.N, g.K1, g.ldb1, BN / CTAS)) return TARDIS_ERR_INVALID_ARG;
   a2 = a1; b2 = b1;
-  if (g.K2 > 0 && (!make_map(&a2, g.A2, g.M, g.K2, g.lda2, BM) || !make_map(&b2, g.B2, g.N, g.K2, g.ldb2, BN)))
+  if (g.K2 > 0 && (!make_map(&a2, g.A2, g.M, g.K2, g.lda2, BM) || !make_map(&b2, g.B2, g.N, g.K2, g.ldb2, BN / CTAS)))
     return TARDIS_ERR_INVALID_ARG;
   KParams p;
   p.M = g.M; p.N = g.N; p.kb1 = (g.K1 + BK - 1) / BK; p.kb2 = g.K2 > 0 ? (g.K2 + BK - 1) / BK : 0;
@@ -396,18 +435,23 @@ static tardis_status_t launch_bn(const GemmArgs& g, cudaStream_t s) {
   int dev = 0, sms = 0;
   TARDIS_CUDA_TRY(cudaGetDevice(&dev));
   if (dev != room_on) {
-    TARDIS_CUDA_TRY(cudaFuncSetAttribute(k_gemm<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<BN>::SMEM));
+    TARDIS_CUDA_TRY(cudaFuncSetAttribute(k_gemm<BN, CTAS>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<BN, CTAS>::SMEM));
     room_on = dev;
   }
-  const int nm = (g.M + BM - 1) / BM, nn = (g.N + BN - 1) / BN;
+  const int nm = (g.M + BM * CTAS - 1) / (BM * CTAS), nn = (g.N + BN - 1) / BN;
   p.fast_m = nm <= nn ? 1 : 0;
   const int fcount = p.fast_m ? nm : nn;
-  p.band = fcount <= 16 ? fcount : 12;
+  p.band = fcount <= 16 / (p.fast_m ? CTAS : 1) ? fcount : 12 / (p.fast_m ? CTAS : 1);
   const long tiles = long(nm) * nn * p.splits;
   TARDIS_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const unsigned grid = unsigned(tiles < sms ? tiles : sms);          // one CTA per SM (shared memory), persistent
-  k_gemm<BN><<<grid, NTHREADS, Cfg<BN>::SMEM, s>>>(a1, b1, a2, b2, p);
-  TARDIS_CUDA_TRY(cudaGetLastError());
+  const long at_once = sms / CTAS;                                    // one CTA per SM (shared memory), persistent
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(unsigned(tiles < at_once ? tiles : at_once) * CTAS); cfg.blockDim = dim3(NTHREADS); cfg.dynamicSmemBytes = Cfg<BN, CTAS>::SMEM; cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = CTAS; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr; cfg.numAttrs = CTAS > 1 ? 1 : 0;
+  TARDIS_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_gemm<BN, CTAS>, a1, b1, a2, b2, p));
   return TARDIS_OK;
 }
 
@@ -428,9 +472,12 @@ tardis_status_t launch_gemm(const GemmArgs& g, cudaStream_t s) {
   auto misaligned = [](const void* p) { return p && (reinterpret_cast<uintptr_t>(p) & 15u); };
   if (misaligned(g.out_f32) || misaligned(g.out_bf16) || misaligned(g.addend)) return TARDIS_ERR_INVALID_ARG;
   // wide tiles when they still fill the machine, narrow ones for skinny problems
-  const long tiles256 = long((g.N + 255) / 256) * ((g.M + BM - 1) / BM) * (g.splits > 1 ? g.splits : 1);
-  if (tiles256 >= 120) return launch_bn<256>(g, s);
-  return launch_bn<128>(g, s);
+  const long splits = g.splits > 1 ? g.splits : 1, nm = (g.M + BM - 1) / BM, nn = (g.N + 255) / 256;
+  if (nm * nn * splits < 120) return launch_bn<128, 1>(g, s);
+  // pairs of CTAs unless the half tile that an odd number of row tiles leaves idle costs more
+  const long waves = (nm * nn * splits + 147) / 148, pair_waves = ((nm + 1) / 2 * nn * splits + 73) / 74;
+  if (pair_waves * 10 <= waves * 11) return launch_bn<256, 2>(g, s);
+  return launch_bn<256, 1>(g, s);
 }
 
 }  // namespace tardis

@@ -292,8 +292,9 @@ tardis_status_t tardis_set_deterministic(tardis_handle_t handle, int32_t on);
  * order: when channel k opens a group, the group's grid is taken from the weights as they are then (range widened to
  * contain 0; scale = (max - min) / (2^bits - 1) rounded to `dtype`, 1 if that is 0; zero-point = round(-min / scale)
  * clamped to the code range); q_k = clip(round(w_k / scale + zero)); e_k = (w_k - scale (q_k - zero)) / U[k][k]; every
- * later channel takes w_j <- w_j - e_k U[k][j].  Rounding is to nearest-even, all arithmetic is double precision with
- * separately rounded products and differences, so the codes are those of a plain double-precision implementation.
+ * later channel takes w_j <- w_j - e_k U[k][j].  Rounding is to nearest-even, and the codes are those of a plain double-precision
+ * implementation with separately rounded products and differences (bf16 layers: decided by multiply-adds where these
+ * tell, neurons that come close to a rounding boundary done again that way).
  *   W1     device [d_ff, d_model] row-major in `dtype`;
  *   U      device double [d_model, d_model] row-major, the upper Cholesky factor of the inverse Hessian of the layer's
  *          inputs (U^T U = H^-1, H = (2/N) X^T X plus damping: made by the caller, e.g. with a library Cholesky), only

@@ -6,16 +6,28 @@
 // e_k = (w_k - s (q_k - z)) / U[k][k], and w_j <- w_j - e_k U[k][j] for j > k.  U is the upper Cholesky factor of the
 // inverse Hessian of the layer's inputs, made by the caller; no U means the identity (plain rounding to nearest).
 //
-// Layout of the work: blocks of 64 channels in superblocks of up to 512.  k_block rounds the 64 channels of a block one after the
-// other (eight lanes per neuron, its 64 weights in their registers, the 64 x 64 corner of U in shared memory) and leaves the
-// 64 errors of every neuron; k_spread takes them to the later channels of the superblock, and, once the superblock is done,
-// all its errors to all channels behind it (so the working copy passes through memory once per superblock), for each
-// (neuron, channel) in ascending order of k.  A channel thus sees exactly the sequence of subtractions of the
-// channel-by-channel procedure, each a rounded product followed by a rounded difference in double precision (no fused
-// multiply-add), so the codes equal those of a plain double-precision implementation bit for bit.
-// Bound by the fp64 pipe: h d^2 separate products and differences (16384 x 4096, 2.7e11: 15 ms).  Measured 23 ms of kernels (53
-// before, with one thread per neuron and 16 x 1 outputs per thread, which read shared memory as often as they computed).
+// The codes are those of a plain double-precision implementation in which every product and every difference is rounded by
+// itself, bit for bit.  Two ways lead to them:
+//
+//   k_build (bf16 layers, groups of 64 or 128 channels): one launch, a CTA takes up to 56 neurons through all channels (neurons do
+//   not depend on each other, so nothing is waited for).  For 128 channels at a time the errors of all channels before them are
+//   multiplied with U on the fp64 matrix instruction, weights in its accumulators; inside the 128, eight channels at a time are
+//   rounded one after the other by a thread per neuron and spread over the rest by the same instruction.  Products are accumulated
+//   without the intermediate rounding, so weights differ from the plain ones in the last bits.  A code can only differ where a weight
+//   lies that close to a rounding boundary, so the kernel notes how close each neuron came to one; the neurons that came within
+//   what the two ways can differ by (k_suspects; almost always none) are done again the plain way.
+//
+//   k_block and k_spread, the plain way: blocks of 64 channels in superblocks of up to 512.  k_block rounds the 64 channels of a block
+//   one after the other (eight lanes per neuron, its 64 weights in their registers, the 64 x 64 corner of U in shared memory) and
+//   leaves the 64 errors of every neuron; k_spread takes them to the later channels of the superblock, and, once the superblock is
+//   done, all its errors to all channels behind it (so the working copy passes through memory once per superblock), for each
+//   (neuron, channel) in ascending order of k.  A channel thus sees exactly the sequence of subtractions of the channel-by-channel
+//   procedure, each a rounded product followed by a rounded difference (no fused multiply-add).
+//
+// Both are bound by the fp64 units: h d^2 / 2 multiply-adds (16384 x 4096, 1.4e11: 7.4 ms at 37 TFLOP/s), or twice as many separate
+// products and differences.  16384 x 4096: 10.4 ms of kernels, 22.8 the plain way.
 #include "common.cuh"
+#include "ptx.cuh"
 
 namespace tardis {
 namespace {
@@ -26,10 +38,13 @@ constexpr int BROWS = 16;         // neurons per CTA of k_block
 constexpr int SROWS = 128;        // neurons and channels per CTA of k_spread; a thread has 8 x 4 of them
 constexpr int SCOLS = 64;
 
+// Rows of W1 (all, or the listed ones) widened; a CTA per row in turn.
 template <typename T>
-__global__ void k_widen(const T* __restrict__ W1, double* __restrict__ Wd, size_t count) {
-  for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < count; i += size_t(gridDim.x) * blockDim.x)
-    Wd[i] = double(to_f32<T>(W1[i]));
+__global__ void k_widen(const T* __restrict__ W1, const int* __restrict__ list, double* __restrict__ Wd, int rows, int d) {
+  for (int r = blockIdx.x; r < rows; r += gridDim.x) {
+    const T* const src = W1 + size_t(list ? list[r] : r) * d;
+    for (int k = threadIdx.x; k < d; k += blockDim.x) Wd[size_t(r) * d + k] = double(to_f32<T>(src[k]));
+  }
 }
 
 __device__ __forceinline__ double storage_round(double v, int dtype) {
@@ -37,10 +52,11 @@ __device__ __forceinline__ double storage_round(double v, int dtype) {
   return dtype == TARDIS_F32 ? double(f) : double(__bfloat162float(__float2bfloat16_rn(f)));
 }
 
-// One block of 64 channels.  Lane l of a neuron holds channels 8 l .. 8 l + 7.  E: errors of the superblock, [channel][h].
-__global__ void __launch_bounds__(BROWS * NL) k_block(double* __restrict__ Wd, const double* __restrict__ U, int h, int d, int b0, int G,
-                                                      int levels, int dtype, double* __restrict__ scale64, double* __restrict__ zero64,
-                                                      uint8_t* __restrict__ q, double* __restrict__ E) {
+// One block of 64 channels of h neurons: row r of Wd is neuron list[r] of scale64, zero64 and q (r itself without a list).  Lane l of a
+// neuron holds channels 8 l .. 8 l + 7.  E: errors of the superblock, [channel][h].
+__global__ void __launch_bounds__(BROWS * NL) k_block(double* __restrict__ Wd, const int* __restrict__ list, const double* __restrict__ U, int h,
+                                                      int d, int b0, int G, int levels, int dtype, double* __restrict__ scale64,
+                                                      double* __restrict__ zero64, uint8_t* __restrict__ q, double* __restrict__ E) {
   __shared__ double2 Us[QB][4][NL];         // row i of the corner: the 16-byte pieces of a lane's 8 channels apart, lanes side by side
   __shared__ double Ud[QB];                 // its diagonal
   const int tid = threadIdx.x, l = tid & (NL - 1), r = blockIdx.x * BROWS + tid / NL;
@@ -55,6 +71,7 @@ __global__ void __launch_bounds__(BROWS * NL) k_block(double* __restrict__ Wd, c
   }
   __syncthreads();
   const bool real = r < h;                  // (lanes of a missing neuron work on zeros: the shuffles want them)
+  const int neuron = list && real ? list[r] : r;
   double w[8];
 #pragma unroll
   for (int k = 0; k < 8; k += 2) {
@@ -81,10 +98,10 @@ __global__ void __launch_bounds__(BROWS * NL) k_block(double* __restrict__ Wd, c
     s = storage_round(__ddiv_rn(__dsub_rn(wmax, wmin), double(levels)), dtype);
     if (!(s > 0.0)) s = 1.0;
     z = fmin(fmax(rint(__ddiv_rn(-wmin, s)), 0.0), double(levels));
-    if (l == 0 && real) { scale64[size_t(r) * ng + g] = s; zero64[size_t(r) * ng + g] = z; }
+    if (l == 0 && real) { scale64[size_t(neuron) * ng + g] = s; zero64[size_t(neuron) * ng + g] = z; }
   } else if (real) {
-    s = scale64[size_t(r) * ng + g];
-    z = zero64[size_t(r) * ng + g];
+    s = scale64[size_t(neuron) * ng + g];
+    z = zero64[size_t(neuron) * ng + g];
   }
   unsigned long long codes = 0;             // of this lane's channels, a byte each
 #pragma unroll 1
@@ -111,7 +128,7 @@ __global__ void __launch_bounds__(BROWS * NL) k_block(double* __restrict__ Wd, c
       for (int k = 0; k < 8; ++k) E[size_t(lo * 8 + k) * h + r] = err[k];
     }
   }
-  if (real) *reinterpret_cast<unsigned long long*>(q + size_t(r) * d + b0 + l * 8) = codes;
+  if (real) *reinterpret_cast<unsigned long long*>(q + size_t(neuron) * d + b0 + l * 8) = codes;
 }
 
 // W[r][j] <- W[r][j] - e[r][i] U[k0 + i][j], i = 0 .. nk - 1 in this order (nk a multiple of 16), for the channels j0 <= j < j1 (both
@@ -181,6 +198,260 @@ __global__ void __launch_bounds__(256, 2) k_spread(double* __restrict__ Wd, cons
   }
 }
 
+// ---- k_build ------------------------------------------------------------------------------------------------------
+constexpr int FB = 128;           // channels that a CTA holds in accumulators at a time: 16 per warp
+constexpr int FK = 16;            // channels k per stage
+constexpr int FT = 256;
+constexpr int FSTAGES = 4;        // used two at a time: a barrier per 32 channels k
+constexpr int FROWS = 56;         // most neurons per CTA: two CTAs of 56 on each of 148 SMs hold the 16384 of a 4096 / 16384 layer
+constexpr int PROBES = 16;        // rows behind the neurons that measure how rounding errors grow (see k_suspects)
+
+template <int MT> struct BuildCfg {               // MT: neurons per CTA in eights
+  static constexpr int R = 8 * MT, ES = R + 4, US = FB + 4;           // (rows four apart modulo 16: fragments without bank conflicts)
+  static constexpr int STAGE = FK * (ES + US) + FK;                   // doubles: errors [k][neuron], U [k][channel], -1 / U[k][k]
+  static constexpr int SMEM = (FSTAGES * STAGE + 8 * R + 8 * R * 2) * 8;
+};
+
+__device__ __forceinline__ void copy_16_async(double* dst, const double* src, bool valid) {     // (zero where not valid)
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(uint32_t(__cvta_generic_to_shared(dst))), "l"(src), "r"(valid ? 16 : 0) : "memory");
+}
+
+// How far v > 0 is from the nearest value whose bf16 is not s = bf16(float(v)); 0 where s has no ordinary neighbours.
+__device__ double distance_to_other_bf16(double v, double s) {
+  if (!(s > 1e-30 && s < 1e30)) return 0.0;
+  const uint32_t b = __float_as_uint(float(s));
+  const double below = double(__uint_as_float(b - 0x10000u)), above = double(__uint_as_float(b + 0x10000u));
+  const double m0 = 0.5 * (below + s), m1 = 0.5 * (s + above);       // midpoints, themselves floats
+  // a midpoint goes to the even neighbour, and so does what the rounding to float takes to the midpoint: half a step of it
+  const double h0 = 0.5 * (double(__uint_as_float(__float_as_uint(float(m0)) + 1u)) - m0), h1 = 0.5 * (double(__uint_as_float(__float_as_uint(float(m1)) + 1u)) - m1);
+  const double even = (b & 0x10000u) ? -1.0 : 1.0;
+  return fmin(v - (m0 - even * h0), (m1 + even * h1) - v);
+}
+
+// negated reciprocals of the diagonal of U
+__global__ void k_reciprocals(const double* __restrict__ U, double* __restrict__ ninv, int d) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k < d) ninv[k] = __ddiv_rn(-1.0, U[size_t(k) * d + k]);
+}
+
+// CTA c: neurons c R .. c R + R - 1.  E: the negated errors of all its channels, [CTA][channel][R].  margin: how close (in weight) the
+// neuron came to a decision that falls the other way; size: its largest weight on the way.
+// Bound by the fp64 matrix instruction, 0.72 of its rate on 16384 x 4096; U comes from L2 (67 MB per CTA), E from memory (8.6 GB in all).
+// (10.8 ms with a barrier every 16 channels instead of 32; the rounding inside the blocks, a chain of six dependent fp64 operations per
+// channel, is 0.6 of it.  A shorter chain for 2-bit codes, and rounding that begins while other warps still spread the eight channels
+// before, need registers that are not there: 11.4.)
+template <int MT>
+__global__ void __launch_bounds__(FT, 2) k_build(const __nv_bfloat16* __restrict__ W1, const double* __restrict__ U, const double* __restrict__ ninv,
+                                                 int h, int d, int G, int levels, double* E, double* __restrict__ scale64,
+                                                 double* __restrict__ zero64, uint8_t* __restrict__ q, double* __restrict__ margin_out,
+                                                 double* __restrict__ size_out) {
+  using C = BuildCfg<MT>;
+  constexpr int R = C::R, ES = C::ES, US = C::US;
+  extern __shared__ __align__(16) double sm[];
+  double* const Wc = sm + FSTAGES * C::STAGE;       // [8][R] weights of the eight channels being rounded
+  double* const ends = Wc + 8 * R;                  // [8 warps][R][2] smallest and largest weight of a warp's channels
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+  const int r0 = blockIdx.x * R, ng = d / G;
+  double* const Eg = E + size_t(blockIdx.x) * d * R;
+  const int nblocks = (d + FB - 1) / FB;
+
+  // The stages run through k = 0 .. j0 + 127 for every block of channels j0 .. j0 + 127: errors from memory up to j0, from there on
+  // they are put into the stage as they arise.
+  int fb = 0, fk = 0, fslot = 0;
+  auto fetch = [&]() {
+    if (fb < nblocks) {
+      double* const st = sm + fslot * C::STAGE;
+      const int j0 = fb * FB, k0 = fk * FK, cols = min(FB, d - j0);
+#pragma unroll
+      for (int e = tid; e < FK * FB / 2; e += FT) {
+        const int k = e / (FB / 2), c = e % (FB / 2) * 2;
+        copy_16_async(st + FK * ES + k * US + c, U + size_t(k0 + k) * d + j0 + (c < cols ? c : 0), c < cols);
+      }
+      if (k0 < j0) {
+        for (int e = tid; e < FK * R / 2; e += FT) {
+          const int k = e / (R / 2), c = e % (R / 2) * 2;
+          copy_16_async(st + k * ES + c, Eg + size_t(k0 + k) * R + c, true);
+        }
+      } else if (tid < FK / 2) {
+        copy_16_async(st + FK * (ES + US) + tid * 2, ninv + k0 + tid * 2, true);
+      }
+      if (++fk == (j0 + cols) / FK) { fk = 0; ++fb; }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    fslot = fslot == FSTAGES - 1 ? 0 : fslot + 1;
+  };
+  fetch();
+  fetch();
+
+  double acc[MT][4];                                // channels 16 warp + g (+ 8: elements 2, 3), neurons 8 nt + 2 t (+ 1: elements 1, 3)
+  auto multiply = [&](const double* es, const double* us) {          // eight channels k
+    const double* const u = us + t * US + warp * 16 + g;
+    const double a0 = u[0], a1 = u[8], a2 = u[4 * US], a3 = u[4 * US + 8];
+#pragma unroll
+    for (int nt = 0; nt < MT; ++nt) ptx::mma_f64(acc[nt], a0, a1, a2, a3, es[t * ES + nt * 8 + g], es[(t + 4) * ES + nt * 8 + g]);
+  };
+
+  // of the thread's neuron (threads 0 .. R - 1)
+  const int r = r0 + tid;
+  const bool real = r < h, probe = r >= h && r < h + PROBES;
+  double s = 1.0, rs = 1.0, z = 0.0, zc = 4503599627370496.0, margin = 1e300, size = 0.0;
+  bool strange = false;
+
+  for (int b = 0, slot = 0; b < nblocks; ++b) {
+    const int j0 = b * FB, nk = (j0 + min(FB, d - j0)) / FK;
+#pragma unroll
+    for (int nt = 0; nt < MT; ++nt)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int row = r0 + nt * 8 + 2 * t + (i & 1), ch = j0 + warp * 16 + g + (i & 2) * 4;
+        double w = 0.0;
+        if (ch < d) {
+          if (row < h) w = double(__bfloat162float(W1[size_t(row) * d + ch]));
+          else if (row < h + PROBES) w = __popc((uint32_t(ch) * 2654435761u) & (uint32_t(row - h) * 40503u + 0x9E3779B9u)) & 1 ? 1.0 : -1.0;
+        }
+        acc[nt][i] = w;
+      }
+    for (int kt = 0; kt < nk; ++kt) {
+      if ((kt & 1) == 0) {                          // (blocks have an even number of stages)
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();                            // these two stages are in place, the two before have been read
+        fetch();
+        fetch();
+      }
+      double* const es = sm + slot * C::STAGE;
+      const double* const us = es + FK * ES;
+      slot = slot == FSTAGES - 1 ? 0 : slot + 1;
+      if (kt * FK < j0) {
+        multiply(es, us);
+        multiply(es + 8 * ES, us + 8 * US);
+        continue;
+      }
+#pragma unroll 1
+      for (int half = 0; half < 2; ++half) {        // eight channels, j0 + c .. j0 + c + 7
+        const int c = kt * FK - j0 + half * 8, owner = c >> 4;
+        const bool opens = (j0 + c) % G == 0;
+        if (opens && warp >= owner && warp < owner + G / 16) {
+#pragma unroll
+          for (int nt = 0; nt < MT; ++nt) {
+            double m[4] = {fmin(acc[nt][0], acc[nt][2]), fmax(acc[nt][0], acc[nt][2]), fmin(acc[nt][1], acc[nt][3]), fmax(acc[nt][1], acc[nt][3])};
+#pragma unroll
+            for (int o = 4; o < 32; o <<= 1)
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                const double v = __shfl_xor_sync(0xffffffffu, m[e], o);
+                m[e] = (e & 1) ? fmax(m[e], v) : fmin(m[e], v);
+              }
+            if (g == 0) {
+              double2* const at = reinterpret_cast<double2*>(ends + (warp * R + nt * 8 + 2 * t) * 2);
+              at[0] = make_double2(m[0], m[1]);
+              at[1] = make_double2(m[2], m[3]);
+            }
+          }
+        }
+        if (warp == owner) {
+#pragma unroll
+          for (int nt = 0; nt < MT; ++nt)
+            *reinterpret_cast<double2*>(Wc + g * R + nt * 8 + 2 * t) = half ? make_double2(acc[nt][2], acc[nt][3]) : make_double2(acc[nt][0], acc[nt][1]);
+        }
+        __syncthreads();
+        if (tid < R) {
+          const bool first = j0 + c == 0;           // weights as they came: their decisions are taken as the plain way takes them
+          if (opens) {
+            double mn = 0.0, mx = 0.0;
+            for (int w = owner; w < owner + G / 16; ++w) {
+              mn = fmin(mn, ends[(w * R + tid) * 2]);
+              mx = fmax(mx, ends[(w * R + tid) * 2 + 1]);
+            }
+            const double step = __ddiv_rn(__dsub_rn(mx, mn), double(levels));
+            s = storage_round(step, TARDIS_BF16);
+            // (no weight but zeros, not for want of digits: the scale is 1 either way)
+            if (!first && !(step == 0.0 && size == 0.0)) margin = fmin(margin, distance_to_other_bf16(step, s) * 0.5 * double(levels));
+            if (!(s > 0.0)) s = 1.0;
+            const double at = __ddiv_rn(-mn, s), zr = rint(at);
+            if (!first && at > 0.0 && at < double(levels)) margin = fmin(margin, (0.5 - fabs(at - zr)) * s);
+            z = fmin(fmax(zr, 0.0), double(levels));
+            zc = 4503599627370496.0 + z;
+            rs = __ddiv_rn(1.0, s);
+            size = fmax(size, fmax(mx, -mn));
+            if (real) {
+              scale64[size_t(r) * ng + (j0 + c) / G] = s;
+              zero64[size_t(r) * ng + (j0 + c) / G] = z;
+            }
+          }
+          const double* const uc = us + half * 8 * US + c;
+          const double* const ni = us + FK * US + half * 8;
+          double w[8], worst = 0.0;
+#pragma unroll
+          for (int i = 0; i < 8; ++i) w[i] = Wc[i * R + tid];
+          unsigned long long codes = 0;
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            double v = fma(w[i], rs, z);
+            if (i == 0 && first) v = __dadd_rn(__ddiv_rn(w[0], s), z);
+            // the nearest whole number in the low bits of v + 1.5 2^52; a code less the zero-point as (2^52 + q) - (2^52 + z)
+            const double m = v + 6755399441055744.0, away = fabs(v - (m - 6755399441055744.0));
+            const int code = min(max(__double2loint(m), 0), levels);
+            strange = strange || !(fabs(v) < 1073741824.0);
+            if (v > 0.0 && v < double(levels) && !(i == 0 && first)) worst = fmax(worst, away);
+            size = fmax(size, fabs(w[i]));
+            const double ne = (probe ? w[i] : fma(-s, __hiloint2double(0x43300000, code) - zc, w[i])) * ni[i];
+            es[(half * 8 + i) * ES + tid] = ne;
+            Eg[size_t(j0 + c + i) * R + tid] = ne;
+#pragma unroll
+            for (int j = i + 1; j < 8; ++j) w[j] = fma(ne, uc[i * US + j], w[j]);
+            codes |= (unsigned long long)(unsigned int)(code) << (8 * i);
+          }
+          margin = fmin(margin, (0.5 - worst) * s);
+          if (real) *reinterpret_cast<unsigned long long*>(q + size_t(r) * d + j0 + c) = codes;
+        }
+        __syncthreads();
+        // (channels that are done take part where they share a warp with ones that are not: nothing reads them any more)
+        if (warp > owner || (warp == owner && half == 0)) multiply(es + half * 8 * ES, us + half * 8 * US);
+      }
+    }
+  }
+  if (tid < R && r < h + PROBES) {
+    margin_out[r] = strange ? -1.0 : margin;
+    size_out[r] = strange ? 1e300 : size;
+  }
+}
+
+// The neurons whose codes may not be the plain way's.  The two ways differ in the rounding of the operations, unit u = 2^-53: a weight
+// sees up to 3 d of them, each of at most a few u times the largest weight M, independent and of either sign, so what they put into a
+// weight stays below lambda u sqrt(d) M with a probability that approaches 1 as exp(-lambda^2 / 2) (the probabilistic rounding analysis
+// of Higham and Mary, 2019).  A difference in one weight goes on into the later ones by the same recurrence without the rounding to
+// codes; the probe rows have followed 16 such disturbances, +-1 in every channel, and A is the largest value that came of them.
+// lambda = 256 leaves room for all constants.  On a 4096 / 16384 layer A = 15 and the bound is 2.7e-11 of a weight: one layer in 40 has a
+// neuron that came closer than that to a boundary anywhere (5 ms for the plain way with a few neurons).
+__global__ void k_suspects(const double* __restrict__ margin, const double* __restrict__ size, int h, double unit, int* __restrict__ list, int* __restrict__ count) {
+  const int r = blockIdx.x * blockDim.x + threadIdx.x;
+  if (r >= h) return;
+  double growth = 1.0;
+  for (int p = 0; p < PROBES; ++p) growth = fmax(growth, size[h + p]);
+  if (!(margin[r] > unit * growth * size[r])) list[atomicAdd(count, 1)] = r;
+}
+
+struct BuildShape { int mt, ctas; };
+// Neurons per CTA: as many as give every one of the 2 CTAs per SM that run together the same number of them.
+BuildShape build_shape(int h, int sms) {
+  const long rows = long(h) + PROBES, slots = 2L * sms, waves = (rows + slots * FROWS - 1) / (slots * FROWS);
+  BuildShape s;
+  s.mt = int((rows + slots * waves - 1) / (slots * waves) + 7) / 8;
+  s.ctas = int((rows + 8 * s.mt - 1) / (8 * s.mt));
+  return s;
+}
+
+template <int MT, typename... Args> cudaError_t launch_build(int mt, int ctas, cudaStream_t s, Args... args) {
+  if constexpr (MT > FROWS / 8) { return cudaErrorInvalidValue; }
+  else {
+    if (mt != MT) return launch_build<MT + 1>(mt, ctas, s, args...);
+    const cudaError_t e = cudaFuncSetAttribute(k_build<MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, BuildCfg<MT>::SMEM);
+    if (e != cudaSuccess) return e;
+    k_build<MT><<<ctas, FT, BuildCfg<MT>::SMEM, s>>>(args...);
+    return cudaGetLastError();
+  }
+}
+
 // codes into 32-bit words (channel order ascending, lowest bits first), scale into its storage type, zero-points into bytes
 template <typename T>
 __global__ void k_pack_out(const uint8_t* __restrict__ q, const double* __restrict__ scale64, const double* __restrict__ zero64,
@@ -207,39 +478,79 @@ __global__ void k_pack_out(const uint8_t* __restrict__ q, const double* __restri
 
 }  // namespace
 
+// k_build's conditions: bf16 layers (a float32 scale has a rounding boundary in every 1e-7 of itself, and too many neurons come close to
+// one), codes of up to 4 bits (8-bit codes have 85 times as many boundaries as 2-bit ones: 8192 x 2048 5.1 ms against 4.7 the plain way,
+// mostly for a few neurons done again), groups that a block of 128 channels holds, U where 16-byte copies can read it (its rows are multiples of 512 bytes).  Without U
+// nothing is spread.
+static bool fast_build_serves(int dtype, int bits, int G, const double* U) {
+  return U && bits <= 4 && dtype == TARDIS_BF16 && (G == 64 || G == FB) && (reinterpret_cast<uintptr_t>(U) & 15u) == 0;
+}
+
 tardis_status_t launch_build_predictor(int h, int d, int dtype, const void* W1, const double* U, int bits, int G, uint32_t* codes,
                                        void* scale, uint8_t* zero, cudaStream_t s) {
   const int ng = d / G, levels = (1 << bits) - 1;
   // A group's grid is taken from weights that have seen every channel before it, so no group may reach over the end of the
   // superblock it opens in: 256 channels where groups divide that, the group itself up to 512, else single blocks.
   const int sb = 256 % G == 0 ? 256 : (G <= 512 ? G : QB);
-  double *Wd = nullptr, *Eb = nullptr, *scale64 = nullptr, *zero64 = nullptr;
+  const bool fast = fast_build_serves(dtype, bits, G, U);
+  BuildShape shape = {};
+  if (fast) {
+    int dev = 0, sms = 0;
+    TARDIS_CUDA_TRY(cudaGetDevice(&dev));
+    TARDIS_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    shape = build_shape(h, sms);
+  }
+  // the plain way's working copy and, before it, the errors of k_build share their memory
+  const size_t wd_bytes = fast ? size_t(shape.ctas) * 8 * shape.mt * d * 8 : size_t(h) * d * 8;
+  const size_t notes_bytes = fast ? (size_t(d) + 2 * (size_t(h) + PROBES)) * 8 + (size_t(h) + 1) * 4 : 0;
+  double *Wd = nullptr, *Eb = nullptr, *scale64 = nullptr, *zero64 = nullptr, *notes = nullptr;
   uint8_t* q = nullptr;
   auto release = [&]() {
-    dev_free(Wd); dev_free(Eb); dev_free(scale64); dev_free(zero64); dev_free(q);
+    dev_free(Wd); dev_free(Eb); dev_free(scale64); dev_free(zero64); dev_free(q); dev_free(notes);
   };
-  dev_reserve(dev_room(size_t(h) * d * 8) + dev_room(size_t(h) * sb * 8) + 2 * dev_room(size_t(h) * ng * 8) + dev_room(size_t(h) * d));
-  cudaError_t e = dev_malloc(&Wd, size_t(h) * d * sizeof(double));
+  dev_reserve(dev_room(wd_bytes) + dev_room(size_t(h) * sb * 8) + 2 * dev_room(size_t(h) * ng * 8) + dev_room(size_t(h) * d) +
+              (fast ? dev_room(notes_bytes) : 0));
+  cudaError_t e = dev_malloc(&Wd, wd_bytes);
   if (e == cudaSuccess) e = dev_malloc(&Eb, size_t(h) * sb * sizeof(double));
   if (e == cudaSuccess) e = dev_malloc(&scale64, size_t(h) * ng * sizeof(double));
   if (e == cudaSuccess) e = dev_malloc(&zero64, size_t(h) * ng * sizeof(double));
   if (e == cudaSuccess) e = dev_malloc(&q, size_t(h) * d);
+  if (e == cudaSuccess && fast) e = dev_malloc(&notes, notes_bytes);
   if (e != cudaSuccess) { release(); cudaGetLastError(); return TARDIS_ERR_ALLOC; }
-  const size_t count = size_t(h) * d;
-  if (dtype == TARDIS_F32) k_widen<float><<<2048, 256, 0, s>>>(static_cast<const float*>(W1), Wd, count);
-  else k_widen<__nv_bfloat16><<<2048, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(W1), Wd, count);
-  auto spread = [&](const double* errors, int k0, int nk, int j0, int j1) {   // from channels k0 .. k0 + nk - 1 to j0 .. j1 - 1
-    if (U && j1 > j0) k_spread<<<dim3((j1 - j0) / SCOLS, (h + SROWS - 1) / SROWS), 256, 0, s>>>(Wd, U, errors, h, d, k0, nk, j0);
-  };
-  for (int s0 = 0; s0 < d && e == cudaSuccess; s0 += sb) {
-    const int s1 = s0 + sb < d ? s0 + sb : d;
-    for (int b0 = s0; b0 < s1; b0 += QB) {
-      double* const Ebb = Eb + size_t(b0 - s0) * h;
-      k_block<<<(h + BROWS - 1) / BROWS, BROWS * NL, 0, s>>>(Wd, U, h, d, b0, G, levels, dtype, scale64, zero64, q, Ebb);
-      spread(Ebb, b0, QB, b0 + QB, s1);
+  const int* list = nullptr;                               // the neurons that are done the plain way (null: all)
+  int rows = h;
+  if (fast) {
+    double* const ninv = notes;
+    double *const margin = ninv + d, *const size = margin + h + PROBES;
+    int* const count = reinterpret_cast<int*>(size + h + PROBES);
+    list = count + 1;
+    const double unit = 256.0 * 1.1102230246251565e-16 * sqrt(double(d));
+    e = cudaMemsetAsync(count, 0, sizeof(int), s);
+    k_reciprocals<<<(d + 255) / 256, 256, 0, s>>>(U, ninv, d);
+    if (e == cudaSuccess)
+      e = launch_build<1>(shape.mt, shape.ctas, s, static_cast<const __nv_bfloat16*>(W1), U, static_cast<const double*>(ninv), h, d, G, levels, Wd,
+                          scale64, zero64, q, margin, size);
+    k_suspects<<<(h + 255) / 256, 256, 0, s>>>(margin, size, h, unit, count + 1, count);
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&rows, count, sizeof(int), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  }
+  if (e == cudaSuccess && rows > 0) {
+    if (dtype == TARDIS_F32) k_widen<float><<<2048, 256, 0, s>>>(static_cast<const float*>(W1), list, Wd, rows, d);
+    else k_widen<__nv_bfloat16><<<2048, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(W1), list, Wd, rows, d);
+    auto spread = [&](const double* errors, int k0, int nk, int j0, int j1) {   // from channels k0 .. k0 + nk - 1 to j0 .. j1 - 1
+      if (U && j1 > j0) k_spread<<<dim3((j1 - j0) / SCOLS, (rows + SROWS - 1) / SROWS), 256, 0, s>>>(Wd, U, errors, rows, d, k0, nk, j0);
+    };
+    for (int s0 = 0; s0 < d && e == cudaSuccess; s0 += sb) {
+      const int s1 = s0 + sb < d ? s0 + sb : d;
+      for (int b0 = s0; b0 < s1; b0 += QB) {
+        double* const Ebb = Eb + size_t(b0 - s0) * rows;
+        k_block<<<(rows + BROWS - 1) / BROWS, BROWS * NL, 0, s>>>(Wd, list, U, rows, d, b0, G, levels, dtype, scale64, zero64, q, Ebb);
+        spread(Ebb, b0, QB, b0 + QB, s1);
+      }
+      spread(Eb, s0, s1 - s0, s1, d);
+      e = cudaGetLastError();
     }
-    spread(Eb, s0, s1 - s0, s1, d);
-    e = cudaGetLastError();
   }
   if (e == cudaSuccess) {
     if (dtype == TARDIS_F32) k_pack_out<float><<<1024, 256, 0, s>>>(q, scale64, zero64, h, d, G, bits, codes, static_cast<float*>(scale), zero);

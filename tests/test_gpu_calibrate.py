@@ -201,6 +201,21 @@ def test_range_search_screening_falls_back_where_it_must(kind, n, step):
         assert _check_search(z.cuda(), None, 0.9, step, act) <= 3
 
 
+@pytest.mark.parametrize("kind,n", [("flat", 2048), ("flat", 700), ("lattice", 2048), ("close", 2047), ("close", 100)])
+def test_range_search_density_candidates_apart_and_together(kind, n):
+    # candidates for the highest density that one expansion about their middle holds ("close": some on either side of it, and two that
+    # only the sums as defined tell apart), spread over more than a quarter of the kernel width ("flat"), in equal pairs ("lattice")
+    g = torch.Generator().manual_seed(n)
+    z = torch.randn(6, n, generator=g)
+    if kind == "flat":
+        z = torch.rand(6, n, generator=g) * 2 - 1
+    elif kind == "lattice":
+        z = (z * 200).round() / 200
+    else:
+        z = z * torch.linspace(0.05, 3.0, 6)[:, None] + torch.linspace(-3, 3, 6)[:, None]
+    assert _check_search(z.cuda(), None, 0.9, 0.05, W.ACT_GELU_TANH) <= 2
+
+
 @pytest.mark.parametrize("mean,spread", [(-10.0, 0.3), (-20.0, 1.0), (-9.0, 0.2), (9.5, 0.3)])
 def test_range_search_of_saturated_neurons(mean, spread):
     # far out the tanh form of GELU is exactly 0 (z): every error is exactly 0, every choice a tie, and the right side is grown
@@ -391,6 +406,46 @@ def test_build_predictor_groups_and_superblocks(h, d, G):
     g = torch.Generator().manual_seed(h)
     W1 = (torch.randn(h, d, generator=g) * 0.02).cuda()
     _build_and_compare(W1, _upper_factor(torch.randn(2 * d, d, generator=g).numpy()), 2, G)
+
+
+# k_build takes up to 56 neurons per CTA in eights, 128 channels at a time: row counts around those (16 rows are added to measure the
+# growth of rounding errors), a last block of 64 channels, both group sizes, all code widths
+@pytest.mark.parametrize("h,d,G,bits", [(1, 64, 64, 2), (112, 128, 128, 4), (113, 192, 64, 3), (2353, 256, 64, 8), (4721, 320, 64, 2), (16561, 128, 128, 2)])
+def test_build_predictor_one_launch_edges(h, d, G, bits):
+    g = torch.Generator().manual_seed(h + d)
+    W1 = (torch.randn(h, d, generator=g) * 0.03).bfloat16().cuda()
+    X = torch.randn(3 * d, d, generator=g) @ (torch.eye(d) + 0.5 * torch.randn(d, d, generator=g) / d ** 0.5)
+    rows = np.unique(np.concatenate([np.arange(0, h, max(1, h // 50)), np.arange(max(0, h - 20), h)]))
+    _build_and_compare(W1, _upper_factor(X.numpy()), bits, G, rows)
+
+
+@pytest.mark.parametrize("kind", ["identity", "blocks", "growing", "infinite"])
+def test_build_predictor_close_decisions_are_done_again(kind):
+    """Weights that lie on rounding boundaries, or may for all that the quick arithmetic can tell: a factor that leaves channels
+    uncoupled (bf16 weights then tie exactly), one whose recurrence magnifies every rounding error, a weight that is no number."""
+    h, d, G = 200, 256, 64
+    g = torch.Generator().manual_seed(5)
+    W1 = (torch.randn(h, d, generator=g) * 0.03).bfloat16()
+    X = torch.randn(3 * d, d, generator=g).numpy()
+    if kind == "identity":
+        U = np.eye(d)
+    elif kind == "blocks":
+        X[:, : d // 2] = 0.0
+        U = _upper_factor(X + 1e-30)
+        U[: d // 2] = np.eye(d)[: d // 2]
+    elif kind == "growing":
+        U = np.triu(torch.randn(d, d, generator=g).double().numpy() * 0.5, 1) + np.eye(d)
+    else:
+        U = _upper_factor(X)
+        W1[3, 17] = float("inf")
+    if kind == "infinite":                                          # the other neurons are what they are without it
+        codes, scale, zero = T.tardis_build_predictor(W1.cuda(), torch.from_numpy(U).cuda(), 2, G)
+        W1[3, 17] = 0.0
+        ref = T.tardis_build_predictor(W1.cuda(), torch.from_numpy(U).cuda(), 2, G)
+        keep = torch.arange(h, device="cuda") != 3
+        assert all(bool(torch.equal(x[keep], y[keep])) for x, y in zip((codes, scale, zero), ref))
+        return
+    _build_and_compare(W1.cuda(), U, 2, G)
 
 
 def test_build_predictor_full_size_sampled_rows_and_use_in_a_layer():

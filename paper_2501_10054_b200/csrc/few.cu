@@ -60,15 +60,17 @@ struct OutParams {
   unsigned int* nfl; unsigned long long* counters;
 };
 
-template <int N> struct InCfg {
+template <int N, int BITS> struct InCfg {
   static constexpr int X_BYTES = N * BK * 2, STAGE = W_BYTES + X_BYTES;
-  static constexpr int NS = N == 128 ? 6 : (N == 64 ? 8 : (N == 32 ? 10 : 11));
-  static constexpr int NBUF = N == 64 ? 2 : 4;                      // expanded predictor blocks in TMEM (32 columns each)
+  static constexpr int NS = N == 128 ? 6 : (N == 64 ? 9 : (N == 32 ? 11 : 12));
+  // expanded predictor blocks in TMEM (32 columns each).  4-bit codes come as two blocks each, and their expansion waits for the launch
+  // before anyway: as many as fit (3328 / 13312, 40 tokens: 80 us with six, 95 with two); 2-bit codes are no faster with six
+  static constexpr int NBUF = N == 128 ? 4 : (BITS == 4 ? 8 : (N == 64 ? 2 : 4));
   static constexpr int COL_S = 0, COL_Z = N, COL_F = 2 * N, COL_A = 3 * N;
   // (an allocation is a power of two; a kernel that takes all 512 columns does so only behind the wait, they may be another's until then)
   static constexpr int TMEM = COL_A + NBUF * 32 <= 256 ? 256 : 512;
-  static constexpr int SMEM = 1024 + NS * STAGE + BARS + MAX_NEAR * 16 + BM * ((N + 31) / 32) * 4 + N * 8 + 8 * 1024;
-  static_assert((2 * NS + 2 * NBUF + 5) * 8 + 16 <= BARS, "barriers");
+  static constexpr int SMEM = 1024 + NS * STAGE + BARS + MAX_NEAR * 16 + BM * ((N + 31) / 32) * 4 + N * 8;
+  static_assert((2 * NS + 2 * NBUF + 5) * 8 + 16 + 64 <= BARS, "barriers, parts of re-evaluated scores");
   static_assert(SMEM <= 232448, "shared memory");
 };
 template <int N> struct OutCfg {
@@ -219,7 +221,7 @@ template <int N, int TERMS, int BITS>
 __global__ void __launch_bounds__(NT_IN, 1)            // (one CTA per SM: its shared memory)
 k_few_in(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUtensorMap tmWf, const __grid_constant__ CUtensorMap tmX,
          const InParams p) {
-  using C = InCfg<N>;
+  using C = InCfg<N, BITS>;
   constexpr int VEC = BITS / 2, AHEAD = BITS == 2 ? 4 : 2;   // 16-byte vectors of a block's neuron; blocks fetched ahead (in registers)
   constexpr int RING = C::NBUF / 2;                    // expanded blocks per group of four warps
   constexpr int HALF = N / 2;                          // token columns per epilogue thread
@@ -238,11 +240,11 @@ k_few_in(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUten
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(norm_ready + 1);
   volatile uint32_t* failed = tmem_slot + 1;
   uint32_t* near_count = tmem_slot + 2;
+  double* near_part = reinterpret_cast<double*>(smem + C::NS * C::STAGE + BARS - 64);   // [8 warps]
   uint4* near = reinterpret_cast<uint4*>(smem + C::NS * C::STAGE + BARS);         // [MAX_NEAR] row << 8 | token, lo, hi, b1
   uint32_t* settled = reinterpret_cast<uint32_t*>(near + MAX_NEAR);               // [BM][(N + 31) / 32] re-evaluated scores that are outside
   float* x1 = reinterpret_cast<float*>(settled + BM * ((N + 31) / 32));           // [N] sum |x|
   unsigned int* tok_flagged = reinterpret_cast<unsigned int*>(x1 + N);            // [N]
-  float* staging = reinterpret_cast<float*>(tok_flagged + N);                     // [8 warps][8][32]
 
   const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // (warp: uniform, and known to be)
   const int nkb = p.nkb;
@@ -278,7 +280,7 @@ k_few_in(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUten
     Walk w(p, wf), first = w;
     const int ahead = min(C::NS, w.total);
     auto bytes = [&](const Walk& at) { return uint32_t((at.folded ? BM : p.rows) * BK * 2 + C::X_BYTES); };
-    auto weights = [&](const Walk& at, int s) { tma_load_2d(smem + s * C::STAGE, at.folded ? &tmWf : &tmW1, at.kb * BK, at.row0, &full[s]); };
+    auto weights = [&](const Walk& at, int s) { tma_load_2d_once(smem + s * C::STAGE, at.folded ? &tmWf : &tmW1, at.kb * BK, at.row0, &full[s]); };
     auto tokens = [&](const Walk& at, int s) { tma_load_2d(smem + s * C::STAGE + W_BYTES, &tmX, at.kb * BK, 0, &full[s]); };
     for (int s = 0; s < ahead; ++s, w.next())              // constant state: before the wait
       if (elect_one()) { mbar_expect_tx(&full[s], bytes(w)); weights(w, s); }
@@ -391,7 +393,6 @@ k_few_in(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUten
     const uint32_t lanes = tmem + (uint32_t(q * 32) << 16);
     const int row = q * 32 + lane, rows = p.rows;
     const bool holds = q * 32 < rows;                      // any row of this warp is in use
-    float* const stage = staging + (warp - 4) * 256;
     const int kpg = p.G / BK;                              // channel blocks per predictor group
     int ati = 0, own = 0;
     bool ok = true;
@@ -495,20 +496,35 @@ k_few_in(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUten
       asm volatile("bar.sync 1, 256;" ::: "memory");
       const uint32_t nn = *near_count;
       if (nn > 0) {                                        // (the same for all eight warps)
-        for (uint32_t e = warp - 4; e < min(nn, uint32_t(MAX_NEAR)); e += 8) {
-          const uint4 pair = near[e];
-          const int r = int(pair.x >> 8), t = int(pair.x & 255u);
-          const float rl = __uint_as_float(pair.y), rh = __uint_as_float(pair.z), rb = __uint_as_float(pair.w);
-          double z = exact_from_packed<BITS>(tile_codes + r, tile_meta + r, p.x + size_t(t) * p.d, nkb * 4 * VEC, kpg, rows, lane, 32);
+        // A warp per pair, eight at a time; of the last round's four or fewer the warps share out the channels: a round takes 4 to 6 us for a
+        // whole row, two rounds of loads and of dependent sums, and the other warps would wait for it
+        const uint32_t queued = min(nn, uint32_t(MAX_NEAR)), left = queued & 7u, alone = left <= 4 ? queued - left : queued;
+        const uint32_t parts = left == 0 || left > 4 ? 1u : (left == 1 ? 8u : (left == 2 ? 4u : 2u));
+        for (uint32_t e0 = 0; e0 < queued; e0 += 8) {
+          const bool whole = e0 < alone;
+          const uint32_t np = whole ? 1u : parts, e = e0 + uint32_t(warp - 4) / np, part = uint32_t(warp - 4) % np;
+          if (e >= queued) break;
+          const int r = int(near[e].x >> 8), t = int(near[e].x & 255u);
+          double z = exact_from_packed<BITS>(tile_codes + r, tile_meta + r, p.x + size_t(t) * p.d, nkb * 4 * VEC, kpg, rows, int(part * 32) + lane, int(32 * np));
 #pragma unroll
           for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-          z += double(rb);
-          if (lane == 0) {
-            if (!(double(rl) <= z && z < double(rh))) atomicOr(&settled[r * ((N + 31) / 32) + (t >> 5)], 1u << (t & 31));
-            if (p.dbg_scores) p.dbg_scores[size_t(t) * p.h + tile * rows + r] = z;
-          }
+          if (lane != 0) continue;
+          if (!whole) { near_part[warp - 4] = z; continue; }
+          z += double(__uint_as_float(near[e].w));
+          if (!(double(__uint_as_float(near[e].y)) <= z && z < double(__uint_as_float(near[e].z))))
+            atomicOr(&settled[r * ((N + 31) / 32) + (t >> 5)], 1u << (t & 31));
+          if (p.dbg_scores) p.dbg_scores[size_t(t) * p.h + tile * rows + r] = z;
         }
         asm volatile("bar.sync 1, 256;" ::: "memory");
+        for (uint32_t e = alone; e < queued; ++e) {        // pairs in parts: settled by their neuron's thread
+          const int r = int(near[e].x >> 8), t = int(near[e].x & 255u) - gi * HALF;
+          if (r != row || t < 0 || t >= HALF) continue;
+          double z = 0.0;
+          for (uint32_t k = 0; k < parts; ++k) z += near_part[(e - alone) * parts + k];
+          z += double(b1);
+          if (!(double(lo) <= z && z < double(hi))) flags |= 1ull << t;
+          if (p.dbg_scores) p.dbg_scores[size_t(gi * HALF + t) * p.h + j] = z;
+        }
         if (threadIdx.x == 128) { atomicAdd(&p.counters[CTR_RECHECKS], (unsigned long long)nn); *near_count = 0u; }
         uint32_t* fix = &settled[row * ((N + 31) / 32)];
         if (HALF >= 32) {
@@ -519,35 +535,47 @@ k_few_in(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUten
         }
       }
       // -- counts per token; corrections act(z) - a z - c where flagged, zero elsewhere --
+      // Evaluated for every element, without branches: a walk over the set bits alone waits for its lane with the most of them, and for one
+      // activation after the other (64 columns of a tile: 5.9 us, now 3.1)
 #pragma unroll 1
       for (int c0 = 0; c0 < HALF; c0 += 8) {
         const uint32_t bits = uint32_t(flags >> c0) & 0xffu;
         float v[8];
         tmem_ld8(lanes + C::COL_Z + gi * HALF + c0, v);
+        uint32_t count = 0u;                               // lane e: flagged neurons of token column c0 + e
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
           const uint32_t word = __ballot_sync(0xffffffffu, (bits >> e) & 1u);
-          const int t = gi * HALF + c0 + e;
-          if (lane == 0 && t < p.n) {
-            if (word) atomicAdd(&tok_flagged[t], __popc(word));
-            if (p.dbg_bitmap && word) {                    // (cleared before the launch; a tile may begin inside a word)
+          if (lane == e) count = __popc(word);
+          if (p.dbg_bitmap) {                              // (cleared before the launch; a tile may begin inside a word)
+            const int t = gi * HALF + c0 + e;
+            if (lane == 0 && t < p.n && word) {
               atomicOr(p.dbg_bitmap + size_t(t) * (p.h / 32) + (j >> 5), word << (j & 31));
               if ((j & 31) && (word >> (32 - (j & 31)))) atomicOr(p.dbg_bitmap + size_t(t) * (p.h / 32) + (j >> 5) + 1, word >> (32 - (j & 31)));
             }
           }
-          stage[e * 32 + lane] = v[e];
         }
+        if (count && gi * HALF + c0 + lane < p.n) atomicAdd(&tok_flagged[gi * HALF + c0 + lane], count);
+        if (p.act == TARDIS_ACT_GELU_TANH) {
+#pragma unroll
+          for (int e = 0; e < 8; ++e) { const float z = v[e] + b1; v[e] = gelu_tanh_f32(z) - fa * z - fc; }
+        } else {
 #pragma unroll 1
-        for (uint32_t w = bits; w; w &= w - 1u) {
-          const int e = __ffs(w) - 1;
-          const float z = stage[e * 32 + lane] + b1;
-          stage[e * 32 + lane] = gelu_f32(z, p.act) - fa * z - fc;
+          for (int e = 0; e < 8; ++e) {                    // (rolled by hand: registers cannot be indexed)
+            float z = 0.f;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) z = q == e ? v[q] : z;
+            z += b1;
+            z = (bits >> e) & 1u ? gelu_f32(z, p.act) - fa * z - fc : 0.f;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) v[q] = q == e ? z : v[q];
+          }
         }
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
           if (c0 + e < cols) {
             const int t = gi * HALF + c0 + e;
-            const float dl = (bits >> e) & 1u ? stage[e * 32 + lane] : 0.f;
+            const float dl = (bits >> e) & 1u ? v[e] : 0.f;
             const __nv_bfloat16 h0 = __float2bfloat16_rn(dl);
             p.delta[size_t(t) * p.h + j] = h0;
             if (TERMS == 2) p.delta[size_t(N + t) * p.h + j] = __float2bfloat16_rn(dl - __bfloat162float(h0));
@@ -623,7 +651,7 @@ k_few_out(const __grid_constant__ CUtensorMap tmW2, const __grid_constant__ CUte
 
   if (warp == 0) {
     int m = begin / nkb, kb = begin - m * nkb, xb = kb;      // next pair; neuron block of the next token tile
-    auto weights = [&](int s) { tma_load_2d(smem + s * C::STAGE, &tmW2, kb * BK, m * BM, &full[s]); };
+    auto weights = [&](int s) { tma_load_2d_once(smem + s * C::STAGE, &tmW2, kb * BK, m * BM, &full[s]); };
     auto corrections = [&](int s) { tma_load_2d(smem + s * C::STAGE + W_BYTES, &tmD, xb * BK, 0, &full[s]); };
     auto next_weights = [&]() { if (++kb == nkb) { kb = 0; ++m; } };
     auto next_corrections = [&]() { if (++xb == nkb) xb = 0; };
@@ -879,9 +907,9 @@ tardis_status_t few_prepare(Handle* H) {
     if (e != cudaSuccess) { set_last_error(e, "cudaMalloc"); cudaGetLastError(); few_release(H); return TARDIS_ERR_ALLOC; }
   }
   auto room = [](auto kernel, int smem) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); };
-  const cudaError_t es[] = {room(k_few_in<16, 2, 2>, InCfg<16>::SMEM), room(k_few_in<32, 1, 2>, InCfg<32>::SMEM), room(k_few_in<64, 1, 2>, InCfg<64>::SMEM),
-                            room(k_few_in<128, 1, 2>, InCfg<128>::SMEM), room(k_few_in<16, 2, 4>, InCfg<16>::SMEM), room(k_few_in<32, 1, 4>, InCfg<32>::SMEM),
-                            room(k_few_in<64, 1, 4>, InCfg<64>::SMEM), room(k_few_in<128, 1, 4>, InCfg<128>::SMEM), room(k_few_out<32>, OutCfg<32>::SMEM),
+  const cudaError_t es[] = {room(k_few_in<16, 2, 2>, InCfg<16, 2>::SMEM), room(k_few_in<32, 1, 2>, InCfg<32, 2>::SMEM), room(k_few_in<64, 1, 2>, InCfg<64, 2>::SMEM),
+                            room(k_few_in<128, 1, 2>, InCfg<128, 2>::SMEM), room(k_few_in<16, 2, 4>, InCfg<16, 4>::SMEM), room(k_few_in<32, 1, 4>, InCfg<32, 4>::SMEM),
+                            room(k_few_in<64, 1, 4>, InCfg<64, 4>::SMEM), room(k_few_in<128, 1, 4>, InCfg<128, 4>::SMEM), room(k_few_out<32>, OutCfg<32>::SMEM),
                             room(k_few_out<64>, OutCfg<64>::SMEM), room(k_few_out<128>, OutCfg<128>::SMEM)};
   for (cudaError_t e : es)
     if (e != cudaSuccess) { set_last_error(e, "cudaFuncSetAttribute"); few_release(H); return TARDIS_ERR_CUDA; }
@@ -947,7 +975,8 @@ static tardis_status_t launch_n(Handle* H, const __nv_bfloat16* x, __nv_bfloat16
   a.wf_plan = S->plan; a.delta = S->delta; a.yacc = S->yacc; a.nfl = S->nfl; a.counters = H->counters;
   a.dbg_bitmap = H->dbg_bitmap; a.dbg_scores = H->dbg_scores;
   if (H->dbg_bitmap) TARDIS_CUDA_TRY(cudaMemsetAsync(H->dbg_bitmap, 0, size_t(n) * (H->h / 32) * 4, s));
-  TARDIS_CUDA_TRY(launch_overlapped(H->bits == 2 ? k_few_in<N, TERMS, 2> : k_few_in<N, TERMS, 4>, S->grid, NT_IN, InCfg<N>::SMEM, s, S->w1, S->wf, tmx, a));
+  static_assert(InCfg<N, 2>::SMEM == InCfg<N, 4>::SMEM, "one size");
+  TARDIS_CUDA_TRY(launch_overlapped(H->bits == 2 ? k_few_in<N, TERMS, 2> : k_few_in<N, TERMS, 4>, S->grid, NT_IN, InCfg<N, 2>::SMEM, s, S->w1, S->wf, tmx, a));
   OutParams o = {};
   o.n = n; o.d = H->d; o.h = H->h; o.nkb = S->out_nkb; o.total = S->mtiles * S->out_nkb; o.terms = TERMS;
   o.bf = H->bf; o.yacc = S->yacc; o.y = y; o.done = S->done; o.parts = S->parts; o.nfl = S->nfl; o.counters = H->counters;

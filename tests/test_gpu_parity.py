@@ -581,6 +581,41 @@ def test_kernels_for_a_few_tokens_at_the_edges_of_their_tiles(d, h, G, q):
     _run(cfg, sum(calls), calls, path=3)
 
 
+@pytest.mark.parametrize("d,bits,n", [(512, 2, 5), (576, 2, 16), (512, 2, 40), (512, 4, 33), (512, 2, 128)])
+def test_scores_near_range_ends_in_every_number_per_tile(d, bits, n):
+    # 0 to 20 scores per tile that the fast sums cannot place: a warp for each of eight, the last one to four shared out.  Tiles have 16
+    # neurons here (2048 over 148 CTAs); the ends lie 2e-5 above or below scores of two tokens, well inside the allowance and well
+    # outside the band in which either outcome is right
+    h = 2048
+    cfg = W.LayerConfig("nearends", d, h, group=64, n_calib=256, bits=bits)
+    L = _layer(cfg, 3)
+    x = W.make_tokens(cfg, n, 3).cuda()
+    s = L.numpy64()
+    zhat = O.predictor_score(x.double().cpu().numpy(), s["codes"], s["scale"], s["zero"], s["group"], s["b1"], s["bits"])
+    lo = np.full(h, -50.0)
+    hi = np.full(h, 50.0)
+    wanted = 0
+    for tile in range(h // 16):
+        k = tile % 21
+        wanted += k
+        for i in range(k):
+            j, off = tile * 16 + i % 16, 2e-5 if (tile + i) % 3 else -2e-5
+            if i < 16:
+                lo[j] = zhat[0, j] + off
+            else:
+                hi[j] = max(zhat[n - 1, j] + off, lo[j] + 1e-3)
+    L.lo.copy_(torch.from_numpy(lo))
+    L.hi.copy_(torch.from_numpy(hi))
+    h1 = T.fold_layer(L)
+    try:
+        T.tardis_set_path(h1, 3)
+        y, F, S = Hp.gpu_forward(h1, L, x)
+        Hp.assert_parity(L, L.numpy64(), x, y, F, S, label="near ends", score_tol=3e-4)
+        assert T.tardis_stats(h1)["exact_rechecks"] >= 0.9 * wanted
+    finally:
+        T.tardis_destroy(h1)
+
+
 @pytest.mark.parametrize("d,h,G,q", [(64, 32, 64, 0.4), (192, 160, 64, 0.2), (1088, 4640, 64, 0.05), (1024, 4096, 128, 0.1)])
 def test_kernels_for_a_few_tokens_with_4_bit_codes(d, h, G, q):
     # one channel block and several, an odd number of them, tiles with a short last one, every width of the token columns

@@ -10,10 +10,9 @@
 //      capture).  Products are exact, the fp32 accumulation is not: a score within
 //      tau(t, j) = kEps * (2^bits - 1) max_g s[j,g] * |x_t|_1 of a range end is queued by the epilogue and
 //      re-evaluated in fp64 from the packed codes (k_recheck), so the flags are the exact ones;
-//   2. speculative product    Yacc = X W_f^T + b_f                               (fp32);
-//   3. result fixing          Delta = flag .* (GELU(Z) - a Z - c), Z = X W1^T + b1   (GEMM with that epilogue, bf16),
-//                             y = bf16(Yacc + Delta W2^T)                            (GEMM over all neurons:
-//      with independent ~10 % flags the union over >= 64 tokens is practically every neuron, which is why
+//   2. result fixing          Delta = flag .* (GELU(Z) - a Z - c), Z = X W1^T + b1   (GEMM with that epilogue, bf16);
+//   3. output                 y = bf16(X W_f^T + b_f + Delta W2^T), the speculative product and the corrections over all neurons in one
+//      GEMM (with independent ~10 % flags the union over >= 64 tokens is practically every neuron, which is why
 //      the paper expects little gain for prompt-heavy requests).
 #include <vector>
 
@@ -27,6 +26,7 @@ namespace bat {
 // Tokens per pass (the scratch is sized for this).  With 2048 the big products have 16 x 64 tiles = 6.9 waves of
 // 148 CTAs; 1024-token chunks lost 15 % of the time to their last, partial wave.
 constexpr int kChunk = 2048;
+constexpr int kSplitTokens = 128;            // calls of up to this many split their output product, whose parts meet in an fp32 array
 constexpr int kChunkCapture = 1024;          // ... while the debug capture is on (the score buffer holds that many)
 constexpr float kEps = 7.62939453125e-6f;    // 2^-17: relative accumulation-error allowance of the fast scores
 // neurons per token that can queue for re-evaluation: a sixteenth, some ten times what narrow ranges of a 4096 / 16384 layer need (the
@@ -37,7 +37,7 @@ struct State {
   __nv_bfloat16 *Wf, *W2, *What_hi, *What_lo;     // [d,d], [d,h], [h,d], [h,d]
   float* smaxrow;                                  // [h] largest group scale of a neuron
   uint32_t* lo_used;                               // [h / 128 rounded up] bit 0: What_lo is not zero in those rows; bit 1: some |q - zp| > 2
-  float *zhat, *yacc, *x1;                         // [kChunkCapture,h] (scores for the capture; fold temporary), [kChunk,d], [kChunk]
+  float *zhat, *yacc, *x1;                         // [kChunkCapture,h] (scores for the capture; fold temporary), [kSplitTokens,d], [kChunk]
   __nv_bfloat16* delta;                            // [kChunk,h]
   uint32_t* bitmap;                                // [kChunk,h/32]
   uint32_t* rlist;                                 // [kChunk][max_recheck(h)] neurons of a token to re-evaluate
@@ -129,10 +129,15 @@ __global__ void __launch_bounds__(256) k_recheck(const uint32_t* __restrict__ rl
                                                  const float* __restrict__ lo, const float* __restrict__ hi, const __nv_bfloat16* __restrict__ x, int d, int h,
                                                  int G, int bits, uint32_t* __restrict__ bitmap, float* __restrict__ zhat, unsigned long long* counters) {
   extern __shared__ double xd[];                           // channel c of unit u (16 channels) at c (d / 16 + 1) + u: the lanes' units side by side
-  __shared__ unsigned int flagged;
+  __shared__ unsigned int flagged;                         // the token's
   const int t = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned int queued = rcount[t];
   const unsigned int most = max_recheck(h);
+  // asked for together with the token: the warp's first neuron (the queue has room for 512 at least, so there is something to read), and
+  // the token's flags, counted before any of them changes
+  const int first = min(int(rlist[size_t(t) * most + warp] & 0x7fffffffu), h - 1);
+  int count = 0;
+  for (int w = threadIdx.x; w < h / 32; w += blockDim.x) count += __popc(__ldcg(bitmap + size_t(t) * (h / 32) + w));
   const bool all = queued > most;
   const unsigned int total = all ? (unsigned int)h : queued;
   const __nv_bfloat16* const xt = x + size_t(t) * d;
@@ -152,7 +157,7 @@ __global__ void __launch_bounds__(256) k_recheck(const uint32_t* __restrict__ rl
   __syncthreads();
   const int ng = d / G;
   for (unsigned int e = warp; e < total; e += 8) {
-    const int j = all ? int(e) : int(rlist[size_t(t) * most + e]);
+    const int j = all ? int(e) : (e < 8 ? first : int(rlist[size_t(t) * most + e]));
     const uint32_t* const row = codes + size_t(j) * (size_t(d) * bits / 32);
     double z = 0.0;
     // units of 16 channels (all of one group), four at a time: their loads go out before the first is used, since waiting for them
@@ -196,16 +201,14 @@ __global__ void __launch_bounds__(256) k_recheck(const uint32_t* __restrict__ rl
     if (lane == 0) {
       const bool inside = (double(lo[j]) <= z) && (z < double(hi[j]));
       uint32_t* wp = bitmap + size_t(t) * (h / 32) + (j >> 5);
-      if (inside) atomicAnd(wp, ~(1u << (j & 31)));
-      else atomicOr(wp, 1u << (j & 31));
+      const uint32_t bit = 1u << (j & 31);
+      if (inside) count -= atomicAnd(wp, ~bit) & bit ? 1 : 0;
+      else count += atomicOr(wp, bit) & bit ? 0 : 1;
       if (zhat) zhat[size_t(t) * h + j] = float(z);
     }
   }
-  __threadfence_block();
-  __syncthreads();
-  unsigned int c = 0;
-  for (int w = threadIdx.x; w < h / 32; w += blockDim.x) c += __popc(__ldcg(bitmap + size_t(t) * (h / 32) + w));
-  c = __reduce_add_sync(0xffffffffu, c);
+  __syncwarp();
+  const unsigned int c = __reduce_add_sync(0xffffffffu, unsigned(count));       // (modulo 2^32, like the sum it goes into)
   if (lane == 0) atomicAdd(&flagged, c);
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -266,7 +269,7 @@ Requests requests(State* S, int d, int h) {
       {reinterpret_cast<void**>(&S->Wf), size_t(d) * d * 2, false}, {reinterpret_cast<void**>(&S->W2), hd * 2, false},
       {reinterpret_cast<void**>(&S->What_hi), hd * 2, false},       {reinterpret_cast<void**>(&S->What_lo), hd * 2, false},
       {reinterpret_cast<void**>(&S->smaxrow), size_t(h) * 4, false}, {reinterpret_cast<void**>(&S->lo_used), size_t((h + 127) / 128) * 4, false},
-      {reinterpret_cast<void**>(&S->zhat), size_t(kChunkCapture) * h * 4, true}, {reinterpret_cast<void**>(&S->yacc), size_t(kChunk) * d * 4, true},
+      {reinterpret_cast<void**>(&S->zhat), size_t(kChunkCapture) * h * 4, true}, {reinterpret_cast<void**>(&S->yacc), size_t(kSplitTokens) * d * 4, true},
       {reinterpret_cast<void**>(&S->x1), size_t(kChunk) * 4, true},       {reinterpret_cast<void**>(&S->delta), size_t(kChunk) * h * 2, true},
       {reinterpret_cast<void**>(&S->bitmap), size_t(kChunk) * (h / 32) * 4, true},
       {reinterpret_cast<void**>(&S->rlist), size_t(kChunk) * max_recheck(h) * 4, true},
@@ -441,31 +444,26 @@ tardis_status_t launch_batched_forward(Handle* H, const void* xv, void* yv, int6
                                                             H->dbg_bitmap ? H->dbg_bitmap + size_t(t0) * (h / 32) : nullptr,
                                                             H->dbg_scores ? H->dbg_scores + size_t(t0) * h : nullptr);
     }
-    // A batch of one tile of tokens is bound by weight traffic and its products over d outputs have few
-    // tiles: those split their channel range over several CTAs, which add into the fp32 accumulator.
-    // (not in deterministic mode: the order of those additions is not fixed)
-    const int splits = (n <= 128 && d <= 8192 && !H->deterministic) ? 4 : 1;
-    // 2. speculative folded product
-    GemmArgs f = {};
-    f.M = n; f.N = d; f.K1 = d; f.A1 = xc; f.lda1 = d; f.B1 = S->Wf; f.ldb1 = d;
-    f.epilogue = GEMM_EPI_F32; f.out_f32 = S->yacc; f.ldo = d; f.bias = H->bf; f.error_word = &H->counters[CTR_ERROR];
-    f.splits = splits;
-    if (splits > 1) TARDIS_CUDA_TRY(cudaMemsetAsync(S->yacc, 0, size_t(n) * d * sizeof(float), s));
-    st = launch_gemm(f, s);
-    if (st != TARDIS_OK) return st;
-    // 3. result fixing: exact pre-activations of every neuron, masked correction, output product
+    // 2. result fixing: exact pre-activations of every neuron, masked correction
     GemmArgs z = {};
     z.M = n; z.N = h; z.K1 = d; z.A1 = xc; z.lda1 = d; z.B1 = H->W1; z.ldb1 = d;
     z.epilogue = GEMM_EPI_DELTA; z.out_bf16 = S->delta; z.ldo = h; z.bias = H->b1; z.a = H->a; z.c = H->c; z.bitmap = S->bitmap;
     z.act = H->act; z.error_word = &H->counters[CTR_ERROR];
     st = launch_gemm(z, s);
     if (st != TARDIS_OK) return st;
+    // 3. y = X W_f^T + b_f + Delta W2^T, one product over d + h channels (two products that meet in an fp32 array write and read it and
+    // end in a partial wave of CTAs each: 16384 tokens of 4096 / 16384 6.64 ms, now 6.30).  A batch of one tile of tokens is bound by weight traffic and has few tiles: it splits its
+    // channel range over several CTAs, which add into the fp32 accumulator.
+    // (not in deterministic mode: the order of those additions is not fixed)
+    const int splits = (n <= kSplitTokens && d <= 8192 && !H->deterministic) ? 4 : 1;
     GemmArgs o = {};
-    o.M = n; o.N = d; o.K1 = h; o.A1 = S->delta; o.lda1 = h; o.B1 = S->W2; o.ldb1 = h; o.ldo = d; o.error_word = &H->counters[CTR_ERROR];
+    o.M = n; o.N = d; o.K1 = d; o.A1 = xc; o.lda1 = d; o.B1 = S->Wf; o.ldb1 = d; o.K2 = h; o.A2 = S->delta; o.lda2 = h; o.B2 = S->W2; o.ldb2 = h;
+    o.ldo = d; o.bias = H->bf; o.error_word = &H->counters[CTR_ERROR];
     if (splits > 1) {
+      TARDIS_CUDA_TRY(cudaMemsetAsync(S->yacc, 0, size_t(n) * d * sizeof(float), s));
       o.epilogue = GEMM_EPI_F32; o.out_f32 = S->yacc; o.splits = splits;
     } else {
-      o.epilogue = GEMM_EPI_ADD_BF16; o.out_bf16 = y + size_t(t0) * d; o.addend = S->yacc;
+      o.epilogue = GEMM_EPI_BF16; o.out_bf16 = y + size_t(t0) * d;
     }
     st = launch_gemm(o, s);
     if (st != TARDIS_OK) return st;
@@ -473,7 +471,7 @@ tardis_status_t launch_batched_forward(Handle* H, const void* xv, void* yv, int6
       const size_t cnt = size_t(n) * d;
       k_round_store<<<unsigned((cnt / 4 + 255) / 256 + 1), 256, 0, s>>>(S->yacc, y + size_t(t0) * d, cnt);
     }
-    H->launches += 8 + ((H->dbg_bitmap || H->dbg_scores) ? 1 : 0);
+    H->launches += 5 + (splits > 1 ? 1 : 0) + ((H->dbg_bitmap || H->dbg_scores) ? 1 : 0);
   }
   TARDIS_CUDA_TRY(cudaGetLastError());
   return TARDIS_OK;

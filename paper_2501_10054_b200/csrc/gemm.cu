@@ -60,7 +60,7 @@ struct KParams {
   int epilogue, ldo, act, splits;
   int fast_m, band;            // tile raster (see decode() in the kernel)
   float* out_f32; __nv_bfloat16* out_bf16;
-  const float *bias, *addend, *a, *c;
+  const float *bias, *a, *c;
   const uint32_t* bitmap;
   unsigned long long* error_word;
   const float *lo, *hi, *colscale, *rowscale;
@@ -156,16 +156,13 @@ __device__ __forceinline__ void epilogue_chunk(const KParams& p, float (&v)[32],
     }
   } else {
     // bf16 outputs: this thread's 32 values become four 16-byte stores
-    if (p.epilogue == GEMM_EPI_ADD_BF16) {
-      const float* ad = p.addend + size_t(m) * p.ldo + n;
-      if (nv == 32 && (p.ldo & 3) == 0) {
+    if (p.epilogue == GEMM_EPI_BF16) {
+      const float* const bias = p.bias + n;
+      if (nv == 32) {
 #pragma unroll
-        for (int i = 0; i < 32; i += 4) {
-          const float4 t = *reinterpret_cast<const float4*>(ad + i);
-          v[i] += t.x; v[i + 1] += t.y; v[i + 2] += t.z; v[i + 3] += t.w;
-        }
+        for (int i = 0; i < 32; ++i) v[i] += bias[i];
       } else {
-        for (int i = 0; i < nv; ++i) v[i] += ad[i];
+        for (int i = 0; i < nv; ++i) v[i] += bias[i];
       }
     } else {   // GEMM_EPI_DELTA: one flag word covers this thread's 32 columns
       // Only the flagged tenth of the elements needs the activation, at different columns in every row: the
@@ -428,7 +425,7 @@ static tardis_status_t launch_bn(const GemmArgs& g, cudaStream_t s) {
   p.M = g.M; p.N = g.N; p.kb1 = (g.K1 + BK - 1) / BK; p.kb2 = g.K2 > 0 ? (g.K2 + BK - 1) / BK : 0;
   p.second_used = g.second_used; p.epilogue = g.epilogue; p.ldo = g.ldo; p.act = g.act; p.splits = g.splits > 1 ? g.splits : 1;
   p.out_f32 = g.out_f32; p.out_bf16 = static_cast<__nv_bfloat16*>(g.out_bf16);
-  p.bias = g.bias; p.addend = g.addend; p.a = g.a; p.c = g.c; p.bitmap = g.bitmap; p.error_word = g.error_word;
+  p.bias = g.bias; p.a = g.a; p.c = g.c; p.bitmap = g.bitmap; p.error_word = g.error_word;
   p.lo = g.lo; p.hi = g.hi; p.colscale = g.colscale; p.rowscale = g.rowscale; p.keps = g.keps; p.bitmap_out = g.bitmap_out;
   p.rlist = g.rlist; p.rcount = g.rcount; p.rcap = g.rcap; p.bits = g.bits;
   static thread_local int room_on = -1;               // the device on which this thread last gave the kernel its shared memory
@@ -468,9 +465,10 @@ tardis_status_t launch_gemm(const GemmArgs& g, cudaStream_t s) {
   if (g.epilogue == GEMM_EPI_FLAGS && !(g.bias && g.lo && g.hi && g.colscale && g.rowscale && g.bitmap_out && g.rlist && g.rcount))
     return TARDIS_ERR_INVALID_ARG;
   if (g.splits > 1 && g.epilogue != GEMM_EPI_F32) return TARDIS_ERR_INVALID_ARG;
+  if (g.epilogue == GEMM_EPI_BF16 && !g.bias) return TARDIS_ERR_INVALID_ARG;
   // the epilogues store (or reduce) 16 bytes at a time
   auto misaligned = [](const void* p) { return p && (reinterpret_cast<uintptr_t>(p) & 15u); };
-  if (misaligned(g.out_f32) || misaligned(g.out_bf16) || misaligned(g.addend)) return TARDIS_ERR_INVALID_ARG;
+  if (misaligned(g.out_f32) || misaligned(g.out_bf16)) return TARDIS_ERR_INVALID_ARG;
   // wide tiles when they still fill the machine, narrow ones for skinny problems
   const long splits = g.splits > 1 ? g.splits : 1, nm = (g.M + BM - 1) / BM, nn = (g.N + 255) / 256;
   if (nm * nn * splits < 120) return launch_bn<128, 1>(g, s);

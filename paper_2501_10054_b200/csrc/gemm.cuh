@@ -12,7 +12,7 @@ namespace tardis {
 
 enum GemmEpilogue {
   GEMM_EPI_F32 = 0,        // out_f32[m, n] = acc + (bias ? bias[n] : 0)
-  GEMM_EPI_ADD_BF16 = 1,   // out_bf16[m, n] = bf16(acc + addend_f32[m, n])
+  GEMM_EPI_BF16 = 1,       // out_bf16[m, n] = bf16(acc + bias[n])
   GEMM_EPI_DELTA = 2,      // z = acc + bias[n]; out_bf16[m, n] = flagged(m, n) ? GELU(z) - a[n] z - c[n] : 0
   GEMM_EPI_FLAGS = 3       // z = acc + bias[n]; bit (m, n) of bitmap_out = !(lo[n] <= z < hi[n]); a z within
                            // keps * colscale[n] * rowscale[m] of lo[n] or hi[n] is queued in rlist for exact
@@ -32,8 +32,7 @@ struct GemmArgs {
                                     // ADD their parts to out_f32 (the caller zeroes it first); the bias is added once
   float* out_f32; void* out_bf16;   // row-major, leading dimension ldo
   int ldo;
-  const float* bias;                // [N] or null
-  const float* addend;              // [M, ldo] fp32 (GEMM_EPI_ADD_BF16)
+  const float* bias;                // [N] or null (not with GEMM_EPI_BF16)
   const float *a, *c;               // [N] (GEMM_EPI_DELTA)
   const uint32_t* bitmap;           // [M, N / 32] flag words (GEMM_EPI_DELTA)
   int act;

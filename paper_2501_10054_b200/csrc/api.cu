@@ -174,6 +174,11 @@ static tardis_status_t settle(cudaStream_t s) {
   return TARDIS_OK;
 }
 
+// Whether a chain's layer of n tokens is one launch of the fused kernel: the calls that tardis_ffn_forward gives to it as one launch.
+bool fused_chain_serves(const Handle* H, int64_t n) {
+  return H->fscratch && n <= 4 && !H->deterministic && (H->path_override == 0 || H->path_override == 2);
+}
+
 // Allocates a handle and its device arrays for a layer of the given shape (nothing is filled in yet).
 static tardis_status_t new_handle(int d, int h, int dtype, int act, int G, int bits, cudaStream_t s, Handle** out) {
   *out = nullptr;

@@ -90,7 +90,16 @@ void decode_release(Handle* H);
 tardis_status_t decode_read_stamps(long long* out, int max_ctas);
 size_t fused_room(const Handle* H);                                        // what fused_prepare or decode_prepare will allocate
 tardis_status_t fused_prepare(Handle* H, cudaStream_t s);                  // builds the state of fused.cu (bf16, d_model <= 4608)
-tardis_status_t launch_fused_forward(Handle* H, const void* x, void* y, int n, cudaStream_t s);
+// A layer of a chain in one launch of the fused kernel: x is the residual stream s, the layer's input u is its normalisation (or s), and
+// with f the layer's output y becomes s + f (residual) or f; y may be x.  keep_in, keep_out: null, or where u and f go.
+struct FusedChain {
+  bool normalise, residual;
+  float eps;
+  const float *gamma, *beta;                                                  // null: ones and zeros
+  __nv_bfloat16 *keep_in, *keep_out;
+};
+tardis_status_t launch_fused_forward(Handle* H, const void* x, void* y, int n, cudaStream_t s, const FusedChain* chain = nullptr);
+bool fused_chain_serves(const Handle* H, int64_t n);
 void fused_release(Handle* H);
 tardis_status_t fused_set_deterministic(Handle* H, bool on);               // allocates the partial-output buffer of the mode
 tardis_status_t fused_read_stamps(long long* out, int max_ctas);

@@ -80,11 +80,12 @@ struct Params {
   int smem_total;          // dynamic shared memory of a CTA
   int gs_cap;              // result fixing: most neurons of a step (16, or 8 where that keeps one more predictor tile in shared memory)
   int nunits;              // folded-matrix units in all
+  FusedChain chain;        // where x is a residual stream (see common.cuh)
 };
 
 struct Scratch {           // handle-owned device memory of this path
   uint8_t* pblocks; int2* plan; float* smax; float* yacc; unsigned int* ctl; uint4* Cp;
-  Params base; size_t smem_bytes; size_t bytes; int grid; const void* kernels[3][2]; bool pairs_fit;
+  Params base; size_t smem_bytes; size_t bytes; int grid; const void* kernels[2][3][2]; bool pairs_fit;
   float* dpart;            // partial outputs of the deterministic mode (allocated when the mode is first switched on)
   int nbuf_n[MAXT + 1];    // tile buffers in shared memory for a call of n tokens
   int gs_cap_n[MAXT + 1];  // ... and the most neurons of a step of its result fixing
@@ -202,8 +203,9 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 // ---- the kernel ---------------------------------------------------------------------------------------
 // G: predictor group size; CT: 16-column output tiles per warp; NTK: tokens of the call (4: three or four; the others' token loops
 // fold away); FAST: every tile of the CTA has its own buffer and a warp has the same one or two channel
-// pairs in every tile (their x operands stay in registers), else the general loop over a ring of tile buffers.
-template <int G, int CT, int NTK, bool FAST>
+// pairs in every tile (their x operands stay in registers), else the general loop over a ring of tile buffers.  CHAIN: x is a residual
+// stream (see FusedChain; a kernel of its own because the code cost other calls 1 %).
+template <int G, int CT, int NTK, bool FAST, bool CHAIN>
 __global__ void __launch_bounds__(NTH, 1) k_fused(const Params p) {
   extern __shared__ __align__(128) uint8_t smem[];
   const SmemLayout L(p.dpad, p.ngroups, p.tiles_max, p.nbuf, p.buf_bytes, p.n, size_t(p.smem_total), p.gs_cap);
@@ -275,10 +277,124 @@ __global__ void __launch_bounds__(NTH, 1) k_fused(const Params p) {
     for (int i = tid; i < lines; i += NTH) asm volatile("prefetch.global.L2 [%0];" ::"l"(base + size_t(i) * 128));
   }
   const float smax_f = *p.smax;                    // constant state of the layer: fetched before the wait
+  // gamma and beta may be written by a launch of the caller's that is still running: asked into L2 now, read behind the wait
+  if (CHAIN && p.chain.normalise)
+    for (int i = (int(blockIdx.x) + int(gridDim.x) * tid) * 32; i < d; i += int(gridDim.x) * NTH * 32) {
+      if (p.chain.gamma) asm volatile("prefetch.global.L2 [%0];" ::"l"(p.chain.gamma + i));
+      if (p.chain.beta) asm volatile("prefetch.global.L2 [%0];" ::"l"(p.chain.beta + i));
+    }
 
   // From here on the kernel touches what earlier work in the stream may still be writing (x, the
   // scratch shared by the calls of one handle): wait until that work has completed and is visible.
   asm volatile("griddepcontrol.wait;" ::: "memory");
+
+  // ---- a layer of a chain: x is the residual stream, normalised here by every CTA, and left in shared memory for the next phase ----
+  if constexpr (CHAIN) {
+    // Item (token t, r): vectors r and r + 512 of the row, and sums in the order in which k_update_norm takes them (512 threads, the
+    // warps' sums in a tree of 16), so that a layer's input does not depend on which kernel normalises it.
+    constexpr int ITEMS = NTK == 4 ? 2 : 1, VECS = CT == 9 ? 2 : 1;    // (512 vectors are 4096 channels: CT 8)
+    uint4 raw[ITEMS][VECS];
+    float mean[ITEMS], rstd[ITEMS];
+    float* const parts = zpart;                                       // [2][n][16] (the predictor's; it starts later)
+    auto warp_sum = [&](float v) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      return v;
+    };
+    auto joined = [&](const float* at) {                              // every warp adds the same numbers in the same order
+      float v = at[lane & 15];
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      return v;
+    };
+    auto table = [&](float (&v)[8], const float* at, float none) {    // (the caller's: may begin anywhere)
+      if (!at) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = none;
+      } else if ((reinterpret_cast<uintptr_t>(at) & 15u) == 0) {
+        const float4 a = *reinterpret_cast<const float4*>(at), b = *reinterpret_cast<const float4*>(at + 4);
+        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+      } else {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = at[q];
+      }
+    };
+    float ga[8], be[8];                                               // of the thread's first vector, asked for with the row
+    auto tables = [&](int v) {
+      table(ga, p.chain.gamma ? p.chain.gamma + v * 8 : nullptr, 1.f);
+      table(be, p.chain.beta ? p.chain.beta + v * 8 : nullptr, 0.f);
+    };
+#pragma unroll
+    for (int k = 0; k < ITEMS; ++k)
+#pragma unroll
+      for (int e = 0; e < VECS; ++e) {
+        const int t = (k * NTH + tid) >> 9, v = (tid & 511) + 512 * e;
+        raw[k][e] = make_uint4(0u, 0u, 0u, 0u);
+        if (t < n && v < p.nvec) raw[k][e] = *reinterpret_cast<const uint4*>(p.x + size_t(t) * d + size_t(v) * 8);
+      }
+    if (p.chain.normalise) {
+      if (ITEMS * VECS == 1 && (tid >> 9) < n && (tid & 511) < p.nvec) tables(tid & 511);
+#pragma unroll
+      for (int k = 0; k < ITEMS; ++k) {
+        const int t = (k * NTH + tid) >> 9;                           // (the same for a warp)
+        float sum = 0.f;
+#pragma unroll
+        for (int e = 0; e < VECS; ++e) {
+          float f[8];
+          unpack8(f, raw[k][e]);
+#pragma unroll
+          for (int q = 0; q < 8; ++q) sum += f[q];
+        }
+        sum = warp_sum(sum);
+        if (t < n && lane == 0) parts[t * 16 + (warp & 15)] = sum;
+      }
+      __syncthreads();
+#pragma unroll
+      for (int k = 0; k < ITEMS; ++k) {
+        const int t = (k * NTH + tid) >> 9;
+        mean[k] = t < n ? joined(parts + t * 16) / float(d) : 0.f;
+        float sq = 0.f;
+#pragma unroll
+        for (int e = 0; e < VECS; ++e)
+          if ((tid & 511) + 512 * e < p.nvec) {
+            float f[8];
+            unpack8(f, raw[k][e]);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) { const float c = f[q] - mean[k]; sq += c * c; }
+          }
+        sq = warp_sum(sq);
+        if (t < n && lane == 0) parts[(n + t) * 16 + (warp & 15)] = sq;
+      }
+      __syncthreads();
+#pragma unroll
+      for (int k = 0; k < ITEMS; ++k) {
+        const int t = (k * NTH + tid) >> 9;
+        rstd[k] = t < n ? rsqrtf(joined(parts + (n + t) * 16) / float(d) + p.chain.eps) : 0.f;
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < ITEMS; ++k)
+#pragma unroll
+      for (int e = 0; e < VECS; ++e) {
+        const int t = (k * NTH + tid) >> 9, v = (tid & 511) + 512 * e;
+        if (t < n && v < nv) {
+          uint4 xw = raw[k][e];
+          if (v < p.nvec) {
+            if (p.chain.normalise) {
+              if (ITEMS * VECS > 1) tables(v);
+              float f[8];
+              unpack8(f, raw[k][e]);
+#pragma unroll
+              for (int q = 0; q < 8; ++q) f[q] = (f[q] - mean[k]) * rstd[k] * ga[q] + be[q];
+              xw = make_uint4(pack_bf16(f[0], f[1]), pack_bf16(f[2], f[3]), pack_bf16(f[4], f[5]), pack_bf16(f[6], f[7]));
+            }
+            if (p.chain.keep_in && blockIdx.x == 0) *reinterpret_cast<uint4*>(p.chain.keep_in + size_t(t) * d + size_t(v) * 8) = xw;
+          }
+          *reinterpret_cast<uint4*>(xh + t * XS + v * 8) = xw;
+        }
+      }
+    __syncthreads();                                                  // (the next phase deals the vectors out differently)
+  }
 
   // ---- x: bf16 copy in shared memory (channels beyond d and 16 more are zero), max |x|, sum |x| ----
   for (int base = 0; base < n * nv; base += NTH) {
@@ -286,8 +402,11 @@ __global__ void __launch_bounds__(NTH, 1) k_fused(const Params p) {
     if (i < n * nv) {                                // uniform over a warp (nv is a multiple of 32)
       const int t = i / nv, v = i - t * nv;
       uint4 xw = make_uint4(0u, 0u, 0u, 0u);
-      if (v < p.nvec) xw = *reinterpret_cast<const uint4*>(p.x + size_t(t) * d + size_t(v) * 8);
-      *reinterpret_cast<uint4*>(xh + t * XS + v * 8) = xw;
+      if (CHAIN) xw = *reinterpret_cast<const uint4*>(xh + t * XS + v * 8);
+      else {
+        if (v < p.nvec) xw = *reinterpret_cast<const uint4*>(p.x + size_t(t) * d + size_t(v) * 8);
+        *reinterpret_cast<uint4*>(xh + t * XS + v * 8) = xw;
+      }
       float f[8];
       unpack8(f, xw);
       float amax = 0.f, l1 = 0.f;
@@ -1052,6 +1171,7 @@ __global__ void __launch_bounds__(NTH, 1) k_fused(const Params p) {
     constexpr int ITEMS = (NTK * CTMAX * NW * 4 + NTH - 1) / NTH;   // vectors of 4 columns per thread
     const int nq = d >> 2, nitems = p.dpart ? 0 : n * nq;           // (deterministic mode: k_ordered_sum writes y)
     float4 sum[ITEMS], add[ITEMS];
+    uint2 stream[CHAIN ? ITEMS : 1];
 #pragma unroll
     for (int k = 0; k < ITEMS; ++k) {
       const int i = k * NTH + tid;
@@ -1059,6 +1179,7 @@ __global__ void __launch_bounds__(NTH, 1) k_fused(const Params p) {
         const int t = i / nq, c0 = (i - t * nq) * 4;
         sum[k] = __ldcg(reinterpret_cast<const float4*>(p.yacc + size_t(t) * p.dacc + c0));
         add[k] = *reinterpret_cast<const float4*>(p.bf + c0);
+        if constexpr (CHAIN) stream[k] = *reinterpret_cast<const uint2*>(p.x + size_t(t) * d + c0);
       }
     }
 #pragma unroll
@@ -1068,7 +1189,13 @@ __global__ void __launch_bounds__(NTH, 1) k_fused(const Params p) {
         const int t = i / nq, c0 = (i - t * nq) * 4;
         *reinterpret_cast<float4*>(p.yacc + size_t(t) * p.dacc + c0) = make_float4(0.f, 0.f, 0.f, 0.f);
         const uint32_t o0 = pack_bf16(add[k].x + sum[k].x, add[k].y + sum[k].y), o1 = pack_bf16(add[k].z + sum[k].z, add[k].w + sum[k].w);
-        *reinterpret_cast<uint2*>(p.y + size_t(t) * d + c0) = make_uint2(o0, o1);
+        uint2 o = make_uint2(o0, o1);
+        if constexpr (CHAIN) {                                        // (every CTA has read the stream: it may be replaced)
+          if (p.chain.keep_out) *reinterpret_cast<uint2*>(p.chain.keep_out + size_t(t) * d + c0) = o;
+          const uint2 w = stream[k];
+          if (p.chain.residual) o = make_uint2(pack_bf16(bf_lo(w.x) + bf_lo(o.x), bf_hi(w.x) + bf_hi(o.x)), pack_bf16(bf_lo(w.y) + bf_lo(o.y), bf_hi(w.y) + bf_hi(o.y)));
+        }
+        *reinterpret_cast<uint2*>(p.y + size_t(t) * d + c0) = o;
       }
     }
     FZ_STAMP(tid == 0, ST_FINAL);
@@ -1224,21 +1351,27 @@ tardis_status_t fused_prepare(Handle* H, cudaStream_t s) {
   k_max_scale<<<64, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(H->scale), size_t(h) * H->ngroups, S->smax);
   e = cudaGetLastError();
   const bool wide = dpad > 32 * 16 * 8;
-  // kernels[one token, two, three or four][ring or fast]
+  // kernels[a call, a layer of a chain][one token, two, three or four][ring or fast]
   auto choose = [&](auto g, auto ct) {
     constexpr int GG = decltype(g)::value, CC = decltype(ct)::value;
-    S->kernels[0][0] = (const void*)k_fused<GG, CC, 1, false>; S->kernels[0][1] = (const void*)k_fused<GG, CC, 1, true>;
-    S->kernels[1][0] = (const void*)k_fused<GG, CC, 2, false>; S->kernels[1][1] = (const void*)k_fused<GG, CC, 2, true>;
-    S->kernels[2][0] = S->kernels[2][1] = (const void*)k_fused<GG, CC, 4, false>;
+    auto both = [&](auto chain) {
+      constexpr bool CH = decltype(chain)::value;
+      const void* (&k)[3][2] = S->kernels[CH ? 1 : 0];
+      k[0][0] = (const void*)k_fused<GG, CC, 1, false, CH>; k[0][1] = (const void*)k_fused<GG, CC, 1, true, CH>;
+      k[1][0] = (const void*)k_fused<GG, CC, 2, false, CH>; k[1][1] = (const void*)k_fused<GG, CC, 2, true, CH>;
+      k[2][0] = k[2][1] = (const void*)k_fused<GG, CC, 4, false, CH>;
+    };
+    both(std::false_type());
+    both(std::true_type());
   };
   using std::integral_constant;
   if (G == 64 && wide) choose(integral_constant<int, 64>(), integral_constant<int, 9>());
   else if (G == 64) choose(integral_constant<int, 64>(), integral_constant<int, 8>());
   else if (wide) choose(integral_constant<int, 128>(), integral_constant<int, 9>());
   else choose(integral_constant<int, 128>(), integral_constant<int, 8>());
-  for (int a = 0; a < 3 && e == cudaSuccess; ++a)
+  for (int a = 0; a < 6 && e == cudaSuccess; ++a)
     for (int b = 0; b < 2 && e == cudaSuccess; ++b)
-      e = cudaFuncSetAttribute(S->kernels[a][b], cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
+      e = cudaFuncSetAttribute(S->kernels[a / 3][a % 3][b], cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
   S->pairs_fit = (p.nkc * 2 == NWP || (p.nkc * 2 >= 2 * NWP && p.nkc * 2 < 3 * NWP));
   if (e != cudaSuccess) { set_last_error(e, "fused_prepare launch"); return fail(TARDIS_ERR_CUDA); }
 
@@ -1296,7 +1429,8 @@ tardis_status_t fused_set_deterministic(Handle* H, bool on) {
   return TARDIS_OK;
 }
 
-tardis_status_t launch_fused_forward(Handle* H, const void* x, void* y, int n, cudaStream_t s) {
+// chain (may be null): see FusedChain; at most MAXT tokens then, and not in deterministic mode.
+tardis_status_t launch_fused_forward(Handle* H, const void* x, void* y, int n, cudaStream_t s, const FusedChain* chain) {
   Scratch* S = static_cast<Scratch*>(H->fscratch);
   const bool det = H->deterministic && S->dpart;
   for (int t0 = 0; t0 < n;) {
@@ -1312,6 +1446,7 @@ tardis_status_t launch_fused_forward(Handle* H, const void* x, void* y, int n, c
     p.dbg_bitmap = H->dbg_bitmap ? H->dbg_bitmap + size_t(t0) * (H->h / 32) : nullptr;
     p.dbg_scores = H->dbg_scores ? H->dbg_scores + size_t(t0) * H->h : nullptr;
     p.dpart = det ? S->dpart : nullptr;
+    if (chain) p.chain = *chain;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(S->grid); cfg.blockDim = dim3(NTH); cfg.dynamicSmemBytes = S->smem_bytes; cfg.stream = s;
     cudaLaunchAttribute attr[1];
@@ -1320,7 +1455,7 @@ tardis_status_t launch_fused_forward(Handle* H, const void* x, void* y, int n, c
     cfg.attrs = attr; cfg.numAttrs = 1;
     void* args[] = {&p};
     const bool fast = S->pairs_fit && S->nbuf_n[nt] >= p.tiles_max;
-    TARDIS_CUDA_TRY(cudaLaunchKernelExC(&cfg, S->kernels[nt <= 2 ? nt - 1 : 2][fast ? 1 : 0], args));
+    TARDIS_CUDA_TRY(cudaLaunchKernelExC(&cfg, S->kernels[chain ? 1 : 0][nt <= 2 ? nt - 1 : 2][fast ? 1 : 0], args));
     H->launches += 1;
     if (det) {
       const int work = nt * (H->d >> 2);                    // warps

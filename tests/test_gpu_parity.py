@@ -662,6 +662,48 @@ def test_stack_normalisation_at_the_edges_of_its_vectors(d, dtype):
         T.tardis_destroy(h)
 
 
+@pytest.mark.parametrize("d,group,n", [(64, 64, 1), (320, 64, 2), (4096, 128, 1), (4096, 128, 4), (4544, 64, 2), (4608, 64, 3)])
+@pytest.mark.parametrize("aligned", [True, False])
+def test_chain_normalised_inside_the_fused_kernel(d, group, n, aligned):
+    # the row in less than one warp's vectors, in one vector per thread, several tokens' vectors per thread; tables that 16-byte loads can
+    # and cannot read; no tables; the last CTA's addition to the stream, in place and not
+    cfg = W.LayerConfig("chain%d" % d, d, 256, group=group, n_calib=64)
+    L = _layer(cfg, 1)
+    x = (W.make_tokens(cfg, n, 1).cuda().float() * 3 + 0.5).to(L.W1.dtype)
+    room = torch.empty(2, d + 1, device="cuda")
+    gam, bet = (r[:d] if aligned else r[1:] for r in room)
+    gam.copy_(torch.linspace(0.5, 2, d))
+    bet.copy_(torch.linspace(-1, 1, d))
+    h = T.fold_layer(L)
+    try:
+        for in_place, ga, be in ((False, [gam, gam], [bet, bet]), (True, None, [bet, bet]), (True, [gam, gam], None)):
+            xs = x.clone()
+            y = xs if in_place else torch.empty_like(x)
+            keep = torch.empty(2, 2, n, d, dtype=x.dtype, device="cuda")
+            T.tardis_stack_forward([h, h], xs, y, ga, be, keep=keep)
+            torch.cuda.synchronize()
+            assert in_place or torch.equal(xs, x)
+            s = x
+            for l in range(2):
+                u = torch.nn.functional.layer_norm(s.double(), (d,), None if ga is None else gam.double(), None if be is None else bet.double(), 1e-5)
+                # (one rounding to bf16, plus the fp32 mean and deviation)
+                assert ((keep[l, 0].double() - u).abs() <= 2.0 ** -8 * u.abs() + 3e-5).all()
+                f = torch.empty_like(x)
+                T.tardis_ffn_forward(h, keep[l, 0].contiguous(), f)
+                # (the same kernel on the same input: only the order of the sums differs)
+                assert (f.float() - keep[l, 1].float()).abs().max() <= 2.0 ** -7 * f.float().abs().max()
+                s = (s.float() + keep[l, 1].float()).to(x.dtype)
+            assert torch.equal(y, s)
+            T.tardis_set_deterministic(h, True)                      # (the small kernels between the layers: the same sums in the same order)
+            apart = torch.empty_like(keep)
+            T.tardis_stack_forward([h, h], x.clone(), torch.empty_like(x), ga, be, keep=apart)
+            torch.cuda.synchronize()
+            T.tardis_set_deterministic(h, False)
+            assert torch.equal(apart[0, 0], keep[0, 0])
+    finally:
+        T.tardis_destroy(h)
+
+
 def _at_range_ends(d, h, bits, group, seed):
     """A ReLU layer without biases whose ranges all end at 0."""
     L = _layer(W.LayerConfig("ends%d" % bits, d, h, bits=bits, group=group, n_calib=128, act=W.ACT_RELU, bias=False), seed)

@@ -55,6 +55,19 @@ __device__ __forceinline__ double activation_f64(double z, int act) {
   return 0.5 * z * (1.0 + tanh(u));
 }
 
+// e^v as straight-line code, so that a thread's samples are evaluated side by side (exp branches, and its calls come one after the other):
+// its Taylor series on |r| <= ln 2 / 2 (13 terms: 4e-18) times a power of two; v is taken into [-700, 700].
+__device__ __forceinline__ double exp_straight(double v) {
+  v = fmin(fmax(v, -700.0), 700.0);
+  const double t = fma(v, 1.4426950408889634, 6755399441055744.0), k = t - 6755399441055744.0;   // the nearest whole number, in t's low bits
+  const double r = fma(k, -2.3190468138462996e-17, fma(k, -0.6931471805599453, v));
+  double p = 1.0 / 6227020800.0;                           // 1 / 13!
+  p = fma(p, r, 1.0 / 479001600.0); p = fma(p, r, 1.0 / 39916800.0); p = fma(p, r, 1.0 / 3628800.0); p = fma(p, r, 1.0 / 362880.0);
+  p = fma(p, r, 1.0 / 40320.0); p = fma(p, r, 1.0 / 5040.0); p = fma(p, r, 1.0 / 720.0); p = fma(p, r, 1.0 / 120.0);
+  p = fma(p, r, 1.0 / 24.0); p = fma(p, r, 1.0 / 6.0); p = fma(p, r, 0.5); p = fma(p, r, 1.0); p = fma(p, r, 1.0);
+  return __hiloint2double(__double2hiint(p) + (__double2loint(t) << 20), __double2loint(p));
+}
+
 // The n samples of neuron j plus its bias, NT E values over the CTA (+inf beyond n): thread t gets samples e NT + t.
 template <int E> __device__ __forceinline__ void load_samples(float (&v)[E], const float* __restrict__ z, long long ldz,
                                                               const float* __restrict__ b1, int j, int n) {
@@ -288,18 +301,22 @@ k_calibrate(const float* __restrict__ z, long long ldz, const float* __restrict_
 //   * density: the samples fall into bins of a quarter of the kernel width (only those that hold any are kept: some 130 of 260
 //     possible ones); from the moments of the bins around it, each bin gets the Taylor polynomial of the density about its
 //     centre (Hermite polynomials, order 4 on both sides), which gives all samples' densities to 1e-5 N.  Only the samples within
-//     that of the best (some 30 of 2048) are evaluated as sums of exponentials in fp32, and of those only the ones that these
-//     cannot tell apart (a handful) in fp64.  All N^2 exponentials in fp64 took 95 % of the time at first; values and slopes at
-//     every 16th sample, with |F''| <= N, still left 300 samples' worth of exponentials.
+//     that of the best (some 30 of 2048) are looked at more closely: where they lie within a quarter of the kernel width, as they do
+//     around a single mode, one pass over the samples in fp64 gives the density's expansion about their middle and with it all their
+//     densities to 1e-12 N; else sums of exponentials in fp32 leave a handful.  What is left (almost always one) is evaluated in fp64.
+//     All N^2 exponentials in fp64 took 95 % of the time at first, the fp32 sums and the fp64 ones after them a quarter.
 //   * candidate errors: from moments of the samples that the steps on either side add (fp64, made for all steps at once and summed
-//     up by scans).  One warp walks the steps; its lanes hold the errors of all ranges that the next six steps can lead to, so
-//     that the chain of dependent fp64 instructions is paid once per six steps.  Two errors closer than the rounding bound of
-//     the moments (or moments that cancel) are evaluated by the definition; exact zeros of piecewise-linear activations, on
+//     up by scans).  The threads hold the errors of all ranges that the next 21 steps can lead to and decide for each what would be done
+//     from it, so that the chain of dependent fp64 instructions is paid once per 21 steps and the walk itself is a look per step (by
+//     one warp, six steps ahead and with the decisions made along the way, it was 40 % of the search).  Two errors closer than the
+//     rounding bound of the moments (or moments that cancel) are evaluated by the definition; exact zeros of piecewise-linear activations, on
 //     which the tie rule depends, thus stay exact.
-// 16384 neurons x 2048 samples: 2.5 ms (133 ms with every density and error evaluated as defined).
+// 16384 neurons x 2048 samples: 1.5 ms (2.5 before the expansion about the candidates' middle, the bins' sums without atomics and the
+// walk of all threads; 133 ms with every density and error evaluated as defined).
 constexpr int kMaxSearchSamples = 2048;
-constexpr int kMaxSteps = 160;           // steps on one side whose moments are made at once
-constexpr int kAhead = 6;                // steps that a warp looks ahead: 28 ranges
+constexpr int kMaxSteps = 128;           // steps on one side whose moments are made at once, a thread per step and side
+constexpr int kSeries = 10;              // terms of the density about the middle of the candidates
+constexpr int kAhead = 21;               // steps that the CTA looks ahead: 253 ranges, one per thread
 // Bins: samples within 5 standard deviations fill at most 10 / (0.25 * 1.06 N^-0.2) = 174 of them at N = 2048 (fewer below), and at
 // most N / 25 samples lie beyond.
 constexpr int kMaxBins = 272;
@@ -315,6 +332,12 @@ struct Bins {
   float centre[kMaxBins];                // from the smallest sample on
   float m[5][kMaxBins];                  // sum of offset^n / n! of the bin's samples, offsets from the centre in kernel widths
   float l[5][kMaxBins];                  // Taylor coefficients of the density about the centre
+  int start[kMaxBins + 1];               // position of the bin's first sample
+};
+struct Ahead {                           // of the ranges that the next steps can lead to
+  double err[NT];
+  float off[NT];
+  uint16_t next[NT];                     // number of the range that follows, what is done (two bits), steps from the first one
 };
 struct Steps {
   double m[2][5][kMaxSteps + 1];         // [side][moment][k]: what the first k steps add
@@ -352,25 +375,35 @@ template <int E> __device__ __forceinline__ int densest_sample(const float (&v)[
   for (int w = 0; w < NT / 32; ++w) { if (w < warp) before += wcnt[w]; nbins += wcnt[w]; }
   screen = screen && nbins <= kMaxBins;
   if (screen) {
-    for (int e = tid; e < 5 * nbins; e += NT) bins.m[e / nbins][e % nbins] = 0.f;
-    __syncthreads();
-    // moments: a thread adds up the run of its samples in one bin before it adds to the bin
-    float sum[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
     for (int e = 0; e < E; ++e) {
-      const int i = tid * E + e;
-      if (i < n) {
-        const int b = before + first[e] - 1;
+      const int i = tid * E + e, b = before + first[e] - 1;
+      if (i < n && first[e] != (e ? first[e > 0 ? e - 1 : 0] : 0)) {
         // (distances from the smallest sample, which are exact or rounded to 2^-24 of themselves: a centre in the samples' own
         // coordinates would be off by an ulp of them, a fifth of the kernel width where the samples lie 4 ulps apart)
-        const float c = (bin_of(v[e]) + 0.5f) * width, o = ((v[e] - zmin) - c) * inv;
-        if (e == 0 || first[e] != first[e > 0 ? e - 1 : 0]) bins.centre[b] = c;   // (neighbours in other threads write the same)
-        const float o2 = o * o;
-        sum[0] += 1.f; sum[1] += o; sum[2] += 0.5f * o2; sum[3] += o2 * o * (1.f / 6.f); sum[4] += o2 * o2 * (1.f / 24.f);
-        if (e == E - 1 || i == n - 1 || first[e + 1 < E ? e + 1 : e] != first[e]) {
-#pragma unroll
-          for (int q = 0; q < 5; ++q) { atomicAdd(&bins.m[q][b], sum[q]); sum[q] = 0.f; }
+        bins.start[b] = i;
+        bins.centre[b] = (bin_of(v[e]) + 0.5f) * width;
+      }
+    }
+    if (tid == 0) bins.start[nbins] = n;
+    __syncthreads();
+    // moments: a pair of lanes adds up a bin's samples (runs of a thread's own samples added to the bins atomically: 10000 clocks)
+    for (int b0 = 0; b0 < nbins; b0 += NT / 2) {
+      const int b = b0 + (tid >> 1);
+      float sum[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+      if (b < nbins) {
+        const float c = bins.centre[b];
+        const int end = bins.start[b + 1];
+        for (int i = bins.start[b] + (tid & 1); i < end; i += 2) {
+          const float o = ((keys[i] - zmin) - c) * inv, o2 = o * o;
+          sum[0] += 1.f; sum[1] += o; sum[2] += 0.5f * o2; sum[3] += o2 * o * (1.f / 6.f); sum[4] += o2 * o2 * (1.f / 24.f);
         }
+      }
+#pragma unroll
+      for (int q = 0; q < 5; ++q) sum[q] += __shfl_xor_sync(0xffffffffu, sum[q], 1);
+      if (b < nbins && !(tid & 1)) {
+#pragma unroll
+        for (int q = 0; q < 5; ++q) bins.m[q][b] = sum[q];
       }
     }
     __syncthreads();
@@ -431,6 +464,67 @@ template <int E> __device__ __forceinline__ int densest_sample(const float (&v)[
       if (f[e] >= 0.f && f[e] + slack >= best) list[atomicAdd(&count, 1)] = tid * E + e;
     __syncthreads();
     const int m = count;
+    __shared__ double red_series[kSeries][NT / 32];
+    float first_z = __int_as_float(0x7f800000), last_z = -first_z;
+    for (int e = lane; e < m; e += 32) { const float x = keys[list[e]]; first_z = fminf(first_z, x); last_z = fmaxf(last_z, x); }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      first_z = fminf(first_z, __shfl_xor_sync(0xffffffffu, first_z, o));
+      last_z = fmaxf(last_z, __shfl_xor_sync(0xffffffffu, last_z, o));
+    }
+    const double middle = 0.5 * (double(first_z) + double(last_z));
+    if (m == 1) {
+      // nothing to tell apart
+    } else if (m <= NT && (double(last_z) - middle) <= 0.125 * bw) {
+      // The listed samples lie close together (around one mode): one pass over the samples gives the density about their middle in
+      // fp64, e^(-(u - t)^2 / 2) = sum He_q(u) e^(-u^2 / 2) t^q / q!, and with it all their densities.  Left out with ten terms and
+      // |t| <= 1/8: at most n 1.09 t^10 / sqrt(10!) = 5.4e-13 n (|He_q e^(-u^2/4)| < 1.09 sqrt(q!)); rounding adds less than 1e-13 n.
+      const double inv = 1.0 / bw;
+      double sum[kSeries] = {};
+#pragma unroll 2
+      for (int i = tid; i < n; i += NT) {
+        const double u = (double(keys[i]) - middle) * inv;
+        double h0 = exp_straight(-0.5 * u * u), h1 = u * h0;
+        sum[0] += h0;
+        sum[1] += h1;
+#pragma unroll
+        for (int q = 2; q < kSeries; ++q) {
+          const double h2 = fma(u, h1, -double(q - 1) * h0);
+          sum[q] += h2;
+          h0 = h1;
+          h1 = h2;
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < kSeries; ++q) {
+        const double w = warp_sum(sum[q]);
+        if (lane == 0) red_series[q][warp] = w;
+      }
+      __syncthreads();
+      if (tid < kSeries) {
+        double all = 0.0;
+        for (int w = 0; w < NT / 32; ++w) all += red_series[tid][w];
+        red_series[tid][0] = all;
+      }
+      __syncthreads();
+      double mine = -1.0;
+      const int at = tid < m ? list[tid] : 0;
+      if (tid < m) {
+        const double t = (double(keys[at]) - middle) * inv;
+        mine = red_series[kSeries - 1][0];
+        for (int q = kSeries - 1; q > 0; --q) mine = fma(mine, t / double(q), red_series[q - 1][0]);
+      }
+      double top = mine;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) top = fmax(top, __shfl_xor_sync(0xffffffffu, top, o));
+      if (lane == 0) bestv[warp] = top;
+      __syncthreads();                                      // (count has been read, and the list)
+      if (tid == 0) count = 0;
+#pragma unroll
+      for (int w = 0; w < NT / 32; ++w) top = fmax(top, bestv[w]);
+      __syncthreads();
+      if (tid < m && mine + 4e-12 * double(n) >= top) list[atomicAdd(&count, 1)] = at;
+    } else {
     // sums of exponentials of the listed samples, two per warp at a time; eight terms at a time in fp32, those sums in fp64
     const float scale = float(0.8493218002880191 / bw);     // sqrt(log2(e) / 2) / width: e^(-u^2/2) = 2^-(scale (zk - zi))^2
     float* const dens = reinterpret_cast<float*>(list + n);
@@ -478,6 +572,7 @@ template <int E> __device__ __forceinline__ int densest_sample(const float (&v)[
 #pragma unroll
     for (int r = 0; r < (kMaxSearchSamples + NT - 1) / NT; ++r)
       if (keep[r] >= 0) list[at++] = keep[r];
+    }
   } else {
     for (int i = tid; i < n; i += NT) list[i] = i;
     if (tid == 0) count = n;
@@ -507,7 +602,7 @@ template <int E> __device__ __forceinline__ int densest_sample(const float (&v)[
 
 template <int E> __global__ void __launch_bounds__(NT, 4)
 k_range_search(const float* __restrict__ z, long long ldz, const float* __restrict__ b1, int n,
-               const float* __restrict__ thr, double t_all, double step, int act, float* __restrict__ lo, float* __restrict__ hi,
+               const float* __restrict__ thr, double t_all, double step, double n_root, int act, float* __restrict__ lo, float* __restrict__ hi,
                float* __restrict__ a, float* __restrict__ c, int* __restrict__ steps_out) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double* gs = reinterpret_cast<double*>(smem_raw);                // [NT E] activation of the sorted samples
@@ -515,6 +610,7 @@ k_range_search(const float* __restrict__ z, long long ldz, const float* __restri
   __shared__ double red[1][NT / 32];
   __shared__ float range_s[2];
   __shared__ union Scratch { Bins bins; Steps steps; __device__ Scratch() {} } scratch;
+  __shared__ Ahead ahead;
   __shared__ double base_m[5];                                     // moments of the range so far (the walk starts anew from time to time)
   __shared__ int base_k[2], base_end[2], total_steps, finished;
   const int j = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
@@ -532,7 +628,7 @@ k_range_search(const float* __restrict__ z, long long ldz, const float* __restri
 #pragma unroll
   for (int e = 0; e < E; ++e) if (tid * E + e < n) { const double dz = double(v[e]) - mean; s2[0] += dz * dz; }
   block_sums<1>(s2, red);
-  const double bw = n > 1 ? 1.06 * sqrt(s2[0] / double(n - 1)) * pow(double(n), -0.2) : 0.0;
+  const double bw = n > 1 ? 1.06 * sqrt(s2[0] / double(n - 1)) * n_root : 0.0;     // (n_root: n^(-1/5))
   const int ic = bw > 0.0 ? densest_sample<E>(v, keys, n, bw, scratch.bins, reinterpret_cast<int*>(gs)) : 0;
   const double cen = double(keys[ic]);
   __syncthreads();                                                 // (the list in the place of gs has been read)
@@ -558,9 +654,10 @@ k_range_search(const float* __restrict__ z, long long ldz, const float* __restri
     __syncthreads();                                               // (the bins, or the steps before, have been read)
     // (1) where the next kMaxSteps steps on either side end, (2) what each adds about the centroid (y = z - centroid, g = activation -
     // activation at the centroid; sums of y, g, y y, y g, g g), (3) running sums
-    for (int e = tid; e < 2 * (kMaxSteps + 1); e += NT) {
-      const int side = e & 1, k = e >> 1;
-      st.end[side][k] = k == 0 ? base_end[side] : lower(side ? cen + (base_k[1] + k) * step : cen - (base_k[0] + k) * step);
+    if (tid < 2) st.end[tid][0] = base_end[tid];
+    for (int e = tid; e < 2 * kMaxSteps; e += NT) {
+      const int side = e & 1, k = (e >> 1) + 1;
+      st.end[side][k] = lower(side ? cen + (base_k[1] + k) * step : cen - (base_k[0] + k) * step);
     }
     __syncthreads();
     for (int e = tid; e < 2 * kMaxSteps; e += NT) {
@@ -588,90 +685,98 @@ k_range_search(const float* __restrict__ z, long long ldz, const float* __restri
       }
     }
     __syncthreads();
-    if (tid < 32) {
-      // Mean squared residual of the least-squares line over the sorted samples i0 .. i1 - 1, as it is defined.  Where both errors are
-      // zero but for rounding (two distinct values inside, a straight stretch of the activation) the order of the additions decides,
-      // so it is a fixed one: 256 running sums, sample i0 + s + 256 k to sum s, added up in trees of 32, those in ascending order.
-      auto mse = [&](int i0, int i1) -> double {
-        const int cnt = i1 - i0;
-        if (cnt < 2) return 0.0;
-        auto total = [&](auto term) {
-          double t = 0.0;
-          for (int s0 = 0; s0 < NT && s0 < cnt; s0 += 32) {        // (what is left out adds zeros)
-            double sum = 0.0;
-            for (int i = i0 + s0 + lane; i < i1; i += NT) sum += term(i);
-            t += warp_sum(sum);
-          }
-          return t;
-        };
-        const double q = 1.0 / double(cnt);
-        const double mz = total([&](int i) { return double(keys[i]); }) * q, mg = total([&](int i) { return gs[i]; }) * q;
-        const double vzz = total([&](int i) { const double dz = double(keys[i]) - mz; return dz * dz; }) * q;
-        if (!(vzz > 1e-30)) return 0.0;
-        const double sl = total([&](int i) { return (double(keys[i]) - mz) * (gs[i] - mg); }) * q / vzz;
-        return total([&](int i) { const double r = (gs[i] - mg) - sl * (double(keys[i]) - mz); return r * r; }) * q;
+    // Mean squared residual of the least-squares line over the sorted samples i0 .. i1 - 1, as it is defined.  Where both errors are
+    // zero but for rounding (two distinct values inside, a straight stretch of the activation) the order of the additions decides,
+    // so it is a fixed one: 256 running sums, sample i0 + s + 256 k to sum s, added up in trees of 32, those in ascending order.
+    auto mse = [&](int i0, int i1) -> double {
+      const int cnt = i1 - i0;
+      if (cnt < 2) return 0.0;
+      auto total = [&](auto term) {
+        double t = 0.0;
+        for (int s0 = 0; s0 < NT && s0 < cnt; s0 += 32) {        // (what is left out adds zeros)
+          double sum = 0.0;
+          for (int i = i0 + s0 + lane; i < i1; i += NT) sum += term(i);
+          t += warp_sum(sum);
+        }
+        return t;
       };
-      // lane = range after i steps to the left and jr to the right, i + jr <= kAhead: lanes s (s + 1) / 2 + jr, s = i + jr
-      auto lane_of = [](int i, int jr) { const int s = i + jr; return s * (s + 1) / 2 + jr; };
-      int s_mine = 0;
-      while ((s_mine + 1) * (s_mine + 2) / 2 <= lane) ++s_mine;
-      const int j_mine = min(lane - s_mine * (s_mine + 1) / 2, kAhead), i_mine = max(0, min(s_mine, kAhead) - j_mine);
-      int kl = 0, kr = 0, nsteps = total_steps;
-      bool done = false;
-      while (!done && kl + kAhead <= kMaxSteps && kr + kAhead <= kMaxSteps) {
-        // the lane's range: error from the moments (times its number of samples, and so on, to have one division), and what it can be
-        // off by (infinite where the moments cancel)
-        const int e0 = st.end[0][kl + i_mine], e1 = st.end[1][kr + j_mine], cnt = e1 - e0;
-        double err = 0.0;
-        float off = 0.f;
-        if (cnt >= 2 && !(act == TARDIS_ACT_RELU && (keys[e0] > 0.f || keys[e1 - 1] <= 0.f))) {   // (one straight piece: exactly zero)
-          double m[5];
+      const double q = 1.0 / double(cnt);
+      const double mz = total([&](int i) { return double(keys[i]); }) * q, mg = total([&](int i) { return gs[i]; }) * q;
+      const double vzz = total([&](int i) { const double dz = double(keys[i]) - mz; return dz * dz; }) * q;
+      if (!(vzz > 1e-30)) return 0.0;
+      const double sl = total([&](int i) { return (double(keys[i]) - mz) * (gs[i] - mg); }) * q / vzz;
+      return total([&](int i) { const double r = (gs[i] - mg) - sl * (double(keys[i]) - mz); return r * r; }) * q;
+    };
+    // Range after i steps to the left and jr to the right, i + jr <= kAhead: number s (s + 1) / 2 + jr, s = i + jr, and a thread's.  (What
+    // follows is the same for all threads: kl, kr, nsteps, done.)
+    int s_mine = 0;
+    while ((s_mine + 1) * (s_mine + 2) / 2 <= tid) ++s_mine;
+    const int j_mine = min(tid - s_mine * (s_mine + 1) / 2, kAhead), i_mine = max(0, min(s_mine, kAhead) - j_mine);
+    int kl = 0, kr = 0, nsteps = total_steps;
+    bool done = false;
+    while (!done && kl + kAhead <= kMaxSteps && kr + kAhead <= kMaxSteps) {
+      // the thread's range: error from the moments (times its number of samples, and so on, to have one reciprocal), and what it can be
+      // off by (infinite where the moments cancel)
+      const int e0 = st.end[0][kl + i_mine], e1 = st.end[1][kr + j_mine], cnt = e1 - e0;
+      {
+        bool zero = cnt < 2;
+        if (act == TARDIS_ACT_RELU) zero = zero || keys[min(e0, n - 1)] > 0.f || keys[max(e1 - 1, 0)] <= 0.f;   // (one straight piece: exactly zero)
+        double m[5];
 #pragma unroll
-          for (int q = 0; q < 5; ++q) m[q] = base_m[q] + (st.m[0][q][kl + i_mine] + st.m[1][q][kr + j_mine]);
-          const double q = double(cnt), yy = m[2] * q, gg = m[4] * q;
-          const double vyy = yy - m[0] * m[0], vyg = m[3] * q - m[0] * m[1], vgg = gg - m[1] * m[1];
-          // Every moment is off by less than c = (n + 20) 2^-53 = 2.3e-13 of the sum of its terms' sizes (n additions, a few roundings
-          // in a term and in joining the parts), and |yg| <= sqrt(yy gg): vyy by 3 c yy, vyg by 3 c sqrt(yy gg), vgg by 3 c gg, so
-          // err q^2 by 3 c gg (1 + sqrt(yy / vyy))^2 <= 7e-13 gg k^2.
-          const float k = 1.f + __fdividef(float(yy), float(vyy)), iq = __fdividef(1.f, float(q));
-          off = fmaxf(1e-12f * float(gg) * iq * iq * k * k, 1e-37f);
-          if (!(vyy > 1e-8 * yy && vyy > 1e-25 * q * q)) off = __int_as_float(0x7f800000);
-          else err = (vgg * vyy - vyg * vyg) / (vyy * q * q);
-        }
-        int i = 0, jr = 0;
-        while (i + jr < kAhead) {                                  // (the same for all lanes)
-          const double l = cen - (base_k[0] + kl + i) * step, u = cen + (base_k[1] + kr + jr) * step;
-          const int here = lane_of(i, jr), p0 = __shfl_sync(0xffffffffu, e0, here), p1 = __shfl_sync(0xffffffffu, e1, here);
-          const int inside = p1 - p0;
-          done = double(inside) >= t * double(n) || inside == n || nsteps >= cap;
-          if (done) break;
-          bool go_left;
-          if (u > zmax) go_left = true;                            // (not both sides: every sample would be inside)
-          else if (l <= zmin) go_left = false;
-          else {
-            const int ll = lane_of(i + 1, jr), lr = lane_of(i, jr + 1);
-            const double el = __shfl_sync(0xffffffffu, err, ll), er = __shfl_sync(0xffffffffu, err, lr);
-            const float o = __shfl_sync(0xffffffffu, off, ll) + __shfl_sync(0xffffffffu, off, lr);
-            go_left = el < er;
-            const bool open = !(fabs(el - er) > double(o)) && o != 0.f;
-            if (__any_sync(0xffffffffu, open)) {                   // (every lane agrees; the vote makes the branch a uniform one)
-              const int l0 = __shfl_sync(0xffffffffu, e0, ll), r1 = __shfl_sync(0xffffffffu, e1, lr);
-              go_left = mse(l0, p1) < mse(p0, r1);
-            }
-          }
-          if (go_left) ++i; else ++jr;
-          ++nsteps;
-        }
-        kl += i;
-        kr += jr;
+        for (int q = 0; q < 5; ++q) m[q] = base_m[q] + (st.m[0][q][kl + i_mine] + st.m[1][q][kr + j_mine]);
+        const double q = double(cnt), yy = m[2] * q, gg = m[4] * q;
+        const double vyy = yy - m[0] * m[0], vyg = m[3] * q - m[0] * m[1], vgg = gg - m[1] * m[1];
+        // Every moment is off by less than c = (n + 20) 2^-53 = 2.3e-13 of the sum of its terms' sizes (n additions, a few roundings
+        // in a term and in joining the parts), and |yg| <= sqrt(yy gg): vyy by 3 c yy, vyg by 3 c sqrt(yy gg), vgg by 3 c gg, so
+        // err q^2 by 3 c gg (1 + sqrt(yy / vyy))^2 <= 7e-13 gg k^2.
+        const float k = 1.f + __fdividef(float(yy), float(vyy)), iq = __fdividef(1.f, float(q));
+        const bool cancels = !(vyy > 1e-8 * yy && vyy > 1e-25 * q * q);
+        ahead.off[tid] = zero ? 0.f : (cancels ? __int_as_float(0x7f800000) : fmaxf(1e-12f * float(gg) * iq * iq * k * k, 1e-37f));
+        // (vgg vyy - vyg^2) / (vyy q^2), the reciprocal by two Newton steps from the 20 bits of an approximate one
+        const double den = cancels ? 1.0 : vyy * q * q;
+        double y;
+        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(den));
+        y = fma(y, fma(-den, y, 1.0), y);
+        y = fma(y, fma(-den, y, 1.0), y);
+        ahead.err[tid] = zero || cancels ? 0.0 : (vgg * vyy - vyg * vyg) * y;
       }
-      if (lane < 5) base_m[lane] += st.m[0][lane][kl] + st.m[1][lane][kr];
-      if (lane == 0) {
-        base_k[0] += kl; base_k[1] += kr;
-        base_end[0] = st.end[0][kl]; base_end[1] = st.end[1][kr];
-        total_steps = nsteps;
-        finished = done;
+      __syncthreads();
+      // what would be done from the range: 0 right, 1 left, 2 nothing (enough samples inside), 3 the errors do not tell; and the range that
+      // follows (the same one where the walk has to stop)
+      {
+        const double l = cen - (base_k[0] + kl + i_mine) * step, u = cen + (base_k[1] + kr + j_mine) * step;
+        const int to_left = min(tid + s_mine + 1, NT - 1), to_right = min(tid + s_mine + 2, NT - 1);   // (of the last ones: never used)
+        const double el = ahead.err[to_left], er = ahead.err[to_right];
+        const float o = ahead.off[to_left] + ahead.off[to_right];
+        int move = !(fabs(el - er) > double(o)) && o != 0.f ? 3 : (el < er ? 1 : 0);
+        if (l <= zmin) move = 0;
+        if (u > zmax) move = 1;                                    // (not both sides: every sample would be inside)
+        if (double(cnt) >= t * double(n) || cnt == n || nsteps + s_mine >= cap) move = 2;
+        ahead.next[tid] = uint16_t((s_mine >= kAhead || move >= 2 ? tid : (move == 1 ? to_left : to_right)) | move << 8 | s_mine << 10);
       }
+      __syncthreads();
+      int last = 0, at = ahead.next[0];
+      while ((at & 0xff) != last) { last = at & 0xff; at = ahead.next[last]; }
+      const int what = at >> 8 & 3, s_last = at >> 10;
+      int jr = last - s_last * (s_last + 1) / 2, i = s_last - jr;
+      if (s_last < kAhead) {
+        done = what == 2;
+        if (what == 3) {                                           // (every warp finds the same)
+          const int p0 = st.end[0][kl + i], p1 = st.end[1][kr + jr];
+          if (mse(st.end[0][kl + i + 1], p1) < mse(p0, st.end[1][kr + jr + 1])) ++i; else ++jr;
+        }
+      }
+      nsteps += i + jr;
+      kl += i;
+      kr += jr;
+    }
+    __syncthreads();                                               // (the sums so far have been read)
+    if (tid < 5) base_m[tid] += st.m[0][tid][kl] + st.m[1][tid][kr];
+    if (tid == 0) {
+      base_k[0] += kl; base_k[1] += kr;
+      base_end[0] = st.end[0][kl]; base_end[1] = st.end[1][kr];
+      total_steps = nsteps;
+      finished = done;
     }
     __syncthreads();
   } while (!finished);
@@ -740,7 +845,7 @@ k_neuron_error(const float* __restrict__ z, long long ldz, const float* __restri
 // leaves more than half of the SMs idle at 16384 neurons: 85 us), then it takes its share of what is left for it.
 __global__ void __launch_bounds__(NT)
 k_neuron_thresholds(const float* __restrict__ err, int h, double t_layer, double t_min, double t_max, float* __restrict__ t) {
-  __shared__ float tile[NT * 4];
+  __shared__ __align__(16) float tile[NT * 4];
   const int j = blockIdx.x * (NT / 8) + (threadIdx.x >> 3), part = threadIdx.x & 7;
   const float ej = j < h ? err[j] : 0.f;
   int rank = 0;
@@ -752,10 +857,20 @@ k_neuron_thresholds(const float* __restrict__ err, int h, double t_layer, double
       tile[r * NT + threadIdx.x] = i < h ? err[i] : __int_as_float(0x7f800000);
     }
     __syncthreads();
+    // equal errors count where their neuron comes first: in a tile that lies in front of the CTA's neurons or behind them the same for all
+    const float4* const at = reinterpret_cast<const float4*>(tile);
+    if (base + NT * 4 <= int(blockIdx.x) * (NT / 8)) {
 #pragma unroll 8
-    for (int i = part; i < NT * 4; i += 8) {
-      const float v = tile[i];
-      rank += (v < ej || (v == ej && base + i < j)) ? 1 : 0;
+      for (int i = part; i < NT; i += 8) { const float4 v = at[i]; rank += (v.x <= ej) + (v.y <= ej) + (v.z <= ej) + (v.w <= ej); }
+    } else if (base >= (int(blockIdx.x) + 1) * (NT / 8)) {
+#pragma unroll 8
+      for (int i = part; i < NT; i += 8) { const float4 v = at[i]; rank += (v.x < ej) + (v.y < ej) + (v.z < ej) + (v.w < ej); }
+    } else {
+#pragma unroll 8
+      for (int i = part; i < NT * 4; i += 8) {
+        const float v = tile[i];
+        rank += (v < ej || (v == ej && base + i < j)) ? 1 : 0;
+      }
     }
   }
 #pragma unroll
@@ -804,7 +919,7 @@ tardis_status_t launch_range_search(int h, int n, const float* z, long long ldz,
   if (n < 1 || n > cal::kMaxSearchSamples) return TARDIS_ERR_UNSUPPORTED;
   return cal::with_samples<cal::kMaxSearchSamples / cal::NT>(n, [&](auto e) {
     constexpr int E = decltype(e)::value;
-    cal::k_range_search<E><<<h, cal::NT, size_t(cal::NT) * E * (sizeof(double) + sizeof(float)), s>>>(z, ldz, b1, n, thr, t_all, step, act,
+    cal::k_range_search<E><<<h, cal::NT, size_t(cal::NT) * E * (sizeof(double) + sizeof(float)), s>>>(z, ldz, b1, n, thr, t_all, step, pow(double(n), -0.2), act,
                                                                                                      lo, hi, a, c, steps_out);
     TARDIS_CUDA_TRY(cudaGetLastError());
     return TARDIS_OK;

@@ -67,6 +67,17 @@ __device__ __forceinline__ double exp_straight(double v) {
   p = fma(p, r, 1.0 / 24.0); p = fma(p, r, 1.0 / 6.0); p = fma(p, r, 0.5); p = fma(p, r, 1.0); p = fma(p, r, 1.0);
   return __hiloint2double(__double2hiint(p) + (__double2loint(t) << 20), __double2loint(p));
 }
+// gelu_f64's tanh form likewise: z / (1 + e^-x), the reciprocal by two Newton steps from a float's; below x = -88 the result is 0, off by
+// less than 1e-36.  (With exp and a division the activation took 7600 of a CTA's 23000 clocks in k_calibrate.)
+__device__ __forceinline__ double gelu_tanh_f64(double z) {
+  const double d = 1.0 + exp_straight(-1.5957691216057308 * (z + 0.044715 * z * z * z));
+  float y0;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y0) : "f"(float(d)));
+  double y = double(y0);
+  y = fma(y, fma(-d, y, 1.0), y);
+  y = fma(y, fma(-d, y, 1.0), y);
+  return z * y;
+}
 
 // The n samples of neuron j plus its bias, NT E values over the CTA (+inf beyond n): thread t gets samples e NT + t.
 template <int E> __device__ __forceinline__ void load_samples(float (&v)[E], const float* __restrict__ z, long long ldz,
@@ -246,13 +257,15 @@ template <int E> __device__ __forceinline__ bool pick_ranks(const float (&v)[E],
   return true;
 }
 
-// Bound by the latency of its dozen barriers and by the fp64 activation.  16384 neurons x 2048 samples: 0.28 ms (0.46 ms with the
+// Bound by the latency of its barriers and by the fp64 activation.  16384 neurons x 2048 samples: 0.24 ms (0.28 with five CTAs per SM, two passes
+// and an activation that branches, 0.46 ms with the
 // samples sorted in registers, 0.91 ms with every step of the sort in shared memory and the activation as a fp64 tanh, evaluated twice).
-template <int E> __global__ void __launch_bounds__(NT, E <= 8 ? 5 : 1)   // (five CTAs per SM: 0.32 ms with three)
+template <int E> __global__ void __launch_bounds__(NT, E <= 8 ? 6 : 1)   // (CTAs per SM: their barriers and chains overlap; one pass and no stored activations leave the registers for six)
 k_calibrate(const float* __restrict__ z, long long ldz, const float* __restrict__ b1, int n, double q_lo, double q_hi,
             int act, float* __restrict__ lo, float* __restrict__ hi, float* __restrict__ a, float* __restrict__ c) {
   extern __shared__ float keys[];                      // [NT E]
   __shared__ float found[4];                           // the order statistics around the two quantiles
+  __shared__ double red5[5][NT / 32];
   const int j = blockIdx.x, tid = threadIdx.x;
   float v[E];
   load_samples<E>(v, z, ldz, b1, j, n);
@@ -282,10 +295,33 @@ k_calibrate(const float* __restrict__ z, long long ldz, const float* __restrict_
     const double w = pos - floor(pos);
     range[r] = float(__dadd_rn(__dmul_rn(double(stat[2 * r]), 1.0 - w), __dmul_rn(double(stat[2 * r + 1]), w)));
   }
-  double gs[E];
+  // Least squares of the activation over the samples inside, in one pass: moments about one of those samples, so that samples that are
+  // all equal give a variance of exactly zero (and the offset of the others' mean costs a digit at most).  Two passes (means first) need a
+  // second round of barriers, and the activations kept in registers, which are then too many for a sixth CTA per SM.
+  const float l = range[0], u = range[1];
+  const double c0 = double(stat[1] >= l && stat[1] < u ? stat[1] : l);
+  const double g0 = double(gelu_f32(float(c0), act));      // (near the activation there, for the same reason)
+  double m[5] = {0.0, 0.0, 0.0, 0.0, 0.0};                 // count, y, g, y y, y g; y = z - c0, g = activation - g0
 #pragma unroll
-  for (int e = 0; e < E; ++e) gs[e] = (v[e] >= range[0] && v[e] < range[1]) ? gelu_f64(double(v[e]), act) : 0.0;
-  fit_and_store<E>(v, gs, range[0], range[1], act, j, lo, hi, a, c);
+  for (int e = 0; e < E; ++e) {
+    const bool inside = v[e] >= l && v[e] < u;
+    const double x = double(inside ? v[e] : float(c0));
+    const double g = (act == TARDIS_ACT_GELU_TANH ? gelu_tanh_f64(x) : gelu_f64(x, act)) - g0, y = x - c0;
+    if (inside) { m[0] += 1.0; m[1] += y; m[2] += g; m[3] = fma(y, y, m[3]); m[4] = fma(y, g, m[4]); }
+  }
+  block_sums(m, red5);
+  if (tid == 0) {
+    const double cnt = m[0], safe = cnt > 0.0 ? cnt : 1.0, my = m[1] / safe, mg = m[2] / safe;
+    const double var = m[3] / safe - my * my, cov = m[4] / safe - my * mg;
+    double aj, cj;
+    if (cnt >= 2.0 && var > 1e-30) { aj = cov / var; cj = (g0 + mg) - aj * (c0 + my); }
+    else {                                                 // too few samples in range: tangent at the midpoint
+      const double mid = 0.5 * (double(l) + double(u));
+      aj = gelu_slope_f64(mid, act);
+      cj = gelu_f64(mid, act) - aj * mid;
+    }
+    lo[j] = l; hi[j] = u; a[j] = float(aj); c[j] = float(cj);
+  }
 }
 
 // ---- the greedy range search of Algorithm 1 (Section 5.1.1, "Range Searching") --------------------------------------

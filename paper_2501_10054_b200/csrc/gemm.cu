@@ -170,6 +170,16 @@ __device__ __forceinline__ void epilogue_chunk(const KParams& p, float (&v)[32],
       // back under the word's mask.
       uint32_t word = p.bitmap[size_t(m) * (p.N / 32) + (n >> 5)];
       if (nv < 32) word &= (1u << nv) - 1u;
+      if (p.act == TARDIS_ACT_GELU_TANH) {
+        // evaluated for every element, without branches: the walk over the set bits below waits for its row with the most of them, one
+        // activation after the other (2048 x 16384 x 4096 with this epilogue 202 us, 210 with the walk, 173 with that of the flags)
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
+          const float4 t = tab[i];
+          const float z = v[i] + t.x, dl = gelu_tanh_f32(z) - t.y * z - t.z;
+          v[i] = (word >> i) & 1u ? dl : 0.f;
+        }
+      } else
 #pragma unroll
       for (int half = 0; half < 32; half += 16) {
 #pragma unroll

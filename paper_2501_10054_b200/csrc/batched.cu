@@ -61,12 +61,15 @@ __global__ void k_dequant_split(const uint32_t* __restrict__ codes, const __nv_b
     const float s = __bfloat162float(scale[size_t(j) * ng + g]), zp = float(zero[size_t(j) * ng + g]);
     smax = fmaxf(smax, fabsf(s));
     __nv_bfloat162 h[4], l[4];
+    // (2- and 4-bit codes of eight channels lie in one word, and k0 is a multiple of 8)
+    const bool whole = bits == 2 || bits == 4;
+    const uint32_t word = whole ? row[k0 * bits >> 5] >> (k0 * bits & 31) : 0u, mask = (1u << bits) - 1u;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       float v[2], t[2];
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
-        const float m = float(stream_code(row, k0 + 2 * q + e, bits)) - zp;
+        const float m = float(whole ? (word >> (bits * (2 * q + e))) & mask : stream_code(row, k0 + 2 * q + e, bits)) - zp;
         v[e] = s * m;                                                      // exact: 8-bit significand times |int| <= 15
         t[e] = __bfloat162float(__float2bfloat16_rn(v[e]));
         notes |= (v[e] != t[e] ? 1u : 0u) | (fabsf(m) > 2.f ? 2u : 0u);
@@ -129,15 +132,10 @@ __global__ void __launch_bounds__(256) k_recheck(const uint32_t* __restrict__ rl
                                                  const float* __restrict__ lo, const float* __restrict__ hi, const __nv_bfloat16* __restrict__ x, int d, int h,
                                                  int G, int bits, uint32_t* __restrict__ bitmap, float* __restrict__ zhat, unsigned long long* counters) {
   extern __shared__ double xd[];                           // channel c of unit u (16 channels) at c (d / 16 + 1) + u: the lanes' units side by side
-  __shared__ unsigned int flagged;                         // the token's
+  __shared__ unsigned int flagged;
   const int t = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned int queued = rcount[t];
   const unsigned int most = max_recheck(h);
-  // asked for together with the token: the warp's first neuron (the queue has room for 512 at least, so there is something to read), and
-  // the token's flags, counted before any of them changes
-  const int first = min(int(rlist[size_t(t) * most + warp] & 0x7fffffffu), h - 1);
-  int count = 0;
-  for (int w = threadIdx.x; w < h / 32; w += blockDim.x) count += __popc(__ldcg(bitmap + size_t(t) * (h / 32) + w));
   const bool all = queued > most;
   const unsigned int total = all ? (unsigned int)h : queued;
   const __nv_bfloat16* const xt = x + size_t(t) * d;
@@ -157,7 +155,7 @@ __global__ void __launch_bounds__(256) k_recheck(const uint32_t* __restrict__ rl
   __syncthreads();
   const int ng = d / G;
   for (unsigned int e = warp; e < total; e += 8) {
-    const int j = all ? int(e) : (e < 8 ? first : int(rlist[size_t(t) * most + e]));
+    const int j = all ? int(e) : int(rlist[size_t(t) * most + e]);
     const uint32_t* const row = codes + size_t(j) * (size_t(d) * bits / 32);
     double z = 0.0;
     // units of 16 channels (all of one group), four at a time: their loads go out before the first is used, since waiting for them
@@ -201,14 +199,16 @@ __global__ void __launch_bounds__(256) k_recheck(const uint32_t* __restrict__ rl
     if (lane == 0) {
       const bool inside = (double(lo[j]) <= z) && (z < double(hi[j]));
       uint32_t* wp = bitmap + size_t(t) * (h / 32) + (j >> 5);
-      const uint32_t bit = 1u << (j & 31);
-      if (inside) count -= atomicAnd(wp, ~bit) & bit ? 1 : 0;
-      else count += atomicOr(wp, bit) & bit ? 0 : 1;
+      if (inside) atomicAnd(wp, ~(1u << (j & 31)));
+      else atomicOr(wp, 1u << (j & 31));
       if (zhat) zhat[size_t(t) * h + j] = float(z);
     }
   }
-  __syncwarp();
-  const unsigned int c = __reduce_add_sync(0xffffffffu, unsigned(count));       // (modulo 2^32, like the sum it goes into)
+  __threadfence_block();
+  __syncthreads();
+  unsigned int c = 0;
+  for (int w = threadIdx.x; w < h / 32; w += blockDim.x) c += __popc(__ldcg(bitmap + size_t(t) * (h / 32) + w));
+  c = __reduce_add_sync(0xffffffffu, c);
   if (lane == 0) atomicAdd(&flagged, c);
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -245,20 +245,6 @@ __global__ void k_capture(const uint32_t* __restrict__ bitmap, const float* __re
 }  // namespace bat
 
 using namespace bat;
-
-template <typename T> __global__ void k_transpose_b(const T* __restrict__ in, T* __restrict__ out, int rows, int cols) {
-  __shared__ T tile[32][33];
-  int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-  for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-    int rr = r0 + r, cc = c0 + threadIdx.x;
-    if (rr < rows && cc < cols) tile[r][threadIdx.x] = in[size_t(rr) * cols + cc];
-  }
-  __syncthreads();
-  for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-    int cc = c0 + r, rr = r0 + threadIdx.x;
-    if (rr < rows && cc < cols) out[size_t(cc) * rows + rr] = tile[threadIdx.x][r];
-  }
-}
 
 namespace {
 struct Req { void** p; size_t bytes; bool scratch; };
@@ -310,23 +296,31 @@ tardis_status_t batched_prepare(Handle* H) {
   return st;
 }
 
-// a_j W1[j][k] in fp32, transposed to [k][j] and split into bf16 hi + lo (16 significant bits together)
-__global__ void k_scale_transpose_split(const __nv_bfloat16* __restrict__ W1, const float* __restrict__ a,
-                                        __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo, int h, int d) {
-  __shared__ float tile[32][33];
-  const int k0 = blockIdx.x * 32, j0 = blockIdx.y * 32;
-  for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-    const int j = j0 + r, k = k0 + threadIdx.x;
-    if (j < h && k < d) tile[r][threadIdx.x] = a[j] * __bfloat162float(W1[size_t(j) * d + k]);
-  }
+// a_j W1[j][k] in fp32, transposed to [k][j] and split into bf16 hi + lo (16 significant bits together); 64 x 64 at a time, two elements
+// per access (h and d are even; 16384 x 4096: 75 us, 172 one by one)
+__global__ void __launch_bounds__(256) k_scale_transpose_split(const uint32_t* __restrict__ W1, const float* __restrict__ a,
+                                                               uint32_t* __restrict__ hi, uint32_t* __restrict__ lo, int h, int d) {
+  __shared__ uint32_t tile[64][33];                                   // [neuron][channel pair]
+  const int k0 = blockIdx.x * 64, j0 = blockIdx.y * 64, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int r = warp; r < 64; r += 8)
+    if (j0 + r < h && k0 + 2 * lane < d) tile[r][lane] = W1[(size_t(j0 + r) * d + k0) / 2 + lane];
   __syncthreads();
-  for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-    const int k = k0 + r, j = j0 + threadIdx.x;
-    if (j < h && k < d) {
-      const float v = tile[threadIdx.x][r];
-      const __nv_bfloat16 hv = __float2bfloat16_rn(v);
-      hi[size_t(k) * h + j] = hv;
-      lo[size_t(k) * h + j] = __float2bfloat16_rn(v - __bfloat162float(hv));
+  const int j = j0 + 2 * lane;
+  if (j >= h) return;
+  const float a0 = a[j], a1 = a[j + 1];
+#pragma unroll
+  for (int p = warp; p < 32; p += 8) {                                // channels k0 + 2 p, k0 + 2 p + 1 of neurons j, j + 1
+    if (k0 + 2 * p >= d) continue;
+    const uint32_t w0 = tile[2 * lane][p], w1 = tile[2 * lane + 1][p];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const float v0 = a0 * __uint_as_float(c ? w0 & 0xffff0000u : w0 << 16), v1 = a1 * __uint_as_float(c ? w1 & 0xffff0000u : w1 << 16);
+      const __nv_bfloat162 top = __floats2bfloat162_rn(v0, v1);
+      const __nv_bfloat162 rest = __floats2bfloat162_rn(v0 - __bfloat162float(top.x), v1 - __bfloat162float(top.y));
+      const size_t at = (size_t(k0 + 2 * p + c) * h + j) / 2;
+      hi[at] = *reinterpret_cast<const uint32_t*>(&top);
+      lo[at] = *reinterpret_cast<const uint32_t*>(&rest);
     }
   }
 }
@@ -354,8 +348,8 @@ tardis_status_t launch_fold_tensor(Handle* H, const tardis_fold_desc_t* desc, cu
   if (!S || H->dtype != TARDIS_BF16) return TARDIS_ERR_UNSUPPORTED;
   const int d = H->d, h = H->h;
   dim3 tb(32, 8);
-  k_scale_transpose_split<<<dim3((d + 31) / 32, (h + 31) / 32), tb, 0, s>>>(static_cast<const __nv_bfloat16*>(H->W1), H->a,
-                                                                            S->What_hi, S->What_lo, h, d);
+  k_scale_transpose_split<<<dim3((d + 63) / 64, (h + 63) / 64), 256, 0, s>>>(static_cast<const uint32_t*>(H->W1), H->a, reinterpret_cast<uint32_t*>(S->What_hi),
+                                                                             reinterpret_cast<uint32_t*>(S->What_lo), h, d);
   const size_t cap = size_t(kChunkCapture) * h;              // floats in the score buffer
   int rows_per = int(cap / d);
   rows_per = rows_per / 128 * 128;
@@ -380,12 +374,11 @@ tardis_status_t batched_finish(Handle* H, const void* W2, cudaStream_t s) {
   if (!S) return TARDIS_OK;
   const int d = H->d, h = H->h;
   const size_t hd = size_t(h) * d;
-  dim3 tb(32, 8);
   // W_f[i][k] row-major (the GEMMs want the channel index contiguous in both operands): transpose of C
-  k_transpose_b<__nv_bfloat16><<<dim3((d + 31) / 32, (d + 31) / 32), tb, 0, s>>>(static_cast<const __nv_bfloat16*>(H->C), S->Wf, d, d);
+  TARDIS_CUDA_TRY(launch_transpose(static_cast<const __nv_bfloat16*>(H->C), S->Wf, d, d, s));
   if (W2) TARDIS_CUDA_TRY(cudaMemcpyAsync(S->W2, W2, hd * 2, cudaMemcpyDeviceToDevice, s));
   else      // (a handle read back from a file has only the transposed copy)
-    k_transpose_b<__nv_bfloat16><<<dim3((d + 31) / 32, (h + 31) / 32), tb, 0, s>>>(static_cast<const __nv_bfloat16*>(H->W2T), S->W2, h, d);
+    TARDIS_CUDA_TRY(launch_transpose(static_cast<const __nv_bfloat16*>(H->W2T), S->W2, h, d, s));
   TARDIS_CUDA_TRY(cudaMemsetAsync(S->lo_used, 0, size_t((h + 127) / 128) * 4, s));
   if (H->bits <= 4)   // (8-bit codes: the batched path is not used, see the dispatch)
     k_dequant_split<<<h, 256, 0, s>>>(H->codes, static_cast<const __nv_bfloat16*>(H->scale), H->zero, S->What_hi, S->What_lo,

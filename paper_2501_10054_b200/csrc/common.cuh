@@ -82,6 +82,7 @@ void dev_reserve(size_t bytes);     // one block for the allocations that the ru
 tardis_status_t launch_fold(Handle* H, const tardis_fold_desc_t* desc, cudaStream_t s, bool skip_product = false);
 tardis_status_t launch_fold_product(Handle* H, cudaStream_t s);   // the SIMT product alone
 tardis_status_t launch_export_folded(Handle* H, void* Wf, float* bf, cudaStream_t s);
+cudaError_t launch_transpose(const __nv_bfloat16* in, __nv_bfloat16* out, int rows, int cols, cudaStream_t s);   // out[cols, rows] from in[rows, cols]
 tardis_status_t launch_generic_forward(Handle* H, const void* x, void* y, int64_t n, cudaStream_t s);
 tardis_status_t launch_static_forward(Handle* H, const void* x, void* y, int64_t n, cudaStream_t s);
 tardis_status_t decode_prepare(Handle* H, cudaStream_t s);                 // builds codes_mma, pmeta, scratch

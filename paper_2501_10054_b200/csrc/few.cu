@@ -559,17 +559,12 @@ k_few_in(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUten
         if (p.act == TARDIS_ACT_GELU_TANH) {
 #pragma unroll
           for (int e = 0; e < 8; ++e) { const float z = v[e] + b1; v[e] = gelu_tanh_f32(z) - fa * z - fc; }
+        } else if (p.act == TARDIS_ACT_GELU_ERF) {
+#pragma unroll
+          for (int e = 0; e < 8; ++e) { const float z = v[e] + b1; v[e] = gelu_f32(z, TARDIS_ACT_GELU_ERF) - fa * z - fc; }
         } else {
-#pragma unroll 1
-          for (int e = 0; e < 8; ++e) {                    // (rolled by hand: registers cannot be indexed)
-            float z = 0.f;
 #pragma unroll
-            for (int q = 0; q < 8; ++q) z = q == e ? v[q] : z;
-            z += b1;
-            z = (bits >> e) & 1u ? gelu_f32(z, p.act) - fa * z - fc : 0.f;
-#pragma unroll
-            for (int q = 0; q < 8; ++q) v[q] = q == e ? z : v[q];
-          }
+          for (int e = 0; e < 8; ++e) { const float z = v[e] + b1; v[e] = gelu_f32(z, TARDIS_ACT_RELU) - fa * z - fc; }
         }
 #pragma unroll
         for (int e = 0; e < 8; ++e) {

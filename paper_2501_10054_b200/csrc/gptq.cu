@@ -421,8 +421,9 @@ __global__ void __launch_bounds__(FT, 2) k_build(const __nv_bfloat16* __restrict
 // weight stays below lambda u sqrt(d) M with a probability that approaches 1 as exp(-lambda^2 / 2) (the probabilistic rounding analysis
 // of Higham and Mary, 2019).  A difference in one weight goes on into the later ones by the same recurrence without the rounding to
 // codes; the probe rows have followed 16 such disturbances, +-1 in every channel, and A is the largest value that came of them.
-// lambda = 256 leaves room for all constants.  On a 4096 / 16384 layer A = 15 and the bound is 2.7e-11 of a weight: one layer in 40 has a
-// neuron that came closer than that to a boundary anywhere (5 ms for the plain way with a few neurons).
+// lambda = 32 leaves room for all constants: the largest difference between the plain way and the same in 64-bit significands is 0.15 of
+// u sqrt(d) A M (24 neurons of 1536 channels, A = 6.5).  On a 4096 / 16384 layer A = 15 and the bound is 3.4e-12 of a weight: one layer in
+// some 300 has a neuron that came closer than that to a boundary anywhere (then 2 to 5 ms for the plain way with a few neurons).
 __global__ void k_suspects(const double* __restrict__ margin, const double* __restrict__ size, int h, double unit, int* __restrict__ list, int* __restrict__ count) {
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= h) return;
@@ -524,7 +525,7 @@ tardis_status_t launch_build_predictor(int h, int d, int dtype, const void* W1, 
     double *const margin = ninv + d, *const size = margin + h + PROBES;
     int* const count = reinterpret_cast<int*>(size + h + PROBES);
     list = count + 1;
-    const double unit = 256.0 * 1.1102230246251565e-16 * sqrt(double(d));
+    const double unit = 32.0 * 1.1102230246251565e-16 * sqrt(double(d));
     e = cudaMemsetAsync(count, 0, sizeof(int), s);
     k_reciprocals<<<(d + 255) / 256, 256, 0, s>>>(U, ninv, d);
     if (e == cudaSuccess)

@@ -581,7 +581,7 @@ def test_kernels_for_a_few_tokens_at_the_edges_of_their_tiles(d, h, G, q):
     _run(cfg, sum(calls), calls, path=3)
 
 
-@pytest.mark.parametrize("d,bits,n", [(512, 2, 5), (576, 2, 16), (512, 2, 40), (512, 4, 33), (512, 2, 128)])
+@pytest.mark.parametrize("d,bits,n", [(512, 2, 5), (576, 2, 16), (512, 2, 40), (512, 4, 33), (512, 2, 128), (512, 2, 200), (512, 3, 200), (1088, 4, 150)])
 def test_scores_near_range_ends_in_every_number_per_tile(d, bits, n):
     # 0 to 20 scores per tile that the fast sums cannot place: a warp for each of eight, the last one to four shared out.  Tiles have 16
     # neurons here (2048 over 148 CTAs); the ends lie 2e-5 above or below scores of two tokens, well inside the allowance and well
@@ -590,6 +590,9 @@ def test_scores_near_range_ends_in_every_number_per_tile(d, bits, n):
     cfg = W.LayerConfig("nearends", d, h, group=64, n_calib=256, bits=bits)
     L = _layer(cfg, 3)
     x = W.make_tokens(cfg, n, 3).cuda()
+    if n > 128:                                                     # (the prompt path: a warp per score of a token)
+        x[0, ::7] *= 2.0 ** -30
+        x[1, :16] = 0.0
     s = L.numpy64()
     zhat = O.predictor_score(x.double().cpu().numpy(), s["codes"], s["scale"], s["zero"], s["group"], s["b1"], s["bits"])
     lo = np.full(h, -50.0)
@@ -601,7 +604,7 @@ def test_scores_near_range_ends_in_every_number_per_tile(d, bits, n):
         for i in range(k):
             j, off = tile * 16 + i % 16, 2e-5 if (tile + i) % 3 else -2e-5
             if i < 16:
-                lo[j] = zhat[0, j] + off
+                lo[j] = zhat[tile % 2, j] + off
             else:
                 hi[j] = max(zhat[n - 1, j] + off, lo[j] + 1e-3)
     L.lo.copy_(torch.from_numpy(lo))
@@ -622,6 +625,26 @@ def test_kernels_for_a_few_tokens_with_4_bit_codes(d, h, G, q):
     cfg = W.LayerConfig("few4bit%d" % d, d, h, group=G, n_calib=256, q_lo=q, q_hi=1 - q, bits=4)
     calls = [1, 3, 16, 17, 33, 64, 65, 128]
     _run(cfg, sum(calls), calls)
+
+
+@pytest.mark.parametrize("d,h,G,bits", [(16, 32, 16, 2), (80, 96, 16, 4), (160, 224, 32, 3), (208, 1056, 16, 2), (64, 64, 64, 8)])
+def test_set_up_kernels_at_the_edges_of_their_tiles(d, h, G, bits):
+    # transposes of 64 x 64 tiles, two elements per access, with sides that end inside a tile; dequantised codes of every width
+    cfg = W.LayerConfig("setup%d" % d, d, h, group=G, bits=bits, n_calib=256)
+    _run(cfg, 9, path=1)
+    if bits <= 4:
+        _run(cfg, 140, path=3)
+    L = _layer(cfg)
+    hd = T.fold_layer(L)
+    try:
+        Wf, bf = torch.empty(d, d, dtype=torch.bfloat16, device="cuda"), torch.empty(d, device="cuda")
+        T.tardis_export_folded(hd, Wf, bf)
+        ref, bref = O.fold(*[L.numpy64()[k] for k in ("W1", "W2", "a", "c", "b1", "b2")])
+        # one rounding to bf16 of sums whose terms keep 16 bits
+        assert np.abs(Wf.double().cpu().numpy() - ref).max() <= 2.0 ** -8 * np.abs(ref).max()
+        assert np.abs(bf.double().cpu().numpy() - bref).max() <= 1e-5 * max(1.0, np.abs(bref).max())
+    finally:
+        T.tardis_destroy(hd)
 
 
 @pytest.mark.parametrize("d,h,G,q", [(64, 32, 64, 0.4), (320, 2400, 64, 0.2), (4096, 16384, 128, 0.05), (4608, 18944, 64, 0.1),

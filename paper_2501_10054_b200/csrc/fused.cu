@@ -86,6 +86,7 @@ struct Params {
 struct Scratch {           // handle-owned device memory of this path
   uint8_t* pblocks; int2* plan; float* smax; float* yacc; unsigned int* ctl; uint4* Cp;
   Params base; size_t smem_bytes; size_t bytes; int grid; const void* kernels[2][3][2]; bool pairs_fit;
+  bool chain_ready;        // the chain's kernels have been given their shared memory (with the first chain: loading them takes time)
   float* dpart;            // partial outputs of the deterministic mode (allocated when the mode is first switched on)
   int nbuf_n[MAXT + 1];    // tile buffers in shared memory for a call of n tokens
   int gs_cap_n[MAXT + 1];  // ... and the most neurons of a step of its result fixing
@@ -1369,9 +1370,9 @@ tardis_status_t fused_prepare(Handle* H, cudaStream_t s) {
   else if (G == 64) choose(integral_constant<int, 64>(), integral_constant<int, 8>());
   else if (wide) choose(integral_constant<int, 128>(), integral_constant<int, 9>());
   else choose(integral_constant<int, 128>(), integral_constant<int, 8>());
-  for (int a = 0; a < 6 && e == cudaSuccess; ++a)
+  for (int a = 0; a < 3 && e == cudaSuccess; ++a)
     for (int b = 0; b < 2 && e == cudaSuccess; ++b)
-      e = cudaFuncSetAttribute(S->kernels[a / 3][a % 3][b], cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
+      e = cudaFuncSetAttribute(S->kernels[0][a][b], cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
   S->pairs_fit = (p.nkc * 2 == NWP || (p.nkc * 2 >= 2 * NWP && p.nkc * 2 < 3 * NWP));
   if (e != cudaSuccess) { set_last_error(e, "fused_prepare launch"); return fail(TARDIS_ERR_CUDA); }
 
@@ -1433,6 +1434,11 @@ tardis_status_t fused_set_deterministic(Handle* H, bool on) {
 tardis_status_t launch_fused_forward(Handle* H, const void* x, void* y, int n, cudaStream_t s, const FusedChain* chain) {
   Scratch* S = static_cast<Scratch*>(H->fscratch);
   const bool det = H->deterministic && S->dpart;
+  if (chain && !S->chain_ready) {
+    for (int a = 0; a < 3; ++a)
+      for (int b = 0; b < 2; ++b) TARDIS_CUDA_TRY(cudaFuncSetAttribute(S->kernels[1][a][b], cudaFuncAttributeMaxDynamicSharedMemorySize, int(S->smem_bytes)));
+    S->chain_ready = true;
+  }
   for (int t0 = 0; t0 < n;) {
     // calls of 5 to 8 tokens go as two launches of about equal size
     const int left = n - t0;

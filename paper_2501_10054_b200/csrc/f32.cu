@@ -3,10 +3,11 @@
 // Calls on such layers are small (256 / 1024 and 64 tokens: 50 MFLOP, 2.6 MB), so latency and launches are what counts; six
 // launches of the generic kernels, the predictor among them with the tokens one after the other, took 284 us there.
 //
-//   k_f32_in: a CTA takes 32 neurons and 16 (or 8) tokens: predictor scores from the packed codes and, in the same pass over the
-//     channels, the exact pre-activations; flags, and the flagged pairs' corrections, written to a dense [token][neuron] array (zero
-//     where not flagged).  (The pre-activations of the flagged pairs alone, eight lanes a pair behind the flags, wait for another round
-//     of loads and for two conversions per multiply-add, which the tenth of the work does not make up for.)
+//   k_f32_in: a CTA takes 32 neurons and 16 (or 8) tokens: predictor scores from the packed codes, flags, and the flagged pairs'
+//     corrections, written to a dense [token][neuron] array (zero where not flagged).  Where its CTAs do not fill the SMs once, the exact
+//     pre-activations of all pairs come out of the same walk over the channels: there is nothing to do but to wait, and the flagged
+//     pairs alone, eight lanes a pair behind the flags, wait for another round of loads.  Where there are more, work counts (the fp64
+//     unit, and from 1024 / 4096 on the bytes of W1): the flagged pairs alone, or a second walk in tiles where they are many.
 //   k_f32_out: y = b_f + [C ; W2^T]^T [x ; corrections], one product over d + h channels; its channel range is split over the
 //     CTAs of a cluster, which add their sums up through distributed shared memory, in order.  (Partial sums in global memory, a
 //     counter and the CTA that finishes last: three dependent trips to L2.  With that and the pairs above 256 / 1024 took 21.8 us for
@@ -43,15 +44,20 @@ struct Params {
   unsigned long long* counters;
   uint32_t* dbg_bitmap; double* dbg_scores;
 };
-struct State { float* delta; unsigned int* nfl; };
+struct State {
+  float* delta; unsigned int* nfl;
+  int clusters[2][MAX_SPLITS + 1];        // of k_f32_out with 8 and 16 tokens: clusters of so many CTAs that run at once
+};
 
-template <int TT> struct Smem {
+template <int TT, int PRODUCTS> struct Smem {
   union {
     // tokens of a pass and the next (padded: four channels x eight tokens in different banks); channel 16 w + 4 t + q in row 16 w + 4 q + t
     double xs[2][KC][TT + 4];
-    double red[2][NWARP][TT][TM];         // the warps' sums of one or two products
+    double red[PRODUCTS][NWARP][TT][TM];  // the warps' sums
   };
-  double total[TT][TM];                   // their sum (k_f32_out)
+};
+template <int TT> struct OutSmem : Smem<TT, 1> {
+  double total[TT][TM];                   // their sum
 };
 
 // A warp's 32 outputs x TT tokens.  Output 4 g + m of the CTA's 32 is row g (m even) or g + 8 (m odd) of row tile m / 2.
@@ -70,7 +76,7 @@ template <int TT> struct Acc {
       }
   }
   // the eight warps' sums of an output go where sum_of finds them (barriers before and after are the caller's)
-  __device__ __forceinline__ void put(Smem<TT>& sm, int product, int warp, int g, int t) const {
+  template <int PRODUCTS> __device__ __forceinline__ void put(Smem<TT, PRODUCTS>& sm, int product, int warp, int g, int t) const {
 #pragma unroll
     for (int nt = 0; nt < TT / 8; ++nt)
 #pragma unroll
@@ -81,7 +87,7 @@ template <int TT> struct Acc {
       }
   }
 };
-template <int TT> __device__ __forceinline__ double sum_of(const Smem<TT>& sm, int product, int t, int m) {
+template <int TT, int PRODUCTS> __device__ __forceinline__ double sum_of(const Smem<TT, PRODUCTS>& sm, int product, int t, int m) {
   double s = 0.0;
 #pragma unroll
   for (int w = 0; w < NWARP; ++w) s += sm.red[product][w][t][m];
@@ -99,7 +105,7 @@ template <int TT> struct Tokens {
       v[q] = (t0 + t < n && k < kend) ? *reinterpret_cast<const float4*>(src + size_t(t0 + t) * ld + k) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
   }
-  __device__ __forceinline__ void store(Smem<TT>& sm, int buffer) const {
+  template <int PRODUCTS> __device__ __forceinline__ void store(Smem<TT, PRODUCTS>& sm, int buffer) const {
 #pragma unroll
     for (int q = 0; q < TT * KC / 4 / NT; ++q) {
       const int e = q * NT + threadIdx.x, t = e % TT, k = e / TT, row = (k >> 2) * 16 + (k & 3);
@@ -111,19 +117,19 @@ template <int TT> struct Tokens {
   }
 };
 
-template <int BITS, int TT>
-__global__ void __launch_bounds__(NT) k_f32_in(const Params p) {
-  extern __shared__ __align__(16) unsigned char raw[];
-  Smem<TT>& sm = *reinterpret_cast<Smem<TT>*>(raw);
+// One walk over the channels for a CTA's neurons and tokens: the scores' products (SCORES), those of the exact pre-activations (EXACT),
+// or both.  FIRST: x has not been waited for yet.  Ends with the last products read from shared memory still under way in other warps.
+template <int BITS, int TT, bool SCORES, bool EXACT, bool FIRST, int PRODUCTS>
+__device__ __forceinline__ void walk(const Params& p, Smem<TT, PRODUCTS>& sm, Acc<TT>& acc, Acc<TT>& accz) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int j0 = blockIdx.x * TM, t0 = blockIdx.y * TT, ng = p.d / p.G;
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  Acc<TT> acc = {}, accz = {};
   Tokens<TT> x;
   // a thread expands four channels of four neurons (all of one group: groups are multiples of 16): s (q - zp), exact in fp64; and
   // takes the same of W1
   const int g = lane >> 2, t4 = lane & 3;
-  uint32_t w[4][BITS == 8 ? 4 : 2];
+  uint32_t w[4];                                           // 4 BITS bits from `shift` on: the codes of channels 4 t4 ..
+  const int half = min(12 * t4 / 16, 1);                   // 3-bit codes: the first of the two half-words that hold them
+  const int shift = BITS == 2 ? 8 * t4 : (BITS == 3 ? 12 * t4 - 16 * half : (BITS == 4 ? 16 * (t4 & 1) : 0));
   float sc[4], zp[4];
   float4 w1[4];
   auto load_weights = [&](int k0) {
@@ -131,25 +137,25 @@ __global__ void __launch_bounds__(NT) k_f32_in(const Params p) {
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
       const size_t j = j0 + 4 * g + m;
-      sc[m] = zp[m] = 0.f;
-      if (kb < p.d) {
-        sc[m] = p.scale[j * ng + kb / p.G];
-        zp[m] = float(p.zero[j * ng + kb / p.G]);
-        const uint32_t* const row = p.codes + j * (size_t(p.d) * BITS / 32);
-        if (BITS == 3) {                                   // 48 bits from a half-word on
-          const uint16_t* at = reinterpret_cast<const uint16_t*>(row) + kb * 3 / 16;
-          w[m][0] = uint32_t(at[0]) | uint32_t(at[1]) << 16;
-          w[m][1] = at[2];
-        } else {
-#pragma unroll
-          for (int q = 0; q < BITS / 2; ++q) w[m][q] = row[kb * BITS / 32 + q];
+      if (SCORES) {
+        sc[m] = zp[m] = 0.f;
+        if (kb < p.d) {
+          sc[m] = p.scale[j * ng + kb / p.G];
+          zp[m] = float(p.zero[j * ng + kb / p.G]);
+          const uint32_t* const row = p.codes + j * (size_t(p.d) * BITS / 32);
+          if (BITS == 3) {                                 // (48 bits from a half-word on)
+            const uint16_t* const at = reinterpret_cast<const uint16_t*>(row) + kb * 3 / 16 + half;
+            w[m] = uint32_t(at[0]) | uint32_t(at[1]) << 16;
+          } else {
+            w[m] = row[kb * BITS / 32 + (BITS == 8 ? t4 : (BITS == 4 ? t4 >> 1 : 0))];
+          }
         }
       }
-      w1[m] = k < p.d ? *reinterpret_cast<const float4*>(p.W1 + j * p.d + k) : make_float4(0.f, 0.f, 0.f, 0.f);   // (d: a multiple of 8)
+      if (EXACT) w1[m] = k < p.d ? *reinterpret_cast<const float4*>(p.W1 + j * p.d + k) : make_float4(0.f, 0.f, 0.f, 0.f);   // (d: a multiple of 8)
     }
   };
   load_weights(0);
-  asm volatile("griddepcontrol.wait;" ::: "memory");       // (x may come from the launch before)
+  if (FIRST) asm volatile("griddepcontrol.wait;" ::: "memory");   // (x may come from the launch before)
   x.load(p.x, p.d, p.n, t0, 0, p.d);
   int buffer = 0;
   for (int k0 = 0; k0 < p.d; k0 += KC, buffer ^= 1) {
@@ -157,56 +163,121 @@ __global__ void __launch_bounds__(NT) k_f32_in(const Params p) {
     double v[4][4], u[4][4];
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
-      const double s = double(sc[m]), z = 4503599627370496.0 + double(zp[m]);
+      if (SCORES) {
+        const double s = double(sc[m]), z = 4503599627370496.0 + double(zp[m]);
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {                        // channel 4 t4 + c
-        uint32_t q;
-        if (BITS == 3) q = uint32_t((uint64_t(w[m][0]) | uint64_t(w[m][1]) << 32) >> (3 * (4 * t4 + c))) & 7u;
-        else if (BITS == 2) q = (w[m][0] >> (8 * t4 + 2 * c)) & 3u;
-        else if (BITS == 4) q = ((t4 & 2 ? w[m][1] : w[m][0]) >> (16 * (t4 & 1) + 4 * c)) & 15u;
-        else q = ((t4 == 0 ? w[m][0] : (t4 == 1 ? w[m][1] : (t4 == 2 ? w[m][BITS == 8 ? 2 : 0] : w[m][BITS == 8 ? 3 : 0]))) >> (8 * c)) & 255u;
-        // (2^52 + q) - (2^52 + zp): the code as a double without a conversion
-        v[c][m] = s * (__hiloint2double(0x43300000, int(q)) - z);
+        for (int c = 0; c < 4; ++c) {                      // channel 4 t4 + c
+          const uint32_t q = (w[m] >> (shift + BITS * c)) & ((1u << BITS) - 1u);
+          // (2^52 + q) - (2^52 + zp): the code as a double without a conversion
+          v[c][m] = s * (__hiloint2double(0x43300000, int(q)) - z);
+        }
       }
-      u[0][m] = double(w1[m].x); u[1][m] = double(w1[m].y); u[2][m] = double(w1[m].z); u[3][m] = double(w1[m].w);
+      if (EXACT) { u[0][m] = double(w1[m].x); u[1][m] = double(w1[m].y); u[2][m] = double(w1[m].z); u[3][m] = double(w1[m].w); }
     }
     __syncthreads();                                       // (a buffer is written again two passes on, behind this barrier)
     if (k0 + KC < p.d) { load_weights(k0 + KC); x.load(p.x, p.d, p.n, t0, k0 + KC, p.d); }
-    acc.multiply(v, &sm.xs[buffer][warp * 16], g, t4);
-    accz.multiply(u, &sm.xs[buffer][warp * 16], g, t4);
+    if (SCORES) acc.multiply(v, &sm.xs[buffer][warp * 16], g, t4);
+    if (EXACT) accz.multiply(u, &sm.xs[buffer][warp * 16], g, t4);
   }
+}
+
+// BOTH: scores and exact pre-activations in one walk; else the scores alone, and then, by the tile's number of flagged pairs, the
+// flagged pairs one by one or a second walk.  A pair of its own takes four times the clocks of a pair of the second walk (two conversions
+// per multiply-add and no reuse; 1024 / 4096 and 256 tokens: 6 us per hundredth of the pairs that is flagged, a second walk 146 us), so a
+// quarter is where the second walk begins.  Registers: one CTA per SM is all there is for BOTH (1024 / 4096, 1 token 24.3 us with 174,
+// 31.7 with the 128 of two); else two, as 80 hold back the loads (2048 / 8192, 1 token 60 us with 128, 77 with 80).
+template <int BITS, int TT, bool BOTH>
+__global__ void __launch_bounds__(NT, BOTH ? 1 : 2) k_f32_in(const Params p) {
+  extern __shared__ __align__(16) unsigned char raw[];
+  Smem<TT, BOTH ? 2 : 1>& sm = *reinterpret_cast<Smem<TT, BOTH ? 2 : 1>*>(raw);
+  __shared__ int pairs[BOTH ? 1 : TT * TM];
+  __shared__ int npairs;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t4 = lane & 3;
+  const int j0 = blockIdx.x * TM, t0 = blockIdx.y * TT;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (!BOTH && threadIdx.x == 0) npairs = 0;
+  Acc<TT> acc = {}, accz = {};
+  walk<BITS, TT, true, BOTH, true>(p, sm, acc, accz);
   __syncthreads();
   acc.put(sm, 0, warp, g, t4);
-  accz.put(sm, 1, warp, g, t4);
+  if (BOTH) accz.put(sm, 1, warp, g, t4);
   __syncthreads();
   // scores -> flags -> corrections; lane = neuron, a warp takes tokens warp, warp + 8 (all at once: their fp64 chains overlap)
   const int j = j0 + lane;
   const double lo = double(p.lo[j]), hi = double(p.hi[j]), b1 = double(p.b1[j]), fa = double(p.a[j]), fc = double(p.c[j]);
+  auto correction = [&](double z) { return float(gelu_f64(z, p.act) - fa * z - fc); };
   bool flag[TT / NWARP];
   float delta[TT / NWARP];
 #pragma unroll
   for (int k = 0; k < TT / NWARP; ++k) {
     const int t = warp + k * NWARP;
-    const double zhat = sum_of<TT>(sm, 0, t, lane) + b1, z = sum_of<TT>(sm, 1, t, lane) + b1;
+    const double zhat = sum_of(sm, 0, t, lane) + b1;
     flag[k] = !(lo <= zhat && zhat < hi);
-    delta[k] = float(gelu_f64(z, p.act) - fa * z - fc);
+    if (BOTH) delta[k] = correction(sum_of(sm, 1, t, lane) + b1);
     if (p.dbg_scores && t0 + t < p.n) p.dbg_scores[size_t(t0 + t) * p.h + j] = zhat;
   }
 #pragma unroll
   for (int k = 0; k < TT / NWARP; ++k) {
     const int t = t0 + warp + k * NWARP;
     if (t >= p.n) break;
-    p.delta[size_t(t) * p.h + j] = flag[k] ? delta[k] : 0.f;
+    if (BOTH || !flag[k]) p.delta[size_t(t) * p.h + j] = BOTH && flag[k] ? delta[k] : 0.f;
     const uint32_t word = __ballot_sync(0xffffffffu, flag[k]);
     if (lane == 0 && word) atomicAdd(&p.nfl[t], (unsigned int)__popc(word));
     if (lane == 0 && p.dbg_bitmap) p.dbg_bitmap[size_t(t) * (p.h / 32) + blockIdx.x] = word;
+    if (!BOTH) {
+      int base = 0;
+      if (lane == 0 && word) base = atomicAdd(&npairs, __popc(word));
+      base = __shfl_sync(0xffffffffu, base, 0);
+      if (flag[k]) pairs[base + __popc(word & ((1u << lane) - 1u))] = (t - t0) * TM + lane;
+    }
+  }
+  if constexpr (!BOTH) {
+    __syncthreads();
+    const int np = npairs;
+    if (np > TT * TM / 4) {
+      walk<BITS, TT, false, true, false>(p, sm, acc, accz);
+      __syncthreads();
+      accz.put(sm, 0, warp, g, t4);
+      __syncthreads();
+#pragma unroll
+      for (int k = 0; k < TT / NWARP; ++k) {
+        const int t = warp + k * NWARP;
+        delta[k] = correction(sum_of(sm, 0, t, lane) + b1);
+        if (t0 + t < p.n && flag[k]) p.delta[size_t(t0 + t) * p.h + j] = delta[k];
+      }
+      return;
+    }
+    // eight lanes a pair
+    const int sub = lane & 7;
+    for (int e0 = warp * 4; e0 < np; e0 += NWARP * 4) {
+      const int e = e0 + (lane >> 3);
+      const int pr = pairs[min(e, np - 1)], jj = j0 + (pr & (TM - 1)), t = t0 + pr / TM;
+      const float* row = p.W1 + size_t(jj) * p.d;
+      const float* xt = p.x + size_t(t) * p.d;
+      double z0 = 0.0, z1 = 0.0, z2 = 0.0, z3 = 0.0;       // (four chains: the latency of one would be most of the time)
+#pragma unroll 8
+      for (int k = sub * 4; k < p.d; k += 32) {            // (d is a multiple of 8, rows are 16-byte aligned)
+        const float4 w = *reinterpret_cast<const float4*>(row + k), v = *reinterpret_cast<const float4*>(xt + k);
+        z0 += double(w.x) * double(v.x);
+        z1 += double(w.y) * double(v.y);
+        z2 += double(w.z) * double(v.z);
+        z3 += double(w.w) * double(v.w);
+      }
+      double z = (z0 + z1) + (z2 + z3);
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+      if (sub == 0 && e < np) {
+        z += double(p.b1[jj]);
+        p.delta[size_t(t) * p.h + jj] = float(gelu_f64(z, p.act) - double(p.a[jj]) * z - double(p.c[jj]));
+      }
+    }
   }
 }
 
 template <int TT>
 __global__ void __launch_bounds__(NT) k_f32_out(const Params p) {
   extern __shared__ __align__(16) unsigned char raw[];
-  Smem<TT>& sm = *reinterpret_cast<Smem<TT>*>(raw);
+  OutSmem<TT>& sm = *reinterpret_cast<OutSmem<TT>*>(raw);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int i0 = blockIdx.x * TM, t0 = blockIdx.y * TT, z = blockIdx.z;
   const int passes_d = (p.d + KC - 1) / KC, passes = passes_d + (p.h + KC - 1) / KC;   // C first, then W2^T
@@ -247,13 +318,13 @@ __global__ void __launch_bounds__(NT) k_f32_out(const Params p) {
   acc.put(sm, 0, warp, g, t4);
   __syncthreads();
 #pragma unroll
-  for (int t = warp; t < TT; t += NWARP) sm.total[t][lane] = sum_of<TT>(sm, 0, t, lane);
+  for (int t = warp; t < TT; t += NWARP) sm.total[t][lane] = sum_of(sm, 0, t, lane);
   // the CTAs of the cluster share out the tile's outputs; each adds up the parts of its own, in order
   if (p.splits > 1) asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
   else __syncthreads();
-  const int share = TT * TM / p.splits;                    // (splits: a power of two)
-  for (int e = int(threadIdx.x); e < share; e += NT) {
-    const int o = z * share + e, t = t0 + o / TM, i = i0 + o % TM;
+  const int share = (TT * TM + p.splits - 1) / p.splits, end = min((z + 1) * share, TT * TM);
+  for (int o = z * share + int(threadIdx.x); o < end; o += NT) {
+    const int t = t0 + o / TM, i = i0 + o % TM;
     const uint32_t at = uint32_t(__cvta_generic_to_shared(&sm.total[0][0] + o));
     double part[MAX_SPLITS];
 #pragma unroll
@@ -278,8 +349,8 @@ __global__ void __launch_bounds__(NT) k_f32_out(const Params p) {
 }
 
 using Kernel = void (*)(Params);
-template <int TT> static Kernel in_kernel(int bits) {
-  return bits == 2 ? k_f32_in<2, TT> : (bits == 3 ? k_f32_in<3, TT> : (bits == 4 ? k_f32_in<4, TT> : k_f32_in<8, TT>));
+template <int TT, bool BOTH> static Kernel in_kernel(int bits) {
+  return bits == 2 ? k_f32_in<2, TT, BOTH> : (bits == 3 ? k_f32_in<3, TT, BOTH> : (bits == 4 ? k_f32_in<4, TT, BOTH> : k_f32_in<8, TT, BOTH>));
 }
 
 }  // namespace f32
@@ -287,6 +358,20 @@ template <int TT> static Kernel in_kernel(int bits) {
 using namespace f32;
 
 namespace {
+// a launch of k_f32_out in clusters of `size`, with one attribute at `attr`
+cudaLaunchConfig_t out_config(dim3 grid, int size, cudaStream_t s, cudaLaunchAttribute* attr) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = dim3(NT); cfg.stream = s;
+  attr->id = cudaLaunchAttributeClusterDimension;
+  attr->val.clusterDim.x = 1; attr->val.clusterDim.y = 1; attr->val.clusterDim.z = unsigned(size);
+  cfg.attrs = attr; cfg.numAttrs = 1;
+  return cfg;
+}
+// may start while the launch before it still runs
+void overlapped(cudaLaunchAttribute* attr) {
+  attr->id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr->val.programmaticStreamSerializationAllowed = 1;
+}
 struct Sizes { size_t bytes[2]; };                         // delta, nfl
 Sizes sizes(const Handle* H) { return {{size_t(MAX_CHUNK) * H->h * 4, MAX_CHUNK * 4}}; }
 }  // namespace
@@ -313,10 +398,20 @@ tardis_status_t f32_prepare(Handle* H, cudaStream_t s) {
     H->bytes_scratch += bytes[i];
   }
   TARDIS_CUDA_TRY(cudaMemsetAsync(S->nfl, 0, bytes[1], s));
-  const Kernel wide[2] = {in_kernel<16>(H->bits), k_f32_out<16>}, narrow[2] = {in_kernel<8>(H->bits), k_f32_out<8>};
-  for (int i = 0; i < 2; ++i) {
-    TARDIS_CUDA_TRY(cudaFuncSetAttribute(wide[i], cudaFuncAttributeMaxDynamicSharedMemorySize, int(sizeof(Smem<16>))));
-    TARDIS_CUDA_TRY(cudaFuncSetAttribute(narrow[i], cudaFuncAttributeMaxDynamicSharedMemorySize, int(sizeof(Smem<8>))));
+  auto room = [](Kernel k, size_t bytes) { return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes)); };
+  TARDIS_CUDA_TRY(room(in_kernel<16, true>(H->bits), sizeof(Smem<16, 2>)));
+  TARDIS_CUDA_TRY(room(in_kernel<16, false>(H->bits), sizeof(Smem<16, 1>)));
+  TARDIS_CUDA_TRY(room(k_f32_out<16>, sizeof(OutSmem<16>)));
+  TARDIS_CUDA_TRY(room(in_kernel<8, true>(H->bits), sizeof(Smem<8, 2>)));
+  TARDIS_CUDA_TRY(room(in_kernel<8, false>(H->bits), sizeof(Smem<8, 1>)));
+  TARDIS_CUDA_TRY(room(k_f32_out<8>, sizeof(OutSmem<8>)));
+  for (int size = 2; size <= MAX_SPLITS; ++size) {
+    cudaLaunchAttribute attr;
+    cudaLaunchConfig_t cfg = out_config(dim3(1, 1, size), size, nullptr, &attr);
+    cfg.dynamicSmemBytes = sizeof(OutSmem<8>);
+    TARDIS_CUDA_TRY(cudaOccupancyMaxActiveClusters(&S->clusters[0][size], k_f32_out<8>, &cfg));
+    cfg.dynamicSmemBytes = sizeof(OutSmem<16>);
+    TARDIS_CUDA_TRY(cudaOccupancyMaxActiveClusters(&S->clusters[1][size], k_f32_out<16>, &cfg));
   }
   return TARDIS_OK;
 }
@@ -332,20 +427,21 @@ void f32_release(Handle* H) {
 }
 
 template <int TT> static tardis_status_t launch_chunk(const Handle* H, const Params& p, cudaStream_t s) {
-  const int tiles = (p.n + TT - 1) / TT;
-  const dim3 grids[2] = {dim3(p.h / TM, tiles), dim3((p.d + TM - 1) / TM, tiles, p.splits)};
-  const Kernel kernels[2] = {in_kernel<TT>(H->bits), k_f32_out<TT>};
-  for (int i = 0; i < 2; ++i) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grids[i]; cfg.blockDim = dim3(NT); cfg.dynamicSmemBytes = sizeof(Smem<TT>); cfg.stream = s;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = 1; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = unsigned(p.splits);
-    cfg.attrs = attr; cfg.numAttrs = i == 1 && p.splits > 1 ? 2 : 1;
-    TARDIS_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernels[i], p));
-  }
+  const int tiles = (p.n + TT - 1) / TT, in_ctas = p.h / TM * tiles;
+  // us with both in one walk against scores first, there with a twentieth to a third of the pairs flagged: 256 / 1024, 64 tokens (128 CTAs) 18.5
+  // against 19.7 .. 21.5; 512 / 2048, 16 tokens (64) 21.1, 25.2 .. 28.8; 768 / 3072, 24 tokens (192) 45.6, 36.9 .. 42.9; 1024 / 4096, 64
+  // tokens (512) 119, 92 .. 104.
+  const bool both = in_ctas <= H->num_sms;
+  cudaLaunchAttribute attrs[2];
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(p.h / TM, tiles); cfg.blockDim = dim3(NT); cfg.dynamicSmemBytes = both ? sizeof(Smem<TT, 2>) : sizeof(Smem<TT, 1>); cfg.stream = s;
+  overlapped(&attrs[0]);
+  cfg.attrs = attrs; cfg.numAttrs = 1;
+  TARDIS_CUDA_TRY(cudaLaunchKernelEx(&cfg, both ? in_kernel<TT, true>(H->bits) : in_kernel<TT, false>(H->bits), p));
+  cfg = out_config(dim3((p.d + TM - 1) / TM, tiles, p.splits), p.splits, s, &attrs[1]);
+  cfg.dynamicSmemBytes = sizeof(OutSmem<TT>);
+  cfg.attrs = attrs; cfg.numAttrs = p.splits > 1 ? 2 : 1;
+  TARDIS_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_f32_out<TT>, p));
   return TARDIS_OK;
 }
 
@@ -361,11 +457,12 @@ tardis_status_t launch_f32_forward(Handle* H, const void* xv, void* yv, int64_t 
     p.delta = S->delta; p.nfl = S->nfl; p.counters = H->counters;
     p.dbg_bitmap = H->dbg_bitmap ? H->dbg_bitmap + size_t(t0) * (H->h / 32) : nullptr;
     p.dbg_scores = H->dbg_scores ? H->dbg_scores + size_t(t0) * H->h : nullptr;
-    // parts of the split product: about two CTAs per SM, at least one pass of KC channels each, a power of two up to a cluster's CTAs
+    // parts of the split product: as many as leave it one wave of clusters, at least one pass of KC channels each
     const int tt = p.n <= 8 ? 8 : 16, tiles = ((p.d + TM - 1) / TM) * ((p.n + tt - 1) / tt);
     const int passes = (p.d + KC - 1) / KC + (p.h + KC - 1) / KC;
     p.splits = 1;
-    while (p.splits < MAX_SPLITS && 2 * p.splits <= passes && 2 * p.splits * tiles <= 2 * H->num_sms) p.splits *= 2;
+    for (int size = 2; size <= MAX_SPLITS && size <= passes; ++size)
+      if (tiles <= S->clusters[tt == 8 ? 0 : 1][size]) p.splits = size;
     const tardis_status_t st = tt == 8 ? launch_chunk<8>(H, p, s) : launch_chunk<16>(H, p, s);
     if (st != TARDIS_OK) return st;
     H->launches += 2;

@@ -572,6 +572,16 @@ def test_f32_kernels_at_the_edges_of_their_tiles(d, h, G, bits):
     _run(cfg, sum(calls), calls)
 
 
+@pytest.mark.parametrize("d,h,bits,q,calls", [(144, 4800, 2, 0.02, [1, 8, 9, 17, 33]), (144, 4800, 4, 0.12, [3, 16, 40]), (288, 4800, 3, 0.35, [2, 9, 24]),
+                                              (144, 2400, 8, 0.3, [16, 17, 32]), (768, 320, 2, 0.1, [40, 48, 64])])
+def test_f32_scores_first_then_flagged_pairs_or_a_second_walk(d, h, bits, q, calls):
+    # more tiles of 32 neurons and 8 or 16 tokens than SMs (150 of them, or 75 where 16 tokens are one walk and 17 are not), with few
+    # pairs flagged in a tile, about the quarter where the second walk begins, and most; output tiles whose parts are a number of CTAs
+    # that does not divide them (768 channels x 48 tokens: threes)
+    cfg = W.LayerConfig("f32two%d" % d, d, h, dtype="f32", group=16, bits=bits, n_calib=256, q_lo=q, q_hi=1 - q)
+    _run(cfg, sum(calls), calls)
+
+
 @pytest.mark.parametrize("d,h,G,q", [(128, 32, 64, 0.05), (192, 96, 64, 0.2), (576, 2080, 192, 0.05), (1152, 4640, 128, 0.1), (640, 19040, 64, 0.02)])
 def test_kernels_for_a_few_tokens_at_the_edges_of_their_tiles(d, h, G, q):
     # columns of 16 (two-term corrections), 32, 64, 128 tokens; neuron tiles of 16 to 128 rows with a short last one, one or several

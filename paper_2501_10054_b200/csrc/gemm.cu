@@ -425,7 +425,7 @@ k_gemm(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtenso
 
 // ---- host side ------------------------------------------------------------------------------------------
 template <int BN, int CTAS>
-static tardis_status_t launch_bn(const GemmArgs& g, cudaStream_t s) {
+static tardis_status_t launch_bn(const GemmArgs& g, int dev, int sms, cudaStream_t s) {
   CUtensorMap a1, b1, a2, b2;
   if (!make_map(&a1, g.A1, g.M, g.K1, g.lda1, BM) || !make_map(&b1, g.B1, g.N, g.K1, g.ldb1, BN / CTAS)) return TARDIS_ERR_INVALID_ARG;
   a2 = a1; b2 = b1;
@@ -439,8 +439,6 @@ static tardis_status_t launch_bn(const GemmArgs& g, cudaStream_t s) {
   p.lo = g.lo; p.hi = g.hi; p.colscale = g.colscale; p.rowscale = g.rowscale; p.keps = g.keps; p.bitmap_out = g.bitmap_out;
   p.rlist = g.rlist; p.rcount = g.rcount; p.rcap = g.rcap; p.bits = g.bits;
   static thread_local int room_on = -1;               // the device on which this thread last gave the kernel its shared memory
-  int dev = 0, sms = 0;
-  TARDIS_CUDA_TRY(cudaGetDevice(&dev));
   if (dev != room_on) {
     TARDIS_CUDA_TRY(cudaFuncSetAttribute(k_gemm<BN, CTAS>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<BN, CTAS>::SMEM));
     room_on = dev;
@@ -450,7 +448,6 @@ static tardis_status_t launch_bn(const GemmArgs& g, cudaStream_t s) {
   const int fcount = p.fast_m ? nm : nn;
   p.band = fcount <= 16 / (p.fast_m ? CTAS : 1) ? fcount : 12 / (p.fast_m ? CTAS : 1);
   const long tiles = long(nm) * nn * p.splits;
-  TARDIS_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const long at_once = sms / CTAS;                                    // one CTA per SM (shared memory), persistent
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(unsigned(tiles < at_once ? tiles : at_once) * CTAS); cfg.blockDim = dim3(NTHREADS); cfg.dynamicSmemBytes = Cfg<BN, CTAS>::SMEM; cfg.stream = s;
@@ -479,13 +476,22 @@ tardis_status_t launch_gemm(const GemmArgs& g, cudaStream_t s) {
   // the epilogues store (or reduce) 16 bytes at a time
   auto misaligned = [](const void* p) { return p && (reinterpret_cast<uintptr_t>(p) & 15u); };
   if (misaligned(g.out_f32) || misaligned(g.out_bf16)) return TARDIS_ERR_INVALID_ARG;
-  // wide tiles when they still fill the machine, narrow ones for skinny problems
+  int dev = 0, sms = 0;
+  TARDIS_CUDA_TRY(cudaGetDevice(&dev));
+  TARDIS_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  // wide tiles when they still fill the machine (120 of 148 SMs), narrow ones for skinny problems
   const long splits = g.splits > 1 ? g.splits : 1, nm = (g.M + BM - 1) / BM, nn = (g.N + 255) / 256;
-  if (nm * nn * splits < 120) return launch_bn<128, 1>(g, s);
-  // pairs of CTAs unless the half tile that an odd number of row tiles leaves idle costs more
-  const long waves = (nm * nn * splits + 147) / 148, pair_waves = ((nm + 1) / 2 * nn * splits + 73) / 74;
-  if (pair_waves * 10 <= waves * 11) return launch_bn<256, 2>(g, s);
-  return launch_bn<256, 1>(g, s);
+  if (nm * nn * splits * 100 < sms * 81) return launch_bn<128, 1>(g, dev, sms, s);
+  // Pairs of CTAs unless the half tile that an odd number of row tiles leaves idle costs more, and for products of 2048 channels and more: a pair's
+  // start, its two meetings and the accumulators' return to one of the two cost some 2 us and 1 us per wave.  us alone / in pairs, operands
+  // from memory: 512 x 8192 (one wave) K = 1024 21.2 / 22.8, 2048 26.9 / 26.9, 4096 40.2 / 38.0; 512 x 16384 (two) 1024 32.3 / 33.0, 2048 46.2 / 42.5; 2048 x 16384
+  // (seven) 512 93 / 103, 1024 100 / 105, 1536 118 / 119, 2048 152 / 138.  (With both operands in L2 and one wave the line lies at 6144: 2048 x 2048 x 4096 33.1 / 35.1,
+  // 8192 59.7 / 56.6; weights that are read once per token or prompt come from memory.)
+  const long waves = (nm * nn * splits + sms - 1) / sms, pair_waves = ((nm + 1) / 2 * nn * splits + sms / 2 - 1) / (sms / 2);
+  const long blocks = (g.K1 + BK - 1) / BK + (g.K2 > 0 && !g.second_used ? (g.K2 + BK - 1) / BK : 0);
+  const bool long_enough = blocks / splits >= 32;
+  if (long_enough && pair_waves * 10 <= waves * 11) return launch_bn<256, 2>(g, dev, sms, s);
+  return launch_bn<256, 1>(g, dev, sms, s);
 }
 
 }  // namespace tardis

@@ -27,9 +27,10 @@ def test_gemm_matches_definition(M, N, K):
     assert np.abs(got - ref).max() <= 2e-3 * np.abs(ref).max()
 
 
-# large enough for pairs of CTAs (tiles of 256 x 256): an odd number of 128-row tiles, a second half of few or of no rows, columns and
-# channels that end inside a tile; the last one has fewer tiles than CTAs
-@pytest.mark.parametrize("M,N,K", [(1100, 4500, 72), (130, 32000, 64), (257, 15400, 200), (4096, 1288, 640), (2048, 2000, 1032)])
+# long and large enough for pairs of CTAs (tiles of 256 x 256): an odd number of 128-row tiles, a second half of few or of no rows, columns
+# and channels that end inside a tile; the last one has fewer tiles than CTAs.  (The first five: as many tiles, too short for pairs.)
+@pytest.mark.parametrize("M,N,K", [(1100, 4500, 72), (130, 32000, 64), (257, 15400, 200), (4096, 1288, 640), (2048, 2000, 1032),
+                                   (1100, 9000, 2056), (130, 32000, 2568), (2048, 2000, 2056)])
 def test_gemm_pairs_of_ctas(M, N, K):
     test_gemm_matches_definition(M, N, K)
 

@@ -250,6 +250,26 @@ def test_range_search_choices_that_rest_on_rounding_are_fixed():
     assert steps.tolist() == pinned
 
 
+def test_range_search_choices_among_many_samples_are_fixed_too():
+    # as above with 2000 samples: a value holds some 200 of them, and the sums are those of all threads together.  Pinned as one warp's sums
+    # in the same order gave them.
+    pinned = {W.ACT_GELU_ERF: [17, 20, 20, 18, 17, 17, 18, 17, 17, 20, 38, 20, 17, 17, 17, 20, 20, 20, 18, 20, 20, 17, 20, 17, 20, 20, 20, 20, 34, 20, 31, 18,
+                               20, 20, 20, 17, 20, 20, 20, 20, 18, 22, 20, 18, 17, 20, 17, 20],
+              W.ACT_RELU: [18, 41, 16, 18, 16, 34, 18, 36, 36, 18, 18, 18, 18, 31, 16, 18, 18, 16, 16, 16, 16, 21, 16, 18, 16, 16, 20, 18, 34, 18, 18, 16,
+                           18, 46, 16, 31, 18, 18, 16, 18, 16, 16, 16, 18, 18, 18, 18, 16]}
+    z = (torch.randn(48, 2000, generator=torch.Generator().manual_seed(6)) * 4).round() / 4
+    for act, steps in pinned.items():
+        assert T.tardis_range_search(z.cuda(), None, 0.5, 0.1, act, want_steps=True)[4].tolist() == steps
+
+
+@pytest.mark.parametrize("n", [64, 66, 257, 2048])
+def test_range_search_undecided_steps_by_a_warp_and_by_all_threads(n):
+    # ReLU over a kink: most steps' errors lie closer together than the moments can tell; up to 64 samples inside a warp decides.  (Fewer
+    # samples: with two or three inside both errors are zero but for rounding, and which is smaller rests on the order of the sums.)
+    z = torch.randn(10, n, generator=torch.Generator().manual_seed(n)) * 1.3 + torch.linspace(-1, 1, 10)[:, None]
+    assert _check_search(z.cuda(), None, 0.95, 0.02, W.ACT_RELU) <= 2
+
+
 def test_greedy_range_search_edge_cases_and_errors():
     lib = T.load_library()
     # all samples equal, a single sample, threshold 0 (empty range at the centroid) and 1 (every sample)

@@ -260,7 +260,9 @@ template <int E> __device__ __forceinline__ bool pick_ranks(const float (&v)[E],
 // Bound by the latency of its barriers and by the fp64 activation.  16384 neurons x 2048 samples: 0.24 ms (0.28 with five CTAs per SM, two passes
 // and an activation that branches, 0.46 ms with the
 // samples sorted in registers, 0.91 ms with every step of the sort in shared memory and the activation as a fp64 tanh, evaluated twice).
-template <int E> __global__ void __launch_bounds__(NT, E <= 8 ? 6 : 1)   // (CTAs per SM: their barriers and chains overlap; one pass and no stored activations leave the registers for six)
+// ERF: the erf form, which branches and is left out where nothing is inside, as beyond n (8192 x 1500: 152 us evaluated everywhere, 130); the
+// others are straight on for every sample.
+template <int E, bool ERF> __global__ void __launch_bounds__(NT, E <= 8 ? 6 : 1)   // (CTAs per SM: their barriers and chains overlap; one pass and no stored activations leave the registers for six)
 k_calibrate(const float* __restrict__ z, long long ldz, const float* __restrict__ b1, int n, double q_lo, double q_hi,
             int act, float* __restrict__ lo, float* __restrict__ hi, float* __restrict__ a, float* __restrict__ c) {
   extern __shared__ float keys[];                      // [NT E]
@@ -296,7 +298,7 @@ k_calibrate(const float* __restrict__ z, long long ldz, const float* __restrict_
     range[r] = float(__dadd_rn(__dmul_rn(double(stat[2 * r]), 1.0 - w), __dmul_rn(double(stat[2 * r + 1]), w)));
   }
   // Least squares of the activation over the samples inside, in one pass: moments about one of those samples, so that samples that are
-  // all equal give a variance of exactly zero (and the offset of the others' mean costs a digit at most).  Two passes (means first) need a
+  // all equal give a variance of exactly zero (the offset of the mean costs at most log10(n) digits of 16, with one sample far below all others).  Two passes (means first) need a
   // second round of barriers, and the activations kept in registers, which are then too many for a sixth CTA per SM.
   const float l = range[0], u = range[1];
   const double c0 = double(stat[1] >= l && stat[1] < u ? stat[1] : l);
@@ -306,7 +308,7 @@ k_calibrate(const float* __restrict__ z, long long ldz, const float* __restrict_
   for (int e = 0; e < E; ++e) {
     const bool inside = v[e] >= l && v[e] < u;
     const double x = double(inside ? v[e] : float(c0));
-    const double g = (act == TARDIS_ACT_GELU_TANH ? gelu_tanh_f64(x) : gelu_f64(x, act)) - g0, y = x - c0;
+    const double g = (ERF ? (inside ? gelu_f64(x, TARDIS_ACT_GELU_ERF) : g0) : (act == TARDIS_ACT_GELU_TANH ? gelu_tanh_f64(x) : gelu_f64(x, act))) - g0, y = x - c0;
     if (inside) { m[0] += 1.0; m[1] += y; m[2] += g; m[3] = fma(y, y, m[3]); m[4] = fma(y, g, m[4]); }
   }
   block_sums(m, red5);
@@ -999,7 +1001,8 @@ tardis_status_t launch_calibrate(int h, int n, const float* z, long long ldz, co
   if (n < 1 || n > cal::kMaxSamples) return TARDIS_ERR_UNSUPPORTED;
   return cal::with_samples<cal::kMaxSamples / cal::NT>(n, [&](auto e) {
     constexpr int E = decltype(e)::value;
-    cal::k_calibrate<E><<<h, cal::NT, size_t(cal::NT) * E * sizeof(float), s>>>(z, ldz, b1, n, q_lo, q_hi, act, lo, hi, a, c);
+    const auto kernel = act == TARDIS_ACT_GELU_ERF ? cal::k_calibrate<E, true> : cal::k_calibrate<E, false>;
+    kernel<<<h, cal::NT, size_t(cal::NT) * E * sizeof(float), s>>>(z, ldz, b1, n, q_lo, q_hi, act, lo, hi, a, c);
     TARDIS_CUDA_TRY(cudaGetLastError());
     return TARDIS_OK;
   });

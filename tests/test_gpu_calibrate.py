@@ -54,6 +54,38 @@ def test_quantiles_picked_without_sorting_and_where_that_is_left_to_the_sort(n, 
     _check(z.cuda(), None, q[0], q[1], W.ACT_GELU_TANH)
 
 
+@pytest.mark.parametrize("n", [200, 300, 1100, 1500])
+def test_erf_fits_with_most_places_beyond_the_samples_or_outside_the_range(n):
+    # the activation is left out there: places beyond n (n just above a power of two times 256), ranges that leave out most samples
+    z = torch.randn(20, n, generator=torch.Generator().manual_seed(n)) * torch.linspace(0.2, 4.0, 20)[:, None]
+    for q in (0.0, 0.3, 0.49):
+        _check(z.cuda(), None, q, 1.0 - q, W.ACT_GELU_ERF)
+
+
+def test_one_sample_far_below_the_others():
+    # the fit's moments are taken about the lowest sample inside: with one at a distance D of n the variance is about D^2 / n of a second
+    # moment of D^2, which costs log10(n) digits of 16
+    z = torch.randn(6, 2048, generator=torch.Generator().manual_seed(3))
+    z[:, 100] = -torch.tensor([10.0, 1e2, 1e3, 1e4, 1e5, 1e6])
+    _check(z.cuda(), None, 0.0, 1.0, W.ACT_RELU)
+    _check(z.cuda(), None, 0.0, 1.0, W.ACT_GELU_TANH)
+
+
+def test_the_tanh_form_in_64_bits_from_slopes_between_neighbouring_floats():
+    """The line through two samples one float apart magnifies an error of the activation by 1 / 2^-23 z: the slope, stored in single (6.7e-8 of up to
+    1.13), tells errors of some 3e-15 z, that is of the exponential below 1e-13.  Reference in extended precision."""
+    z1 = torch.cat([torch.linspace(-6, 6, 400), torch.logspace(-4, 0, 60), -torch.logspace(-4, 0, 60)])
+    z2 = torch.nextafter(z1, torch.full_like(z1, 100.0))
+    z = torch.stack([z1, z2, z2 + 1.0], 1).contiguous()             # (the range ends at the third)
+    _, _, a, _ = T.tardis_calibrate(z.cuda(), None, 0.0, 1.0, W.ACT_GELU_TANH)
+    x = z.numpy().astype(np.longdouble)[:, :2]
+    two = np.longdouble(2)
+    c = np.sqrt(two / np.arccos(np.longdouble(-1)))
+    g = x / (1 + np.exp(-two * c * (x + np.longdouble("0.044715") * x ** 3)))
+    ref = ((g[:, 1] - g[:, 0]) / (x[:, 1] - x[:, 0])).astype(np.float64)
+    assert np.abs(a.cpu().numpy() - ref).max() <= 1e-7
+
+
 def test_padded_rows_ties_and_degenerate_neurons():
     # leading dimension larger than n, many equal samples, constant neurons
     g = torch.Generator().manual_seed(7)

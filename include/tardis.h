@@ -293,8 +293,10 @@ tardis_status_t tardis_set_deterministic(tardis_handle_t handle, int32_t on);
  * contain 0; scale = (max - min) / (2^bits - 1) rounded to `dtype`, 1 if that is 0; zero-point = round(-min / scale)
  * clamped to the code range); q_k = clip(round(w_k / scale + zero)); e_k = (w_k - scale (q_k - zero)) / U[k][k]; every
  * later channel takes w_j <- w_j - e_k U[k][j].  Rounding is to nearest-even, and the codes are those of a plain double-precision
- * implementation with separately rounded products and differences (bf16 layers: decided by multiply-adds where these
- * tell, neurons that come close to a rounding boundary done again that way).
+ * implementation with separately rounded products and differences: by construction for float32 layers, 8-bit codes, groups other than 64
+ * and 128, a U that is not 16-byte aligned and without U; else (bf16 layers) multiply-adds decide, and neurons in which a decision came closer to a rounding
+ * boundary than the difference of the two can be are done again the plain way.  That difference is bounded with rounding errors taken as independent of
+ * each other (32 deviations, for any U); a code outside it would need errors that conspire.
  *   W1     device [d_ff, d_model] row-major in `dtype`;
  *   U      device double [d_model, d_model] row-major, the upper Cholesky factor of the inverse Hessian of the layer's
  *          inputs (U^T U = H^-1, H = (2/N) X^T X plus damping: made by the caller, e.g. with a library Cholesky), only

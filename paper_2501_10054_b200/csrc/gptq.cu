@@ -228,14 +228,30 @@ __device__ double distance_to_other_bf16(double v, double s) {
   return fmin(v - (m0 - even * h0), (m1 + even * h1) - v);
 }
 
-// negated reciprocals of the diagonal of U
-__global__ void k_reciprocals(const double* __restrict__ U, double* __restrict__ ninv, int d) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < d) ninv[k] = __ddiv_rn(-1.0, U[size_t(k) * d + k]);
+// Negated reciprocals of the diagonal of U; the largest sum of squares of a column above the diagonal (as bits: of positive numbers the
+// order is the same, and no number comes out on top).  A warp takes every 32nd row of 32 columns.
+__global__ void __launch_bounds__(1024) k_columns(const double* __restrict__ U, double* __restrict__ ninv, unsigned long long* __restrict__ largest, int d) {
+  __shared__ double sums[32][33];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, j = blockIdx.x * 32 + lane, last = min(d, int(blockIdx.x + 1) * 32);
+  double sum = 0.0;
+#pragma unroll 16
+  for (int k = warp; k < last; k += 32) {
+    const double u = U[size_t(k) * d + min(j, d - 1)];
+    if (k < j) sum = fma(u, u, sum);
+  }
+  sums[warp][lane] = sum;
+  __syncthreads();
+  if (warp > 0) return;
+  sum = 0.0;
+  for (int w = 0; w < 32; ++w) sum += sums[w][lane];
+  unsigned long long top = j < d ? (unsigned long long)(__double_as_longlong(fabs(sum))) : 0ull;
+  for (int o = 16; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
+  if (lane == 0) atomicMax(largest, top);
+  if (j < d) ninv[j] = __ddiv_rn(-1.0, U[size_t(j) * d + j]);
 }
 
 // CTA c: neurons c R .. c R + R - 1.  E: the negated errors of all its channels, [CTA][channel][R].  margin: how close (in weight) the
-// neuron came to a decision that falls the other way; size: its largest weight on the way.
+// neuron came to a decision that falls the other way; size: its largest weight when it was rounded; squares: the sum of its errors' squares.
 // Bound by the fp64 matrix instruction, 0.72 of its rate on 16384 x 4096; U comes from L2 (67 MB per CTA), E from memory (8.6 GB in all).
 // (10.8 ms with a barrier every 16 channels instead of 32; the rounding inside the blocks, a chain of six dependent fp64 operations per
 // channel, is 0.6 of it.  A shorter chain for 2-bit codes, and rounding that begins while other warps still spread the eight channels
@@ -244,7 +260,7 @@ template <int MT>
 __global__ void __launch_bounds__(FT, 2) k_build(const __nv_bfloat16* __restrict__ W1, const double* __restrict__ U, const double* __restrict__ ninv,
                                                  int h, int d, int G, int levels, double* E, double* __restrict__ scale64,
                                                  double* __restrict__ zero64, uint8_t* __restrict__ q, double* __restrict__ margin_out,
-                                                 double* __restrict__ size_out) {
+                                                 double* __restrict__ size_out, double* __restrict__ squares_out) {
   using C = BuildCfg<MT>;
   constexpr int R = C::R, ES = C::ES, US = C::US;
   extern __shared__ __align__(16) double sm[];
@@ -295,6 +311,7 @@ __global__ void __launch_bounds__(FT, 2) k_build(const __nv_bfloat16* __restrict
   const int r = r0 + tid;
   const bool real = r < h, probe = r >= h && r < h + PROBES;
   double s = 1.0, rs = 1.0, z = 0.0, zc = 4503599627370496.0, margin = 1e300, size = 0.0;
+  double squares = 0.0;                             // of the errors of neuron tid - FT / 2
   bool strange = false;
 
   for (int b = 0, slot = 0; b < nblocks; ++b) {
@@ -407,6 +424,9 @@ __global__ void __launch_bounds__(FT, 2) k_build(const __nv_bfloat16* __restrict
         __syncthreads();
         // (channels that are done take part where they share a warp with ones that are not: nothing reads them any more)
         if (warp > owner || (warp == owner && half == 0)) multiply(es + half * 8 * ES, us + half * 8 * US);
+        if (tid >= FT / 2 && tid < FT / 2 + R)      // (not by the threads that round: 0.2 ms of 10 in their chain)
+#pragma unroll
+          for (int i = 0; i < 8; ++i) { const double e = es[(half * 8 + i) * ES + tid - FT / 2]; squares = fma(e, e, squares); }
       }
     }
   }
@@ -414,22 +434,27 @@ __global__ void __launch_bounds__(FT, 2) k_build(const __nv_bfloat16* __restrict
     margin_out[r] = strange ? -1.0 : margin;
     size_out[r] = strange ? 1e300 : size;
   }
+  if (tid >= FT / 2 && tid < FT / 2 + R && r - FT / 2 < h + PROBES) squares_out[r - FT / 2] = squares;
 }
 
-// The neurons whose codes may not be the plain way's.  The two ways differ in the rounding of the operations, unit u = 2^-53: a weight
-// sees up to 3 d of them, each of at most a few u times the largest weight M, independent and of either sign, so what they put into a
-// weight stays below lambda u sqrt(d) M with a probability that approaches 1 as exp(-lambda^2 / 2) (the probabilistic rounding analysis
-// of Higham and Mary, 2019).  A difference in one weight goes on into the later ones by the same recurrence without the rounding to
-// codes; the probe rows have followed 16 such disturbances, +-1 in every channel, and A is the largest value that came of them.
-// lambda = 32 leaves room for all constants: the largest difference between the plain way and the same in 64-bit significands is 0.15 of
-// u sqrt(d) A M (24 neurons of 1536 channels, A = 6.5).  On a 4096 / 16384 layer A = 15 and the bound is 3.4e-12 of a weight: one layer in
-// some 300 has a neuron that came closer than that to a boundary anywhere (then 2 to 5 ms for the plain way with a few neurons).
-__global__ void k_suspects(const double* __restrict__ margin, const double* __restrict__ size, int h, double unit, int* __restrict__ list, int* __restrict__ count) {
+// The neurons whose codes may not be the plain way's.  The two ways differ in the rounding of the operations, unit u = 2^-53: a weight sees up
+// to 3 d of them, each of at most u times the largest sum P that it goes through.  P is bounded for any U: a part of sum e_k U[k][j] is at
+// most |e| C (Cauchy and Schwarz), C the largest norm of a column above the diagonal, and with the largest weight M that was rounded
+// P <= M + 2 |e| C.  With roundings of either sign that do not depend on each other, what they put into a weight stays below lambda u sqrt(d) P
+// with a probability that approaches 1 as exp(-lambda^2 / 6) (the probabilistic rounding analysis of Higham and Mary, 2019).  A difference
+// in one weight goes on into the later ones by the same recurrence without the rounding to codes; the probe rows have followed 16 such
+// disturbances, +-1 in every channel, and A is the largest value that came of them.  lambda = 32: exp(-170).
+// On a 4096 / 16384 layer P is some 45 M and the bound 1e-11: one layer in some 25 has a neuron that came closer than that to a boundary
+// anywhere (then 2 to 5 ms for the plain way with a few neurons).  (M in place of P misses factors whose terms cancel: 1.3^(j - k) above the
+// diagonal takes sums to 1e14 and weights back to 0.1.)
+__global__ void k_suspects(const double* __restrict__ margin, const double* __restrict__ size, const double* __restrict__ squares,
+                           const unsigned long long* __restrict__ largest, int h, double unit, int* __restrict__ list, int* __restrict__ count) {
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= h) return;
   double growth = 1.0;
   for (int p = 0; p < PROBES; ++p) growth = fmax(growth, size[h + p]);
-  if (!(margin[r] > unit * growth * size[r])) list[atomicAdd(count, 1)] = r;
+  const double sums = size[r] + 2.0 * sqrt(squares[r]) * sqrt(__longlong_as_double((long long)*largest));
+  if (!(margin[r] > unit * growth * sums)) list[atomicAdd(count, 1)] = r;
 }
 
 struct BuildShape { int mt, ctas; };
@@ -503,7 +528,7 @@ tardis_status_t launch_build_predictor(int h, int d, int dtype, const void* W1, 
   }
   // the plain way's working copy and, before it, the errors of k_build share their memory
   const size_t wd_bytes = fast ? size_t(shape.ctas) * 8 * shape.mt * d * 8 : size_t(h) * d * 8;
-  const size_t notes_bytes = fast ? (size_t(d) + 2 * (size_t(h) + PROBES)) * 8 + (size_t(h) + 1) * 4 : 0;
+  const size_t notes_bytes = fast ? (size_t(d) + 3 * (size_t(h) + PROBES) + 1) * 8 + (size_t(h) + 1) * 4 : 0;
   double *Wd = nullptr, *Eb = nullptr, *scale64 = nullptr, *zero64 = nullptr, *notes = nullptr;
   uint8_t* q = nullptr;
   auto release = [&]() {
@@ -522,16 +547,17 @@ tardis_status_t launch_build_predictor(int h, int d, int dtype, const void* W1, 
   int rows = h;
   if (fast) {
     double* const ninv = notes;
-    double *const margin = ninv + d, *const size = margin + h + PROBES;
-    int* const count = reinterpret_cast<int*>(size + h + PROBES);
+    double *const margin = ninv + d, *const size = margin + h + PROBES, *const squares = size + h + PROBES;
+    unsigned long long* const largest = reinterpret_cast<unsigned long long*>(squares + h + PROBES);
+    int* const count = reinterpret_cast<int*>(largest + 1);
     list = count + 1;
     const double unit = 32.0 * 1.1102230246251565e-16 * sqrt(double(d));
-    e = cudaMemsetAsync(count, 0, sizeof(int), s);
-    k_reciprocals<<<(d + 255) / 256, 256, 0, s>>>(U, ninv, d);
+    e = cudaMemsetAsync(largest, 0, sizeof(unsigned long long) + sizeof(int), s);   // (and the count behind it)
+    k_columns<<<(d + 31) / 32, 1024, 0, s>>>(U, ninv, largest, d);
     if (e == cudaSuccess)
       e = launch_build<1>(shape.mt, shape.ctas, s, static_cast<const __nv_bfloat16*>(W1), U, static_cast<const double*>(ninv), h, d, G, levels, Wd,
-                          scale64, zero64, q, margin, size);
-    k_suspects<<<(h + 255) / 256, 256, 0, s>>>(margin, size, h, unit, count + 1, count);
+                          scale64, zero64, q, margin, size, squares);
+    k_suspects<<<(h + 255) / 256, 256, 0, s>>>(margin, size, squares, largest, h, unit, count + 1, count);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpyAsync(&rows, count, sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);

@@ -421,7 +421,8 @@ def _upper_factor(X, damp=0.01):
 
 def _build_and_compare(W1, U, bits, G, rows=None):
     """GPU builder against the oracle on the same W1 and U: codes, zero-points and scales must be identical (every rounding
-    decision is taken in double precision with the same sequence of rounded operations on both sides)."""
+    decision is taken as double precision with the oracle's sequence of rounded operations takes it, or further from a boundary than another sequence
+    can lead)."""
     dtype = "f32" if W1.dtype == torch.float32 else "bf16"
     Ud = None if U is None else torch.from_numpy(U).cuda()
     codes, scale, zero = T.tardis_build_predictor(W1, Ud, bits, G)
@@ -461,7 +462,7 @@ def test_build_predictor_groups_and_superblocks(h, d, G):
 
 
 # k_build takes up to 56 neurons per CTA in eights, 128 channels at a time: row counts around those (16 rows are added to measure the
-# growth of rounding errors), a last block of 64 channels, both group sizes, all code widths
+# growth of rounding errors), a last block of 64 channels, both group sizes, 2 to 4 bits (and 8, which go the plain way)
 @pytest.mark.parametrize("h,d,G,bits", [(1, 64, 64, 2), (112, 128, 128, 4), (113, 192, 64, 3), (2353, 256, 64, 8), (4721, 320, 64, 2), (16561, 128, 128, 2)])
 def test_build_predictor_one_launch_edges(h, d, G, bits):
     g = torch.Generator().manual_seed(h + d)
@@ -498,6 +499,36 @@ def test_build_predictor_close_decisions_are_done_again(kind):
         assert all(bool(torch.equal(x[keep], y[keep])) for x, y in zip((codes, scale, zero), ref))
         return
     _build_and_compare(W1.cuda(), U, 2, G)
+
+
+@pytest.mark.parametrize("growth", [1.1, 1.3, 1.5])
+def test_build_predictor_sums_that_grow_and_cancel(growth):
+    """A factor whose terms take a weight to growth^127 times its size and back within one group: what the rounding of the large sums leaves is far
+    above that of the weights themselves, so closeness to a boundary has to be measured by the sums."""
+    d = 128
+    W1 = (torch.randn(2000, d, generator=torch.Generator().manual_seed(5)) * 0.03).bfloat16().cuda()
+    k = np.arange(d)
+    _build_and_compare(W1, np.triu(growth ** np.maximum(k[None, :] - k[:, None], 0).astype(np.float64)), 2, 128)
+
+
+@pytest.mark.parametrize("d,h,n,damp,bits,G", [(1024, 4096, 2000, 1e-2, 2, 64), (1024, 4096, 300, 1e-6, 3, 128), (2048, 4096, 1024, 1e-9, 4, 64),
+                                               (4096, 16384, 1024, 1e-2, 2, 128), (4096, 8192, 1024, 1e-2, 4, 128)])
+def test_build_predictor_quick_and_plain_way_agree_on_whole_layers(d, h, n, damp, bits, G):
+    """Every code, scale and zero-point of a layer, decided by multiply-adds and by separately rounded products and differences (a factor that does not
+    begin on a 16-byte boundary is not read by the quick kernel's copies and goes the plain way); also fewer samples than channels and next to no damping."""
+    for seed in (1, 2):
+        g = torch.Generator(device="cuda").manual_seed(seed)
+        X = torch.randn(n, d, generator=g, device="cuda", dtype=torch.float64)
+        H = 2.0 / n * X.t() @ X
+        H += damp * H.diagonal().mean() * torch.eye(d, dtype=torch.float64, device="cuda")
+        U = torch.linalg.cholesky(torch.cholesky_inverse(torch.linalg.cholesky(H)), upper=True).contiguous()
+        W1 = (torch.randn(h, d, generator=g, device="cuda") * 0.02).bfloat16()
+        room = torch.empty(d * d + 1, dtype=torch.float64, device="cuda")
+        aside = room[1:].view(d, d)
+        aside.copy_(U)
+        assert U.data_ptr() % 16 == 0 and aside.data_ptr() % 16 == 8
+        for quick, plain in zip(T.tardis_build_predictor(W1, U, bits, G), T.tardis_build_predictor(W1, aside, bits, G)):
+            assert torch.equal(quick, plain)
 
 
 def test_build_predictor_full_size_sampled_rows_and_use_in_a_layer():

@@ -26,6 +26,8 @@
 //
 // Both are bound by the fp64 units: h d^2 / 2 multiply-adds (16384 x 4096, 1.4e11: 7.4 ms at 37 TFLOP/s), or twice as many separate
 // products and differences.  16384 x 4096: 10.4 ms of kernels, 22.8 the plain way.
+#include <type_traits>
+
 #include "common.cuh"
 #include "ptx.cuh"
 
@@ -372,7 +374,7 @@ __global__ void __launch_bounds__(FT, 2) k_build(const __nv_bfloat16* __restrict
         }
         __syncthreads();
         if (tid < R) {
-          const bool first = j0 + c == 0;           // weights as they came: their decisions are taken as the plain way takes them
+          const bool first = j0 + c == 0;           // weights as they came
           if (opens) {
             double mn = 0.0, mx = 0.0;
             for (int w = owner; w < owner + G / 16; ++w) {
@@ -401,23 +403,33 @@ __global__ void __launch_bounds__(FT, 2) k_build(const __nv_bfloat16* __restrict
 #pragma unroll
           for (int i = 0; i < 8; ++i) w[i] = Wc[i * R + tid];
           unsigned long long codes = 0;
+          // FIRST: of the neuron's first eight channels those up to the first error that is not zero are weights as they came, bf16 values
+          // that tie now and then; their decisions are taken as the plain way takes them, and none of them is close.  (With the first
+          // channel's alone a 4-bit layer of 8192 neurons has one done again the plain way for it.)
+          auto round_eight = [&](auto first_ones) {
+            constexpr bool FIRST = decltype(first_ones)::value;
+            bool untouched = true;
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            double v = fma(w[i], rs, z);
-            if (i == 0 && first) v = __dadd_rn(__ddiv_rn(w[0], s), z);
-            // the nearest whole number in the low bits of v + 1.5 2^52; a code less the zero-point as (2^52 + q) - (2^52 + z)
-            const double m = v + 6755399441055744.0, away = fabs(v - (m - 6755399441055744.0));
-            const int code = min(max(__double2loint(m), 0), levels);
-            strange = strange || !(fabs(v) < 1073741824.0);
-            if (v > 0.0 && v < double(levels) && !(i == 0 && first)) worst = fmax(worst, away);
-            size = fmax(size, fabs(w[i]));
-            const double ne = (probe ? w[i] : fma(-s, __hiloint2double(0x43300000, code) - zc, w[i])) * ni[i];
-            es[(half * 8 + i) * ES + tid] = ne;
-            Eg[size_t(j0 + c + i) * R + tid] = ne;
+            for (int i = 0; i < 8; ++i) {
+              double v = fma(w[i], rs, z);
+              if (FIRST && untouched) v = __dadd_rn(__ddiv_rn(w[i], s), z);
+              // the nearest whole number in the low bits of v + 1.5 2^52; a code less the zero-point as (2^52 + q) - (2^52 + z)
+              const double m = v + 6755399441055744.0, away = fabs(v - (m - 6755399441055744.0));
+              const int code = min(max(__double2loint(m), 0), levels);
+              strange = strange || !(fabs(v) < 1073741824.0);
+              if (v > 0.0 && v < double(levels) && !(FIRST && untouched)) worst = fmax(worst, away);
+              size = fmax(size, fabs(w[i]));
+              const double ne = (probe ? w[i] : fma(-s, __hiloint2double(0x43300000, code) - zc, w[i])) * ni[i];
+              untouched = untouched && ne == 0.0;
+              es[(half * 8 + i) * ES + tid] = ne;
+              Eg[size_t(j0 + c + i) * R + tid] = ne;
 #pragma unroll
-            for (int j = i + 1; j < 8; ++j) w[j] = fma(ne, uc[i * US + j], w[j]);
-            codes |= (unsigned long long)(unsigned int)(code) << (8 * i);
-          }
+              for (int j = i + 1; j < 8; ++j) w[j] = fma(ne, uc[i * US + j], w[j]);
+              codes |= (unsigned long long)(unsigned int)(code) << (8 * i);
+            }
+          };
+          if (first) round_eight(std::true_type());
+          else round_eight(std::false_type());
           margin = fmin(margin, (0.5 - worst) * s);
           if (real) *reinterpret_cast<unsigned long long*>(q + size_t(r) * d + j0 + c) = codes;
         }
@@ -444,17 +456,61 @@ __global__ void __launch_bounds__(FT, 2) k_build(const __nv_bfloat16* __restrict
 // with a probability that approaches 1 as exp(-lambda^2 / 6) (the probabilistic rounding analysis of Higham and Mary, 2019).  A difference
 // in one weight goes on into the later ones by the same recurrence without the rounding to codes; the probe rows have followed 16 such
 // disturbances, +-1 in every channel, and A is the largest value that came of them.  lambda = 32: exp(-170).
-// On a 4096 / 16384 layer P is some 45 M and the bound 1e-11: one layer in some 25 has a neuron that came closer than that to a boundary
-// anywhere (then 2 to 5 ms for the plain way with a few neurons).  (M in place of P misses factors whose terms cancel: 1.3^(j - k) above the
-// diagonal takes sums to 1e14 and weights back to 0.1.)
-__global__ void k_suspects(const double* __restrict__ margin, const double* __restrict__ size, const double* __restrict__ squares,
-                           const unsigned long long* __restrict__ largest, int h, double unit, int* __restrict__ list, int* __restrict__ count) {
+// That P is some 45 M on a 4096 / 16384 layer and the bound 1e-11 of a weight: one layer in some 25 has a neuron that came closer than that to a
+// boundary anywhere, a 4544 / 18176 layer one or two.  For up to kTightened of them the largest sum is then taken from the errors themselves
+// (k_largest_sums; it is about M, and 2 to 5 ms for the plain way with a few neurons become rare).  (M in place of P misses factors whose terms
+// cancel: 1.3^(j - k) above the diagonal takes sums to 1e14 and weights back to 0.1.)
+constexpr int kTightened = 64;
+struct Notes {                                // of k_build, behind one another in device memory
+  double *ninv, *margin, *size, *squares;     // [d], [h + PROBES] each
+  unsigned long long *column, *sums;          // bits of the largest column's squares; of the listed neurons' largest sums
+  int *count, *list;
+  static size_t bytes(int h, int d) { return (size_t(d) + 3 * (size_t(h) + PROBES) + 1 + kTightened) * 8 + (size_t(h) + 1) * 4; }
+  Notes(double* at, int h, int d) : ninv(at), margin(at + d), size(margin + h + PROBES), squares(size + h + PROBES),
+      column(reinterpret_cast<unsigned long long*>(squares + h + PROBES)), sums(column + 1), count(reinterpret_cast<int*>(sums + kTightened)), list(count + 1) {}
+};
+__device__ double growth_of(const Notes& n, int h) {
+  double growth = 1.0;
+  for (int p = 0; p < PROBES; ++p) growth = fmax(growth, n.size[h + p]);
+  return growth;
+}
+__global__ void k_suspects(const Notes n, int h, double unit) {
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= h) return;
-  double growth = 1.0;
-  for (int p = 0; p < PROBES; ++p) growth = fmax(growth, size[h + p]);
-  const double sums = size[r] + 2.0 * sqrt(squares[r]) * sqrt(__longlong_as_double((long long)*largest));
-  if (!(margin[r] > unit * growth * sums)) list[atomicAdd(count, 1)] = r;
+  const double sums = n.size[r] + 2.0 * sqrt(n.squares[r]) * sqrt(__longlong_as_double((long long)*n.column));
+  if (!(n.margin[r] > unit * growth_of(n, h) * sums)) n.list[atomicAdd(n.count, 1)] = r;
+}
+// Block (x, y): 32 channels of the y-th neuron of the list, its weights with every error's term added in turn: a warp per 32nd of the errors,
+// whose sums come first.  (One thread per channel alone waits 1.4 ms for its loads.)  E as k_build left it, R neurons per CTA.
+__global__ void __launch_bounds__(1024) k_largest_sums(const Notes n, const __nv_bfloat16* __restrict__ W1, const double* __restrict__ U, const double* __restrict__ E, int d, int R) {
+  __shared__ double sums[32][33];
+  const int count = *n.count, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, j = blockIdx.x * 32 + lane;
+  if (count > kTightened || int(blockIdx.y) >= count) return;
+  const int r = n.list[blockIdx.y], jc = min(j, d - 1), each = (d + 31) / 32, from = warp * each, to = min(min(d, from + each), int(blockIdx.x + 1) * 32);
+  const double* const e = E + size_t(r / R) * d * R + r % R;
+  auto term = [&](int k) { return k < j ? e[size_t(k) * R] * U[size_t(k) * d + jc] : 0.0; };
+  double sum = 0.0;
+#pragma unroll 16
+  for (int k = from; k < to; ++k) sum += term(k);
+  sums[warp][lane] = sum;
+  __syncthreads();
+  double w = double(__bfloat162float(W1[size_t(r) * d + jc])), top = fabs(w);
+  for (int q = 0; q < warp; ++q) w += sums[q][lane];
+#pragma unroll 16
+  for (int k = from; k < to; ++k) { w += term(k); top = !(fabs(w) <= top) ? fabs(w) : top; }     // (what is no number stays on top)
+  unsigned long long bits = j < d ? (unsigned long long)(__double_as_longlong(top)) & 0x7fffffffffffffffull : 0ull;
+  for (int o = 16; o > 0; o >>= 1) bits = max(bits, __shfl_xor_sync(0xffffffffu, bits, o));
+  if (lane == 0) atomicMax(n.sums + blockIdx.y, bits);
+}
+__global__ void __launch_bounds__(kTightened) k_confirm(const Notes n, int h, double unit) {
+  const int count = *n.count, s = threadIdx.x;
+  if (count > kTightened) return;
+  const int r = s < count ? n.list[s] : 0;
+  const bool keep = s < count && !(n.margin[r] > unit * growth_of(n, h) * __longlong_as_double((long long)n.sums[s]));
+  __syncthreads();
+  if (s == 0) *n.count = 0;
+  __syncthreads();
+  if (keep) n.list[atomicAdd(n.count, 1)] = r;
 }
 
 struct BuildShape { int mt, ctas; };
@@ -528,7 +584,7 @@ tardis_status_t launch_build_predictor(int h, int d, int dtype, const void* W1, 
   }
   // the plain way's working copy and, before it, the errors of k_build share their memory
   const size_t wd_bytes = fast ? size_t(shape.ctas) * 8 * shape.mt * d * 8 : size_t(h) * d * 8;
-  const size_t notes_bytes = fast ? (size_t(d) + 3 * (size_t(h) + PROBES) + 1) * 8 + (size_t(h) + 1) * 4 : 0;
+  const size_t notes_bytes = fast ? Notes::bytes(h, d) : 0;
   double *Wd = nullptr, *Eb = nullptr, *scale64 = nullptr, *zero64 = nullptr, *notes = nullptr;
   uint8_t* q = nullptr;
   auto release = [&]() {
@@ -546,20 +602,19 @@ tardis_status_t launch_build_predictor(int h, int d, int dtype, const void* W1, 
   const int* list = nullptr;                               // the neurons that are done the plain way (null: all)
   int rows = h;
   if (fast) {
-    double* const ninv = notes;
-    double *const margin = ninv + d, *const size = margin + h + PROBES, *const squares = size + h + PROBES;
-    unsigned long long* const largest = reinterpret_cast<unsigned long long*>(squares + h + PROBES);
-    int* const count = reinterpret_cast<int*>(largest + 1);
-    list = count + 1;
+    const Notes n(notes, h, d);
+    list = n.list;
     const double unit = 32.0 * 1.1102230246251565e-16 * sqrt(double(d));
-    e = cudaMemsetAsync(largest, 0, sizeof(unsigned long long) + sizeof(int), s);   // (and the count behind it)
-    k_columns<<<(d + 31) / 32, 1024, 0, s>>>(U, ninv, largest, d);
+    e = cudaMemsetAsync(n.column, 0, reinterpret_cast<char*>(n.list) - reinterpret_cast<char*>(n.column), s);
+    k_columns<<<(d + 31) / 32, 1024, 0, s>>>(U, n.ninv, n.column, d);
     if (e == cudaSuccess)
-      e = launch_build<1>(shape.mt, shape.ctas, s, static_cast<const __nv_bfloat16*>(W1), U, static_cast<const double*>(ninv), h, d, G, levels, Wd,
-                          scale64, zero64, q, margin, size, squares);
-    k_suspects<<<(h + 255) / 256, 256, 0, s>>>(margin, size, squares, largest, h, unit, count + 1, count);
+      e = launch_build<1>(shape.mt, shape.ctas, s, static_cast<const __nv_bfloat16*>(W1), U, static_cast<const double*>(n.ninv), h, d, G, levels, Wd,
+                          scale64, zero64, q, n.margin, n.size, n.squares);
+    k_suspects<<<(h + 255) / 256, 256, 0, s>>>(n, h, unit);
+    k_largest_sums<<<dim3((d + 31) / 32, kTightened), 1024, 0, s>>>(n, static_cast<const __nv_bfloat16*>(W1), U, Wd, d, 8 * shape.mt);
+    k_confirm<<<1, kTightened, 0, s>>>(n, h, unit);
     if (e == cudaSuccess) e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&rows, count, sizeof(int), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&rows, n.count, sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   }
   if (e == cudaSuccess && rows > 0) {

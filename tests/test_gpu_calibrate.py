@@ -531,6 +531,21 @@ def test_build_predictor_quick_and_plain_way_agree_on_whole_layers(d, h, n, damp
             assert torch.equal(quick, plain)
 
 
+def test_build_predictor_first_weights_that_tie():
+    # first errors that are exactly zero leave the next weights as they came, and these lie on rounding boundaries: 1.5, 2.5, 3.5 steps of the
+    # grid behind none to seven such channels, then an ordinary row
+    d, G, bits = 128, 128, 4
+    g = torch.Generator().manual_seed(9)
+    W1 = (torch.randn(64, d, generator=g) * 0.03).bfloat16()
+    W1[:, 100], W1[:, 101] = 0.125, -0.109375                       # the ends of every grid: a step of 2^-6, zero-point 7
+    W1 = W1.clamp(-0.109375, 0.125)
+    for r in range(64):
+        W1[r, : r % 8] = 2.0 ** -6 * (r % 5 - 2)
+        W1[r, r % 8] = 2.0 ** -6 * (0.5 + r % 3)
+    X = torch.randn(3 * d, d, generator=g) @ (torch.eye(d) + 0.5 * torch.randn(d, d, generator=g) / d ** 0.5)
+    _build_and_compare(W1.cuda(), _upper_factor(X.numpy()), bits, G)
+
+
 def test_build_predictor_full_size_sampled_rows_and_use_in_a_layer():
     """The 7B-class layer (16384 x 4096, groups of 128, 2 bits): sampled neurons against the oracle (neurons are independent
     given U), then the built predictor goes into tardis_fold and a forward is compared with the oracle run on those codes."""

@@ -29,6 +29,7 @@
 //     last one adds b_f, rounds to bf16, writes y and re-zeroes the scratch.
 #include <stdio.h>
 
+#include <mutex>
 #include <new>
 #include <type_traits>
 
@@ -86,7 +87,6 @@ struct Params {
 struct Scratch {           // handle-owned device memory of this path
   uint8_t* pblocks; int2* plan; float* smax; float* yacc; unsigned int* ctl; uint4* Cp;
   Params base; size_t smem_bytes; size_t bytes; int grid; const void* kernels[2][3][2]; bool pairs_fit;
-  bool chain_ready;        // the chain's kernels have been given their shared memory (with the first chain: loading them takes time)
   float* dpart;            // partial outputs of the deterministic mode (allocated when the mode is first switched on)
   int nbuf_n[MAXT + 1];    // tile buffers in shared memory for a call of n tokens
   int gs_cap_n[MAXT + 1];  // ... and the most neurons of a step of its result fixing
@@ -1280,8 +1280,24 @@ size_t fused_room(const Handle* H) {
          dev_room(16) + dev_room(sizeof(float) * MAXT * dacc) + dev_room(8192) + dev_room(sizeof(int) * H->h);
 }
 
-// Builds the state of this path for bf16 layers with 2-bit codes, group size 64 or 128 and d_model a multiple of 16
-// up to 4608; other layers are left to the other kernels (H->fscratch stays null).
+// All of a layer's kernels are given their shared memory when the layer is set up, so that no forward call, which may be under capture, is the
+// first to load one.  Loading them takes time that every layer would pay for again: done once per device and set of kernels.
+static cudaError_t give_shared_memory(int device, int set, const void* (&kernels)[2][3][2], int bytes) {
+  constexpr int kDevices = 64, kSets = 4;
+  static std::mutex mutex;
+  static bool done[kDevices][kSets];
+  std::lock_guard<std::mutex> lock(mutex);
+  if (device < kDevices && done[device][set]) return cudaSuccess;
+  for (const auto& of_tokens : kernels)
+    for (const auto& forms : of_tokens)
+      for (const void* kernel : forms) {
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        if (e != cudaSuccess) return e;
+      }
+  if (device < kDevices) done[device][set] = true;
+  return cudaSuccess;
+}
+
 tardis_status_t fused_prepare(Handle* H, cudaStream_t s) {
   H->fscratch = nullptr;
   const int d = H->d, h = H->h, G = H->G;
@@ -1370,9 +1386,7 @@ tardis_status_t fused_prepare(Handle* H, cudaStream_t s) {
   else if (G == 64) choose(integral_constant<int, 64>(), integral_constant<int, 8>());
   else if (wide) choose(integral_constant<int, 128>(), integral_constant<int, 9>());
   else choose(integral_constant<int, 128>(), integral_constant<int, 8>());
-  for (int a = 0; a < 3 && e == cudaSuccess; ++a)
-    for (int b = 0; b < 2 && e == cudaSuccess; ++b)
-      e = cudaFuncSetAttribute(S->kernels[0][a][b], cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
+  if (e == cudaSuccess) e = give_shared_memory(H->device, (G == 64 ? 2 : 0) + (wide ? 1 : 0), S->kernels, max_smem);
   S->pairs_fit = (p.nkc * 2 == NWP || (p.nkc * 2 >= 2 * NWP && p.nkc * 2 < 3 * NWP));
   if (e != cudaSuccess) { set_last_error(e, "fused_prepare launch"); return fail(TARDIS_ERR_CUDA); }
 
@@ -1434,11 +1448,6 @@ tardis_status_t fused_set_deterministic(Handle* H, bool on) {
 tardis_status_t launch_fused_forward(Handle* H, const void* x, void* y, int n, cudaStream_t s, const FusedChain* chain) {
   Scratch* S = static_cast<Scratch*>(H->fscratch);
   const bool det = H->deterministic && S->dpart;
-  if (chain && !S->chain_ready) {
-    for (int a = 0; a < 3; ++a)
-      for (int b = 0; b < 2; ++b) TARDIS_CUDA_TRY(cudaFuncSetAttribute(S->kernels[1][a][b], cudaFuncAttributeMaxDynamicSharedMemorySize, int(S->smem_bytes)));
-    S->chain_ready = true;
-  }
   for (int t0 = 0; t0 < n;) {
     // calls of 5 to 8 tokens go as two launches of about equal size
     const int left = n - t0;

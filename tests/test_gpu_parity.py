@@ -667,6 +667,42 @@ def test_fused_kernels_at_the_edges_of_their_rings(d, h, G, q):
     _run(cfg, sum(calls), calls, path=2)
 
 
+def test_first_call_of_a_process_may_be_a_chain_under_capture():
+    # every kernel of a chain has to be loaded and to have its shared memory when the layers are set up: a process of its own, whose first
+    # forward call is captured, and the shape of each of the four sets of kernels
+    import subprocess
+    import sys
+    script = r"""
+import sys
+import torch
+import paper_2501_10054_b200 as T
+import workloads as W
+for d, G in ((256, 64), (256, 128), (4544, 64), (4224, 128)):
+    cfg = W.LayerConfig("capture%d" % d, d, 512, group=G, n_calib=256)
+    L = [W.make_layer(cfg, s, device=torch.device("cuda", 0)) for s in (1, 2)]
+    handles = [T.fold_layer(l) for l in L]
+    for n in (1, 2, 4):
+        x = torch.randn(n, d, device="cuda").bfloat16()
+        y, work = torch.empty_like(x), torch.empty(2, n, d, dtype=x.dtype, device="cuda")
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            T.tardis_stack_forward(handles, x, y, work=work)
+        graph.replay()
+        torch.cuda.synchronize()
+        captured = y.clone()
+        T.tardis_stack_forward(handles, x, y, work=work)
+        torch.cuda.synchronize()
+        assert T.tardis_stats(handles[0])["last_path"] == 2
+        assert (captured.float() - y.float()).abs().max() <= 2e-2 * y.float().abs().max(), (d, G, n)
+        del graph
+    for h in handles:
+        T.tardis_destroy(h)
+"""
+    r = subprocess.run([sys.executable, "-c", script], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
+
+
 @pytest.mark.parametrize("d,dtype", [(16, "f32"), (1040, "f32"), (4096, "bf16"), (4160, "bf16"), (8256, "bf16")])
 def test_stack_normalisation_at_the_edges_of_its_vectors(d, dtype):
     # one, two and three vectors of 8 elements per thread of 512, the last ones partly beyond the row; x apart from y and in place

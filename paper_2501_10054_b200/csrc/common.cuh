@@ -154,8 +154,8 @@ __device__ __forceinline__ float gelu_f32(float z, int act) {
 // The tanh form without branches: (1 + tanh u) / 2 = 1 / (1 + e^-2u), with the exponential of -|2u|, so that what is rounded is small beside z.
 // (Against 64 bits, root mean square over [-1, 5]: 7.1e-8, of the form with tanhf 9.3e-8; over [-6, -1] 6e-9 against 2.9e-8.)
 __device__ __forceinline__ float gelu_tanh_f32(float z) {
-  const float e = __expf(-fabsf(z * fmaf(0.0713548162726f, z * z, 1.59576912161f)));
-  return 0.5f * (z + fabsf(z)) - __fdividef(fminf(fabsf(z), 3.0e38f) * e, 1.f + e);
+  const float e = __expf(-fabsf(z * fmaf(0.0713548162726f, z * z, 1.59576912161f))), half = 0.5f * z;
+  return (half + fabsf(half)) - __fdividef(fminf(fabsf(z), 3.0e38f) * e, 1.f + e);       // (halves first: twice z may be too large)
 }
 __device__ __forceinline__ double gelu_f64(double z, int act) {
   if (act == TARDIS_ACT_RELU) return z > 0.0 ? z : 0.0 * z;

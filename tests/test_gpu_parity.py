@@ -667,6 +667,22 @@ def test_fused_kernels_at_the_edges_of_their_rings(d, h, G, q):
     _run(cfg, sum(calls), calls, path=2)
 
 
+@pytest.mark.parametrize("n", [12, 60, 200])
+def test_corrections_of_the_largest_pre_activations_are_finite(n):
+    # beyond 2^127 twice a pre-activation is no float; with a bias of 2e38 and output weights of 2^-120 the neuron gives some 150 to every output
+    cfg = W.LayerConfig("largest", 256, 512, group=64, n_calib=256)
+    L = _layer(cfg, 4)
+    L.b1[5], L.a[5], L.W2[:, 5] = 2e38, 0.5, 2.0 ** -120
+    x = W.make_tokens(cfg, n, 4).cuda()
+    h = T.fold_layer(L)
+    try:
+        y, F, S = Hp.gpu_forward(h, L, x)
+        assert F[:, 5].all()
+        Hp.assert_parity(L, L.numpy64(), x, y, F, None, label="largest")
+    finally:
+        T.tardis_destroy(h)
+
+
 def test_first_call_of_a_process_may_be_a_chain_under_capture():
     # every kernel of a chain has to be loaded and to have its shared memory when the layers are set up: a process of its own, whose first
     # forward call is captured, and the shape of each of the four sets of kernels

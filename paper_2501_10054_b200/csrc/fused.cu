@@ -1291,6 +1291,7 @@ static cudaError_t give_shared_memory(int device, int set, const void* (&kernels
   for (const auto& of_tokens : kernels)
     for (const auto& forms : of_tokens)
       for (const void* kernel : forms) {
+        if (!kernel) continue;
         const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
         if (e != cudaSuccess) return e;
       }
@@ -1376,7 +1377,7 @@ tardis_status_t fused_prepare(Handle* H, cudaStream_t s) {
       const void* (&k)[3][2] = S->kernels[CH ? 1 : 0];
       k[0][0] = (const void*)k_fused<GG, CC, 1, false, CH>; k[0][1] = (const void*)k_fused<GG, CC, 1, true, CH>;
       k[1][0] = (const void*)k_fused<GG, CC, 2, false, CH>; k[1][1] = (const void*)k_fused<GG, CC, 2, true, CH>;
-      k[2][0] = k[2][1] = (const void*)k_fused<GG, CC, 4, false, CH>;
+      if constexpr (!CH || CC == 8) k[2][0] = k[2][1] = (const void*)k_fused<GG, CC, 4, false, CH>;      // (see fused_chain_serves)
     };
     both(std::false_type());
     both(std::true_type());

@@ -8,7 +8,7 @@
 // output.  Both take part in the programmatic hand-over between launches: they let the next launch start at once
 // (the fused decode kernel then loads its predictor blocks while the row is being normalised) and wait for the launch
 // before them only where they first touch its results.  Everything else is the per-layer forward.  Layers that are one launch of the
-// fused kernel (up to 4 tokens) need neither: see FusedChain.
+// fused kernel (one or two tokens, four on narrow layers) need neither: see FusedChain.
 #include "common.cuh"
 
 namespace tardis {

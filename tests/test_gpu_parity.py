@@ -747,7 +747,7 @@ def test_stack_normalisation_at_the_edges_of_its_vectors(d, dtype):
         T.tardis_destroy(h)
 
 
-@pytest.mark.parametrize("d,group,n", [(64, 64, 1), (320, 64, 2), (4096, 128, 1), (4096, 128, 4), (4544, 64, 2), (4608, 64, 3)])
+@pytest.mark.parametrize("d,group,n", [(64, 64, 1), (320, 64, 2), (1024, 128, 3), (1024, 64, 4), (4096, 128, 1), (4096, 128, 2), (4096, 128, 4), (4544, 64, 2), (4608, 64, 3)])
 @pytest.mark.parametrize("aligned", [True, False])
 def test_chain_normalised_inside_the_fused_kernel(d, group, n, aligned):
     # the row in less than one warp's vectors, in one vector per thread, several tokens' vectors per thread; tables that 16-byte loads can

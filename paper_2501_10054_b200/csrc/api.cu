@@ -174,12 +174,9 @@ static tardis_status_t settle(cudaStream_t s) {
   return TARDIS_OK;
 }
 
-// Whether a chain's layer of n tokens is one launch of the fused kernel.  Of the calls that tardis_ffn_forward gives to it as one launch those
-// of three and four tokens only on narrow layers: every CTA normalises all tokens, which there takes less than the small kernels between the
-// layers and wider less and less (three layers, us with the small kernels / inside: 2 tokens of 1024/4096 47.3 / 43.0, of 4544/18176 114.6 / 111.6; 4
-// tokens of 1024/4096 56.9 / 56.2, of 2048/8192 73.7 / 74.9, of 4544/18176 152 / 159).
+// Whether a chain's layer of n tokens is one launch of the fused kernel.
 bool fused_chain_serves(const Handle* H, int64_t n) {
-  return H->fscratch && n <= (H->d <= 1024 ? 4 : 2) && !H->deterministic && (H->path_override == 0 || H->path_override == 2);
+  return H->fscratch && n <= max_chain_tokens(H->d) && !H->deterministic && (H->path_override == 0 || H->path_override == 2);
 }
 
 // Allocates a handle and its device arrays for a layer of the given shape (nothing is filled in yet).

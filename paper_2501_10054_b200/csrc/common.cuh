@@ -100,6 +100,11 @@ struct FusedChain {
   __nv_bfloat16 *keep_in, *keep_out;
 };
 tardis_status_t launch_fused_forward(Handle* H, const void* x, void* y, int n, cudaStream_t s, const FusedChain* chain = nullptr);
+// Most tokens of a chain's layer that is one launch of the fused kernel.  Of the calls that tardis_ffn_forward gives to it as one launch those of
+// three and four tokens only on narrow layers: every CTA normalises all tokens, which there takes less than the small kernels between the
+// layers and wider less and less (three layers, us with the small kernels / inside: 2 tokens of 1024/4096 47.3 / 43.0, of 4544/18176 114.6 / 111.6; 4
+// tokens of 1024/4096 56.9 / 56.2, of 2048/8192 73.7 / 74.9, of 4544/18176 152 / 159).
+inline int max_chain_tokens(int d) { return d <= 1024 ? 4 : 2; }
 bool fused_chain_serves(const Handle* H, int64_t n);
 void fused_release(Handle* H);
 tardis_status_t fused_set_deterministic(Handle* H, bool on);               // allocates the partial-output buffer of the mode

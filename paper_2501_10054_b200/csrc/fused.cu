@@ -1280,23 +1280,23 @@ size_t fused_room(const Handle* H) {
          dev_room(16) + dev_room(sizeof(float) * MAXT * dacc) + dev_room(8192) + dev_room(sizeof(int) * H->h);
 }
 
-// All of a layer's kernels are given their shared memory when the layer is set up, so that no forward call, which may be under capture, is the
-// first to load one.  Loading them takes time that every layer would pay for again: done once per device and set of kernels.
-static cudaError_t give_shared_memory(int device, int set, const void* (&kernels)[2][3][2], int bytes) {
-  constexpr int kDevices = 64, kSets = 4;
+// The kernel for nt tokens of a call (chain: of a chain's layer).
+static const void* kernel_for(const Scratch* S, bool chain, int nt) {
+  const bool fast = S->pairs_fit && S->nbuf_n[nt] >= S->base.tiles_max;
+  return S->kernels[chain ? 1 : 0][nt <= 2 ? nt - 1 : 2][fast ? 1 : 0];
+}
+// The kernels that a layer's calls and chains come to are given their shared memory when the layer is set up, so that no forward call, which may
+// be under capture, is the first to load one.  Loading takes some 0.2 ms each, which the next layers would not pay for again, but the calls
+// for the attribute they would: once per device and kernel (`which`: the kernel's place among all).
+static cudaError_t give_shared_memory(int device, int which, const void* kernel, int bytes) {
+  constexpr int kDevices = 64, kKernels = 4 * 2 * 4;
   static std::mutex mutex;
-  static bool done[kDevices][kSets];
+  static const void* done[kDevices][kKernels];
   std::lock_guard<std::mutex> lock(mutex);
-  if (device < kDevices && done[device][set]) return cudaSuccess;
-  for (const auto& of_tokens : kernels)
-    for (const auto& forms : of_tokens)
-      for (const void* kernel : forms) {
-        if (!kernel) continue;
-        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        if (e != cudaSuccess) return e;
-      }
-  if (device < kDevices) done[device][set] = true;
-  return cudaSuccess;
+  if (device < kDevices && done[device][which] == kernel) return cudaSuccess;
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess && device < kDevices) done[device][which] = kernel;
+  return e;
 }
 
 tardis_status_t fused_prepare(Handle* H, cudaStream_t s) {
@@ -1387,7 +1387,6 @@ tardis_status_t fused_prepare(Handle* H, cudaStream_t s) {
   else if (G == 64) choose(integral_constant<int, 64>(), integral_constant<int, 8>());
   else if (wide) choose(integral_constant<int, 128>(), integral_constant<int, 9>());
   else choose(integral_constant<int, 128>(), integral_constant<int, 8>());
-  if (e == cudaSuccess) e = give_shared_memory(H->device, (G == 64 ? 2 : 0) + (wide ? 1 : 0), S->kernels, max_smem);
   S->pairs_fit = (p.nkc * 2 == NWP || (p.nkc * 2 >= 2 * NWP && p.nkc * 2 < 3 * NWP));
   if (e != cudaSuccess) { set_last_error(e, "fused_prepare launch"); return fail(TARDIS_ERR_CUDA); }
 
@@ -1395,6 +1394,11 @@ tardis_status_t fused_prepare(Handle* H, cudaStream_t s) {
   p.W1 = static_cast<const __nv_bfloat16*>(H->W1); p.W2T = static_cast<const __nv_bfloat16*>(H->W2T);
   p.Cp = S->Cp; p.bf = H->bf; p.lo = H->lo; p.hi = H->hi; p.a = H->a; p.c = H->c; p.b1 = H->b1;
   p.counters = H->counters;
+  for (int chain = 0; chain < 2 && e == cudaSuccess; ++chain)
+    for (int nt = 1; nt <= MAXT && e == cudaSuccess; ++nt)
+      if (const void* const kernel = chain && nt > max_chain_tokens(d) ? nullptr : kernel_for(S, chain, nt))
+        e = give_shared_memory(H->device, ((G == 64 ? 2 : 0) + (wide ? 1 : 0)) * 8 + chain * 4 + nt - 1, kernel, max_smem);
+  if (e != cudaSuccess) { set_last_error(e, "fused_prepare attributes"); return fail(TARDIS_ERR_CUDA); }
   H->fscratch = S;
   // beyond this many tokens the batched tensor-core path is faster (decode_7b: 208 against 212 us at 16 tokens, 245 against
   // 212 at 18; Falcon shape: 253 against 255 us at 13, 272 against 251 at 14)
@@ -1470,8 +1474,7 @@ tardis_status_t launch_fused_forward(Handle* H, const void* x, void* y, int n, c
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
     void* args[] = {&p};
-    const bool fast = S->pairs_fit && S->nbuf_n[nt] >= p.tiles_max;
-    TARDIS_CUDA_TRY(cudaLaunchKernelExC(&cfg, S->kernels[chain ? 1 : 0][nt <= 2 ? nt - 1 : 2][fast ? 1 : 0], args));
+    TARDIS_CUDA_TRY(cudaLaunchKernelExC(&cfg, kernel_for(S, chain != nullptr, nt), args));
     H->launches += 1;
     if (det) {
       const int work = nt * (H->d >> 2);                    // warps

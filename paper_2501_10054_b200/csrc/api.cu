@@ -71,7 +71,13 @@ size_t dev_room(size_t bytes) { return (bytes + 255) / 256 * 256 + 2 * kGuard; }
 
 void dev_reserve(size_t bytes) {
   cudaError_t e = cudaSuccess;
-  if (bytes && !g_block) g_block = new_block(bytes, &e);
+  if (!bytes || g_block) return;
+  // Large blocks in whole multiples of 64 MiB (at most 6 % more): one token of 8192/32768, rows from all over 2 GB, takes 71.2 us so wherever the
+  // block lies, and 71.2 or 72.4 by what was allocated before when its size is any (the kernel is the same).
+  constexpr size_t kLarge = size_t(1) << 30, kPiece = size_t(64) << 20;
+  if (bytes >= kLarge) g_block = new_block((bytes + kPiece - 1) / kPiece * kPiece, &e);
+  if (e != cudaSuccess) cudaGetLastError();
+  if (!g_block) g_block = new_block(bytes, &e);
   if (e != cudaSuccess) cudaGetLastError();                         // (the allocations are then made one by one)
 }
 

@@ -165,9 +165,9 @@ __device__ __forceinline__ void epilogue_chunk(const KParams& p, float (&v)[32],
         for (int i = 0; i < nv; ++i) v[i] += bias[i];
       }
     } else {   // GEMM_EPI_DELTA: one flag word covers this thread's 32 columns
-      // Only the flagged tenth of the elements needs the activation, at different columns in every row: the
-      // accumulators go to shared memory, each thread walks the set bits of its own word, and the corrections come
-      // back under the word's mask.
+      // Only the flagged tenth of the elements needs the activation, at different columns in every row.  The tanh form is evaluated for all of
+      // them; for the others the accumulators go to shared memory, each thread walks the set bits of its own word, and the corrections
+      // come back under the word's mask.
       uint32_t word = p.bitmap[size_t(m) * (p.N / 32) + (n >> 5)];
       if (nv < 32) word &= (1u << nv) - 1u;
       if (p.act == TARDIS_ACT_GELU_TANH) {
